@@ -81,6 +81,8 @@ struct SlotHost {
   float* out_stage = nullptr;
 };
 
+constexpr int kFuseSlots = 8;  // most slots of a workspace whose scalar steps are fused
+
 struct Workspace {
   std::string key;
   std::vector<SlotHost> slots;
@@ -98,6 +100,7 @@ struct Workspace {
   int n_sten = 0;
   int sten_ty = 32;             // stencil tile height of this workspace (autotuned)
   bool tuned = false;
+  bool fuse = false;            // scalar steps inside the update and stencil (few slots)
   WorkItem *d_l1 = nullptr, *d_l3 = nullptr;  // tiles of the low-mode products
   int n_l1 = 0, n_l3 = 0;
   // tensor-core problems (mixed modes): kMirClasses entries per slot, the slot's own descriptor
@@ -510,7 +513,8 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   d.sten_ty = 32;
   d.n_sten_tiles = d.n_st_tiles;
   const size_t N = (size_t)nx * ny;
-  d.n_vec_items = (int)((N + kVecChunk - 1) / kVecChunk);
+  d.vec_chunk = vec_chunk_of((long long)N);
+  d.n_vec_items = (int)((N + d.vec_chunk - 1) / d.vec_chunk);
   const int n_gm = (d.nxp / 128) * (d.nyp / 64);
   d.n_gm_tiles = n_gm;
   d.n_tc_tiles = n_gm;
@@ -930,6 +934,14 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   if (!rc) rc = upload(&W->d_prep, prep);
   if (rc) return rc;
   W->n_sten = W->n_st;
+  // Few slots: every block of the update and of the stencil forms the slot's scalars itself, which
+  // saves two launches an iteration (1024^2 solve: 334 -> 328 ms); with many slots, each met by
+  // every block in turn, the repeated sums cost as much as the launches.
+  W->fuse = count <= kFuseSlots;
+  for (const SlotHost& h : W->slots) {
+    const int pq_parts = ((h.d.ny + 15) / 16) * ((h.d.nx + kStTileX - 1) / kStTileX);
+    if (std::max(pq_parts, h.d.n_prec_parts) > kFuseParts) W->fuse = false;
+  }
   W->n_l1 = (int)l1.size();
   W->n_l3 = (int)l3.size();
   W->n_fold = (int)fold.size();
@@ -974,6 +986,7 @@ static int get_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bool
 static LaunchCfg cfg_of(ext_ctx* ctx, Workspace* W, int which) {
   LaunchCfg c;
   c.wait_cycles = ctx->opt.wait_cycles;
+  c.pdl = !ctx->opt.profile;  // a profiled kernel is bracketed by event records
   c.slots = W->d_slots;
   c.tcp = W->d_tcp;
   c.stream = W->stream ? W->stream : ctx->stream;
@@ -1078,7 +1091,8 @@ static void harvest(ext_ctx* ctx) {
   cudaGetLastError();
 }
 
-static void launch_prec(ext_ctx* ctx, Workspace* W, int mode) {
+// with_finish = false: the next stencil forms rho and beta from the partials itself
+static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish = true) {
   LaunchCfg g = cfg_of(ctx, W, 2);
   if (ctx->tc) {
     // residual slices: unfolded slots directly, folded slots per mirror class
@@ -1096,6 +1110,9 @@ static void launch_prec(ext_ctx* ctx, Workspace* W, int mode) {
       c1.slots = cm.slots = c3.slots = W->d_tcp;
       cm.grid = std::max(1, std::min(W->n_l3, ctx->sm_count * 8));  // the middle: small blocks
       timed(ctx, EXT_KERNEL_LOW_FWD, [&] { launch_low_tc(c1, 0, mode, ctx->split, ctx->d_err); }, g.stream);
+      // the middle starts on a free device: blocks placed as the forward product's leave would load
+      // the SMs unevenly (15 us more per application on a batch of 48 grids)
+      cm.pdl = false;
       timed(ctx, EXT_KERNEL_LOW_MID, [&] { launch_low_mid(cm, mode, ctx->split); }, g.stream);
       timed(ctx, EXT_KERNEL_LOW_INV, [&] { launch_low_tc(c3, 1, mode, ctx->split, ctx->d_err); }, g.stream);
     }
@@ -1104,6 +1121,7 @@ static void launch_prec(ext_ctx* ctx, Workspace* W, int mode) {
     // CUDA-core transforms over the transform problems: a folded slot's classes get their
     // residuals from the fold first
     g.slots = W->d_tcp;
+    g.pdl = false;  // measured slower with it (64^2 grid: 32.0 -> 32.6 ms a solve)
     if (W->n_unfold > 0)
       timed(ctx, EXT_KERNEL_FOLD, [&] { launch_simt_fold(cfg_of(ctx, W, 8), mode); }, g.stream);
   }
@@ -1115,6 +1133,7 @@ static void launch_prec(ext_ctx* ctx, Workspace* W, int mode) {
   }
   if (W->n_unfold > 0)
     timed(ctx, EXT_KERNEL_UNFOLD, [&] { launch_unfold(cfg_of(ctx, W, 8), mode); }, g.stream);
+  if (!with_finish) return;
   const LaunchCfg f = cfg_of(ctx, W, 3);  // one block per slot
   timed(ctx, EXT_KERNEL_PREC_FINISH, [&] { launch_prec_finish(f, mode); }, f.stream);
 }
@@ -1122,12 +1141,15 @@ static void launch_prec(ext_ctx* ctx, Workspace* W, int mode) {
 static void enqueue_iterations(ext_ctx* ctx, Workspace* W, int iters) {
   const LaunchCfg st = cfg_of(ctx, W, 0), vc = cfg_of(ctx, W, 1);
   const LaunchCfg sc = cfg_of(ctx, W, 4);
+  const bool fuse = W->fuse;
   for (int i = 0; i < iters; ++i) {
-    timed(ctx, EXT_KERNEL_STENCIL, [&] { launch_stencil(sc, W->aniso, W->sten_ty, ctx->d_err); }, st.stream);
+    // the first stencil follows a pass with its own finish (the tail's, or the first one)
+    const bool fz = fuse && i > 0;
+    timed(ctx, EXT_KERNEL_STENCIL, [&] { launch_stencil(sc, W->aniso, W->sten_ty, ctx->d_err, fz); }, st.stream);
     const LaunchCfg pf = cfg_of(ctx, W, 3);  // one block per slot
-    timed(ctx, EXT_KERNEL_PQ_FINISH, [&] { launch_pq_finish(pf); }, st.stream);
-    timed(ctx, EXT_KERNEL_UPDATE, [&] { launch_update(vc); }, st.stream);
-    launch_prec(ctx, W, 0);
+    if (!fuse) timed(ctx, EXT_KERNEL_PQ_FINISH, [&] { launch_pq_finish(pf); }, st.stream);
+    timed(ctx, EXT_KERNEL_UPDATE, [&] { launch_update(vc, fuse); }, st.stream);
+    launch_prec(ctx, W, 0, !fuse || i + 1 == iters);
   }
   timed(ctx, EXT_KERNEL_TRUE_RESIDUAL, [&] { launch_true_residual(st); }, st.stream);
   launch_prec(ctx, W, 1);
@@ -1984,11 +2006,11 @@ int ext_apply_biharmonic(ext_ctx* ctx, const ext_problem* prob, const float* phi
   BX_CUDA(cudaMemcpyAsync(sl.d.z, p, 4 * N, cudaMemcpyDeviceToDevice, s));
   BX_CUDA(cudaMemsetAsync(sl.d.z_lo, 0, 4 * N, s));
   const int it0 = 0, on = 1;
-  const double zero = 0.0;
+  const float zero[2] = {0.f, 0.f};
   char* dsc = reinterpret_cast<char*>(W->d_sc);
   BX_CUDA(cudaMemcpyAsync(dsc + offsetof(SlotScalars, it), &it0, sizeof(int), cudaMemcpyHostToDevice, s));
   BX_CUDA(cudaMemcpyAsync(dsc + offsetof(SlotScalars, active), &on, sizeof(int), cudaMemcpyHostToDevice, s));
-  BX_CUDA(cudaMemcpyAsync(dsc + offsetof(SlotScalars, beta), &zero, sizeof(double), cudaMemcpyHostToDevice, s));
+  BX_CUDA(cudaMemcpyAsync(dsc + offsetof(SlotScalars, beta_f), zero, sizeof(zero), cudaMemcpyHostToDevice, s));
   const LaunchCfg sc = cfg_of(ctx, W, 4);
   timed(ctx, EXT_KERNEL_STENCIL, [&] { launch_stencil(sc, W->aniso, W->sten_ty, ctx->d_err); });
   BX_CUDA(cudaGetLastError());

@@ -26,8 +26,16 @@ constexpr int kLowAutoSide = 2048;  // low_modes = 2: grids with a side of at le
 constexpr long long kLowAutoNodes = 2048LL * 2048;  // low_modes = 2: or calls with this many nodes
 constexpr int kLowNS = 6;           // integer slices per operand of the low-mode products
 constexpr int kLowK3 = 64;          // k extent of the inverse low-mode product (32 modes, zero-padded)
-constexpr int kVecChunk = 4096;     // elements per work item of the vector kernels
 constexpr int kVecThreads = 256;
+constexpr int kVecStep = 4 * kVecThreads;  // elements a block moves with one vector per thread
+// Elements per work item of the vector kernels (a function of the grid alone, so that the partial
+// sums do not depend on the call): one step up to 2^17 nodes and two up to 2^21 (more blocks at
+// once: the update of a 389 x 251 grid, 24 blocks of four steps before, went from about 13 to 7 us,
+// that of a 1024^2 grid from 14 to 12 us), four beyond (less per-item overhead: 43 us a launch on 48
+// grids of 5.1 M nodes against 61 with one step everywhere).
+constexpr int vec_chunk_of(long long nodes) {
+  return kVecStep * (nodes <= 1LL << 17 ? 1 : nodes <= 1LL << 21 ? 2 : 4);
+}
 
 enum Bc : int { BC_SYM = 0, BC_PER = 1, BC_DIR = 2 };
 
@@ -37,12 +45,13 @@ enum : int { ST_OK = 0, ST_RUNNING = 1, ST_ENOTCONV = -5, ST_EBREAKDOWN = -6 };
 // Per-slot scalars, FP64 where they feed CG.  Written only by the last work item of a slot.
 struct __align__(16) SlotScalars {
   double bb;        // ||b||^2
-  double rho;       // r.z of the current z
+  double rho2[2];   // r.z of the current z at [it & 1], of the previous iteration's at the other
   double pq;        // p.Ap of the current direction
   double zq;        // z_new.q_old (flexible beta)
   double rr;        // ||r||^2, recursive
   double rr_true;   // ||b - A xhat||^2 at the last replacement
   double alpha, beta;
+  float alpha_f[2], beta_f[2];  // the same as double-float pairs, for the kernels that apply them
   double rtol2;     // rtol^2
   double rr_ref;    // ||r||^2 at the last residual replacement
   double delta2;    // replace the residual once ||r||^2 < delta2 * rr_ref
@@ -57,7 +66,6 @@ struct __align__(16) SlotScalars {
   unsigned cnt[6];  // completion counters of the last-item reductions, one per kernel kind
   int n_known;      // known nodes, counted by the set-up kernel
   int bexp;         // the iteration solves A x' = 2^bexp b; the answer is x = 2^-bexp x'
-  double rho_prev;  // r.z of the previous iteration (Fletcher-Reeves beta)
   // error estimate: in CG, ||x* - x_k||_A^2 = sum_{j >= k} alpha_j rho_j, so the terms of the last
   // kErrDelay iterations over the sum of all terms estimate the relative A-norm error of the
   // iterate kErrDelay steps before the end (an upper estimate for the returned one)
@@ -74,7 +82,8 @@ struct SlotDesc {
   int n_st_tiles;    // grid tiles of the set-up, residual and slicing kernels: ceil(nx/64) * ceil(ny/32)
   int n_sten_tiles;  // tiles of the stencil kernel: ceil(nx/64) * ceil(ny/sten_ty)
   int sten_ty;       // the stencil kernel's tile height (16 or 32)
-  int n_vec_items;   // vector chunks: ceil(nx*ny / kVecChunk)
+  int vec_chunk;     // elements per vector work item
+  int n_vec_items;   // vector work items: ceil(nx*ny / vec_chunk)
   int n_gm_tiles;    // output tiles of one transform stage
   float wc, wex, wey, wd, wfx, wfy;  // stencil weights (hi), scaled so that max(a, c) = 1
   float wc_l, wex_l, wey_l, wd_l, wfx_l, wfy_l;  // low parts (anisotropic grids only)
@@ -160,6 +169,19 @@ struct WorkItem {
   int slot;
   int tile;   // tile / chunk index within the slot
 };
+
+// Programmatic dependent launch.  The kernels of an iteration follow one another at 2-10 us
+// each, so the launch gap between them counts: each is launched with programmatic serialization
+// and calls pdl_wait before it reads anything an earlier kernel wrote (the descriptors and work
+// lists it may read before: no kernel writes them).  griddepcontrol.wait returns once the previous
+// grid has completed and its writes are visible; only then does the block release the next grid
+// (launch_dependents), so that at most two grids of a stream are in flight and a grid's
+// completion implies that of every earlier one.  Every block of every such kernel makes the
+// call, whether or not it has work.  Without the launch attribute both instructions do nothing.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // ------------------------------------------------------------------------------------------
 // Reductions
@@ -296,25 +318,38 @@ struct CompDot {
   __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
 
-// Block sum of compensated per-thread accumulators: FP32 TwoSum reductions inside each warp,
-// FP64 only across the block's warps (thread 0).  Result valid in thread 0.  `sh` >= 32 doubles.
-template <int NT>
-__device__ __forceinline__ double block_sum_comp(CompDot d, double* sh) {
+// Compensated sum of (s, c) pairs over groups of W consecutive lanes in a fixed butterfly; every
+// lane of a group gets the group's pair.
+template <int W>
+__device__ __forceinline__ void group_sum_pair(float& s, float& c) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float s2 = __shfl_xor_sync(0xffffffffu, d.s, o);
-    const float c2 = __shfl_xor_sync(0xffffffffu, d.c, o);
+  for (int o = W / 2; o > 0; o >>= 1) {
+    const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
+    const float c2 = __shfl_xor_sync(0xffffffffu, c, o);
     float e;
-    two_sum(d.s, s2, d.s, e);
-    d.c = __fadd_rn(d.c, __fadd_rn(c2, e));
+    two_sum(s, s2, s, e);
+    c = __fadd_rn(c, __fadd_rn(c2, e));
   }
+}
+
+// Block sum of compensated per-thread accumulators by FP32 TwoSum butterflies, inside the warps
+// and then across them; FP64 only for the result.  The SM adds two FP64 numbers a cycle (a warp
+// instruction takes 16), so FP64 stays out of every step that each warp would repeat.  Result
+// valid in thread 0.  `sh` >= NT / 32 float2.
+template <int NT>
+__device__ __forceinline__ double block_sum_comp(CompDot d, float2* sh) {
+  static_assert(NT / 32 == 8, "eight warps");
+  group_sum_pair<32>(d.s, d.c);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) sh[w] = d.value();
+  if (l == 0) sh[w] = make_float2(d.s, d.c);
   __syncthreads();
   double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < NT / 32; ++k) t += sh[k];
+  if (w == 0) {
+    const float2 v = sh[l & 7];
+    float s = v.x, c = v.y;
+    group_sum_pair<8>(s, c);
+    if (l == 0) t = (double)s + (double)c;
+  }
   return t;
 }
 
@@ -459,23 +494,88 @@ __device__ __forceinline__ float spectral_weight(const SlotDesc& S, int kx, int 
   return spectral_weight_of(S.wnorm, s);
 }
 
-// Last item of stage 3 (thread 0): r.z, z.q -> rho, beta (flexible or Fletcher-Reeves).
+// The per-slot scalar steps.  Each is computed either by one block per slot in a launch of its own
+// (k_pq_finish, k_prec_finish) or, for workspaces of few slots, by every block of the kernel that
+// needs the result (the update and the next stencil), from the same partial sums in the same
+// order, so both give the same bits; then only the block of the slot's tile 0 writes the scalars,
+// and none of the fields it writes is read by the other blocks of that kernel.
+constexpr int kFuseParts = 2048;  // most partial sums a consumer kernel adds up itself
+
+// Sum of p[i * stride], i < n, by the calling warp: lane l adds i = l, l + 32, ... on four chains, the
+// lanes in a fixed butterfly; the order depends on n alone.  Every lane gets the sum.  One warp: the
+// FP64 pipe (two lanes a cycle and SM) is the limit, so more warps would only add butterflies.
+__device__ __forceinline__ double warp_sum_strided(const double* p, int n, int stride) {
+  const int l = threadIdx.x & 31;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  int i = l;
+  for (; i + 96 < n; i += 128) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] += __ldcg(p + (size_t)(i + 32 * k) * stride);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    if (i + 32 * k < n) a[k] += __ldcg(p + (size_t)(i + 32 * k) * stride);
+  return warp_sum((a[0] + a[1]) + (a[2] + a[3]));
+}
+// One warp: the sum of the slot's p.q partials.
+__device__ __forceinline__ double sum_pq(const SlotDesc& S) {
+  return warp_sum_strided(S.pq_part, ((S.ny + 15) >> 4) * ((S.nx + kStTileX - 1) / kStTileX), 1);
+}
+// One warp: the sums of the slot's r.z and (for the flexible beta and mode 2) z.q partials.
+__device__ __forceinline__ void sum_rz(const SlotDesc& S, bool with_zq, double& rz, double& zq) {
+  rz = warp_sum_strided(S.part + 2, S.n_prec_parts, 4);
+  zq = with_zq ? warp_sum_strided(S.part + 3, S.n_prec_parts, 4) : 0.0;
+}
+
+// alpha = rho / p.q is usable (p.q > 0, everything finite)
+__device__ __forceinline__ bool pq_ok(const SlotScalars* sc, double pq) {
+  return pq > 0.0 && isfinite(pq) && isfinite(sc->rho2[sc->it & 1]);
+}
+// One thread: record p.q and alpha, or the breakdown.
+__device__ __forceinline__ void finish_pq(SlotScalars* sc, double pq) {
+  sc->pq = pq;
+  if (!pq_ok(sc, pq)) {
+    sc->status = ST_EBREAKDOWN;
+    sc->active = 0;
+    sc->fold = 1;  // the tail replaces the residual and reports the best iterate
+    return;
+  }
+  const double rho = sc->rho2[sc->it & 1];
+  sc->alpha = rho / pq;
+  const f2 af = df_of(sc->alpha);
+  sc->alpha_f[0] = af.hi;
+  sc->alpha_f[1] = af.lo;
+  const double aro = sc->alpha * rho;
+  sc->aro_total += aro;
+  sc->aro_ring[sc->aro_n % kErrDelay] = aro;
+  sc->aro_n += 1;
+}
+
+// beta of the next direction (flexible or Fletcher-Reeves); 0 before the first iteration.
+__device__ __forceinline__ double prec_beta(const SlotScalars* sc, double rz, double zq) {
+  if (sc->it == 0) return 0.0;
+  return sc->flexible ? -zq / sc->pq : rz / sc->rho2[(sc->it & 1) ^ 1];
+}
+__device__ __forceinline__ void record_preconditioner(SlotScalars* sc, double rz, double zq, double beta) {
+  sc->zq = zq;
+  sc->rho2[sc->it & 1] = rz;
+  sc->beta = beta;
+  const f2 bf = df_of(beta);
+  sc->beta_f[0] = bf.hi;
+  sc->beta_f[1] = bf.lo;
+}
+// One thread: record rho and beta, or the breakdown.  Mode 1 (the pass after a residual
+// replacement) recomputes them for the same iteration.
 __device__ __forceinline__ void finish_preconditioner(const SlotDesc& S, double rz, double zq,
                                                       int mode) {
   SlotScalars* sc = S.sc;
   if (mode == 2) {
-    sc->rho = rz;
+    sc->rho2[0] = rz;
     sc->zq = zq;
     return;
   }
-  // Mode 1 recomputes, after a residual replacement, the beta of the iteration whose mode-0
-  // pass already ran: its Fletcher-Reeves denominator is the r.z from before that pass.
-  if (mode == 0) sc->rho_prev = sc->rho;
-  double beta = 0.0;
-  if (sc->it > 0) beta = sc->flexible ? -zq / sc->pq : rz / sc->rho_prev;
-  sc->rho = rz;
-  sc->zq = zq;
-  sc->beta = beta;
+  const double beta = prec_beta(sc, rz, zq);
+  record_preconditioner(sc, rz, zq, beta);
   if (!isfinite(rz) || !isfinite(beta)) {
     sc->status = ST_EBREAKDOWN;
     sc->active = 0;

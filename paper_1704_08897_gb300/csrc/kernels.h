@@ -20,7 +20,27 @@ struct LaunchCfg {
   int grid;
   cudaStream_t stream;
   long long wait_cycles = 0;  // bound of the kernels' pipeline waits (0: the default bound)
+  // programmatic dependent launch: the grid may start its prologue while the stream's previous
+  // kernel still runs (every kernel launched this way begins its reads with pdl_wait)
+  bool pdl = false;
 };
+
+// Launch `kernel` under `c` (its stream and dependence form).
+template <class... KArgs, class... Args>
+inline void launch_cfg(const LaunchCfg& c, void (*kernel)(KArgs...), int grid, int threads, size_t smem,
+                       Args... args) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((unsigned)grid);
+  lc.blockDim = dim3((unsigned)threads);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = c.stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = c.pdl ? 1 : 0;
+  cudaLaunchKernelEx(&lc, kernel, KArgs(args)...);
+}
 
 // host helpers (api.cu): stencil weights of (L_y (+) L_x)^2 for spacings hx, hy; the problem
 // checks every entry point applies (EXT_OK or EXT_EINVAL); whether a pointer is device (or
@@ -34,13 +54,15 @@ void launch_setup(const LaunchCfg& c, const float* const* phis, const float* con
                   const int* dirs);
 void launch_rhs_scale(const LaunchCfg& c);
 // err receives 1 if a bounded wait for a tensor copy ran out; tile_y = 16 or 32 (tiles 64 wide)
-void launch_stencil(const LaunchCfg& c, bool aniso, int tile_y, int* err);
+// fuse_prec: the blocks form rho and beta from the preconditioner's partials themselves
+void launch_stencil(const LaunchCfg& c, bool aniso, int tile_y, int* err, bool fuse_prec = false);
 int stencil_blocks_per_sm(int tile_y);
 // shared-memory carveout of the stencil kernels (once per process and device)
 cudaError_t stencil_init();
 // per-slot p.q -> alpha (after the stencil)
 void launch_pq_finish(const LaunchCfg& c);
-void launch_update(const LaunchCfg& c);
+// fuse_pq: the blocks form alpha from the stencil's partials themselves
+void launch_update(const LaunchCfg& c, bool fuse_pq = false);
 void launch_true_residual(const LaunchCfg& c);
 void launch_output(const LaunchCfg& c, const float* const* fs, float* const* outs);
 void launch_output64(const SlotDesc* slot, int n, const float* f, double* out, cudaStream_t s);

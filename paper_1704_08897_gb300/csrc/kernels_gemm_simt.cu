@@ -72,6 +72,7 @@ k_prec_simt(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ ite
   const int arow = t >> 1, acol = (t & 1) * 4;  // A tile 128 x 8: 4 per thread and plane
   const int brow = t >> 2, bcol = (t & 3) * 2;  // B tile  64 x 8: 2 per thread and plane
   const int total = *n_items;
+  pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
     const WorkItem item = items[w];
     const SlotDesc& S = slots[item.slot];
@@ -230,6 +231,7 @@ __global__ void __launch_bounds__(256)
 k_simt_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
             const WorkItem* __restrict__ items, const int* __restrict__ n_items, int mode) {
   const int total = *n_items;
+  pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
     const WorkItem it = items[w];
@@ -265,15 +267,15 @@ k_simt_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp
 }
 
 void launch_simt_fold(const LaunchCfg& c, int mode) {
-  k_simt_fold<<<c.grid, 256, 0, c.stream>>>(c.slots, c.tcp, c.items, c.n_items, mode);
+  launch_cfg(c, k_simt_fold, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
 }
 
 void launch_prec_simt(const LaunchCfg& c, int stage, int mode) {
   switch (stage) {
-    case 0: k_prec_simt<0><<<c.grid, NT, 0, c.stream>>>(c.slots, c.items, c.n_items, mode); break;
-    case 1: k_prec_simt<1><<<c.grid, NT, 0, c.stream>>>(c.slots, c.items, c.n_items, mode); break;
-    case 2: k_prec_simt<2><<<c.grid, NT, 0, c.stream>>>(c.slots, c.items, c.n_items, mode); break;
-    default: k_prec_simt<3><<<c.grid, NT, 0, c.stream>>>(c.slots, c.items, c.n_items, mode); break;
+    case 0: launch_cfg(c, k_prec_simt<0>, c.grid, NT, 0, c.slots, c.items, c.n_items, mode); break;
+    case 1: launch_cfg(c, k_prec_simt<1>, c.grid, NT, 0, c.slots, c.items, c.n_items, mode); break;
+    case 2: launch_cfg(c, k_prec_simt<2>, c.grid, NT, 0, c.slots, c.items, c.n_items, mode); break;
+    default: launch_cfg(c, k_prec_simt<3>, c.grid, NT, 0, c.slots, c.items, c.n_items, mode); break;
   }
 }
 

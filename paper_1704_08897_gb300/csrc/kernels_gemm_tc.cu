@@ -287,6 +287,7 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem;
+  pdl_wait();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -713,6 +714,7 @@ k_tc_prepare(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ it
              const int* __restrict__ n_items, int mode) {
   const int total = *n_items;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
     const WorkItem it = items[w];
     const SlotDesc& S = slots[it.slot];
@@ -795,6 +797,7 @@ k_tc_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
           const WorkItem* __restrict__ items, const int* __restrict__ n_items, int mode) {
   const int total = *n_items;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
     const WorkItem it = items[w];
     const SlotDesc& S = slots[it.slot];
@@ -887,9 +890,10 @@ k_tc_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
 __global__ void __launch_bounds__(256)
 k_unfold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
          const WorkItem* __restrict__ items, const int* __restrict__ n_items, int mode) {
-  __shared__ float red[8][4];
+  __shared__ float4 red[8];
   const int total = *n_items;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
     const WorkItem it = items[w];
     const SlotDesc& S = slots[it.slot];
@@ -945,34 +949,20 @@ k_unfold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
         if (with_zq) c_zq.add(zh, zl, qh[t], ql[t]);
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      float e;
-      const float a1 = __shfl_xor_sync(0xffffffffu, c_rz.s, o), a2 = __shfl_xor_sync(0xffffffffu, c_rz.c, o);
-      two_sum(c_rz.s, a1, c_rz.s, e);
-      c_rz.c = __fadd_rn(c_rz.c, __fadd_rn(a2, e));
-      const float b1 = __shfl_xor_sync(0xffffffffu, c_zq.s, o), b2 = __shfl_xor_sync(0xffffffffu, c_zq.c, o);
-      two_sum(c_zq.s, b1, c_zq.s, e);
-      c_zq.c = __fadd_rn(c_zq.c, __fadd_rn(b2, e));
-    }
-    if (lane == 0) {
-      red[warp][0] = c_rz.s;
-      red[warp][1] = c_rz.c;
-      red[warp][2] = c_zq.s;
-      red[warp][3] = c_zq.c;
-    }
+    // the tile's sums: butterflies inside the warps and, by warp 0, across the eight
+    group_sum_pair<32>(c_rz.s, c_rz.c);
+    if (with_zq) group_sum_pair<32>(c_zq.s, c_zq.c);
+    if (lane == 0) red[warp] = make_float4(c_rz.s, c_rz.c, c_zq.s, c_zq.c);
     __syncthreads();
-    if (threadIdx.x == 0) {
-      CompDot t_rz, t_zq;
-      for (int k = 0; k < 8; ++k) {  // the warps in order
-        float e;
-        two_sum(t_rz.s, red[k][0], t_rz.s, e);
-        t_rz.c = __fadd_rn(t_rz.c, __fadd_rn(red[k][1], e));
-        two_sum(t_zq.s, red[k][2], t_zq.s, e);
-        t_zq.c = __fadd_rn(t_zq.c, __fadd_rn(red[k][3], e));
+    if (warp == 0) {
+      const float4 v = red[lane & 7];
+      float sv = v.x, cv = v.y, sq = v.z, cq = v.w;
+      group_sum_pair<8>(sv, cv);
+      if (with_zq) group_sum_pair<8>(sq, cq);
+      if (lane == 0) {
+        S.part[it.tile * 4 + 2] = (double)sv + (double)cv;
+        S.part[it.tile * 4 + 3] = with_zq ? (double)sq + (double)cq : 0.0;
       }
-      S.part[it.tile * 4 + 2] = t_rz.value();
-      S.part[it.tile * 4 + 3] = t_zq.value();
     }
     __syncthreads();
   }
@@ -1058,6 +1048,7 @@ k_low_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem;
+  pdl_wait();
   uint32_t ph_full = 0, ph_done = 0;
   int inflight = 0;     // thread 0: tensor copies issued and not yet waited for (0 or 1)
   int mma_pending = 0;  // thread 0: MMAs committed and not yet waited for (0 or 1)
@@ -1284,6 +1275,7 @@ k_low_inv(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem;
+  pdl_wait();
   // thread 0's barrier bookkeeping: phases and the waits still owed
   uint32_t ph_fa = 0, ph_fb[2] = {0, 0}, ph_md[2] = {0, 0};
   int owe_fa = 0, owe_fb[2] = {0, 0}, owe_md[2] = {0, 0};
@@ -1457,6 +1449,7 @@ k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   __shared__ __align__(16) float qs[2][kLowM][kQsStride];  // Qx_low rows of the block: hi, lo
   const int total = *n_items;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
     const WorkItem it = items[w];
     const SlotDesc& S = slots[it.slot];
@@ -1529,10 +1522,10 @@ template <bool BF16>
 void launch_all(const LaunchCfg& c, int stage, int mode, int* err) {
   const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
   switch (stage) {
-    case 0: k_prec_tc<BF16, 0><<<c.grid, kThreads, SMEM_BYTES, c.stream>>>(c.slots, c.items, c.n_items, mode, err, wc); break;
-    case 1: k_prec_tc<BF16, 1><<<c.grid, kThreads, SMEM_BYTES, c.stream>>>(c.slots, c.items, c.n_items, mode, err, wc); break;
-    case 2: k_prec_tc<BF16, 2><<<c.grid, kThreads, SMEM_BYTES, c.stream>>>(c.slots, c.items, c.n_items, mode, err, wc); break;
-    default: k_prec_tc<BF16, 3><<<c.grid, kThreads, SMEM_BYTES, c.stream>>>(c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 0: launch_cfg(c, k_prec_tc<BF16, 0>, c.grid, kThreads, SMEM_BYTES, c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 1: launch_cfg(c, k_prec_tc<BF16, 1>, c.grid, kThreads, SMEM_BYTES, c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 2: launch_cfg(c, k_prec_tc<BF16, 2>, c.grid, kThreads, SMEM_BYTES, c.slots, c.items, c.n_items, mode, err, wc); break;
+    default: launch_cfg(c, k_prec_tc<BF16, 3>, c.grid, kThreads, SMEM_BYTES, c.slots, c.items, c.n_items, mode, err, wc); break;
   }
 }
 
@@ -1582,26 +1575,26 @@ cudaError_t tc_init() {
 void launch_low_tc(const LaunchCfg& c, int kind, int mode, int split_kind, int* err) {
   const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
   if (split_kind == 0) {
-    if (kind == 0) k_low_tc<false><<<c.grid, kLowThreads, kLowSmem, c.stream>>>(c.slots, c.items, c.n_items, mode, err, wc);
-    else k_low_inv<false><<<c.grid, kLowInvThreads, kLowInvSmem, c.stream>>>(c.slots, c.items, c.n_items, mode, err, wc);
+    if (kind == 0) launch_cfg(c, k_low_tc<false>, c.grid, kLowThreads, kLowSmem, c.slots, c.items, c.n_items, mode, err, wc);
+    else launch_cfg(c, k_low_inv<false>, c.grid, kLowInvThreads, kLowInvSmem, c.slots, c.items, c.n_items, mode, err, wc);
   } else {
-    if (kind == 0) k_low_tc<true><<<c.grid, kLowThreads, kLowSmem, c.stream>>>(c.slots, c.items, c.n_items, mode, err, wc);
-    else k_low_inv<true><<<c.grid, kLowInvThreads, kLowInvSmem, c.stream>>>(c.slots, c.items, c.n_items, mode, err, wc);
+    if (kind == 0) launch_cfg(c, k_low_tc<true>, c.grid, kLowThreads, kLowSmem, c.slots, c.items, c.n_items, mode, err, wc);
+    else launch_cfg(c, k_low_inv<true>, c.grid, kLowInvThreads, kLowInvSmem, c.slots, c.items, c.n_items, mode, err, wc);
   }
 }
 
 void launch_low_mid(const LaunchCfg& c, int mode, int split_kind) {
-  if (split_kind == 0) k_low_mid<false><<<c.grid, 256, 0, c.stream>>>(c.slots, c.items, c.n_items, mode);
-  else k_low_mid<true><<<c.grid, 256, 0, c.stream>>>(c.slots, c.items, c.n_items, mode);
+  if (split_kind == 0) launch_cfg(c, k_low_mid<false>, c.grid, 256, 0, c.slots, c.items, c.n_items, mode);
+  else launch_cfg(c, k_low_mid<true>, c.grid, 256, 0, c.slots, c.items, c.n_items, mode);
 }
 
 void launch_tc_fold(const LaunchCfg& c, int mode, int split_kind) {
-  if (split_kind == 0) k_tc_fold<false><<<c.grid, 256, 0, c.stream>>>(c.slots, c.tcp, c.items, c.n_items, mode);
-  else k_tc_fold<true><<<c.grid, 256, 0, c.stream>>>(c.slots, c.tcp, c.items, c.n_items, mode);
+  if (split_kind == 0) launch_cfg(c, k_tc_fold<false>, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
+  else launch_cfg(c, k_tc_fold<true>, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
 }
 
 void launch_unfold(const LaunchCfg& c, int mode) {
-  k_unfold<<<c.grid, 256, 0, c.stream>>>(c.slots, c.tcp, c.items, c.n_items, mode);
+  launch_cfg(c, k_unfold, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
 }
 
 void launch_prec_tc(const LaunchCfg& c, int stage, int mode, int split_kind, int* err) {
@@ -1610,8 +1603,8 @@ void launch_prec_tc(const LaunchCfg& c, int stage, int mode, int split_kind, int
 }
 
 void launch_prec_tc_prepare(const LaunchCfg& c, int mode, int split_kind) {
-  if (split_kind == 0) k_tc_prepare<false><<<c.grid, 256, 0, c.stream>>>(c.slots, c.items, c.n_items, mode);
-  else k_tc_prepare<true><<<c.grid, 256, 0, c.stream>>>(c.slots, c.items, c.n_items, mode);
+  if (split_kind == 0) launch_cfg(c, k_tc_prepare<false>, c.grid, 256, 0, c.slots, c.items, c.n_items, mode);
+  else launch_cfg(c, k_tc_prepare<true>, c.grid, 256, 0, c.slots, c.items, c.n_items, mode);
 }
 
 }  // namespace bx

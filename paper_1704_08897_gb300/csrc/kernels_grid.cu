@@ -223,8 +223,9 @@ k_setup(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
         sc->rr = sbs;
         sc->rr_true = sbs;
         sc->rr_ref = sbs;
-        sc->rho = 0.0;
+        sc->rho2[0] = sc->rho2[1] = 0.0;
         sc->beta = 0.0;
+        sc->beta_f[0] = sc->beta_f[1] = 0.f;
         sc->alpha = 0.0;
         sc->it = 0;
         sc->fold = 0;
@@ -393,22 +394,7 @@ __device__ __forceinline__ void stencil_issue_next(const SlotDesc* __restrict__ 
   }
 }
 
-// Compensated sum of (s, c) pairs over the lanes of groups of W consecutive lanes (W = 16 or 32),
-// in a fixed butterfly; the group's total (as FP64) is valid in every lane of the group.
-template <int W>
-__device__ __forceinline__ double group_sum_comp(float s, float c) {
-#pragma unroll
-  for (int o = W / 2; o > 0; o >>= 1) {
-    const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
-    const float c2 = __shfl_xor_sync(0xffffffffu, c, o);
-    float e;
-    two_sum(s, s2, s, e);
-    c = __fadd_rn(c, __fadd_rn(c2, e));
-  }
-  return (double)s + (double)c;
-}
-
-template <bool ANISO, int TY>
+template <bool ANISO, int TY, bool FUSE>
 __global__ void __launch_bounds__(kStThreads, StGeom<TY>::kBlocksPerSm)
 k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
           const int* __restrict__ n_items, int* __restrict__ err, long long wait_cycles) {
@@ -418,7 +404,10 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
       (reinterpret_cast<uintptr_t>(st_smem_raw) + 127) & ~static_cast<uintptr_t>(127));
   __shared__ __align__(8) uint64_t full[2];
   __shared__ int s_abort;
-  __shared__ double blk_sm[TY / 16][kStThreads / 32];  // p.q of each warp in each 16-row block
+  __shared__ float2 blk_sm[TY / 16][kStThreads / 32];  // p.q of each warp in each 16-row block
+  __shared__ float2 s_beta;                            // FUSE: beta of slot beta_slot
+  int beta_slot = -1;
+  f2 beta_fused = {0.f, 0.f};
   const int total = *n_items;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -429,6 +418,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
+  pdl_wait();
   volatile int* abort_flag = &s_abort;
   int w_issue = blockIdx.x, n_issued = 0;  // thread 0: the tensor-copy cursor
   int n_used = 0;                          // copied windows consumed (uniform over the block)
@@ -438,7 +428,24 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     const SlotDesc& S = slots[it.slot];
     SlotScalars* sc = S.sc;
     if (!sc->active) continue;
-    const f2 beta = df_of(sc->beta);
+    if (FUSE && it.slot != beta_slot) {
+      // r.z, z.q -> beta in this block; the tile-0 block records the scalars.  A breakdown (a
+      // non-finite r.z or beta) reaches p.q and rho, where the update finds it.
+      if (threadIdx.x < 32) {
+        double rz, zq;
+        sum_rz(S, sc->flexible != 0, rz, zq);
+        if (threadIdx.x == 0) {
+          const double b = prec_beta(sc, rz, zq);
+          const f2 bf = df_of(b);
+          s_beta = make_float2(bf.hi, bf.lo);
+          if (it.tile == 0) record_preconditioner(sc, rz, zq, b);
+        }
+      }
+      __syncthreads();
+      beta_fused = f2{s_beta.x, s_beta.y};
+      beta_slot = it.slot;
+    }
+    const f2 beta = FUSE ? beta_fused : f2{sc->beta_f[0], sc->beta_f[1]};
     const int par = sc->it & 1;
     const float* __restrict__ pold = S.p[par];
     const float* __restrict__ pold_lo = S.p_lo[par];
@@ -609,8 +616,8 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
           }
         }
         if (j & 1) {  // the end of a 16-row block: every lane joins the butterfly
-          const double blk = group_sum_comp<32>(dot.s, dot.c);
-          if (lane == 0) blk_sm[j >> 1][threadIdx.x >> 5] = blk;
+          group_sum_pair<32>(dot.s, dot.c);
+          if (lane == 0) blk_sm[j >> 1][threadIdx.x >> 5] = make_float2(dot.s, dot.c);
           dot = CompDotDF{};
         }
       }
@@ -638,8 +645,8 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
           dot.add(pvh, pvl, qv.hi, qv.lo);
         }
         if ((j & 3) == 3) {
-          const double blk = group_sum_comp<32>(dot.s, dot.c);
-          if (lane == 0) blk_sm[j >> 2][threadIdx.x >> 5] = blk;
+          group_sum_pair<32>(dot.s, dot.c);
+          if (lane == 0) blk_sm[j >> 2][threadIdx.x >> 5] = make_float2(dot.s, dot.c);
           dot = CompDotDF{};
         }
       }
@@ -647,12 +654,14 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     __syncthreads();  // the window set is free for the copies started at the next copied tile
     // the 16-row blocks of the tile (TY / 16 of them, so the partials do not depend on TY); the
     // next tile writes blk_sm only after its own block barriers, which these threads join later
-    if (threadIdx.x < TY / 16) {
-      const int by = (y0 >> 4) + threadIdx.x;
-      double acc = 0.0;
-#pragma unroll
-      for (int w = 0; w < kStThreads / 32; ++w) acc += blk_sm[threadIdx.x][w];
-      if (16 * by < S.ny) S.pq_part[by * nbx + x0 / kStTileX] = acc;
+    if (threadIdx.x < 32) {
+      const int j = (lane >> 3) & (TY / 16 - 1);  // eight lanes per block, one per warp's pair
+      const float2 v = blk_sm[j][lane & 7];
+      float sv = v.x, cv = v.y;
+      group_sum_pair<8>(sv, cv);
+      const int by = (y0 >> 4) + j;
+      if ((lane & 7) == 0 && lane < TY / 2 && 16 * by < S.ny)
+        S.pq_part[by * nbx + x0 / kStTileX] = (double)sv + (double)cv;
     }
   }
   if (threadIdx.x == 0) {
@@ -668,106 +677,107 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
 
 // One block per slot (the slot's tile-0 item of the per-slot list): p.q from the stencil's
 // block partials (64 x 16 nodes) in a fixed order, alpha = rho / p.q, breakdown detection.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(32)
 k_pq_finish(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
             const int* __restrict__ n_items) {
-  __shared__ double red[64];
   const int total = *n_items;
+  pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
-    const WorkItem it = items[w];
-    if (it.tile != 0) continue;
-    const SlotDesc& S = slots[it.slot];
-    SlotScalars* sc = S.sc;
-    if (!sc->active) continue;
-    double a = 0.0, b = 0.0;
-    const int nparts = ((S.ny + 15) >> 4) * ((S.nx + kStTileX - 1) / kStTileX);
-    for (int t = threadIdx.x; t < nparts; t += blockDim.x) a += __ldcg(&S.pq_part[t]);
-    block_sum2<256>(a, b, red);
-    if (threadIdx.x == 0) {
-      sc->pq = a;
-      if (!(a > 0.0) || !isfinite(a) || !isfinite(sc->rho)) {
-        sc->status = ST_EBREAKDOWN;
-        sc->active = 0;
-        sc->fold = 1;  // the tail replaces the residual and reports the best iterate
-      } else {
-        sc->alpha = sc->rho / a;
-        const double aro = sc->alpha * sc->rho;
-        sc->aro_total += aro;
-        sc->aro_ring[sc->aro_n % kErrDelay] = aro;
-        sc->aro_n += 1;
-      }
-    }
-    __syncthreads();
+    const SlotDesc& S = slots[items[w].slot];
+    if (!S.sc->active) continue;
+    const double pq = sum_pq(S);
+    __syncwarp();  // every lane has read `active`
+    if (threadIdx.x == 0) finish_pq(S.sc, pq);
   }
 }
 
 // ---------------------------------------------------------------------------------------------
 // Iteration, stage 2: x += alpha p, r -= alpha q (all double-float), partial ||r||^2.  The last
-// item advances the iteration count and decides stop / residual replacement.  Each thread moves
-// 16-byte vectors (4 elements per access) of every plane; all loads are issued before any
-// arithmetic.
+// item advances the iteration count and decides stop / residual replacement.  Bound by HBM on large
+// batches (48 B a node; 43 us on 5.1 M nodes, 84% of the measured copy rate) and by the chain of
+// dependent loads and reductions on one grid.  Each thread moves one 16-byte vector of every plane
+// per step, four blocks per SM (64 registers): 128 KB of loads in flight per SM.  alpha arrives as
+// a double-float pair: an FP64 division or conversion repeated by every thread costs more than a
+// step's loads.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kVecThreads)
+template <bool FUSE>
+__global__ void __launch_bounds__(kVecThreads, 4)
 k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
          const int* __restrict__ n_items) {
-  __shared__ double red[64];
-  __shared__ int s_last;
+  __shared__ float2 red[kVecThreads / 32];
+  __shared__ float2 s_alpha;  // FUSE: alpha of slot pq_slot, and whether the slot runs
+  __shared__ int s_run, s_last;
+  int pq_slot = -1;
+  f2 alpha = {0.f, 0.f};
+  bool run = false;
   const int total = *n_items;
+  pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
     const WorkItem it = items[w];
     const SlotDesc& S = slots[it.slot];
     SlotScalars* sc = S.sc;
-    if (!sc->active) continue;
-    const f2 alpha = df_of(sc->alpha);
+    if (FUSE) {
+      if (it.slot != pq_slot) {
+        if (threadIdx.x < 32) {
+          const bool act = sc->active != 0;  // one reading for the whole block
+          const double pq = sum_pq(S);
+          if (threadIdx.x == 0) {
+            const bool ok = act && pq_ok(sc, pq);
+            const f2 af = ok ? df_of(sc->rho2[sc->it & 1] / pq) : f2{0.f, 0.f};
+            s_alpha = make_float2(af.hi, af.lo);
+            s_run = ok;
+            if (act && it.tile == 0) finish_pq(sc, pq);
+          }
+        }
+        __syncthreads();
+        alpha = f2{s_alpha.x, s_alpha.y};
+        run = s_run != 0;
+        pq_slot = it.slot;
+        __syncthreads();  // s_alpha and s_run are written again for the next slot
+      }
+      // a breakdown: every block finds the same one, the tile-0 block records it
+      if (!run) continue;
+    } else {
+      if (!sc->active) continue;
+      alpha = f2{sc->alpha_f[0], sc->alpha_f[1]};
+    }
     const f2 nalpha = {-alpha.hi, -alpha.lo};
     const int pi = (sc->it & 1) ^ 1;
     const float* __restrict__ p = S.p[pi];
     const float* __restrict__ p_lo = S.p_lo[pi];
     const int n = S.nx * S.ny;
-    const int e0 = it.tile * kVecChunk;
-    const int e1 = min(n, e0 + kVecChunk);
+    const int chunk = S.vec_chunk;
+    const int e0 = it.tile * chunk;
+    const int e1 = min(n, e0 + chunk);
     CompDotDF dot;
-    constexpr int kStep = 4 * kVecThreads;
-    constexpr int kVec = kVecChunk / kStep;
-    if (e0 + kVecChunk <= n) {
-      // full chunk: kU 16-byte vectors of every plane in flight per thread, loads first
-      constexpr int kU = 2;
-      static_assert(kVec % kU == 0, "unroll");
+    if (e0 + chunk <= n) {
+      // one 16-byte vector of every plane per thread and step, every load before any use
 #pragma unroll 1
-      for (int j0 = 0; j0 < kVec; j0 += kU) {
-        float4 ph[kU], pl[kU], qh[kU], ql[kU], rh[kU], rl[kU], xh[kU], xl[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const int e = e0 + (j0 + u) * kStep + 4 * threadIdx.x;
-          ph[u] = __ldg(reinterpret_cast<const float4*>(p + e));
-          pl[u] = __ldg(reinterpret_cast<const float4*>(p_lo + e));
-          qh[u] = __ldg(reinterpret_cast<const float4*>(S.q + e));
-          ql[u] = __ldg(reinterpret_cast<const float4*>(S.q_lo + e));
-          rh[u] = *reinterpret_cast<const float4*>(S.r + e);
-          rl[u] = *reinterpret_cast<const float4*>(S.r_lo + e);
-          xh[u] = *reinterpret_cast<const float4*>(S.xhi + e);
-          xl[u] = *reinterpret_cast<const float4*>(S.xlo + e);
-        }
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const int e = e0 + (j0 + u) * kStep + 4 * threadIdx.x;
-          df_axpy(xh[u].x, xl[u].x, alpha, ph[u].x, pl[u].x);
-          df_axpy(xh[u].y, xl[u].y, alpha, ph[u].y, pl[u].y);
-          df_axpy(xh[u].z, xl[u].z, alpha, ph[u].z, pl[u].z);
-          df_axpy(xh[u].w, xl[u].w, alpha, ph[u].w, pl[u].w);
-          df_axpy(rh[u].x, rl[u].x, nalpha, qh[u].x, ql[u].x);
-          df_axpy(rh[u].y, rl[u].y, nalpha, qh[u].y, ql[u].y);
-          df_axpy(rh[u].z, rl[u].z, nalpha, qh[u].z, ql[u].z);
-          df_axpy(rh[u].w, rl[u].w, nalpha, qh[u].w, ql[u].w);
-          *reinterpret_cast<float4*>(S.xhi + e) = xh[u];
-          *reinterpret_cast<float4*>(S.xlo + e) = xl[u];
-          *reinterpret_cast<float4*>(S.r + e) = rh[u];
-          *reinterpret_cast<float4*>(S.r_lo + e) = rl[u];
-          dot.add(rh[u].x, rl[u].x, rh[u].x, rl[u].x);
-          dot.add(rh[u].y, rl[u].y, rh[u].y, rl[u].y);
-          dot.add(rh[u].z, rl[u].z, rh[u].z, rl[u].z);
-          dot.add(rh[u].w, rl[u].w, rh[u].w, rl[u].w);
-        }
+      for (int e = e0 + 4 * threadIdx.x; e < e1; e += kVecStep) {
+        const float4 ph = __ldg(reinterpret_cast<const float4*>(p + e));
+        const float4 pl = __ldg(reinterpret_cast<const float4*>(p_lo + e));
+        const float4 qh = __ldg(reinterpret_cast<const float4*>(S.q + e));
+        const float4 ql = __ldg(reinterpret_cast<const float4*>(S.q_lo + e));
+        float4 rh = *reinterpret_cast<const float4*>(S.r + e);
+        float4 rl = *reinterpret_cast<const float4*>(S.r_lo + e);
+        float4 xh = *reinterpret_cast<const float4*>(S.xhi + e);
+        float4 xl = *reinterpret_cast<const float4*>(S.xlo + e);
+        df_axpy(xh.x, xl.x, alpha, ph.x, pl.x);
+        df_axpy(xh.y, xl.y, alpha, ph.y, pl.y);
+        df_axpy(xh.z, xl.z, alpha, ph.z, pl.z);
+        df_axpy(xh.w, xl.w, alpha, ph.w, pl.w);
+        df_axpy(rh.x, rl.x, nalpha, qh.x, ql.x);
+        df_axpy(rh.y, rl.y, nalpha, qh.y, ql.y);
+        df_axpy(rh.z, rl.z, nalpha, qh.z, ql.z);
+        df_axpy(rh.w, rl.w, nalpha, qh.w, ql.w);
+        *reinterpret_cast<float4*>(S.xhi + e) = xh;
+        *reinterpret_cast<float4*>(S.xlo + e) = xl;
+        *reinterpret_cast<float4*>(S.r + e) = rh;
+        *reinterpret_cast<float4*>(S.r_lo + e) = rl;
+        dot.add(rh.x, rl.x, rh.x, rl.x);
+        dot.add(rh.y, rl.y, rh.y, rl.y);
+        dot.add(rh.z, rl.z, rh.z, rl.z);
+        dot.add(rh.w, rl.w, rh.w, rl.w);
       }
     } else {
       for (int k = e0 + threadIdx.x; k < e1; k += blockDim.x) {
@@ -785,10 +795,9 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
     const double rr = block_sum_comp<kVecThreads>(dot.as_comp(), red);
     if (threadIdx.x == 0) S.part[it.tile * 4 + 0] = rr;
     if (last_item_block(&sc->cnt[2], S.n_vec_items, &s_last)) {
-      double sums[1];
-      reduce_partials<kVecThreads, 1>(S.part, S.n_vec_items, sums, red);
+      double s = 0.0;
+      if (threadIdx.x < 32) s = warp_sum_strided(S.part, S.n_vec_items, 4);
       if (threadIdx.x == 0) {
-        const double s = sums[0];
         sc->rr = s;
         const int itn = sc->it + 1;
         sc->it = itn;
@@ -815,6 +824,7 @@ k_true_residual(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__
   __shared__ double red[64];
   __shared__ int s_last;
   const int total = *n_items;
+  pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
     const WorkItem it = items[w];
     const SlotDesc& S = slots[it.slot];
@@ -881,26 +891,20 @@ k_true_residual(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__
 // transform work list) reduces the per-tile r.z and z.q partials in a fixed order and forms rho
 // and beta (flexible or Fletcher-Reeves), or flags breakdown.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(32)
 k_prec_finish(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
               const int* __restrict__ n_items, int mode) {
-  __shared__ double red[64];
   const int total = *n_items;
+  pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
-    const WorkItem it = items[w];
-    if (it.tile != 0) continue;
-    const SlotDesc& S = slots[it.slot];
+    const SlotDesc& S = slots[items[w].slot];
     SlotScalars* sc = S.sc;
     const int run = mode == 0 ? sc->active : (mode == 1 ? sc->need_prec : 1);
     if (!run) continue;
-    double a = 0.0, b = 0.0;
-    for (int t = threadIdx.x; t < S.n_prec_parts; t += blockDim.x) {
-      a += S.part[t * 4 + 2];
-      b += S.part[t * 4 + 3];
-    }
-    block_sum2<256>(a, b, red);
-    if (threadIdx.x == 0) finish_preconditioner(S, a, b, mode);
-    __syncthreads();
+    double rz, zq;
+    sum_rz(S, sc->flexible != 0 || mode == 2, rz, zq);
+    __syncwarp();  // every lane has read the flags
+    if (threadIdx.x == 0) finish_preconditioner(S, rz, zq, mode);
   }
 }
 
@@ -918,8 +922,8 @@ k_output(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
     const float* f = fs[it.slot];
     float* out = outs[it.slot];
     const int n = S.nx * S.ny;
-    const int e0 = it.tile * kVecChunk;
-    const int e1 = min(n, e0 + kVecChunk);
+    const int e0 = it.tile * S.vec_chunk;
+    const int e1 = min(n, e0 + S.vec_chunk);
     const int be = S.sc->bexp;  // x = 2^-bexp x'
     for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x)
       out[e] = S.mask[e] ? (float)ldexp((double)S.xhi[e] + (double)S.xlo[e], -be) : f[e];
@@ -957,6 +961,7 @@ k_apply(const SlotDesc* __restrict__ slots, const float* __restrict__ p, float* 
     }
     __syncthreads();
     double pq = 0.0;
+  bool run = false;
     for (int k = threadIdx.x; k < kStTileX * kStTileY; k += blockDim.x) {
       const int ly = k / kStTileX, lx = k - ly * kStTileX;
       const int gx = x0 + lx, gy = y0 + ly;
@@ -984,54 +989,62 @@ void launch_setup(const LaunchCfg& c, const float* const* phis, const float* con
 void launch_rhs_scale(const LaunchCfg& c) {
   k_rhs_scale<<<c.grid, kStThreads, 0, c.stream>>>(c.slots, c.items, c.n_items);
 }
-template <int TY>
+template <int TY, bool FUSE>
 static void launch_stencil_ty(const LaunchCfg& c, bool aniso, int* err, long long wc) {
   constexpr int smem = StGeom<TY>::kSmemBytes;
   if (aniso)
-    k_stencil<true, TY><<<c.grid, kStThreads, smem, c.stream>>>(c.slots, c.items, c.n_items, err, wc);
+    launch_cfg(c, k_stencil<true, TY, FUSE>, c.grid, kStThreads, smem, c.slots, c.items, c.n_items, err, wc);
   else
-    k_stencil<false, TY><<<c.grid, kStThreads, smem, c.stream>>>(c.slots, c.items, c.n_items, err, wc);
+    launch_cfg(c, k_stencil<false, TY, FUSE>, c.grid, kStThreads, smem, c.slots, c.items, c.n_items, err, wc);
 }
-void launch_stencil(const LaunchCfg& c, bool aniso, int tile_y, int* err) {
+void launch_stencil(const LaunchCfg& c, bool aniso, int tile_y, int* err, bool fuse_prec) {
   const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
-  if (tile_y == 16) launch_stencil_ty<16>(c, aniso, err, wc);
-  else launch_stencil_ty<32>(c, aniso, err, wc);
+  if (fuse_prec) {
+    if (tile_y == 16) launch_stencil_ty<16, true>(c, aniso, err, wc);
+    else launch_stencil_ty<32, true>(c, aniso, err, wc);
+  } else {
+    if (tile_y == 16) launch_stencil_ty<16, false>(c, aniso, err, wc);
+    else launch_stencil_ty<32, false>(c, aniso, err, wc);
+  }
 }
 int stencil_blocks_per_sm(int tile_y) {
   return tile_y == 16 ? StGeom<16>::kBlocksPerSm : StGeom<32>::kBlocksPerSm;
 }
-template <bool ANISO, int TY>
+template <bool ANISO, int TY, bool FUSE>
 static cudaError_t stencil_attr() {
   // the window sets live in dynamic shared memory; all of the SM's shared memory to the
   // carveout, so that kBlocksPerSm blocks fit
-  const cudaError_t e = cudaFuncSetAttribute(k_stencil<ANISO, TY>,
+  const cudaError_t e = cudaFuncSetAttribute(k_stencil<ANISO, TY, FUSE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              StGeom<TY>::kSmemBytes);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_stencil<ANISO, TY>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  return cudaFuncSetAttribute(k_stencil<ANISO, TY, FUSE>, cudaFuncAttributePreferredSharedMemoryCarveout,
                               cudaSharedmemCarveoutMaxShared);
 }
 cudaError_t stencil_init() {
-  const cudaError_t e[4] = {stencil_attr<false, 32>(), stencil_attr<true, 32>(),
-                            stencil_attr<false, 16>(), stencil_attr<true, 16>()};
+  const cudaError_t e[8] = {stencil_attr<false, 32, false>(), stencil_attr<true, 32, false>(),
+                            stencil_attr<false, 16, false>(), stencil_attr<true, 16, false>(),
+                            stencil_attr<false, 32, true>(),  stencil_attr<true, 32, true>(),
+                            stencil_attr<false, 16, true>(),  stencil_attr<true, 16, true>()};
   for (cudaError_t x : e)
     if (x != cudaSuccess) return x;
   return cudaSuccess;
 }
 void launch_pq_finish(const LaunchCfg& c) {
-  k_pq_finish<<<c.grid, 256, 0, c.stream>>>(c.slots, c.items, c.n_items);
+  launch_cfg(c, k_pq_finish, c.grid, 32, 0, c.slots, c.items, c.n_items);
 }
-void launch_update(const LaunchCfg& c) {
-  k_update<<<c.grid, kVecThreads, 0, c.stream>>>(c.slots, c.items, c.n_items);
+void launch_update(const LaunchCfg& c, bool fuse_pq) {
+  if (fuse_pq) launch_cfg(c, k_update<true>, c.grid, kVecThreads, 0, c.slots, c.items, c.n_items);
+  else launch_cfg(c, k_update<false>, c.grid, kVecThreads, 0, c.slots, c.items, c.n_items);
 }
 void launch_true_residual(const LaunchCfg& c) {
-  k_true_residual<<<c.grid, kStThreads, 0, c.stream>>>(c.slots, c.items, c.n_items);
+  launch_cfg(c, k_true_residual, c.grid, kStThreads, 0, c.slots, c.items, c.n_items);
 }
 void launch_output(const LaunchCfg& c, const float* const* fs, float* const* outs) {
   k_output<<<c.grid, kVecThreads, 0, c.stream>>>(c.slots, c.items, c.n_items, fs, outs);
 }
 void launch_prec_finish(const LaunchCfg& c, int mode) {
-  k_prec_finish<<<c.grid, 256, 0, c.stream>>>(c.slots, c.items, c.n_items, mode);
+  launch_cfg(c, k_prec_finish, c.grid, 32, 0, c.slots, c.items, c.n_items, mode);
 }
 void launch_output64(const SlotDesc* slot, int n, const float* f, double* out, cudaStream_t s) {
   int grid = (n + kVecThreads - 1) / kVecThreads;
