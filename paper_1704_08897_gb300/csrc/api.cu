@@ -588,7 +588,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
           L.o_tt1 = take(2 * NS * Npc);
           L.o_tt2 = take(2 * NS * Npc);
           L.o_tt3 = take(2 * NS * Npc);
-          L.o_maps = take(8 * sizeof(CUtensorMap));
+          L.o_maps = take(kTcMaps * sizeof(CUtensorMap));
           L.o_ex = take(4 * (Npc / 64));
         } else {
           L.o_s1 = take(8 * Npc);
@@ -782,7 +782,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     t.tc_eb[3] = plan_exps(qy, 0);  // Qy rows
     BX_CUDA(cudaMemset(t.tc_r, 0, 2 * (low ? kLowNS : NS) * Npc));
     BX_CUDA(cudaMemset(A + L.o_ex, 0, 4 * nex));
-    CUtensorMap maps[8];
+    CUtensorMap maps[kTcMaps];
     const size_t pxp = (size_t)t.nxp * t.nxp, pyp = (size_t)t.nyp * t.nyp;
     uint16_t* qxb = (uint16_t*)qx->tc;
     uint16_t* qyb = (uint16_t*)qy->tc;
@@ -796,6 +796,10 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     if (!rc3) rc3 = make_tmap(&maps[5], qyb + NS * pyp, bf, t.nyp, (uint64_t)NS * t.nyp, 64);
     if (!rc3) rc3 = make_tmap(&maps[6], qxb, bf, t.nxp, (uint64_t)NS * t.nxp, 64);
     if (!rc3) rc3 = make_tmap(&maps[7], qyb, bf, t.nyp, (uint64_t)NS * t.nyp, 64);
+    // the stages' results as they are stored, tile by tile: T1, T2, T3
+    if (!rc3) rc3 = make_tmap(&maps[8], t.tc_t1, bf, t.nyp, (uint64_t)NS * t.nxp, 32);
+    if (!rc3) rc3 = make_tmap(&maps[9], t.tc_t2, bf, t.nxp, (uint64_t)NS * t.nyp, 32);
+    if (!rc3) rc3 = make_tmap(&maps[10], t.tc_t3, bf, t.nyp, (uint64_t)NS * t.nxp, 32);
     if (rc3) return rc3;
     BX_CUDA(cudaMemcpy(A + L.o_maps, maps, sizeof(maps), cudaMemcpyHostToDevice));
     t.lowm_x = t.lowm_y = 0;
@@ -1739,7 +1743,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   double* part = (double*)take(sizeof(double) * 4 * (size_t)tiles3);
   float* lam = (float*)take(sizeof(float) * ((size_t)Y * X + Z));
   SlotScalars* sc = (SlotScalars*)take(sizeof(SlotScalars));
-  void* maps = take(6 * 8 * sizeof(CUtensorMap));
+  void* maps = take(6 * kTcMaps * sizeof(CUtensorMap));
   SlotDesc* descs = (SlotDesc*)take(7 * sizeof(SlotDesc));
   if (!S0 || !SA || !SB || !E0 || !EA || !EB || !part || !lam || !sc || !maps || !descs) {
     g_last_error = "cudaMalloc of the 3-D tensor-core workspace failed";
@@ -1785,7 +1789,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   const size_t pl[3] = {(size_t)X * X, (size_t)Y * Y, (size_t)Z * Z};
   auto QT = [&](int ax) { return (void*)(q[ax] + NS * pl[ax]); };  // Q^T planes follow the Q planes
   auto QQ = [&](int ax) { return (void*)q[ax]; };
-  CUtensorMap m[6][8];
+  CUtensorMap m[6][kTcMaps];
   memset(m, 0, sizeof(m));
   // [0]: residual slicing, rows (z, y), columns x
   d[0].nx = X; d[0].ny = Z * Y; d[0].nxp = X; d[0].nyp = Z * Y;
@@ -1796,27 +1800,32 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   int rc = make_tmap(&m[0][0], S0, bf, X, (uint64_t)NS * Z * Y, 128);
   if (!rc) rc = make_tmap(&m[0][4], QT(0), bf, X, (uint64_t)NS * X, 64);
   d[1].tc_e[0] = E0; d[1].tc_eb[0] = plan_exps(P[0], 1); d[1].tc_t1 = SA; d[1].tc_e[1] = EA;
+  if (!rc) rc = make_tmap(&m[0][8], SA, bf, (uint64_t)Z * Y, (uint64_t)NS * X, 32);
   // [2] F2 (stage-0 form): A = SA as [X Z][Y], B = Qy^T -> SB [Y][X Z]
   d[2].nyp = X * Z; d[2].nxp = Y; d[2].nx = Y; d[2].ny = X * Z;
   if (!rc) rc = make_tmap(&m[1][0], SA, bf, Y, (uint64_t)NS * X * Z, 128);
   if (!rc) rc = make_tmap(&m[1][4], QT(1), bf, Y, (uint64_t)NS * Y, 64);
   d[2].tc_e[0] = EA; d[2].tc_eb[0] = plan_exps(P[1], 1); d[2].tc_t1 = SB; d[2].tc_e[1] = EB;
+  if (!rc) rc = make_tmap(&m[1][8], SB, bf, (uint64_t)X * Z, (uint64_t)NS * Y, 32);
   // [3] F3 (stage-1 form, weights): A = SB as [Y X][Z], B = Qz^T -> SA [Z][Y X]
   d[3].nxp = Y * X; d[3].nyp = Z; d[3].nx = Y * X; d[3].ny = Z;
   if (!rc) rc = make_tmap(&m[2][1], SB, bf, Z, (uint64_t)NS * Y * X, 128);
   if (!rc) rc = make_tmap(&m[2][5], QT(2), bf, Z, (uint64_t)NS * Z, 64);
   d[3].tc_e[1] = EB; d[3].tc_eb[1] = plan_exps(P[2], 1); d[3].tc_t2 = SA; d[3].tc_e[2] = EA;
   d[3].lamx = lam; d[3].lamy = lam + (size_t)Y * X; d[3].wnorm = (float)(smin * smin);
+  if (!rc) rc = make_tmap(&m[2][9], SA, bf, (uint64_t)Y * X, (uint64_t)NS * Z, 32);
   // [4] I1 (stage-2 form): A = SA as [Z Y][X], B = Qx -> SB [X][Z Y]
   d[4].nyp = Z * Y; d[4].nxp = X; d[4].nx = X; d[4].ny = Z * Y;
   if (!rc) rc = make_tmap(&m[3][2], SA, bf, X, (uint64_t)NS * Z * Y, 128);
   if (!rc) rc = make_tmap(&m[3][6], QQ(0), bf, X, (uint64_t)NS * X, 64);
   d[4].tc_e[2] = EA; d[4].tc_eb[2] = plan_exps(P[0], 0); d[4].tc_t3 = SB; d[4].tc_e[3] = EB;
+  if (!rc) rc = make_tmap(&m[3][10], SB, bf, (uint64_t)Z * Y, (uint64_t)NS * X, 32);
   // [5] I2 (stage-2 form): A = SB as [X Z][Y], B = Qy -> SA [Y][X Z]
   d[5].nyp = X * Z; d[5].nxp = Y; d[5].nx = Y; d[5].ny = X * Z;
   if (!rc) rc = make_tmap(&m[4][2], SB, bf, Y, (uint64_t)NS * X * Z, 128);
   if (!rc) rc = make_tmap(&m[4][6], QQ(1), bf, Y, (uint64_t)NS * Y, 64);
   d[5].tc_e[2] = EB; d[5].tc_eb[2] = plan_exps(P[1], 0); d[5].tc_t3 = SA; d[5].tc_e[3] = EA;
+  if (!rc) rc = make_tmap(&m[4][10], SA, bf, (uint64_t)X * Z, (uint64_t)NS * Y, 32);
   // [6] I3 (stage-3 form): A = SA as [Y X][Z], B = Qz -> z[Z][Y X] masked, r.z per tile
   d[6].nxp = Y * X; d[6].nyp = Z; d[6].nx = Y * X; d[6].ny = Z;
   if (!rc) rc = make_tmap(&m[5][3], SA, bf, Z, (uint64_t)NS * Y * X, 128);
@@ -1827,7 +1836,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   d[6].q = const_cast<float*>(io.qh); d[6].q_lo = const_cast<float*>(io.ql);
   d[6].z = io.zh; d[6].z_lo = io.zl; d[6].mask = const_cast<uint8_t*>(io.mask); d[6].part = part;
   BX_CUDA(cudaMemcpy(maps, m, sizeof(m), cudaMemcpyHostToDevice));
-  for (int k = 1; k < 7; ++k) d[k].tmaps = (const char*)maps + (size_t)(k - 1) * 8 * sizeof(CUtensorMap);
+  for (int k = 1; k < 7; ++k) d[k].tmaps = (const char*)maps + (size_t)(k - 1) * kTcMaps * sizeof(CUtensorMap);
   BX_CUDA(cudaMemcpy(descs, d, sizeof(d), cudaMemcpyHostToDevice));
   // work items: [0] 32 rows x 128 columns; the products tiles of 128 x 64 (M x N)
   static const int kForm[7] = {-1, 0, 0, 1, 2, 2, 3};

@@ -57,6 +57,7 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
 constexpr long long kShortBudget = 100000;
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           long long budget = kWaitCycles) {
+  if (mbar_test(bar, parity)) return true;  // the usual case for a producer or issuer that is ahead
   const long long t0 = clock64();
   const bool short_budget = budget < kShortBudget;
   while (!(short_budget ? mbar_test(bar, parity) : mbar_try(bar, parity))) {

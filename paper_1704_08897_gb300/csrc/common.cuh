@@ -20,6 +20,7 @@ constexpr int kStThreads = 256;
 // left than the halo so that a copy starts on a 16-byte boundary.
 constexpr int kStWinX = kStTileX + 8;
 constexpr int kStWinY = kStTileY + 4;
+constexpr int kTcMaps = 11;         // transform tensor maps per problem
 constexpr int kStMaps = 7;          // stencil tensor maps per slot
 constexpr int kLowM = 32;           // low modes per axis computed in high precision
 constexpr int kLowAutoSide = 2048;  // low_modes = 2: grids with a side of at least this many nodes
@@ -126,7 +127,8 @@ struct SlotDesc {
   void* tc_t3;       // [NS][nxp][nyp]
   int8_t* tc_e[4];   // block exponents of the A operand of stage s: [rows][K/128]
   const int8_t* tc_eb[4];  // block exponents of the B operand of stage s (transform matrices)
-  const void* tmaps; // 8 CUtensorMap (64-byte aligned): A operand of stages 0..3, B of 0..3
+  const void* tmaps; // kTcMaps CUtensorMap (64-byte aligned): A operand of stages 0..3, B of 0..3,
+                     // the results of stages 0..2 (store boxes)
   const void* st_maps;  // kStMaps CUtensorMap for the stencil's tensor copies (z, z_lo, p[0],
                         // p_lo[0], p[1], p_lo[1], mask); null when a mask row is not a multiple
                         // of 16 bytes
@@ -478,11 +480,13 @@ __device__ __forceinline__ int ghost(int i, int n, int bc, float& sgn) {
   return i < 0 ? -i - 2 : 2 * n - i;
 }
 
-// wnorm / s^2 by the approximate division (at most 2 ulp for s^2 in [2^-126, 2^126]; s^2 of the
-// grids' eigenvalue sums stays far inside that range).  The preconditioner is only an
+// wnorm / s^2 by the approximate reciprocal (at most 2 ulp in all; s^2 of the grids' eigenvalue
+// sums, 1e-18 to 300, stays far inside the normal range).  The preconditioner is only an
 // approximation of the inverse, so a 2-ulp change of its weights is immaterial.
 __device__ __forceinline__ float spectral_weight_of(float wnorm, float s) {
-  return __fdividef(wnorm, s * s);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s * s));
+  return wnorm * r;
 }
 
 // Spectral weight 1/(lam_y + lam_x)^2, normalised to <= 1; zero for padding and the constant

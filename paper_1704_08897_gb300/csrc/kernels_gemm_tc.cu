@@ -22,16 +22,30 @@
 // error along K; the stage outputs stay double-float (hi, lo) pairs and are sliced from them
 // directly, and the last stage writes z as a double-float pair.  Three slices on
 // 64-blocks (24 bits) cost this operator 30-80% more CG iterations than exact transforms; four on
-// 128-blocks come within 5-10% of them.  The writer of the next stage's operand computes its
-// block exponents with a four-warp maximum and stores the slices transposed (Out[n][m],
-// coalesced along m).
+// 128-blocks come within 5-10% of them.
 //
 // Kernel structure (one CTA per SM, persistent over the (slot, tile) work list):
-//   warp 0      : TMA producer: 128B-swizzled K-major tiles of the four slices of A and B
-//   warp 1      : TMEM allocation; lane 0 issues the MMAs and the tcgen05.commit arrivals
-//   warps 2..17 : four per TMEM lane quarter (32 rows), each owning 16 of the tile's 64 columns:
+//   warp 0      : TMA producer: 128B-swizzled K-major tiles of the slices of A and B, two 64-deep
+//                 steps of 96 KB
+//   warp 1      : TMEM allocation; issues the MMAs and the tcgen05.commit arrivals
+//   warps 2..17 : four per TMEM lane quarter (32 rows), each owning a quarter of the tile's columns:
 //                 exact k-block sums -> compensated registers -> the stage's epilogue
 //                 (eigenvalue weights; masking and per-tile r.z, z.q partials in stage 3).
+//
+// What bounds it.  A step's ten products take 1,700 SM cycles at the measured BF16 peak; the
+// k-loop runs at 1,660 (clock stamps, 1024^2 grid).  Getting there took the issuing warp out of
+// the way: run by one lane under a divergent branch it spent 62 cycles an MMA on moving the
+// descriptors to uniform registers and 300 a wait, 2,050 a step, so the whole warp now runs the
+// loop (uniform descriptors, one elected lane issues) and a wait first tests its barrier without
+// reading the clock.  Per-plane barriers for A (earlier refills, but five waits and commits a step)
+// measured 3,250 cycles a step; 32-deep steps with a 64-byte swizzle were no faster either.
+// Then the epilogue: it reads TMEM in the 16x256b shape, whose register layout is that of an
+// 8 x 8 matrix fragment: a thread holds four rows by a few columns, so row and column factors need a
+// few shuffles, a column's maximum over the rows three exchanges, and the 16-bit slices leave by
+// transposing stmatrix into a swizzled staging tile that tensor stores write out while the next
+// tile runs.  (With one row per thread a tile took 64 two-byte stores and about 80 shuffles per
+// thread.)  What is left after the last k-block is FP32 issue: about 1,300 cycles for the merge, 2,000
+// for slicing and storing, 2,000 for stage 1's weights.
 // Every wait on an mbarrier is bounded; on time-out the CTA raises an error flag, drains its
 // outstanding copies and MMAs, frees its TMEM and returns.
 #include <cuda.h>
@@ -45,29 +59,36 @@
 namespace bx {
 namespace {
 
-constexpr int BM = 128, BN = 64, BK = 64;  // BK: one 128-byte swizzle atom per pipeline stage
+constexpr int BM = 128, BK = 64;  // BK: one 128-byte swizzle atom per pipeline step
 constexpr int KC = 128;                     // k per exponent / exact accumulation block
-constexpr int KPC = KC / BK;                // pipeline stages per accumulation block
-constexpr int NS = 4;                            // slices per operand
+constexpr int KPC = KC / BK;                // pipeline steps per accumulation block
+constexpr int NS = 4;                       // slices per operand of the transform stages
 constexpr int kEpiWarps = 16;
-constexpr int kColGroups = kEpiWarps / 4;        // epilogue warps per TMEM lane quarter
-constexpr int kEpiCols = BN / kColGroups;        // tile columns per epilogue warp
-static_assert(kEpiCols % 16 == 0 && kEpiCols <= 32, "epilogue column split");
-static_assert(KC % BK == 0 && KC <= BM && BM % KC == 0, "exponent blocks within a tile");
-constexpr int kLdCols = kEpiWarps == 16 ? 4 : 8;  // TMEM columns per load (register budget)
+static_assert(KC % BK == 0 && KC == BM, "one exponent block per tile column");
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 // One CTA per SM.  Each of the SM's four schedulers owns a quarter of the register file and
 // holds up to ceil(warps / 4) of the CTA's warps.
 constexpr int kMaxRegs = (16384 / (32 * ((kThreads / 32 + 3) / 4))) & ~7;
 constexpr int kChunks = 2;                       // TMEM ring of k-block accumulator sets
-constexpr int kSetCols = NS * BN;                // one accumulator per slice order
-constexpr int kTmemCols = 512;                   // power of two >= kChunks * kSetCols
-static_assert(kChunks * kSetCols <= kTmemCols, "TMEM columns");
-constexpr int STAGES = 2;
+constexpr int kTmemCols = 512;                   // power of two >= kChunks * sets
 constexpr int A_PLANE = BM * BK * 2;
-constexpr int B_PLANE = BN * BK * 2;
-constexpr int STAGE_BYTES = NS * (A_PLANE + B_PLANE);
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 2048;
+constexpr int STAGES = 2;
+
+// Tile geometry by the number of slices: shared memory holds the A ring, the two B steps and the
+// staging tile of the outgoing slices.
+template <int NSL>
+struct TcGeom {
+  static constexpr int BN = NSL == 4 ? 64 : 32;   // tile columns
+  static constexpr int kCb = BN / 32;             // 8-column blocks per epilogue warp
+  static constexpr int kEpiCols = 8 * kCb;        // tile columns per epilogue warp
+  static constexpr int kBPlane = BN * BK * 2;
+  static constexpr int kStageBytes = NSL * (A_PLANE + kBPlane);  // one 64-deep step of both operands
+  static constexpr int kStage = NSL * 32 * BM * 2;  // staging: [slice][64-row half][column] 128 B rows
+  static constexpr int kSetCols = NSL * BN;       // one accumulator per slice order
+  static constexpr int kSmem = STAGES * kStageBytes + kStage + 1024 + 2048;
+  static_assert(kChunks * kSetCols <= kTmemCols, "TMEM columns");
+  static_assert(kSmem <= 232448, "shared memory of an SM's block");
+};
 
 struct Ctl {
   uint64_t full[STAGES];
@@ -77,10 +98,8 @@ struct Ctl {
   uint64_t drain;
   uint32_t tmem;
   int abort_flag;
-  int last;
-  int pad;
-  float red[kEpiWarps][4];  // stage 3: per-warp compensated r.z and z.q
-  float colmax[kColGroups][4][kEpiCols];  // [column group][lane quarter][column]
+  float4 red[kEpiWarps];                  // stage 3: per-warp compensated r.z and z.q
+  float colmax[4][16][4];                 // [column group][column][lane quarter]
 };
 static_assert(sizeof(Ctl) <= 2048, "control block too large");
 
@@ -111,32 +130,42 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
+// One lane of the (converged) warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-[[maybe_unused]] __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-        "=r"(v[15])
-      : "r"(taddr));
-}
-[[maybe_unused]] __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
                : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+// Sixteen TMEM lanes by eight columns as a matrix fragment: lane l of the warp gets columns
+// 2 (l % 4), 2 (l % 4) + 1 of rows l / 4 (v[0], v[1]) and l / 4 + 8 (v[2], v[3]).
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
                : "r"(taddr));
 }
-template <int N>
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&v)[N]) {
-  if constexpr (N == 16) tmem_ld16(taddr, v);
-  else if constexpr (N == 8) tmem_ld8(taddr, v);
-  else tmem_ld4(taddr, v);
+// Four 8 x 8 matrices of 16-bit values (fragments v[0..3]: lane l holds columns 2 (l % 4), + 1 of row
+// l / 4) stored transposed: lanes 8 k .. 8 k + 7 give the addresses of matrix k's columns.
+__device__ __forceinline__ void stmatrix4_t(uint32_t saddr, const uint32_t (&v)[4]) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(v[0]),
+               "r"(v[1]), "r"(v[2]), "r"(v[3])
+               : "memory");
+}
+__device__ __forceinline__ void tma_store_2d(const void* tmap, uint32_t saddr, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(tmap)),
+               "r"(saddr), "r"(c0), "r"(c1)
+               : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -148,53 +177,65 @@ __device__ __forceinline__ float ld_early(const float* p) {
   return v;
 }
 
+__device__ __forceinline__ unsigned ld_keep(const void* p) {
+  unsigned v;
+  asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+
 // 2^e as a float for e in the normal range, 0 below it.
 __device__ __forceinline__ float pow2f(int e) {
   return e < -126 ? 0.f : __int_as_float((min(e, 127) + 127) << 23);
 }
 
-// Exponent E of a block whose largest magnitude is amax: amax < 2^E (0 for an all-zero block);
-// for blocks wider than 64 also amax 2^(8-E) < 255.5, so the leading slice stays within +-255.
+// Exponent E of a block whose largest magnitude is amax: amax < 2^E and amax 2^(8-E) < 255.5, so the
+// leading slice stays within +-256 (0 for an all-zero block).
 __device__ __forceinline__ int block_exp(float amax) {
   if (!(amax > 0.f)) return 0;
   int e;
   frexpf(amax, &e);
-  if (KC > 64 && amax * pow2f(8 - e) >= 255.5f) ++e;
-  return max(e, -90);  // keeps 2^(32-E) and 2^(E-16-8d) normal
+  if (amax * pow2f(8 - e) >= 255.5f) ++e;
+  return max(e, -70);  // keeps 2^(48-E) and 2^(E-16-8d) normal
 }
 
-// The NS integer slices of double-float values (hi, lo) for block exponent E, given s = 2^(8-E) and
-// is = 2^(E-8) (all the powers of two involved are normal for the exponents block_exp returns),
-// on two lanes with their own block factors: each step takes the integer of the leading plane,
-// removes it exactly (FMA; the product is exact) and renormalises the remainder with the lo plane
-// (TwoSum), so the slices carry the value to 2^-32 of the block whatever its size; the last
-// slice is rounded to an integer.  The 16-bit codes are returned as (lane x, lane y) pairs.
-// Every slice is an integer of magnitude at most 256, which keeps the two per-value conversions
-// off the (quarter-rate) conversion pipe: the rounding to the nearest integer (ties to even) adds
-// and removes 1.5 * 2^23 on packed FP32x2, exact for magnitudes below 2^22; and such an integer is
-// exact in BF16, whose bits are then the upper half of the FP32 bits (one byte permutation packs
-// the two lanes' codes).  FP16 codes come from the packed two-value conversion.
-template <bool BF16, int NSL = NS>
-__device__ __forceinline__ void slice_codes2_df(float2 vh, float2 vl, float2 s, float2 is,
+// The NSL integer slices of double-float values (hi, lo) for block exponent E, given up = 2^(16-E)
+// and dn = -2^(E-16), on two lanes with their own block factors.  The value is taken sixteen bits
+// at a time: w = the integer nearest to the leading plane at that scale, removed exactly (the
+// product is exact in the FMA), the remainder joined with the lo plane; and each w is cut into its
+// two digits w = 256 c0 + c1, |c1| <= 128.  The slices carry the value to 2^-32 (NSL = 4) or 2^-48
+// (6) of the block.  Roundings to the nearest integer add and remove 1.5 * 2^23 on packed FP32x2
+// (exact for magnitudes below 2^22; ties to even); a digit is an integer of magnitude at most 256,
+// exact in BF16, whose bits are the upper half of the FP32 bits (one byte permutation packs the two
+// lanes' codes).  FP16 codes come from the packed two-value conversion.  About 4 packed operations
+// a digit; the form before, one digit at a time with a renormalised remainder, took 12.
+template <bool BF16, int NSL>
+__device__ __forceinline__ void slice_codes2_df(float2 vh, float2 vl, float2 up, float2 dn,
                                                 uint32_t (&code)[NSL]) {
+  static_assert(NSL == 4 || NSL == 6, "slices in pairs");
   const float2 rnd = make_float2(12582912.f, 12582912.f), rnd_n = make_float2(-12582912.f, -12582912.f);
-  float2 rh = vh, rl = vl, up = s, down = make_float2(-is.x, -is.y);
+  float2 rh = vh, rl = vl;
 #pragma unroll
-  for (int k = 0; k < NSL; ++k) {
-    const float2 t = __fmul2_rn(rh, up);
-    const float2 c = __fadd2_rn(__fadd2_rn(t, rnd), rnd_n);
-    if (k + 1 < NSL) {
-      const float2 h = __ffma2_rn(c, down, rh);
-      two_sum2(h, rl, rh, rl);
+  for (int k = 0; k < NSL; k += 2) {
+    const float2 w = __fadd2_rn(__fadd2_rn(__fmul2_rn(rh, up), rnd), rnd_n);
+    if (k + 2 < NSL) {
+      const float2 h = __ffma2_rn(w, dn, rh);
+      if (k + 4 < NSL) two_sum2(h, rl, rh, rl);
+      else rh = __fadd2_rn(h, rl);
+      up = mul2(65536.f, up);
+      dn = mul2(1.52587890625e-05f, dn);
     }
-    up = mul2(256.f, up);
-    down = mul2(0.00390625f, down);
-    if (BF16) {
-      code[k] = __byte_perm(__float_as_uint(c.x), __float_as_uint(c.y), 0x7632);
-    } else {
-      const __half2 h2 = __floats2half2_rn(c.x, c.y);
-      code[k] = static_cast<uint32_t>(__half_as_ushort(__low2half(h2))) |
-                (static_cast<uint32_t>(__half_as_ushort(__high2half(h2))) << 16);
+    float2 c[2];
+    c[0] = __fadd2_rn(__ffma2_rn(w, make_float2(0.00390625f, 0.00390625f), rnd), rnd_n);
+    c[1] = __ffma2_rn(c[0], make_float2(-256.f, -256.f), w);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      if (BF16) {
+        code[k + j] = __byte_perm(__float_as_uint(c[j].x), __float_as_uint(c[j].y), 0x7632);
+      } else {
+        const __half2 h2 = __floats2half2_rn(c[j].x, c[j].y);
+        code[k + j] = static_cast<uint32_t>(__half_as_ushort(__low2half(h2))) |
+                      (static_cast<uint32_t>(__half_as_ushort(__high2half(h2))) << 16);
+      }
     }
   }
 }
@@ -205,29 +246,6 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// Column maxima of a warp's C x 32 block (v[i]: column i of this lane's row), by a transposing
-// butterfly: at each step a lane keeps the half of its columns selected by its lane bit and takes
-// the partner's copy of that half.  Returns, in lane l, the maximum over all 32 rows of column
-// l mod C.  C - 1 exchanges instead of the C * 5 of one reduction per column.
-template <int C>
-__device__ __forceinline__ float column_max(float (&v)[C], int lane) {
-  if (C == 16) {
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], __shfl_xor_sync(0xffffffffu, v[i], 16));
-  }
-#pragma unroll
-  for (int w = C / 2; w >= 1; w /= 2) {
-    const bool up = (lane & w) != 0;
-#pragma unroll
-    for (int i = 0; i < w; ++i) {
-      const float keep = up ? v[i + w] : v[i];
-      const float give = up ? v[i] : v[i + w];
-      v[i] = fmaxf(keep, __shfl_xor_sync(0xffffffffu, give, w));
-    }
-  }
-  return v[0];
-}
-
 __device__ __forceinline__ bool slot_runs(const SlotScalars* sc, int mode) {
   return mode == 0 ? sc->active != 0 : (mode == 1 ? sc->need_prec != 0 : true);
 }
@@ -236,29 +254,71 @@ __device__ __forceinline__ void epi_bar() {
   asm volatile("bar.sync 1, %0;" ::"r"(32 * kEpiWarps) : "memory");
 }
 
+// Barrier of the epilogue warps that also tells whether any of them has failed.
+__device__ __forceinline__ bool epi_vote(bool fail) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, 1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(any)
+      : "r"(fail ? 1u : 0u), "r"(32 * kEpiWarps)
+      : "memory");
+  return any != 0;
+}
+
 struct TcStage {
   int M, N, K;
-  void* out;        // next stage's slices, or nullptr in the last stage
-  int8_t* eout;     // next stage's block exponents [N][M/64]
+  int8_t* eout;     // next stage's block exponents [N][M/128]
 };
 
 __device__ __forceinline__ TcStage tc_stage(const SlotDesc& S, int stage) {
   switch (stage) {
-    case 0: return {S.nyp, S.nxp, S.nxp, S.tc_t1, S.tc_e[1]};
-    case 1: return {S.nxp, S.nyp, S.nyp, S.tc_t2, S.tc_e[2]};
-    case 2: return {S.nyp, S.nxp, S.nxp, S.tc_t3, S.tc_e[3]};
-    default: return {S.nxp, S.nyp, S.nyp, nullptr, nullptr};
+    case 0: return {S.nyp, S.nxp, S.nxp, S.tc_e[1]};
+    case 1: return {S.nxp, S.nyp, S.nyp, S.tc_e[2]};
+    case 2: return {S.nyp, S.nxp, S.nxp, S.tc_e[3]};
+    default: return {S.nxp, S.nyp, S.nyp, nullptr};
   }
 }
 
-template <bool BF16, int STAGE>
+// Merge of one pair of columns' order sums (exact integers) into the compensated pair (hi, lo);
+// scl = 2^(E_A + E_B - 16) of the two columns.  Four slices: orders 1..3 are combined first, their
+// roundings are 2^-24 of terms 2^-8 below hi.  Six: orders 0..2 by TwoSum, 3..5 in plain FP32.
+template <int NSL>
+__device__ __forceinline__ void merge_orders(const float2 (&v)[NSL], float2 scl, float2& hi, float2& lo) {
+  const float2 q8 = make_float2(0.00390625f, 0.00390625f);
+  float2 er;
+  if constexpr (NSL == 4) {
+    const float2 w = __ffma2_rn(v[3], q8, v[2]);
+    const float2 u = __ffma2_rn(w, q8, v[1]);
+    const float2 t0 = __fmul2_rn(v[0], scl);
+    const float2 t1 = __fmul2_rn(u, __fmul2_rn(scl, q8));
+    two_sum2(hi, t0, hi, er);
+    lo = add2(lo, add2(er, t1));
+  } else {
+    const float2 w = __ffma2_rn(__ffma2_rn(v[5], q8, v[4]), q8, v[3]);
+    const float2 s1 = __fmul2_rn(scl, q8), s2 = __fmul2_rn(s1, q8);
+    two_sum2(hi, __fmul2_rn(v[0], scl), hi, er);
+    lo = add2(lo, er);
+    two_sum2(hi, __fmul2_rn(v[1], s1), hi, er);
+    lo = add2(lo, er);
+    two_sum2(hi, __fmul2_rn(v[2], s2), hi, er);
+    lo = add2(lo, add2(er, __fmul2_rn(w, __fmul2_rn(s2, q8))));
+  }
+}
+
+template <bool BF16, int STAGE, int NSL>
 __global__ void __maxnreg__(kMaxRegs)
 k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
           const int* __restrict__ n_items, int mode, int* __restrict__ err, long long wait_cycles) {
+  using G = TcGeom<NSL>;
+  constexpr int BN = G::BN, kCb = G::kCb, kEpiCols = G::kEpiCols;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  Ctl* ctl = reinterpret_cast<Ctl*>(smem + STAGES * STAGE_BYTES);
+  unsigned char* sO = smem + STAGES * G::kStageBytes;
+  Ctl* ctl = reinterpret_cast<Ctl*>(sO + G::kStage);
   volatile int* abort_flag = &ctl->abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int total = *n_items;
@@ -287,107 +347,113 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem;
-  pdl_wait();
+  // Each role reads its first tile's item and descriptor, which no kernel writes, before it waits
+  // for the previous kernel (pdl_wait): those dependent loads took 1 us after the wait.
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      int stage = 0, issued = 0;
-      uint32_t phase = 0;
-      for (int w = blockIdx.x; w < total && !*abort_flag; w += gridDim.x) {
+      struct Tile {
+        const SlotScalars* sc;
+        const unsigned char *ma, *mb;
+        int M, N, steps, m0, n0;
+      };
+      auto tile_of = [&](int w) {
         const WorkItem it = items[w];
         const SlotDesc& S = slots[it.slot];
-        if (!slot_runs(S.sc, mode)) continue;
         const TcStage v = tc_stage(S, STAGE);
-        const void* ma = static_cast<const unsigned char*>(S.tmaps) + 128 * STAGE;
-        const void* mb = static_cast<const unsigned char*>(S.tmaps) + 128 * (4 + STAGE);
-        tmap_acquire(ma);
-        tmap_acquire(mb);
         const int mt = v.M / BM;
-        const int m0 = (it.tile % mt) * BM, n0 = (it.tile / mt) * BN;
-        for (int kb = 0; kb < v.K / BK; ++kb) {
-          if (!mbar_wait(&ctl->empty[stage], phase ^ 1, abort_flag, wait_cycles)) break;
-          mbar_expect_tx(&ctl->full[stage], STAGE_BYTES);
-          unsigned char* sa = smem + stage * STAGE_BYTES;
-          unsigned char* sb = sa + NS * A_PLANE;
+        Tile t = {S.sc, static_cast<const unsigned char*>(S.tmaps) + 128 * STAGE,
+                  static_cast<const unsigned char*>(S.tmaps) + 128 * (4 + STAGE), v.M, v.N, v.K / BK,
+                  (it.tile % mt) * BM, (it.tile / mt) * BN};
+        tmap_acquire(t.ma);
+        tmap_acquire(t.mb);
+        return t;
+      };
+      Tile t = {};
+      if (blockIdx.x < total) t = tile_of(blockIdx.x);
+      pdl_wait();
+      int n = 0;  // steps issued
+      for (int w = blockIdx.x; w < total && !*abort_flag; w += gridDim.x) {
+        if (w != blockIdx.x) t = tile_of(w);
+        if (!slot_runs(t.sc, mode)) continue;
+        for (int kb = 0; kb < t.steps; ++kb) {
+          const int st = n % STAGES;
+          unsigned char* sa = smem + st * G::kStageBytes;
+          unsigned char* sb = sa + NSL * A_PLANE;
+          if (!mbar_wait(&ctl->empty[st], ((n / STAGES) & 1) ^ 1, abort_flag, wait_cycles)) break;
+          mbar_expect_tx(&ctl->full[st], G::kStageBytes);
 #pragma unroll
-          for (int p = 0; p < NS; ++p) tma_load_2d(sa + p * A_PLANE, ma, &ctl->full[stage], kb * BK, p * v.M + m0);
+          for (int p = 0; p < NSL; ++p)
+            tma_load_2d(sa + p * A_PLANE, t.ma, &ctl->full[st], kb * BK, p * t.M + t.m0);
 #pragma unroll
-          for (int p = 0; p < NS; ++p) tma_load_2d(sb + p * B_PLANE, mb, &ctl->full[stage], kb * BK, p * v.N + n0);
-          ++issued;
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
+          for (int p = 0; p < NSL; ++p)
+            tma_load_2d(sb + p * G::kBPlane, t.mb, &ctl->full[st], kb * BK, p * t.N + t.n0);
+          ++n;
         }
       }
       if (*abort_flag) {
-        // let the copies already issued (at most one per ring slot) land before the CTA leaves
-        int s = stage;
-        uint32_t ph = phase;
-        for (int k = 0; k < STAGES && k < issued; ++k) {
-          if (s == 0) {
-            s = STAGES - 1;
-            ph ^= 1;
-          } else {
-            --s;
-          }
-          const long long t0 = clock64();
-          while (!mbar_try(&ctl->full[s], ph) && clock64() - t0 < kWaitCycles / 4) {
-          }
+        // let the copies already issued (the last into each stage) land before the CTA leaves
+        const long long t0 = clock64();
+        for (int s = 0; s < STAGES; ++s) {
+          const int k = (n - s + STAGES - 1) / STAGES;  // steps issued into stage s
+          if (k > 0)
+            while (!mbar_try(&ctl->full[s], (k - 1) & 1) && clock64() - t0 < kWaitCycles / 4) {
+            }
         }
       }
     }
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      int stage = 0, chunk = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x) {
-        const WorkItem it = items[w];
-        const SlotDesc& S = slots[it.slot];
-        if (!slot_runs(S.sc, mode)) continue;
-        const TcStage v = tc_stage(S, STAGE);
-        for (int kb = 0; kb < v.K / BK; ++kb) {
-          const int half_kb = kb % KPC;  // position inside the accumulation block
-          const int cb = chunk % kChunks;
-          if ((half_kb == 0 &&
-               !mbar_wait(&ctl->tempty[cb], ((chunk / kChunks) & 1) ^ 1, abort_flag, wait_cycles)) ||
-              !mbar_wait(&ctl->full[stage], phase, abort_flag, wait_cycles)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t dset = tmem_base + cb * kSetCols;
-          const uint32_t sa = smem_u32(smem + stage * STAGE_BYTES);
-          const uint32_t sb = sa + NS * A_PLANE;
+    // the whole warp runs the loop, so that the descriptors stay in uniform registers; one elected
+    // lane issues
+    const bool elected = elect_one();
+    int n = 0, chunk = 0;
+    bool ok = true;
+    const SlotScalars* sc = nullptr;
+    int k_tile = 0;
+    auto tile_of = [&](int w) {
+      const SlotDesc& S = slots[items[w].slot];
+      sc = S.sc;
+      k_tile = tc_stage(S, STAGE).K;
+    };
+    if (blockIdx.x < total) tile_of(blockIdx.x);
+    pdl_wait();
+    for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+      if (w != blockIdx.x) tile_of(w);
+      if (!__any_sync(0xffffffffu, slot_runs(sc, mode))) continue;
+      const int steps = __reduce_max_sync(0xffffffffu, k_tile / BK);
+      for (int kb = 0; kb < steps; ++kb) {
+        const int half_kb = kb % KPC;  // position inside the accumulation block
+        const int cb = chunk % kChunks, st = n % STAGES;
+        bool got = half_kb != 0 || mbar_wait(&ctl->tempty[cb], ((chunk / kChunks) & 1) ^ 1, abort_flag, wait_cycles);
+        got = got && mbar_wait(&ctl->full[st], (n / STAGES) & 1, abort_flag, wait_cycles);
+        ok = __all_sync(0xffffffffu, got);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t dset = tmem_base + cb * G::kSetCols;
+        const uint64_t ad = sdesc(smem_u32(smem + st * G::kStageBytes));
+        const uint64_t bd = sdesc(smem_u32(smem + st * G::kStageBytes + NSL * A_PLANE));
+        if (elected) {
+          // slice pa of A against the B slices 0 .. NSL-1-pa stacked along N (adjacent in shared
+          // memory): one MMA adds A_pa B_pb to the accumulator of order pa + pb for every pb,
+          // since the order accumulators are adjacent in TMEM the same way; the first MMA of an
+          // accumulation block (pa = 0) starts all orders afresh
 #pragma unroll
-          for (int j = 0; j < BK / 16; ++j) {
+            for (int j = 0; j < BK / 16; ++j)
 #pragma unroll
-            for (int pa = 0; pa < NS; ++pa) {
-              // slice pa of A against the B slices 0 .. NS-1-pa stacked along N (adjacent in
-              // shared memory): one MMA adds A_pa B_pb to the accumulator of order pa + pb for
-              // every pb, since the order accumulators are adjacent in TMEM the same way
-              const uint64_t ad = sdesc(sa + pa * A_PLANE) + 2 * j;
-              const uint64_t bd = sdesc(sb) + 2 * j;
-              // the first MMA of an accumulation block (pa = 0) starts all NS orders afresh
-              umma(dset + pa * BN, ad, bd, idesc_f16(BF16, BM, (NS - pa) * BN),
-                   (half_kb > 0 || j > 0 || pa > 0) ? 1u : 0u);
-            }
-          }
-          umma_commit(&ctl->empty[stage]);
-          if (half_kb == KPC - 1) {
-            umma_commit(&ctl->tfull[cb]);
-            ++chunk;
-          }
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
+              for (int pa = 0; pa < NSL; ++pa)
+                umma(dset + pa * BN, ad + ((pa * A_PLANE) >> 4) + 2 * j, bd + 2 * j, idesc_f16(BF16, BM, (NSL - pa) * BN),
+                     (half_kb > 0 || j > 0 || pa > 0) ? 1u : 0u);
+          umma_commit(&ctl->empty[st]);
+          if (half_kb == KPC - 1) umma_commit(&ctl->tfull[cb]);
         }
+        ++n;
+        if (half_kb == KPC - 1) ++chunk;
       }
+    }
+    if (elected) {
       // all MMAs issued by this thread complete before TMEM can be released
       umma_commit(&ctl->drain);
       const long long t0 = clock64();
@@ -398,12 +464,24 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   } else {
     // ------------------------------------------------------------------ epilogue
     const int quarter = warp & 3;            // TMEM lanes 32*quarter .. +31
-    const int group = (warp - 2) >> 2;       // columns kEpiCols*group .. +kEpiCols-1 of the tile
     const int ew = warp - 2;
-    const int row = quarter * 32 + lane;
+    const int group = ew >> 2;               // columns 32 cb + 8 group .. + 7 of the tile, cb < kCb
+    // the thread's rows of the quarter: 8 rb + t4, rb = 0..3; its columns: 2 tc + e, e = 0, 1, of each
+    // of the group's column blocks (one packed pair per rb and cb)
+    const int t4 = lane >> 2, tc = lane & 3;
     const bool col_lane = lane < kEpiCols;   // lanes that own one of the warp's columns
     int chunk = 0;
-    for (int w = blockIdx.x; w < total && !*abort_flag; w += gridDim.x) {
+    if (blockIdx.x < total) {
+      // the first tile's descriptor into this SM's L1
+      const SlotDesc& S = slots[items[blockIdx.x].slot];
+      if (lane < static_cast<int>((sizeof(SlotDesc) + 127) / 128)) {
+        const unsigned first = ld_keep(reinterpret_cast<const char*>(&S) + 128 * lane);
+        if (first == 0x7fedcba9u) __nanosleep(1);  // the load has a use
+      }
+    }
+    pdl_wait();
+    // the epilogue warps leave the list only together, at a vote: after an abort their waits fail
+    for (int w = blockIdx.x; w < total; w += gridDim.x) {
       const WorkItem it = items[w];
       const SlotDesc& S = slots[it.slot];
       SlotScalars* sc = S.sc;
@@ -411,16 +489,16 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
       const TcStage v = tc_stage(S, STAGE);
       const int mt = v.M / BM;
       const int m0 = (it.tile % mt) * BM, n0 = (it.tile / mt) * BN;
-      const int m = m0 + row;
-      const int ncol0 = n0 + group * kEpiCols;
+      const int mq = m0 + 32 * quarter;          // first row of the quarter
+      const int ng = n0 + 8 * group;             // first column of the group (block cb: + 32 cb)
+      const int n_mine = ng + 32 * (lane >> 3) + (lane & 7);  // a column lane's column
       const int kblocks = v.K / KC;
       if (STAGE == 3 && col_lane && !S.mir_out) {
         // the r, q and mask entries read after the last k-block: start them towards L2 now
-        const int n = ncol0 + lane;
-        const int mr = min(m0 + 32 * quarter, S.nx - 1);
-        if (n < S.ny && m0 + 32 * quarter < S.nx) {
-          const size_t g = static_cast<size_t>(n) * S.nx + mr;
-          const size_t g1 = static_cast<size_t>(n) * S.nx + min(mr + 31, S.nx - 1);
+        const int n = n_mine;
+        if (n < S.ny && mq < S.nx) {
+          const size_t g = static_cast<size_t>(n) * S.nx + mq;
+          const size_t g1 = static_cast<size_t>(n) * S.nx + min(mq + 31, S.nx - 1);
           asm volatile("prefetch.global.L2 [%0];" ::"l"(S.r + g));
           asm volatile("prefetch.global.L2 [%0];" ::"l"(S.r + g1));
           asm volatile("prefetch.global.L2 [%0];" ::"l"(S.q + g));
@@ -428,272 +506,291 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
           asm volatile("prefetch.global.L2 [%0];" ::"l"(S.mask + g));
         }
       }
-      // stage 1's eigenvalues, read now so their latency hides behind the k-blocks
-      // and everything else the weights read from the descriptor, so that nothing is loaded after
-      // the k-blocks: the row's flags, and per column lane a flag word (bit 0: the column is in the
-      // grid, bit 1: it is in the low-mode block) that the weight loop takes by shuffles
-      float lamx_m = 0.f, lamy_mine = 0.f, wnorm = 0.f;
-      bool row_in = false, row_low = false;
-      uint32_t col_flags = 0;
+      // stage 1's eigenvalues, read now (the MMA waits hide their latency) with the grid's edge
+      // folded in: a row or column outside it makes the eigenvalue sum negative, and its weight zero
+      float lamx[4], lamy[2 * kCb], wnorm = 0.f;
       if (STAGE == 1) {
-        // issued here, not where the compiler would sink them: the MMA waits hide their latency
-        row_in = m < S.nx;
-        row_low = m < S.lowm_x;
-        if (row_in) lamx_m = ld_early(S.lamx + m);
-        const int n_mine = ncol0 + lane;
-        if (col_lane && n_mine < S.ny) {
-          lamy_mine = ld_early(S.lamy + n_mine);
-          col_flags = 1u | (n_mine < S.lowm_y ? 2u : 0u);
+#pragma unroll
+        for (int rb = 0; rb < 4; ++rb) {
+          const int m = mq + 8 * rb + t4;
+          lamx[rb] = m < S.nx ? ld_early(S.lamx + m) : -INFINITY;
+        }
+#pragma unroll
+        for (int c = 0; c < 2 * kCb; ++c) {
+          const int n = ng + 32 * (c >> 1) + 2 * tc + (c & 1);
+          lamy[c] = n < S.ny ? ld_early(S.lamy + n) : -INFINITY;
         }
         wnorm = ld_early(&S.wnorm);
       }
-      const int8_t* ea_row = S.tc_e[STAGE] + static_cast<size_t>(m) * kblocks;
-      const int8_t* eb_col = S.tc_eb[STAGE] + static_cast<size_t>(ncol0 + (col_lane ? lane : 0)) * kblocks;
-      // compensated (hi, lo) pairs of the warp's columns, two columns per packed register pair
-      float2 hi[kEpiCols / 2], lo[kEpiCols / 2];
+      const int8_t* ea_row = S.tc_e[STAGE] + static_cast<size_t>(mq + lane) * kblocks;
+      const int8_t* eb_col = S.tc_eb[STAGE] + static_cast<size_t>(col_lane ? n_mine : ng) * kblocks;
+      // compensated (hi, lo) pairs, one packed register pair per (rb, cb)
+      float2 hi[kCb][4], lo[kCb][4];
 #pragma unroll
-      for (int i = 0; i < kEpiCols / 2; ++i) {
-        hi[i] = make_float2(0.f, 0.f);
-        lo[i] = make_float2(0.f, 0.f);
-      }
-      bool fail_all = false;
-      for (int kb = 0; kb < kblocks; ++kb) {
-        const int cb = chunk % kChunks;
-        // scale of the block sums: 2^(E_A + E_B - 16), as an exact product of two powers of two
-        const float sa = pow2f(static_cast<int>(ea_row[kb]) - 16);
-        const float sb_mine = pow2f(eb_col[kb]);
-        // all epilogue warps leave together if any of them gave up waiting
-        const uint32_t fail =
-            mbar_wait(&ctl->tfull[cb], (chunk / kChunks) & 1, abort_flag, wait_cycles) ? 0u : 1u;
-        uint32_t any_fail;
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t"
-            "setp.ne.u32 p, %1, 0;\n\t"
-            "bar.red.or.pred q, 1, %2, p;\n\t"
-            "selp.u32 %0, 1, 0, q;\n\t}"
-            : "=r"(any_fail)
-            : "r"(fail), "r"(32 * kEpiWarps)
-            : "memory");
-        if (any_fail) {
-          fail_all = true;
-          break;
+      for (int cb = 0; cb < kCb; ++cb)
+#pragma unroll
+        for (int rb = 0; rb < 4; ++rb) {
+          hi[cb][rb] = make_float2(0.f, 0.f);
+          lo[cb][rb] = make_float2(0.f, 0.f);
         }
+      bool fail = false;
+      for (int kb = 0; kb < kblocks; ++kb) {
+        const int cs = chunk % kChunks;
+        // factors of the block sums, 2^(E_A - 16) of the lane's row and 2^E_B of its column
+        const float sa_mine = pow2f(static_cast<int>(ea_row[kb]) - 16);
+        const float sb_mine = pow2f(eb_col[kb]);
+        // a warp that gives up waiting leaves with the others at the vote after the k-blocks
+        if (!fail) fail = !mbar_wait(&ctl->tfull[cs], (chunk / kChunks) & 1, abort_flag, wait_cycles);
         tc_fence_after();
-        const uint32_t base =
-            tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + cb * kSetCols + group * kEpiCols;
+        float sa[4];
 #pragma unroll
-        for (int hc = 0; hc < kEpiCols / kLdCols; ++hc) {
-          uint32_t s0[kLdCols], s1[kLdCols], s2[kLdCols], s3[kLdCols];
-          tmem_ld<kLdCols>(base + hc * kLdCols, s0);
-          tmem_ld<kLdCols>(base + BN + hc * kLdCols, s1);
-          tmem_ld<kLdCols>(base + 2 * BN + hc * kLdCols, s2);
-          tmem_ld<kLdCols>(base + 3 * BN + hc * kLdCols, s3);
-          tmem_wait_ld();
-          if (hc == kEpiCols / kLdCols - 1) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&ctl->tempty[cb]);
-          }
-          // two columns per step on packed FP32x2; per column the operations and their order
-          // are those of the scalar merge
-          const float2 q8 = make_float2(0.00390625f, 0.00390625f);
+        for (int rb = 0; rb < 4; ++rb) sa[rb] = __shfl_sync(0xffffffffu, sa_mine, 8 * rb + t4);
+        const uint32_t base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + cs * G::kSetCols + ng - n0;
 #pragma unroll
-          for (int i = 0; i < kLdCols; i += 2) {
-            const int c = hc * kLdCols + i;
-            const float2 scl = mul2(sa, make_float2(__shfl_sync(0xffffffffu, sb_mine, c),
-                                                    __shfl_sync(0xffffffffu, sb_mine, c + 1)));
-            const float2 v0 = make_float2(__uint_as_float(s0[i]), __uint_as_float(s0[i + 1]));
-            const float2 v1 = make_float2(__uint_as_float(s1[i]), __uint_as_float(s1[i + 1]));
-            const float2 v2 = make_float2(__uint_as_float(s2[i]), __uint_as_float(s2[i + 1]));
-            const float2 v3 = make_float2(__uint_as_float(s3[i]), __uint_as_float(s3[i + 1]));
-            // orders 1..3 combined first: their roundings are 2^-24 of terms 2^-8 below hi
-            const float2 w = __ffma2_rn(v3, q8, v2);
-            const float2 u = __ffma2_rn(w, q8, v1);
-            const float2 t0 = __fmul2_rn(v0, scl);
-            const float2 t1 = __fmul2_rn(u, __fmul2_rn(scl, q8));
-            float2 er;
-            two_sum2(hi[c / 2], t0, hi[c / 2], er);
-            lo[c / 2] = add2(lo[c / 2], add2(er, t1));
+        for (int cb = 0; cb < kCb; ++cb) {
+          const float2 sb = make_float2(__shfl_sync(0xffffffffu, sb_mine, 8 * cb + 2 * tc),
+                                        __shfl_sync(0xffffffffu, sb_mine, 8 * cb + 2 * tc + 1));
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t o[NSL][4];
+#pragma unroll
+            for (int d = 0; d < NSL; ++d)
+              tmem_ld_frag(base + (static_cast<uint32_t>(16 * h) << 16) + d * BN + 32 * cb, o[d]);
+            tmem_wait_ld();
+            if (cb == kCb - 1 && h == 1) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&ctl->tempty[cs]);
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+              const int rb = 2 * h + r;
+              float2 x[NSL];
+#pragma unroll
+              for (int d = 0; d < NSL; ++d)
+                x[d] = make_float2(__uint_as_float(o[d][2 * r]), __uint_as_float(o[d][2 * r + 1]));
+              merge_orders<NSL>(x, mul2(sa[rb], sb), hi[cb][rb], lo[cb][rb]);
+            }
           }
         }
         ++chunk;
       }
-      if (fail_all) break;
-      // the column sums as normalised double-float pairs (val, vlo)
-      float val[kEpiCols], vlo[kEpiCols];
+      // the sums as normalised double-float pairs
 #pragma unroll
-      for (int i = 0; i < kEpiCols / 2; ++i) {
-        const f2x2 v = df_norm2(hi[i], lo[i]);
-        val[2 * i] = v.hi.x;
-        val[2 * i + 1] = v.hi.y;
-        vlo[2 * i] = v.lo.x;
-        vlo[2 * i + 1] = v.lo.y;
-      }
-      if (STAGE == 1) {
-        // weight 1/(lam_y + lam_x)^2 (normalised); lam_y of the warp's columns via shuffles
+      for (int cb = 0; cb < kCb; ++cb)
 #pragma unroll
-        for (int i = 0; i < kEpiCols; ++i) {
-          const float s = __shfl_sync(0xffffffffu, lamy_mine, i) + lamx_m;
-          const uint32_t f = __shfl_sync(0xffffffffu, col_flags, i);
-          // the low block (m < lowm_x, n < lowm_y) comes from the six-slice products instead
-          const bool ok = row_in && (f & 1u) && (s > 0.f) && !(row_low && (f & 2u));
-          const f2 wv = df_mul(f2{val[i], vlo[i]}, spectral_weight_of(wnorm, s));
-          val[i] = ok ? wv.hi : 0.f;
-          vlo[i] = ok ? wv.lo : 0.f;
+        for (int rb = 0; rb < 4; ++rb) {
+          const f2x2 t = df_norm2(hi[cb][rb], lo[cb][rb]);
+          hi[cb][rb] = t.hi;
+          lo[cb][rb] = t.lo;
         }
+      if (STAGE == 1) {
+        // weight 1/(lam_y + lam_x)^2 (normalised); the low block (m < lowm_x, n < lowm_y) comes
+        // from the six-slice products instead
+        const bool low_tile = S.lowm_x != 0 && mq == 0 && ng < kLowM;
+        const int lowx = S.lowm_x, lowy = S.lowm_y;
+#pragma unroll
+        for (int cb = 0; cb < kCb; ++cb)
+#pragma unroll
+          for (int rb = 0; rb < 4; ++rb) {
+            const float s0 = lamy[2 * cb] + lamx[rb], s1 = lamy[2 * cb + 1] + lamx[rb];
+            bool ok0 = s0 > 0.f, ok1 = s1 > 0.f;
+            if (low_tile && 8 * rb + t4 < lowx) {
+              ok0 = ok0 && ng + 32 * cb + 2 * tc >= lowy;
+              ok1 = ok1 && ng + 32 * cb + 2 * tc + 1 >= lowy;
+            }
+            const float2 wt = make_float2(ok0 ? spectral_weight_of(wnorm, s0) : 0.f,
+                                          ok1 ? spectral_weight_of(wnorm, s1) : 0.f);
+            const float2 p = __fmul2_rn(hi[cb][rb], wt);
+            const float2 e = __ffma2_rn(lo[cb][rb], wt, __ffma2_rn(hi[cb][rb], wt, neg2(p)));
+            const f2x2 t = df_norm2(p, e);
+            hi[cb][rb] = t.hi;
+            lo[cb][rb] = t.lo;
+          }
       }
       if (STAGE <= 2) {
-        // block exponents of the next operand: rows n, k-blocks of KC consecutive m (lane quarters
-        // 32q .. 32q+31 of this tile; KC/32 quarters per block, KC <= BM)
-        float av[kEpiCols];
+        // block exponents of the next operand: row n, k-block of the tile's 128 m.  The largest
+        // magnitude of each column: over the thread's rows, then by halving exchanges over the
+        // lanes of equal tc, after which the lane holds one column
+        float mx[2 * kCb];
 #pragma unroll
-        for (int i = 0; i < kEpiCols; ++i) av[i] = fabsf(val[i]);
-        const float mine = column_max<kEpiCols>(av, lane);
-        if (col_lane) ctl->colmax[group][quarter][lane] = mine;
-        epi_bar();
-        float bmax = 0.f;
-        const int q0 = (quarter / (KC / 32)) * (KC / 32);
+        for (int c = 0; c < 2 * kCb; ++c) {
+          mx[c] = 0.f;
+#pragma unroll
+          for (int rb = 0; rb < 4; ++rb)
+            mx[c] = fmaxf(mx[c], fabsf((c & 1) ? hi[c >> 1][rb].y : hi[c >> 1][rb].x));
+        }
+        int col = 2 * tc;
+        if (kCb == 2) {
+          const bool up = (lane & 16) != 0;
+          const float g0 = __shfl_xor_sync(0xffffffffu, up ? mx[0] : mx[2 % (2 * kCb)], 16);
+          const float g1 = __shfl_xor_sync(0xffffffffu, up ? mx[1] : mx[3 % (2 * kCb)], 16);
+          mx[0] = fmaxf(up ? mx[2 % (2 * kCb)] : mx[0], g0);
+          mx[1] = fmaxf(up ? mx[3 % (2 * kCb)] : mx[1], g1);
+          col += up ? 8 : 0;
+        } else {
+#pragma unroll
+          for (int c = 0; c < 2; ++c) mx[c] = fmaxf(mx[c], __shfl_xor_sync(0xffffffffu, mx[c], 16));
+        }
+        {
+          const bool up = (lane & 8) != 0;
+          const float g = __shfl_xor_sync(0xffffffffu, up ? mx[0] : mx[1], 8);
+          mx[0] = fmaxf(up ? mx[1] : mx[0], g);
+          col += up ? 1 : 0;
+        }
+        mx[0] = fmaxf(mx[0], __shfl_xor_sync(0xffffffffu, mx[0], 4));
+        if ((lane & 4) == 0 && (kCb == 2 || (lane & 16) == 0)) ctl->colmax[group][col][quarter] = mx[0];
+        // the staging tile is free once the previous tile's stores have read it
+        if (ew == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        if (epi_vote(fail)) break;
+        int E_mine = 0;
         if (col_lane) {
-#pragma unroll
-          for (int q = 0; q < KC / 32; ++q) bmax = fmaxf(bmax, ctl->colmax[group][q0 + q][lane]);
+          const float4 q = *reinterpret_cast<const float4*>(ctl->colmax[group][lane]);
+          E_mine = block_exp(fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)));
         }
-        const int E_mine = block_exp(bmax);
-        const float s_mine = pow2f(8 - E_mine), is_mine = pow2f(E_mine - 8);
-        // no second barrier before colmax is rewritten: that happens after the next tile's first
-        // k-block, whose failure vote every epilogue warp joins only after these reads
-        const size_t plane = static_cast<size_t>(v.M) * v.N;
-        uint16_t* out = static_cast<uint16_t*>(v.out);
+        // slices, transposed into the staging tile, one 32-column block of the tile at a time: row n of
+        // 64 m (128 bytes), 16-byte chunks permuted by n % 8 (the tensor stores' 128-byte swizzle;
+        // conflict-free here)
+        const void* mo = static_cast<const unsigned char*>(S.tmaps) + 128 * (8 + STAGE);
+        if (ew == 0 && lane == 0) tmap_acquire(mo);
+        const uint32_t so = smem_u32(sO) + (((quarter >> 1) * 32 + 8 * group + (lane & 7)) << 7) +
+                            (((((quarter & 1) << 2) + (lane >> 3)) ^ (lane & 7)) << 4);
 #pragma unroll
-        for (int i = 0; i < kEpiCols; i += 2) {
-          const float2 s2 = make_float2(__shfl_sync(0xffffffffu, s_mine, i), __shfl_sync(0xffffffffu, s_mine, i + 1));
-          const float2 is2 =
-              make_float2(__shfl_sync(0xffffffffu, is_mine, i), __shfl_sync(0xffffffffu, is_mine, i + 1));
-          uint32_t code[NS];
-          slice_codes2_df<BF16>(make_float2(val[i], val[i + 1]), make_float2(vlo[i], vlo[i + 1]), s2,
-                                is2, code);
-          const size_t i0 = static_cast<size_t>(ncol0 + i) * v.M + m, i1 = i0 + v.M;
+        for (int cb = 0; cb < kCb; ++cb) {
+          const int e0 = __shfl_sync(0xffffffffu, E_mine, 8 * cb + 2 * tc);
+          const int e1 = __shfl_sync(0xffffffffu, E_mine, 8 * cb + 2 * tc + 1);
+          const float2 up = make_float2(pow2f(16 - e0), pow2f(16 - e1));
+          const float2 dn = make_float2(-pow2f(e0 - 16), -pow2f(e1 - 16));
+          uint32_t code[4][NSL];
 #pragma unroll
-          for (int q = 0; q < NS; ++q) {
-            out[q * plane + i0] = static_cast<uint16_t>(code[q] & 0xffffu);
-            out[q * plane + i1] = static_cast<uint16_t>(code[q] >> 16);
+          for (int rb = 0; rb < 4; ++rb) slice_codes2_df<BF16, NSL>(hi[cb][rb], lo[cb][rb], up, dn, code[rb]);
+          if (cb > 0) {
+            // the previous column block's stores have read the staging tile
+            if (ew == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            epi_bar();
+          }
+#pragma unroll
+          for (int q = 0; q < NSL; ++q) {
+            const uint32_t f[4] = {code[0][q], code[1][q], code[2][q], code[3][q]};
+            stmatrix4_t(so + (q * 2 * 32 << 7), f);
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          epi_bar();
+          if (ew == 0 && lane == 0) {
+#pragma unroll
+            for (int q = 0; q < NSL; ++q)
+#pragma unroll
+              for (int h = 0; h < 2; ++h)
+                tma_store_2d(mo, smem_u32(sO) + ((q * 2 + h) * 32 << 7), m0 + 64 * h, q * v.N + n0 + 32 * cb);
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           }
         }
-        if (quarter == q0 && col_lane)
-          v.eout[static_cast<size_t>(ncol0 + lane) * (v.M / KC) + (m0 + 32 * quarter) / KC] =
-              static_cast<int8_t>(E_mine);
+        if (quarter == 0 && col_lane)
+          v.eout[static_cast<size_t>(n_mine) * (v.M / KC) + m0 / KC] = static_cast<int8_t>(E_mine);
       } else {
+        if (epi_vote(fail)) break;
         CompDotDF c_rz, c_zq;
-        const bool with_zq = S.mir_out == 0 && (sc->flexible != 0 || mode == 2);
-        if (m < S.nx) {
-          constexpr int kGrp = 8;
-          static_assert(kEpiCols % kGrp == 0, "stage-3 load groups");
+        const bool mir_out = S.mir_out != 0;
+        const bool with_zq = !mir_out && (sc->flexible != 0 || mode == 2);
+        const int nx = S.nx, ny = S.ny;
+        const size_t nn = static_cast<size_t>(nx) * ny;
+        float* __restrict__ zh = S.z;
+        float* __restrict__ zl = S.z_lo;
+        const float* lz = S.lowm_x ? S.low_z : nullptr;
 #pragma unroll
-          for (int g8 = 0; g8 < kEpiCols; g8 += kGrp) {
-            if (S.lowm_x) {
-              // the low-mode part first: the 32-bit stages' result plus zl, one double-float value
-              const size_t nn = static_cast<size_t>(S.nx) * S.ny;
-              float wh[kGrp], wl[kGrp];
+        for (int cb = 0; cb < kCb; ++cb) {
+          // the eight values' nodes: g < 0 outside the grid
+          int g[4][2];
 #pragma unroll
-              for (int i = 0; i < kGrp; ++i) {
-                const int n = ncol0 + g8 + i;
-                const size_t g = static_cast<size_t>(n < S.ny ? n : 0) * S.nx + m;
-                wh[i] = S.low_z[g];
-                wl[i] = S.low_z[nn + g];
-              }
+          for (int rb = 0; rb < 4; ++rb)
 #pragma unroll
-              for (int i = 0; i < kGrp; ++i) {
-                const f2 zsum = df_add(f2{val[g8 + i], vlo[g8 + i]}, f2{wh[i], wl[i]});
-                val[g8 + i] = zsum.hi;
-                vlo[g8 + i] = zsum.lo;
-              }
+            for (int e = 0; e < 2; ++e) {
+              const int m = mq + 8 * rb + t4, n = ng + 32 * cb + 2 * tc + e;
+              g[rb][e] = (m < nx && n < ny) ? n * nx + m : -1;
             }
-            if (S.mir_out) {
-              // one mirror class of a folded slot: its result g, unmasked (k_unfold combines the
-              // classes, masks and forms the dot products)
+          if (lz) {
+            // the low-mode part first: the 32-bit stages' result plus zl, one double-float value
+            float wh[4][2], wl[4][2];
 #pragma unroll
-              for (int i = 0; i < kGrp; ++i) {
-                const int n = ncol0 + g8 + i;
-                if (n < S.ny) {
-                  S.z[n * S.nx + m] = val[g8 + i];
-                  S.z_lo[n * S.nx + m] = vlo[g8 + i];
-                }
+            for (int rb = 0; rb < 4; ++rb)
+#pragma unroll
+              for (int e = 0; e < 2; ++e) {
+                const int gi = max(g[rb][e], 0);
+                wh[rb][e] = lz[gi];
+                wl[rb][e] = lz[nn + gi];
               }
-              continue;
-            }
-            float rv[kGrp], rl[kGrp], qv[kGrp], ql[kGrp];
-            uint8_t mk[kGrp];
 #pragma unroll
-            for (int i = 0; i < kGrp; ++i) {  // issue the group's loads together
-              const int n = ncol0 + g8 + i;
-              const int g = (n < S.ny ? n : 0) * S.nx + m;
-              rv[i] = S.r[g];
-              rl[i] = S.r_lo[g];
-              // z.q enters only the flexible beta
-              qv[i] = with_zq ? S.q[g] : 0.f;
-              ql[i] = with_zq ? S.q_lo[g] : 0.f;
-              mk[i] = n < S.ny ? S.mask[g] : 0;
-            }
-#pragma unroll
-            for (int i = 0; i < kGrp; ++i) {
-              const int n = ncol0 + g8 + i;
-              if (n < S.ny) {
-                const float zh = mk[i] ? val[g8 + i] : 0.f;
-                const float zl = mk[i] ? vlo[g8 + i] : 0.f;
-                S.z[n * S.nx + m] = zh;
-                S.z_lo[n * S.nx + m] = zl;
-                c_rz.add(rv[i], rl[i], zh, zl);
-                c_zq.add(zh, zl, qv[i], ql[i]);
-              }
+            for (int rb = 0; rb < 4; ++rb) {
+              const f2 a = df_add(f2{hi[cb][rb].x, lo[cb][rb].x}, f2{wh[rb][0], wl[rb][0]});
+              const f2 b = df_add(f2{hi[cb][rb].y, lo[cb][rb].y}, f2{wh[rb][1], wl[rb][1]});
+              hi[cb][rb] = make_float2(a.hi, b.hi);
+              lo[cb][rb] = make_float2(a.lo, b.lo);
             }
           }
-        }
-        if (S.mir_out) continue;  // a class problem leaves no partial sums
-        // tile partials of r.z and z.q (FP32-compensated inside the warp)
+          if (mir_out) {
+            // one mirror class of a folded slot: its result g, unmasked (k_unfold combines the
+            // classes, masks and forms the dot products)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          float e;
-          const float a1 = __shfl_xor_sync(0xffffffffu, c_rz.s, o), a2 = __shfl_xor_sync(0xffffffffu, c_rz.c, o);
-          two_sum(c_rz.s, a1, c_rz.s, e);
-          c_rz.c = __fadd_rn(c_rz.c, __fadd_rn(a2, e));
-          const float b1 = __shfl_xor_sync(0xffffffffu, c_zq.s, o), b2 = __shfl_xor_sync(0xffffffffu, c_zq.c, o);
-          two_sum(c_zq.s, b1, c_zq.s, e);
-          c_zq.c = __fadd_rn(c_zq.c, __fadd_rn(b2, e));
+            for (int rb = 0; rb < 4; ++rb) {
+              if (g[rb][0] >= 0) {
+                zh[g[rb][0]] = hi[cb][rb].x;
+                zl[g[rb][0]] = lo[cb][rb].x;
+              }
+              if (g[rb][1] >= 0) {
+                zh[g[rb][1]] = hi[cb][rb].y;
+                zl[g[rb][1]] = lo[cb][rb].y;
+              }
+            }
+            continue;
+          }
+          float rv[4][2], rl[4][2], qv[4][2], ql[4][2];
+          uint8_t mk[4][2];
+#pragma unroll
+          for (int rb = 0; rb < 4; ++rb)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {  // issue the block's loads together
+              const int gi = max(g[rb][e], 0);
+              rv[rb][e] = S.r[gi];
+              rl[rb][e] = S.r_lo[gi];
+              // z.q enters only the flexible beta
+              qv[rb][e] = with_zq ? S.q[gi] : 0.f;
+              ql[rb][e] = with_zq ? S.q_lo[gi] : 0.f;
+              mk[rb][e] = g[rb][e] >= 0 ? S.mask[gi] : 0;
+            }
+#pragma unroll
+          for (int rb = 0; rb < 4; ++rb)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              if (g[rb][e] < 0) continue;
+              const float a = mk[rb][e] ? (e ? hi[cb][rb].y : hi[cb][rb].x) : 0.f;
+              const float b = mk[rb][e] ? (e ? lo[cb][rb].y : lo[cb][rb].x) : 0.f;
+              zh[g[rb][e]] = a;
+              zl[g[rb][e]] = b;
+              c_rz.add(rv[rb][e], rl[rb][e], a, b);
+              if (with_zq) c_zq.add(a, b, qv[rb][e], ql[rb][e]);
+            }
         }
-        if (lane == 0) {
-          ctl->red[ew][0] = c_rz.s;
-          ctl->red[ew][1] = c_rz.c;
-          ctl->red[ew][2] = c_zq.s;
-          ctl->red[ew][3] = c_zq.c;
-        }
+        if (mir_out) continue;  // a class problem leaves no partial sums
+        // tile partials of r.z and z.q: butterflies in the warps, then across them by warp 0;
+        // k_prec_finish forms rho and beta from them
+        group_sum_pair<32>(c_rz.s, c_rz.c);
+        if (with_zq) group_sum_pair<32>(c_zq.s, c_zq.c);
+        if (lane == 0) ctl->red[ew] = make_float4(c_rz.s, c_rz.c, c_zq.s, c_zq.c);
         epi_bar();
         if (ew == 0) {
-          // the warps' compensated pairs, summed the same way across lanes 0 .. kEpiWarps-1
-          CompDot t_rz, t_zq;
-          if (lane < kEpiWarps) {
-            t_rz.s = ctl->red[lane][0];
-            t_rz.c = ctl->red[lane][1];
-            t_zq.s = ctl->red[lane][2];
-            t_zq.c = ctl->red[lane][3];
-          }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            float e;
-            const float a1 = __shfl_xor_sync(0xffffffffu, t_rz.s, o), a2 = __shfl_xor_sync(0xffffffffu, t_rz.c, o);
-            two_sum(t_rz.s, a1, t_rz.s, e);
-            t_rz.c = __fadd_rn(t_rz.c, __fadd_rn(a2, e));
-            const float b1 = __shfl_xor_sync(0xffffffffu, t_zq.s, o), b2 = __shfl_xor_sync(0xffffffffu, t_zq.c, o);
-            two_sum(t_zq.s, b1, t_zq.s, e);
-            t_zq.c = __fadd_rn(t_zq.c, __fadd_rn(b2, e));
-          }
-          // tile partials; k_prec_finish forms rho and beta from them
+          const float4 t = ctl->red[lane % kEpiWarps];
+          float sv = t.x, cv = t.y, sq = t.z, cq = t.w;
+          group_sum_pair<kEpiWarps>(sv, cv);
+          if (with_zq) group_sum_pair<kEpiWarps>(sq, cq);
           if (lane == 0) {
-            S.part[it.tile * 4 + 2] = t_rz.value();
-            S.part[it.tile * 4 + 3] = t_zq.value();
+            S.part[it.tile * 4 + 2] = (double)sv + (double)cv;
+            S.part[it.tile * 4 + 3] = with_zq ? (double)sq + (double)cq : 0.0;
           }
         }
-        // ctl->red is rewritten only after the next tile's first k-block (see stages 0..2)
+        // ctl->red is rewritten only after the next tile's vote, which this warp joins later
       }
     }
+    if (STAGE <= 2 && ew == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
 
   tc_fence_before();
@@ -756,7 +853,7 @@ k_tc_prepare(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ it
 #pragma unroll
       for (int k = 0; k < kPairs; ++k) amax = fmaxf(amax, fmaxf(fabsf(v[j][k].x), fabsf(v[j][k].y)));
       const int E = block_exp(warp_max(amax));
-      const float s = pow2f(8 - E), is = pow2f(E - 8);
+      const float s = pow2f(16 - E), is = -pow2f(E - 16);
 #pragma unroll
       for (int k = 0; k < kPairs; ++k) {
         const size_t idx = (static_cast<size_t>(y) * S.nxp + x0 + 64 * k + 2 * lane) / 2;
@@ -862,7 +959,7 @@ k_tc_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
 #pragma unroll
       for (int k = 0; k < 2; ++k) amax = fmaxf(amax, fmaxf(fabsf(ch[c][k].x), fabsf(ch[c][k].y)));
       const int E = block_exp(warp_max(amax));
-      const float up = pow2f(8 - E), is = pow2f(E - 8);
+      const float up = pow2f(16 - E), is = -pow2f(E - 16);
       const size_t plane = static_cast<size_t>(T.nyp) * T.nxp;
       uint32_t* out32 = static_cast<uint32_t*>(T.tc_r);
 #pragma unroll
@@ -1010,15 +1107,6 @@ struct LowCtl {
   uint32_t tmem;
   int abort_flag;
 };
-
-// Exponent of a block whose largest magnitude is amax: amax < 2^E and amax 2^(8-E) < 255.5.
-__device__ __forceinline__ int low_block_exp(float amax) {
-  if (!(amax > 0.f)) return 0;
-  int e;
-  frexpf(amax, &e);
-  if (amax * pow2f(8 - e) >= 255.5f) ++e;
-  return max(e, -90);
-}
 
 template <bool BF16>
 __global__ void __launch_bounds__(kLowThreads, 1)
@@ -1423,11 +1511,11 @@ k_low_inv(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
 
 // The slices of one double-float value on a single lane (the packed routine on lane x).
 template <bool BF16>
-__device__ __forceinline__ void slice_codes_df(float vh, float vl, float s, float is,
+__device__ __forceinline__ void slice_codes_df(float vh, float vl, float up, float dn,
                                                uint16_t (&code)[kLowNS]) {
   uint32_t c2[kLowNS];
-  slice_codes2_df<BF16, kLowNS>(make_float2(vh, 0.f), make_float2(vl, 0.f), make_float2(s, s),
-                                make_float2(is, is), c2);
+  slice_codes2_df<BF16, kLowNS>(make_float2(vh, 0.f), make_float2(vl, 0.f), make_float2(up, up),
+                                make_float2(dn, dn), c2);
 #pragma unroll
   for (int k = 0; k < kLowNS; ++k) code[k] = static_cast<uint16_t>(c2[k] & 0xffffu);
 }
@@ -1498,9 +1586,9 @@ k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         const int x = xb + rb + r;
         const CompDotDF2& d = acc[r / 2];
         const f2 j = (r & 1) ? df_norm(d.s.y, d.c.y) : df_norm(d.s.x, d.c.x);
-        const int E = low_block_exp(warp_max(fabsf(j.hi)));
+        const int E = block_exp(warp_max(fabsf(j.hi)));
         uint16_t code[kLowNS];
-        slice_codes_df<BF16>(j.hi, j.lo, pow2f(8 - E), pow2f(E - 8), code);
+        slice_codes_df<BF16>(j.hi, j.lo, pow2f(16 - E), -pow2f(E - 16), code);
 #pragma unroll
         for (int p = 0; p < kLowNS; ++p) {
           jt[p * plane + static_cast<size_t>(x) * kLowK3 + lane] = code[p];
@@ -1515,17 +1603,18 @@ k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
 
 template <bool BF16, int STAGE>
 cudaError_t set_attr() {
-  return cudaFuncSetAttribute(k_prec_tc<BF16, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+  return cudaFuncSetAttribute(k_prec_tc<BF16, STAGE, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              TcGeom<NS>::kSmem);
 }
 
 template <bool BF16>
 void launch_all(const LaunchCfg& c, int stage, int mode, int* err) {
   const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
   switch (stage) {
-    case 0: launch_cfg(c, k_prec_tc<BF16, 0>, c.grid, kThreads, SMEM_BYTES, c.slots, c.items, c.n_items, mode, err, wc); break;
-    case 1: launch_cfg(c, k_prec_tc<BF16, 1>, c.grid, kThreads, SMEM_BYTES, c.slots, c.items, c.n_items, mode, err, wc); break;
-    case 2: launch_cfg(c, k_prec_tc<BF16, 2>, c.grid, kThreads, SMEM_BYTES, c.slots, c.items, c.n_items, mode, err, wc); break;
-    default: launch_cfg(c, k_prec_tc<BF16, 3>, c.grid, kThreads, SMEM_BYTES, c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 0: launch_cfg(c, k_prec_tc<BF16, 0, NS>, c.grid, kThreads, TcGeom<NS>::kSmem, c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 1: launch_cfg(c, k_prec_tc<BF16, 1, NS>, c.grid, kThreads, TcGeom<NS>::kSmem, c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 2: launch_cfg(c, k_prec_tc<BF16, 2, NS>, c.grid, kThreads, TcGeom<NS>::kSmem, c.slots, c.items, c.n_items, mode, err, wc); break;
+    default: launch_cfg(c, k_prec_tc<BF16, 3, NS>, c.grid, kThreads, TcGeom<NS>::kSmem, c.slots, c.items, c.n_items, mode, err, wc); break;
   }
 }
 
@@ -1538,11 +1627,11 @@ bool tc_supported() {
     cudaGetLastError();
     return false;
   }
-  if (p.major != 10 || p.sharedMemPerBlockOptin < static_cast<size_t>(SMEM_BYTES)) return false;
+  if (p.major != 10 || p.sharedMemPerBlockOptin < static_cast<size_t>(TcGeom<NS>::kSmem)) return false;
   // one CTA of kThreads threads at kMaxRegs registers each must fit an SM
   int blocks = 0;
   if (set_attr<true, 0>() != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_prec_tc<true, 0>, kThreads, SMEM_BYTES) !=
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_prec_tc<true, 0, NS>, kThreads, TcGeom<NS>::kSmem) !=
           cudaSuccess) {
     cudaGetLastError();
     return false;
