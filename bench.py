@@ -234,7 +234,7 @@ class ClockSampler:
 # ----------------------------------------------------------------------------------------------
 def kernel_hash(kind, prec="fp32"):
     if kind.startswith("prec") or kind in ("split", "fold", "unfold") or kind.startswith("low"):
-        f = "kernels_gemm_simt.cu" if prec == "fp32" else "kernels_gemm_tc.cu"
+        f = "kernels_gemm_tc.cu"
     else:
         f = "kernels_grid.cu"
     with open(os.path.join(CSRC, f), "rb") as fh:

@@ -54,10 +54,10 @@ thread_local std::string g_last_error;
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct PlanDev {
-  int n = 0, np = 0, bc = 0;
+  int n = 0, np = 0, bc = 0, ns = 0;
   int cls = -1;   // -1: the axis basis; 0 / 1: its even / odd mirror class (n = ceil(nfull / 2))
   int nfull = 0;  // nodes of the axis
-  float* q = nullptr;   // [2][np][np]: hi plane, lo plane
+  float* q = nullptr;   // [2][np][np]: hi plane, lo plane (3-D CUDA-core products only)
   float* qt = nullptr;  // [2][np][np]
   std::vector<double> lam;
   void* tc = nullptr;   // tensor-core operand planes: [Q planes][Q^T planes], 2-byte elements
@@ -144,8 +144,8 @@ struct ext_ctx {
   std::map<int, PlanDev> plans;
   std::map<std::string, Workspace*> ws;
   std::mutex api_mu;  // serialises ext_solve* and the serving worker on the stream
-  bool tc = false;    // mixed modes: tensor-core preconditioner
-  int split = 0;      // type of the exact integer operand slices: 0 = FP16, 1 = BF16
+  int ns = 4;         // integer slices per transform operand: 4 (mixed modes) or 6 (FP32 mode)
+  int split = 0;      // their type: 0 = FP16, 1 = BF16
   int* d_err = nullptr;   // device flag raised by a bounded wait that ran out
   int* h_err = nullptr;   // pinned copy
   // launch accounting and optional per-kernel timing (ext_options.profile)
@@ -229,11 +229,13 @@ static int make_tmap_2d(CUtensorMap* m, void* base, CUtensorMapDataType type, ui
   return EXT_OK;
 }
 
-// Tensor-core operand planes: `rows` rows of `inner` 16-bit slices; boxes of 64 x box_rows,
-// 128-byte swizzle.
-static int make_tmap(CUtensorMap* m, void* base, bool bf16, uint64_t inner, uint64_t rows, uint32_t box_rows) {
+// Tensor-core operand planes: `rows` rows of `inner` 16-bit slices; boxes of box_k x box_rows, one
+// swizzle atom wide (box_k = 64: 128 bytes; 32: 64 bytes).
+static int make_tmap(CUtensorMap* m, void* base, bool bf16, uint64_t inner, uint64_t rows, uint32_t box_rows,
+                     uint32_t box_k = 64) {
   return make_tmap_2d(m, base, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
-                      inner, rows, 64, box_rows, CU_TENSOR_MAP_SWIZZLE_128B);
+                      inner, rows, box_k, box_rows,
+                      box_k == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 // Stencil windows: the hi and lo planes of z, p[0], p[1] as FP32 boxes of the tile plus its halo
@@ -279,10 +281,9 @@ static int block_exp_host(const double* v, size_t stride, int count) {
 // Q and Q^T of one axis (n nodes, rule bc) as block-scaled slices, zero-padded to np x np, with
 // their exponents: h = [Q slices (NS planes)][Q^T slices (NS planes)], each plane [np][np];
 // ex = [exponents of Q rows][exponents of Q^T rows], each [np][np / KB].
-static void slice_plan_basis(const AxisBasis& B, int np, int split, std::vector<uint16_t>& h,
+static void slice_plan_basis(const AxisBasis& B, int np, int split, int NS, std::vector<uint16_t>& h,
                              std::vector<int8_t>& ex) {
   const int n = B.n;
-  const int NS = tc_planes(split);
   const int KB = tc_block();  // k per block exponent of the sliced operands
   const int nkb = np / KB;
   const size_t plane = (size_t)np * np;
@@ -311,7 +312,7 @@ static void slice_plan_basis(const AxisBasis& B, int np, int split, std::vector<
 
 static void slice_plan_host(int n, int bc, int np, int split, std::vector<uint16_t>& h,
                             std::vector<int8_t>& ex) {
-  slice_plan_basis(make_axis_basis(n, bc), np, split, h, ex);
+  slice_plan_basis(make_axis_basis(n, bc), np, split, 4, h, ex);
 }
 
 static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P) {
@@ -323,7 +324,7 @@ static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P) {
   std::vector<uint16_t> h;
   std::vector<int8_t> ex;
   const AxisBasis B = plan_basis(P->nfull, P->bc, P->cls);
-  slice_plan_basis(B, P->np, ctx->split, h, ex);
+  slice_plan_basis(B, P->np, ctx->split, ctx->ns, h, ex);
   const size_t bytes = 2 * h.size() + ex.size();
   if (cudaMalloc(&P->tc, bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -333,6 +334,8 @@ static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P) {
   BX_CUDA(cudaMemcpy(P->tc, h.data(), 2 * h.size(), cudaMemcpyHostToDevice));
   BX_CUDA(cudaMemcpy((char*)P->tc + 2 * h.size(), ex.data(), ex.size(), cudaMemcpyHostToDevice));
   P->tc_split = ctx->split;
+  P->ns = ctx->ns;
+  if (ctx->ns == 6) return EXT_OK;  // no low-mode correction in FP32 mode
   // low-mode operands of the same basis
   if (P->low) {
     cudaFree(P->low);
@@ -390,7 +393,7 @@ static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P) {
 static const int8_t* plan_exps(const PlanDev* P, int t) {
   const size_t plane = (size_t)P->np * P->np;
   const size_t nkb = P->np / tc_block();
-  return (const int8_t*)((const char*)P->tc + 2 * 2 * (size_t)tc_planes(P->tc_split) * plane) +
+  return (const int8_t*)((const char*)P->tc + 2 * 2 * (size_t)P->ns * plane) +
          t * (size_t)P->np * nkb;
 }
 
@@ -409,18 +412,26 @@ static int get_plan(ext_ctx* ctx, int n, int bc, int cls, PlanDev** out) {
   P.bc = bc;
   P.np = pad_to(B.n, kPad);
   P.lam = B.lam;
+  auto res = ctx->plans.emplace(key, std::move(P));
+  *out = &res.first->second;
+  return EXT_OK;
+}
+
+// The plan's double-float planes of Q and Q^T (the 3-D CUDA-core products).
+static int ensure_df_plan(PlanDev* P) {
+  if (P->q) return EXT_OK;
   std::vector<float> q, qt;
-  padded_df(B, P.np, q, qt);
-  const size_t bytes = 2 * (size_t)P.np * P.np * sizeof(float);
-  if (cudaMalloc(&P.q, bytes) != cudaSuccess || cudaMalloc(&P.qt, bytes) != cudaSuccess) {
+  padded_df(plan_basis(P->nfull, P->bc, P->cls), P->np, q, qt);
+  const size_t bytes = 2 * (size_t)P->np * P->np * sizeof(float);
+  if (cudaMalloc(&P->q, bytes) != cudaSuccess || cudaMalloc(&P->qt, bytes) != cudaSuccess) {
     cudaGetLastError();
+    cudaFree(P->q);
+    P->q = P->qt = nullptr;
     g_last_error = "cudaMalloc of transform plan failed";
     return EXT_ENOMEM;
   }
-  BX_CUDA(cudaMemcpy(P.q, q.data(), bytes, cudaMemcpyHostToDevice));
-  BX_CUDA(cudaMemcpy(P.qt, qt.data(), bytes, cudaMemcpyHostToDevice));
-  auto res = ctx->plans.emplace(key, std::move(P));
-  *out = &res.first->second;
+  BX_CUDA(cudaMemcpy(P->q, q.data(), bytes, cudaMemcpyHostToDevice));
+  BX_CUDA(cudaMemcpy(P->qt, qt.data(), bytes, cudaMemcpyHostToDevice));
   return EXT_OK;
 }
 
@@ -515,9 +526,9 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   const size_t N = (size_t)nx * ny;
   d.vec_chunk = vec_chunk_of((long long)N);
   d.n_vec_items = (int)((N + d.vec_chunk - 1) / d.vec_chunk);
-  const int n_gm = (d.nxp / 128) * (d.nyp / 64);
+  const int bn = tc_tile_cols(ctx->ns), bk = tc_step_k(ctx->ns);
+  const int n_gm = (d.nxp / 128) * (d.nyp / bn);
   d.n_gm_tiles = n_gm;
-  d.n_tc_tiles = n_gm;
   set_weights(d, prob.hx, prob.hy);
   // the tensor-core transforms fold an axis by its mirror symmetry where both classes, padded,
   // fit in the padded axis: each stage then does half the products
@@ -528,14 +539,12 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   }
   d.mhx = (d.mir & 1) ? mirror_half(nx) : nx;
   d.mhy = (d.mir & 2) ? mirror_half(ny) : ny;
-  // fold items: mixed modes 8 class rows x 128 columns (a warp per row); CUDA cores 32 x 8 class
-  // nodes (one per thread, the unfold tiles)
-  d.n_fold_items = !d.mir ? 0 : ctx->tc ? ((d.mhy + 7) / 8) * ((d.mhx + 127) / 128) : 0;
-  d.n_prep_items = (ctx->tc && !d.mir) ? ((ny + kStTileY - 1) / kStTileY) * ((nx + 127) / 128) : 0;
+  // fold items: 8 class rows x 128 columns (a warp per row)
+  d.n_fold_items = !d.mir ? 0 : ((d.mhy + 7) / 8) * ((d.mhx + 127) / 128);
+  d.n_prep_items = !d.mir ? ((ny + kStTileY - 1) / kStTileY) * ((nx + 127) / 128) : 0;
   d.n_unfold_tiles = d.mir ? ((d.mhx + 31) / 32) * ((d.mhy + 7) / 8) : 0;
   d.n_prec_parts = d.mir ? d.n_unfold_tiles : n_gm;
   const int n_part = std::max(std::max(d.n_st_tiles, d.n_vec_items), std::max(n_gm, d.n_unfold_tiles));
-  const size_t Np = (size_t)d.nxp * d.nyp;
   // arena layout
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
@@ -546,10 +555,6 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   const size_t o_q = take(4 * N), o_z = take(4 * N), o_mask = take(N);
   const size_t o_rl = take(4 * N), o_p0l = take(4 * N), o_p1l = take(4 * N);
   const size_t o_ql = take(4 * N), o_zl = take(4 * N);
-  // CUDA-core transform intermediates (hi, lo planes) of an unfolded slot
-  const size_t fp = (ctx->tc || d.mir) ? 0 : 4 * Np;
-  const size_t o_t1 = take(fp), o_t2 = take(fp), o_t3 = take(fp);
-  const size_t o_t1l = take(fp), o_t2l = take(fp), o_t3l = take(fp);
   const size_t o_lx = take(4 * (size_t)d.nxp), o_ly = take(4 * (size_t)d.nyp);
   size_t o_io = 0;
   if (host_io) o_io = take(12 * N);
@@ -561,20 +566,19 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     PlanDev *px = nullptr, *py = nullptr;
     size_t o_tr = 0, o_tt1 = 0, o_tt2 = 0, o_tt3 = 0, o_maps = 0, o_ex = 0, o_lx = 0, o_ly = 0;
     size_t o_g = 0, o_lh = 0, o_ljt = 0, o_ljte = 0, o_lz = 0, o_lmaps = 0;
-    size_t o_s1 = 0, o_s2 = 0, o_s3 = 0, o_cr = 0;  // CUDA-core class problems: T1..T3, residual
   };
   std::vector<TcLay> tl;
-  const int NS = ctx->tc ? tc_planes(ctx->split) : 0;
+  const int NS = ctx->ns;
   // the low-mode correction: always (1), never (0), or (2) for grids of side >= 2048 and for every
   // grid of a call whose grids hold >= 2048^2 nodes together (large_call): there the correction's
   // kernels run at throughput and the iterations they save outweigh their cost; on one smaller
   // grid they are latency-bound and cost more than they save
-  const bool low = ctx->tc && (ctx->opt.low_modes == 1 ||
+  const bool low = NS == 4 && (ctx->opt.low_modes == 1 ||
                                (ctx->opt.low_modes == 2 &&
                                 (std::max(nx, ny) >= kLowAutoSide || large_call)));
-  // transform problems: in mixed modes always (the slot itself or its classes), on the CUDA
-  // cores only for a folded slot (its classes; an unfolded slot runs on its own buffers)
-  if (ctx->tc || d.mir) {
+  const int nr = low ? kLowNS : NS;  // slices of the residual
+  // transform problems: the slot itself or its classes
+  {
     for (int cy = 0; cy < ((d.mir & 2) ? 2 : 1); ++cy)
       for (int cx = 0; cx < ((d.mir & 1) ? 2 : 1); ++cx) {
         TcLay L;
@@ -583,18 +587,13 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
         if (!rc) rc = get_plan(ctx, ny, prob.bc_y, (d.mir & 2) ? cy : -1, &L.py);
         if (rc) return rc;
         const size_t Npc = (size_t)L.px->np * L.py->np;
-        if (ctx->tc) {
-          L.o_tr = take(2 * (low ? kLowNS : NS) * Npc);
+        {
+          L.o_tr = take(2 * nr * Npc);
           L.o_tt1 = take(2 * NS * Npc);
           L.o_tt2 = take(2 * NS * Npc);
           L.o_tt3 = take(2 * NS * Npc);
           L.o_maps = take(kTcMaps * sizeof(CUtensorMap));
           L.o_ex = take(4 * (Npc / 64));
-        } else {
-          L.o_s1 = take(8 * Npc);
-          L.o_s2 = take(8 * Npc);
-          L.o_s3 = take(8 * Npc);
-          L.o_cr = take(8 * (size_t)L.px->n * L.py->n);
         }
         if (d.mir) {
           L.o_lx = take(4 * (size_t)L.px->np);
@@ -638,12 +637,6 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   d.q_lo = (float*)(A + o_ql);
   d.z_lo = (float*)(A + o_zl);
   d.mask = (uint8_t*)(A + o_mask);
-  d.t1 = (float*)(A + o_t1);
-  d.t2 = (float*)(A + o_t2);
-  d.t3 = (float*)(A + o_t3);
-  d.t1_lo = (float*)(A + o_t1l);
-  d.t2_lo = (float*)(A + o_t2l);
-  d.t3_lo = (float*)(A + o_t3l);
   d.st_maps = nullptr;
   if (st_copy) {
     CUtensorMap smaps[kStMaps];
@@ -652,10 +645,6 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     BX_CUDA(cudaMemcpy(A + o_smaps, smaps, sizeof(smaps), cudaMemcpyHostToDevice));
     d.st_maps = A + o_smaps;
   }
-  d.qx = px->q;
-  d.qxt = px->qt;
-  d.qy = py->q;
-  d.qyt = py->qt;
   if (host_io) {
     s.phi_stage = (float*)(A + o_io);
     s.f_stage = s.phi_stage + N;
@@ -696,49 +685,6 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     SlotDesc t = d;  // the slot's fields; a class problem overrides its domain and operands below
     PlanDev* qx = L.px;
     PlanDev* qy = L.py;
-    if (!ctx->tc) {
-      // a class problem on the CUDA cores: its residual (formed by the fold kernel), T1..T3, the
-      // class bases as double-float planes, its eigenvalues and its result g
-      t.nx = qx->n;
-      t.ny = qy->n;
-      t.nxp = qx->np;
-      t.nyp = qy->np;
-      t.n_gm_tiles = (t.nxp / 128) * (t.nyp / 64);
-      t.mir = 0;
-      t.mir_out = 1;
-      t.mask = nullptr;
-      t.b = nullptr;
-      t.xhi = t.xlo = nullptr;
-      t.q = t.q_lo = nullptr;
-      t.p[0] = t.p[1] = t.p_lo[0] = t.p_lo[1] = nullptr;
-      t.part = t.pq_part = nullptr;
-      t.st_maps = nullptr;
-      const size_t Npc = (size_t)t.nxp * t.nyp, nc = (size_t)t.nx * t.ny;
-      t.t1 = (float*)(A + L.o_s1);
-      t.t1_lo = t.t1 + Npc;
-      t.t2 = (float*)(A + L.o_s2);
-      t.t2_lo = t.t2 + Npc;
-      t.t3 = (float*)(A + L.o_s3);
-      t.t3_lo = t.t3 + Npc;
-      t.r = (float*)(A + L.o_cr);
-      t.r_lo = t.r + nc;
-      t.qx = qx->q;
-      t.qxt = qx->qt;
-      t.qy = qy->q;
-      t.qyt = qy->qt;
-      t.z = (float*)(A + L.o_g);
-      t.z_lo = t.z + nc;
-      std::vector<float> lxc(t.nxp, 0.f), lyc(t.nyp, 0.f);
-      for (int k = 0; k < t.nx; ++k) lxc[k] = (float)(qx->lam[k] * a);
-      for (int k = 0; k < t.ny; ++k) lyc[k] = (float)(qy->lam[k] * c);
-      BX_CUDA(cudaMemcpy(A + L.o_lx, lxc.data(), 4 * lxc.size(), cudaMemcpyHostToDevice));
-      BX_CUDA(cudaMemcpy(A + L.o_ly, lyc.data(), 4 * lyc.size(), cudaMemcpyHostToDevice));
-      t.lamx = (const float*)(A + L.o_lx);
-      t.lamy = (const float*)(A + L.o_ly);
-      t.lowm_x = t.lowm_y = 0;
-      s.tcp[L.c] = t;
-      continue;
-    }
     int rc2 = ensure_tc_plan(ctx, qx);
     if (!rc2) rc2 = ensure_tc_plan(ctx, qy);
     if (rc2) return rc2;
@@ -747,7 +693,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
       t.ny = qy->n;
       t.nxp = qx->np;
       t.nyp = qy->np;
-      t.n_gm_tiles = t.n_tc_tiles = (t.nxp / 128) * (t.nyp / 64);
+      t.n_gm_tiles = (t.nxp / 128) * (t.nyp / bn);
       t.mir = 0;
       t.mir_out = 1;
       // only the transform fields are live: grid vectors of the slot stay out of reach
@@ -757,7 +703,6 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
       t.r = t.r_lo = t.q = t.q_lo = nullptr;
       t.p[0] = t.p[1] = t.p_lo[0] = t.p_lo[1] = nullptr;
       t.part = t.pq_part = nullptr;
-      t.t1 = t.t2 = t.t3 = t.t1_lo = t.t2_lo = t.t3_lo = nullptr;
       t.st_maps = nullptr;
       t.z = (float*)(A + L.o_g);  // the class result g, [ny][nx] hi then lo
       t.z_lo = t.z + (size_t)t.nx * t.ny;
@@ -771,6 +716,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     }
     const size_t Npc = (size_t)t.nxp * t.nyp, nex = Npc / 64;
     t.tc_r = A + L.o_tr;
+    t.tc_nr = nr;
     t.tc_t1 = A + L.o_tt1;
     t.tc_t2 = A + L.o_tt2;
     t.tc_t3 = A + L.o_tt3;
@@ -780,22 +726,22 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     t.tc_eb[1] = plan_exps(qy, 1);  // Qy^T rows
     t.tc_eb[2] = plan_exps(qx, 0);  // Qx rows
     t.tc_eb[3] = plan_exps(qy, 0);  // Qy rows
-    BX_CUDA(cudaMemset(t.tc_r, 0, 2 * (low ? kLowNS : NS) * Npc));
+    BX_CUDA(cudaMemset(t.tc_r, 0, 2 * nr * Npc));
     BX_CUDA(cudaMemset(A + L.o_ex, 0, 4 * nex));
     CUtensorMap maps[kTcMaps];
     const size_t pxp = (size_t)t.nxp * t.nxp, pyp = (size_t)t.nyp * t.nyp;
     uint16_t* qxb = (uint16_t*)qx->tc;
     uint16_t* qyb = (uint16_t*)qy->tc;
     // A operands: r planes [P][nyp][nxp], T1 [P][nxp][nyp], T2 [P][nyp][nxp], T3 [P][nxp][nyp]
-    int rc3 = make_tmap(&maps[0], t.tc_r, bf, t.nxp, (uint64_t)NS * t.nyp, 128);
-    if (!rc3) rc3 = make_tmap(&maps[1], t.tc_t1, bf, t.nyp, (uint64_t)NS * t.nxp, 128);
-    if (!rc3) rc3 = make_tmap(&maps[2], t.tc_t2, bf, t.nxp, (uint64_t)NS * t.nyp, 128);
-    if (!rc3) rc3 = make_tmap(&maps[3], t.tc_t3, bf, t.nyp, (uint64_t)NS * t.nxp, 128);
+    int rc3 = make_tmap(&maps[0], t.tc_r, bf, t.nxp, (uint64_t)NS * t.nyp, 128, bk);
+    if (!rc3) rc3 = make_tmap(&maps[1], t.tc_t1, bf, t.nyp, (uint64_t)NS * t.nxp, 128, bk);
+    if (!rc3) rc3 = make_tmap(&maps[2], t.tc_t2, bf, t.nxp, (uint64_t)NS * t.nyp, 128, bk);
+    if (!rc3) rc3 = make_tmap(&maps[3], t.tc_t3, bf, t.nyp, (uint64_t)NS * t.nxp, 128, bk);
     // B operands: Qx^T, Qy^T, Qx, Qy planes
-    if (!rc3) rc3 = make_tmap(&maps[4], qxb + NS * pxp, bf, t.nxp, (uint64_t)NS * t.nxp, 64);
-    if (!rc3) rc3 = make_tmap(&maps[5], qyb + NS * pyp, bf, t.nyp, (uint64_t)NS * t.nyp, 64);
-    if (!rc3) rc3 = make_tmap(&maps[6], qxb, bf, t.nxp, (uint64_t)NS * t.nxp, 64);
-    if (!rc3) rc3 = make_tmap(&maps[7], qyb, bf, t.nyp, (uint64_t)NS * t.nyp, 64);
+    if (!rc3) rc3 = make_tmap(&maps[4], qxb + NS * pxp, bf, t.nxp, (uint64_t)NS * t.nxp, bn, bk);
+    if (!rc3) rc3 = make_tmap(&maps[5], qyb + NS * pyp, bf, t.nyp, (uint64_t)NS * t.nyp, bn, bk);
+    if (!rc3) rc3 = make_tmap(&maps[6], qxb, bf, t.nxp, (uint64_t)NS * t.nxp, bn, bk);
+    if (!rc3) rc3 = make_tmap(&maps[7], qyb, bf, t.nyp, (uint64_t)NS * t.nyp, bn, bk);
     // the stages' results as they are stored, tile by tile: T1, T2, T3
     if (!rc3) rc3 = make_tmap(&maps[8], t.tc_t1, bf, t.nyp, (uint64_t)NS * t.nxp, 32);
     if (!rc3) rc3 = make_tmap(&maps[9], t.tc_t2, bf, t.nxp, (uint64_t)NS * t.nyp, 32);
@@ -830,11 +776,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     s.tcp[L.c] = t;
   }
   s.n_tcp = (int)tl.size();
-  if (ctx->tc && !d.mir) d = s.tcp[0];  // the slot is its own problem (k_tc_prepare reads it)
-  if (!ctx->tc && !d.mir) {             // the slot's own transforms on the CUDA cores
-    s.tcp[0] = d;
-    s.n_tcp = 1;
-  }
+  if (!d.mir) d = s.tcp[0];  // the slot is its own problem (k_tc_prepare reads it)
   return EXT_OK;
 }
 
@@ -904,7 +846,7 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
     tc_items(s, i, gm, l1, l3, tcl);
     for (int t = 0; t < d.n_fold_items; ++t) fold.push_back({i, t});
     for (int t = 0; t < d.n_unfold_tiles; ++t) unfold.push_back({i, t});
-    if (ctx->tc && !d.mir)
+    if (!d.mir)
       for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
   }
   longest_first_tc(gm, W->slots);
@@ -1098,41 +1040,29 @@ static void harvest(ext_ctx* ctx) {
 // with_finish = false: the next stencil forms rho and beta from the partials itself
 static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish = true) {
   LaunchCfg g = cfg_of(ctx, W, 2);
-  if (ctx->tc) {
-    // residual slices: unfolded slots directly, folded slots per mirror class
-    if (W->n_prep > 0)
-      timed(ctx, EXT_KERNEL_SPLIT, [&] { launch_prec_tc_prepare(cfg_of(ctx, W, 10), mode, ctx->split); },
-            g.stream);
-    if (W->n_fold > 0)
-      timed(ctx, EXT_KERNEL_FOLD, [&] { launch_tc_fold(cfg_of(ctx, W, 7), mode, ctx->split); }, g.stream);
-    // the transform kernels run over the tensor-core problems
-    g.slots = W->d_tcp;
-    g.grid = std::max(1, std::min(W->n_gm, ctx->sm_count));
-    if (W->n_l1 > 0) {
-      // the lowest modes in high precision: forward product, middle, inverse product
-      LaunchCfg c1 = cfg_of(ctx, W, 5), cm = cfg_of(ctx, W, 6), c3 = cfg_of(ctx, W, 6);
-      c1.slots = cm.slots = c3.slots = W->d_tcp;
-      cm.grid = std::max(1, std::min(W->n_l3, ctx->sm_count * 8));  // the middle: small blocks
-      timed(ctx, EXT_KERNEL_LOW_FWD, [&] { launch_low_tc(c1, 0, mode, ctx->split, ctx->d_err); }, g.stream);
-      // the middle starts on a free device: blocks placed as the forward product's leave would load
-      // the SMs unevenly (15 us more per application on a batch of 48 grids)
-      cm.pdl = false;
-      timed(ctx, EXT_KERNEL_LOW_MID, [&] { launch_low_mid(cm, mode, ctx->split); }, g.stream);
-      timed(ctx, EXT_KERNEL_LOW_INV, [&] { launch_low_tc(c3, 1, mode, ctx->split, ctx->d_err); }, g.stream);
-    }
-  }
-  if (!ctx->tc) {
-    // CUDA-core transforms over the transform problems: a folded slot's classes get their
-    // residuals from the fold first
-    g.slots = W->d_tcp;
-    g.pdl = false;  // measured slower with it (64^2 grid: 32.0 -> 32.6 ms a solve)
-    if (W->n_unfold > 0)
-      timed(ctx, EXT_KERNEL_FOLD, [&] { launch_simt_fold(cfg_of(ctx, W, 8), mode); }, g.stream);
+  // residual slices: unfolded slots directly, folded slots per mirror class
+  if (W->n_prep > 0)
+    timed(ctx, EXT_KERNEL_SPLIT, [&] { launch_prec_tc_prepare(cfg_of(ctx, W, 10), mode, ctx->split); }, g.stream);
+  if (W->n_fold > 0)
+    timed(ctx, EXT_KERNEL_FOLD, [&] { launch_tc_fold(cfg_of(ctx, W, 7), mode, ctx->split); }, g.stream);
+  // the transform kernels run over the tensor-core problems
+  g.slots = W->d_tcp;
+  g.grid = std::max(1, std::min(W->n_gm, ctx->sm_count));
+  if (W->n_l1 > 0) {
+    // the lowest modes in high precision: forward product, middle, inverse product
+    LaunchCfg c1 = cfg_of(ctx, W, 5), cm = cfg_of(ctx, W, 6), c3 = cfg_of(ctx, W, 6);
+    c1.slots = cm.slots = c3.slots = W->d_tcp;
+    cm.grid = std::max(1, std::min(W->n_l3, ctx->sm_count * 8));  // the middle: small blocks
+    timed(ctx, EXT_KERNEL_LOW_FWD, [&] { launch_low_tc(c1, 0, mode, ctx->split, ctx->d_err); }, g.stream);
+    // the middle starts on a free device: blocks placed as the forward product's leave would load
+    // the SMs unevenly (15 us more per application on a batch of 48 grids)
+    cm.pdl = false;
+    timed(ctx, EXT_KERNEL_LOW_MID, [&] { launch_low_mid(cm, mode, ctx->split); }, g.stream);
+    timed(ctx, EXT_KERNEL_LOW_INV, [&] { launch_low_tc(c3, 1, mode, ctx->split, ctx->d_err); }, g.stream);
   }
   for (int s = 0; s < 4; ++s) {
     timed(ctx, EXT_KERNEL_PREC0 + s, [&] {
-      if (!ctx->tc) launch_prec_simt(g, s, mode);
-      else launch_prec_tc(g, s, mode, ctx->split, ctx->d_err);
+      launch_prec_tc(g, s, mode, ctx->split, ctx->ns, ctx->d_err);
     }, g.stream);
   }
   if (W->n_unfold > 0)
@@ -1554,10 +1484,10 @@ int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out) {
   ctx->sm_count = prop.multiProcessorCount;
   ctx->cc_major = prop.major;
   ctx->cc_minor = prop.minor;
-  if (o.prec != EXT_PREC_FP32 && !(prop.major == 10 && tc_supported())) return EXT_ENOTSUP;
-  ctx->tc = o.prec != EXT_PREC_FP32;
-  ctx->split = o.prec == EXT_PREC_MIXED_BF16 ? 1 : 0;
-  if (ctx->tc) BX_CUDA(tc_init());
+  if (!(prop.major == 10 && tc_supported())) return EXT_ENOTSUP;
+  ctx->ns = o.prec == EXT_PREC_FP32 ? 6 : 4;
+  ctx->split = o.prec == EXT_PREC_MIXED_FP16 ? 0 : 1;
+  BX_CUDA(tc_init());
   BX_CUDA(stencil_init());
   BX_CUDA(cudaMalloc(&ctx->d_err, sizeof(int)));
   BX_CUDA(cudaMemset(ctx->d_err, 0, sizeof(int)));
@@ -1681,9 +1611,11 @@ static int args3(ext_ctx* ctx, const ext_problem3* p, Solve3Args& a) {
   a.h[1] = p->hy;
   a.h[2] = p->hz;
   const int n[3] = {p->nx, p->ny, p->nz};
+  const bool on_tc = p->nx % 128 == 0 && p->ny % 128 == 0 && p->nz % 128 == 0;
   for (int ax = 0; ax < 3; ++ax) {
     PlanDev* P = nullptr;
-    const int rc = get_plan(ctx, n[ax], a.bc[ax], -1, &P);
+    int rc = get_plan(ctx, n[ax], a.bc[ax], -1, &P);
+    if (!rc && !on_tc) rc = ensure_df_plan(P);
     if (rc) return rc;
     a.q[ax] = P->q;
     a.qt[ax] = P->qt;
@@ -1695,12 +1627,12 @@ static int args3(ext_ctx* ctx, const ext_problem3* p, Solve3Args& a) {
   a.true_res_every = ctx->opt.true_res_every;
   a.replace_factor = ctx->opt.replace_factor;
   a.stream = ctx->stream;
-  if (ctx->tc && p->nx % 128 == 0 && p->ny % 128 == 0 && p->nz % 128 == 0)
+  if (on_tc)
     a.tc_build = [ctx, &a](const Tc3Io& io, Tc3& t) { return tc3_build(ctx, a, io, t); };
   return EXT_OK;
 }
 
-// The 3-D transforms on the tensor cores (mixed modes, every side a multiple of 128).  Each of
+// The 3-D transforms on the tensor cores (every side a multiple of 128).  Each of
 // the six products contracts the contiguous axis of its operand and writes its result with that
 // axis first, exactly the form of the 2-D stage kernels, so every product is one launch of
 // k_prec_tc over a descriptor whose dimensions are the box's: with X, Y, Z the sides, the
@@ -1712,7 +1644,7 @@ static int args3(ext_ctx* ctx, const ext_problem3* p, Solve3Args& a) {
 static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t) {
   const int X = a.nx, Y = a.ny, Z = a.nz;
   const size_t N3 = (size_t)X * Y * Z;
-  const int NS = tc_planes(ctx->split);
+  const int NS = ctx->ns, bn = tc_tile_cols(NS), bk = tc_step_k(NS);
   const bool bf = ctx->split == 1;
   PlanDev* P[3];
   {
@@ -1739,7 +1671,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   int8_t* E0 = (int8_t*)take(N3 / 128);
   int8_t* EA = (int8_t*)take(N3 / 128);
   int8_t* EB = (int8_t*)take(N3 / 128);
-  const int tiles3 = ((Y * X) / 128) * (Z / 64);
+  const int tiles3 = ((Y * X) / 128) * (Z / bn);
   double* part = (double*)take(sizeof(double) * 4 * (size_t)tiles3);
   float* lam = (float*)take(sizeof(float) * ((size_t)Y * X + Z));
   SlotScalars* sc = (SlotScalars*)take(sizeof(SlotScalars));
@@ -1794,42 +1726,42 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   // [0]: residual slicing, rows (z, y), columns x
   d[0].nx = X; d[0].ny = Z * Y; d[0].nxp = X; d[0].nyp = Z * Y;
   d[0].r = const_cast<float*>(io.rh); d[0].r_lo = const_cast<float*>(io.rl);
-  d[0].tc_r = S0; d[0].tc_e[0] = E0;
+  d[0].tc_r = S0; d[0].tc_nr = NS; d[0].tc_e[0] = E0;
   // [1] F1 (stage-0 form): A = r slices [Z Y][X], B = Qx^T -> SA [X][Z Y]
   d[1].nyp = Z * Y; d[1].nxp = X; d[1].nx = X; d[1].ny = Z * Y;
-  int rc = make_tmap(&m[0][0], S0, bf, X, (uint64_t)NS * Z * Y, 128);
-  if (!rc) rc = make_tmap(&m[0][4], QT(0), bf, X, (uint64_t)NS * X, 64);
+  int rc = make_tmap(&m[0][0], S0, bf, X, (uint64_t)NS * Z * Y, 128, bk);
+  if (!rc) rc = make_tmap(&m[0][4], QT(0), bf, X, (uint64_t)NS * X, bn, bk);
   d[1].tc_e[0] = E0; d[1].tc_eb[0] = plan_exps(P[0], 1); d[1].tc_t1 = SA; d[1].tc_e[1] = EA;
   if (!rc) rc = make_tmap(&m[0][8], SA, bf, (uint64_t)Z * Y, (uint64_t)NS * X, 32);
   // [2] F2 (stage-0 form): A = SA as [X Z][Y], B = Qy^T -> SB [Y][X Z]
   d[2].nyp = X * Z; d[2].nxp = Y; d[2].nx = Y; d[2].ny = X * Z;
-  if (!rc) rc = make_tmap(&m[1][0], SA, bf, Y, (uint64_t)NS * X * Z, 128);
-  if (!rc) rc = make_tmap(&m[1][4], QT(1), bf, Y, (uint64_t)NS * Y, 64);
+  if (!rc) rc = make_tmap(&m[1][0], SA, bf, Y, (uint64_t)NS * X * Z, 128, bk);
+  if (!rc) rc = make_tmap(&m[1][4], QT(1), bf, Y, (uint64_t)NS * Y, bn, bk);
   d[2].tc_e[0] = EA; d[2].tc_eb[0] = plan_exps(P[1], 1); d[2].tc_t1 = SB; d[2].tc_e[1] = EB;
   if (!rc) rc = make_tmap(&m[1][8], SB, bf, (uint64_t)X * Z, (uint64_t)NS * Y, 32);
   // [3] F3 (stage-1 form, weights): A = SB as [Y X][Z], B = Qz^T -> SA [Z][Y X]
   d[3].nxp = Y * X; d[3].nyp = Z; d[3].nx = Y * X; d[3].ny = Z;
-  if (!rc) rc = make_tmap(&m[2][1], SB, bf, Z, (uint64_t)NS * Y * X, 128);
-  if (!rc) rc = make_tmap(&m[2][5], QT(2), bf, Z, (uint64_t)NS * Z, 64);
+  if (!rc) rc = make_tmap(&m[2][1], SB, bf, Z, (uint64_t)NS * Y * X, 128, bk);
+  if (!rc) rc = make_tmap(&m[2][5], QT(2), bf, Z, (uint64_t)NS * Z, bn, bk);
   d[3].tc_e[1] = EB; d[3].tc_eb[1] = plan_exps(P[2], 1); d[3].tc_t2 = SA; d[3].tc_e[2] = EA;
   d[3].lamx = lam; d[3].lamy = lam + (size_t)Y * X; d[3].wnorm = (float)(smin * smin);
   if (!rc) rc = make_tmap(&m[2][9], SA, bf, (uint64_t)Y * X, (uint64_t)NS * Z, 32);
   // [4] I1 (stage-2 form): A = SA as [Z Y][X], B = Qx -> SB [X][Z Y]
   d[4].nyp = Z * Y; d[4].nxp = X; d[4].nx = X; d[4].ny = Z * Y;
-  if (!rc) rc = make_tmap(&m[3][2], SA, bf, X, (uint64_t)NS * Z * Y, 128);
-  if (!rc) rc = make_tmap(&m[3][6], QQ(0), bf, X, (uint64_t)NS * X, 64);
+  if (!rc) rc = make_tmap(&m[3][2], SA, bf, X, (uint64_t)NS * Z * Y, 128, bk);
+  if (!rc) rc = make_tmap(&m[3][6], QQ(0), bf, X, (uint64_t)NS * X, bn, bk);
   d[4].tc_e[2] = EA; d[4].tc_eb[2] = plan_exps(P[0], 0); d[4].tc_t3 = SB; d[4].tc_e[3] = EB;
   if (!rc) rc = make_tmap(&m[3][10], SB, bf, (uint64_t)Z * Y, (uint64_t)NS * X, 32);
   // [5] I2 (stage-2 form): A = SB as [X Z][Y], B = Qy -> SA [Y][X Z]
   d[5].nyp = X * Z; d[5].nxp = Y; d[5].nx = Y; d[5].ny = X * Z;
-  if (!rc) rc = make_tmap(&m[4][2], SB, bf, Y, (uint64_t)NS * X * Z, 128);
-  if (!rc) rc = make_tmap(&m[4][6], QQ(1), bf, Y, (uint64_t)NS * Y, 64);
+  if (!rc) rc = make_tmap(&m[4][2], SB, bf, Y, (uint64_t)NS * X * Z, 128, bk);
+  if (!rc) rc = make_tmap(&m[4][6], QQ(1), bf, Y, (uint64_t)NS * Y, bn, bk);
   d[5].tc_e[2] = EB; d[5].tc_eb[2] = plan_exps(P[1], 0); d[5].tc_t3 = SA; d[5].tc_e[3] = EA;
   if (!rc) rc = make_tmap(&m[4][10], SA, bf, (uint64_t)X * Z, (uint64_t)NS * Y, 32);
   // [6] I3 (stage-3 form): A = SA as [Y X][Z], B = Qz -> z[Z][Y X] masked, r.z per tile
   d[6].nxp = Y * X; d[6].nyp = Z; d[6].nx = Y * X; d[6].ny = Z;
-  if (!rc) rc = make_tmap(&m[5][3], SA, bf, Z, (uint64_t)NS * Y * X, 128);
-  if (!rc) rc = make_tmap(&m[5][7], QQ(2), bf, Z, (uint64_t)NS * Z, 64);
+  if (!rc) rc = make_tmap(&m[5][3], SA, bf, Z, (uint64_t)NS * Y * X, 128, bk);
+  if (!rc) rc = make_tmap(&m[5][7], QQ(2), bf, Z, (uint64_t)NS * Z, bn, bk);
   if (rc) return rc;
   d[6].tc_e[3] = EA; d[6].tc_eb[3] = plan_exps(P[2], 0);
   d[6].r = const_cast<float*>(io.rh); d[6].r_lo = const_cast<float*>(io.rl);
@@ -1845,7 +1777,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   for (int k = 1; k < 7; ++k) {
     const bool mrows_y = kForm[k] == 0 || kForm[k] == 2;  // M = nyp in the stage-0/2 forms
     const int M = mrows_y ? d[k].nyp : d[k].nxp, N = mrows_y ? d[k].nxp : d[k].nyp;
-    for (int tt = 0; tt < (M / 128) * (N / 64); ++tt) items[k].push_back({k, tt});
+    for (int tt = 0; tt < (M / 128) * (N / bn); ++tt) items[k].push_back({k, tt});
   }
   int counts[7];
   for (int k = 0; k < 7; ++k) {
@@ -1864,6 +1796,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   t.d_counts = dc;
   t.d_descs = descs;
   t.split = ctx->split;
+  t.ns = NS;
   t.d_err = ctx->d_err;
   t.wait_cycles = ctx->opt.wait_cycles;
   t.sm_count = ctx->sm_count;
@@ -2226,7 +2159,7 @@ static int serve_rebuild_lists(ext_ctx* ctx) {
     tc_items(h, i, gm, l1, l3, tcl);
     for (int t = 0; t < d.n_fold_items; ++t) fold.push_back({i, t});
     for (int t = 0; t < d.n_unfold_tiles; ++t) unfold.push_back({i, t});
-    if (ctx->tc && !d.mir)
+    if (!d.mir)
       for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
     sl.push_back({i, 0});
   }

@@ -105,23 +105,13 @@ struct SlotDesc {
   float* p_lo[2];
   float* q_lo;
   float* z_lo;
-  // transform intermediates of the CUDA-core path, padded [.][.] row-major, double-float planes
-  float* t1;         // [nxp][nyp]
-  float* t2;         // [nyp][nxp]
-  float* t3;         // [nxp][nyp]
-  float* t1_lo;
-  float* t2_lo;
-  float* t3_lo;
-  const float* qx;   // [nxp][nxp]  Qx[x][k] (hi); the lo plane follows at + nxp * nxp
-  const float* qxt;  // [nxp][nxp]  Qx^T
-  const float* qy;
-  const float* qyt;
   const float* lamx; // [nxp] eigenvalues of T_x (scaled), padding entries never read
   const float* lamy;
   float wnorm;       // 1 / w_max, so that the scaled weights are <= 1
   int zero_mode;     // 1: drop the (0,0) mode (both axes symmetric/periodic)
-  // tensor-core path: block-scaled integer slices (NS 16-bit planes) and their TMA descriptors
-  void* tc_r;        // [NS][nyp][nxp]  residual
+  // transforms: block-scaled integer slices (NS = 4 or 6 16-bit planes) and their TMA descriptors
+  void* tc_r;        // [tc_nr][nyp][nxp]  residual
+  int tc_nr;         // its slices: NS, or 6 where the low-mode correction reads them
   void* tc_t1;       // [NS][nxp][nyp]
   void* tc_t2;       // [NS][nyp][nxp]
   void* tc_t3;       // [NS][nxp][nyp]
@@ -132,7 +122,6 @@ struct SlotDesc {
   const void* st_maps;  // kStMaps CUtensorMap for the stencil's tensor copies (z, z_lo, p[0],
                         // p_lo[0], p[1], p_lo[1], mask); null when a mask row is not a multiple
                         // of 16 bytes
-  int n_tc_tiles;    // output tiles of one tensor-core transform stage
   // Low-mode correction of the tensor-core preconditioner: the modes kx < lowm_x, ky < lowm_y
   // (the smoothest, with the largest weights) are left out of the four 32-bit transform stages and
   // added from thin transforms with six slices per operand (about 48 bits).  0 = off.
@@ -487,15 +476,6 @@ __device__ __forceinline__ float spectral_weight_of(float wnorm, float s) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s * s));
   return wnorm * r;
-}
-
-// Spectral weight 1/(lam_y + lam_x)^2, normalised to <= 1; zero for padding and the constant
-// mode when both axes are symmetric/periodic (pseudo-inverse).
-__device__ __forceinline__ float spectral_weight(const SlotDesc& S, int kx, int ky) {
-  if (kx >= S.nx || ky >= S.ny) return 0.f;
-  const float s = S.lamy[ky] + S.lamx[kx];
-  if (!(s > 0.f)) return 0.f;
-  return spectral_weight_of(S.wnorm, s);
 }
 
 // The per-slot scalar steps.  Each is computed either by one block per slot in a launch of its own

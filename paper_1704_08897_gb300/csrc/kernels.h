@@ -71,22 +71,17 @@ void launch_prec_finish(const LaunchCfg& c, int mode);
 void launch_apply(const SlotDesc* slot, int n_tiles, bool aniso, const float* p, float* q,
                   double* part, cudaStream_t s);
 
-// fast Poisson preconditioner, FP32 CUDA-core transform products (kernels_gemm_simt.cu).
-// stage 0..3 = forward x, forward y (+ eigenvalue weights), inverse x, inverse y (+ mask, dots).
-// mode 0: slots with active iterations; mode 1: slots with a pending preconditioner pass;
-// mode 2: every slot (verification entry point).
-void launch_prec_simt(const LaunchCfg& c, int stage, int mode);
-// the mirror classes' residuals of folded slots in double-float (c.slots = slots, c.tcp = the
-// transform problems, items: the unfold tiles of 32 x 8 class nodes)
-void launch_simt_fold(const LaunchCfg& c, int mode);
-
-// tensor-core variant (kernels_gemm_tc.cu): exact block-scaled integer slice planes stored as
-// FP16 (split_kind 0) or BF16 (split_kind 1); err receives 1 if a bounded wait ran out.
-void launch_prec_tc(const LaunchCfg& c, int stage, int mode, int split_kind, int* err);
+// fast Poisson preconditioner (kernels_gemm_tc.cu): exact block-scaled integer slice planes stored
+// as FP16 (split_kind 0) or BF16 (split_kind 1), ns = 4 of them (mixed modes) or 6 (FP32 mode, BF16
+// only).  stage 0..3 = forward x, forward y (+ eigenvalue weights), inverse x, inverse y (+ mask,
+// dots).  mode 0: slots with active iterations; mode 1: slots with a pending preconditioner pass;
+// mode 2: every slot (verification entry point).  err receives 1 if a bounded wait ran out.
+void launch_prec_tc(const LaunchCfg& c, int stage, int mode, int split_kind, int ns, int* err);
 // residual -> integer slice planes of the first stage's A operand, slots with no folded axis
 // (items of 32 rows x 128 columns)
 void launch_prec_tc_prepare(const LaunchCfg& c, int mode, int split_kind);
-int tc_planes(int split_kind);
+int tc_tile_cols(int ns);  // columns of a stage's output tile
+int tc_step_k(int ns);     // k per pipeline step of a stage (the copies' box width)
 // low-mode correction of the tensor-core preconditioner: kind 0 = forward product with the tiles'
 // shares of G (one CTA per 128 rows of y), kind 1 = inverse product (one CTA per 128 rows of x,
 // walking the y-tiles); the middle step one block per (problem, 128 rows of x)
@@ -108,7 +103,7 @@ struct Tc3 {
   const WorkItem* d_items[7] = {};
   const int* d_counts = nullptr;  // [7]
   int n_items[7] = {};
-  int split = 0;
+  int split = 0, ns = 4;
   int* d_err = nullptr;
   long long wait_cycles = 0;
   int sm_count = 148;

@@ -1,7 +1,14 @@
 // Fast Poisson preconditioner (Sec. 2.2 / Algorithm 1) on the 5th-generation tensor cores.
 //
-// The four separable transform products of the preconditioner (stage equations in
-// kernels_gemm_simt.cu) run as tcgen05 MMAs with FP16 or BF16 operands and FP32 accumulation.
+// z = M Q_y W Q_y^T (M r) Q_x W ... written separably on the padded rectangle:
+//   stage 0: T1[kx][y]  = sum_x r[y][x]  Qx[x][kx]       (forward transform along x)
+//   stage 1: T2[ky][kx] = w(ky,kx) sum_y T1[kx][y] Qy[y][ky]   (along y, times 1/(lam+mu)^2)
+//   stage 2: T3[x][ky]  = sum_kx T2[ky][kx] Qx[x][kx]    (inverse along x)
+//   stage 3: z[y][x]    = mask(y,x) sum_ky T3[x][ky] Qy[y][ky] (inverse along y), plus partial
+//            r.z, z.q per tile (reduced by k_prec_finish or the next stencil)
+// Every stage is D[m][n] = sum_k A[m][k] B[n][k] with both operands k-contiguous, written out
+// transposed (Out[n][m]) so the next stage again reads a k-contiguous operand.  The products run
+// as tcgen05 MMAs with FP16 or BF16 operands and FP32 accumulation.
 // This operator is so ill-conditioned that a plain 16-bit operand ruins the preconditioner, and
 // even float hi/lo operand splits lose too much in the tensor core's truncating FP32
 // accumulation.  The products are therefore made exact:
@@ -23,6 +30,10 @@
 // directly, and the last stage writes z as a double-float pair.  Three slices on
 // 64-blocks (24 bits) cost this operator 30-80% more CG iterations than exact transforms; four on
 // 128-blocks come within 5-10% of them.
+//
+// FP32 mode runs the same kernels with six slices per operand (48 bits of each 128-block, orders
+// 0..5, 21 products), the accuracy of its double-float vectors: it takes the FP64 iteration's count
+// plus 10-20%.  Its tiles are 128 x 32 (six accumulators twice in TMEM) and its steps 32 deep.
 //
 // Kernel structure (one CTA per SM, persistent over the (slot, tile) work list):
 //   warp 0      : TMA producer: 128B-swizzled K-major tiles of the slices of A and B, two 64-deep
@@ -59,26 +70,26 @@
 namespace bx {
 namespace {
 
-constexpr int BM = 128, BK = 64;  // BK: one 128-byte swizzle atom per pipeline step
+constexpr int BM = 128;
 constexpr int KC = 128;                     // k per exponent / exact accumulation block
-constexpr int KPC = KC / BK;                // pipeline steps per accumulation block
-constexpr int NS = 4;                       // slices per operand of the transform stages
 constexpr int kEpiWarps = 16;
-static_assert(KC % BK == 0 && KC == BM, "one exponent block per tile column");
+static_assert(KC == BM, "one exponent block per tile column");
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 // One CTA per SM.  Each of the SM's four schedulers owns a quarter of the register file and
 // holds up to ceil(warps / 4) of the CTA's warps.
 constexpr int kMaxRegs = (16384 / (32 * ((kThreads / 32 + 3) / 4))) & ~7;
 constexpr int kChunks = 2;                       // TMEM ring of k-block accumulator sets
 constexpr int kTmemCols = 512;                   // power of two >= kChunks * sets
-constexpr int A_PLANE = BM * BK * 2;
 constexpr int STAGES = 2;
 
-// Tile geometry by the number of slices: shared memory holds the A ring, the two B steps and the
-// staging tile of the outgoing slices.
+// Tile geometry by the number of slices: shared memory holds two steps of both operands and the
+// staging tile of the outgoing slices; six slices of a 64-deep step would not fit twice.
 template <int NSL>
 struct TcGeom {
   static constexpr int BN = NSL == 4 ? 64 : 32;   // tile columns
+  static constexpr int BK = NSL == 4 ? 64 : 32;   // one swizzle atom (128 or 64 bytes) per pipeline step
+  static constexpr int KPC = KC / BK;             // pipeline steps per accumulation block
+  static constexpr int A_PLANE = BM * BK * 2;
   static constexpr int kCb = BN / 32;             // 8-column blocks per epilogue warp
   static constexpr int kEpiCols = 8 * kCb;        // tile columns per epilogue warp
   static constexpr int kBPlane = BN * BK * 2;
@@ -103,14 +114,17 @@ struct Ctl {
 };
 static_assert(sizeof(Ctl) <= 2048, "control block too large");
 
-// UMMA shared-memory descriptor: K-major operand, 128-byte swizzle, 8-row core groups 1024 B apart.
+// UMMA shared-memory descriptor: K-major operand, rows of K 16-bit values swizzled over 2 K = 128 or
+// 64 bytes, 8-row core groups 16 K bytes apart.
+template <int K = 64>
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
+  static_assert(K == 64 || K == 32, "swizzle atoms");
   uint64_t d = 0;
   d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
   d |= static_cast<uint64_t>(1) << 16;          // leading-dimension offset (unused here)
-  d |= static_cast<uint64_t>(1024 >> 4) << 32;  // stride between 8-row groups
+  d |= static_cast<uint64_t>(16 * K >> 4) << 32;  // stride between 8-row groups
   d |= static_cast<uint64_t>(1) << 46;          // descriptor version
-  d |= static_cast<uint64_t>(2) << 61;          // 128-byte swizzle
+  d |= static_cast<uint64_t>(K == 64 ? 2 : 4) << 61;  // 128- or 64-byte swizzle
   return d;
 }
 // Instruction descriptor of kind::f16: FP32 accumulator, both operands K-major, M x N tile.
@@ -313,7 +327,8 @@ __global__ void __maxnreg__(kMaxRegs)
 k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
           const int* __restrict__ n_items, int mode, int* __restrict__ err, long long wait_cycles) {
   using G = TcGeom<NSL>;
-  constexpr int BN = G::BN, kCb = G::kCb, kEpiCols = G::kEpiCols;
+  constexpr int BN = G::BN, kCb = G::kCb, kEpiCols = G::kEpiCols, BK = G::BK, KPC = G::KPC;
+  constexpr int A_PLANE = G::A_PLANE;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -433,8 +448,8 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         if (!ok) break;
         tc_fence_after();
         const uint32_t dset = tmem_base + cb * G::kSetCols;
-        const uint64_t ad = sdesc(smem_u32(smem + st * G::kStageBytes));
-        const uint64_t bd = sdesc(smem_u32(smem + st * G::kStageBytes + NSL * A_PLANE));
+        const uint64_t ad = sdesc<BK>(smem_u32(smem + st * G::kStageBytes));
+        const uint64_t bd = sdesc<BK>(smem_u32(smem + st * G::kStageBytes + NSL * A_PLANE));
         if (elected) {
           // slice pa of A against the B slices 0 .. NSL-1-pa stacked along N (adjacent in shared
           // memory): one MMA adds A_pa B_pb to the accumulator of order pa + pb for every pb,
@@ -857,17 +872,17 @@ k_tc_prepare(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ it
 #pragma unroll
       for (int k = 0; k < kPairs; ++k) {
         const size_t idx = (static_cast<size_t>(y) * S.nxp + x0 + 64 * k + 2 * lane) / 2;
-        if (S.lowm_x) {
-          // six slices: the first four are stage 0's operand, all six the low-mode product's
+        if (S.tc_nr == kLowNS) {
+          // six slices (mixed modes: the first four are stage 0's operand, all six the low-mode product's)
           uint32_t code[kLowNS];
           slice_codes2_df<BF16, kLowNS>(v[j][k], vl[j][k], make_float2(s, s), make_float2(is, is), code);
 #pragma unroll
           for (int q = 0; q < kLowNS; ++q) out32[q * (plane / 2) + idx] = code[q];
         } else {
-          uint32_t code[NS];
-          slice_codes2_df<BF16, NS>(v[j][k], vl[j][k], make_float2(s, s), make_float2(is, is), code);
+          uint32_t code[4];
+          slice_codes2_df<BF16, 4>(v[j][k], vl[j][k], make_float2(s, s), make_float2(is, is), code);
 #pragma unroll
-          for (int q = 0; q < NS; ++q) out32[q * (plane / 2) + idx] = code[q];
+          for (int q = 0; q < 4; ++q) out32[q * (plane / 2) + idx] = code[q];
         }
       }
       if (lane == 0) S.tc_e[0][static_cast<size_t>(y) * kblocks + x0 / KC] = static_cast<int8_t>(E);
@@ -965,16 +980,16 @@ k_tc_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         const size_t idx = (static_cast<size_t>(y) * T.nxp + xb * KC + 64 * k + 2 * lane) / 2;
-        if (T.lowm_x) {
+        if (T.tc_nr == kLowNS) {
           uint32_t code[kLowNS];
           slice_codes2_df<BF16, kLowNS>(ch[c][k], cl[c][k], make_float2(up, up), make_float2(is, is), code);
 #pragma unroll
           for (int q = 0; q < kLowNS; ++q) out32[q * (plane / 2) + idx] = code[q];
         } else {
-          uint32_t code[NS];
-          slice_codes2_df<BF16, NS>(ch[c][k], cl[c][k], make_float2(up, up), make_float2(is, is), code);
+          uint32_t code[4];
+          slice_codes2_df<BF16, 4>(ch[c][k], cl[c][k], make_float2(up, up), make_float2(is, is), code);
 #pragma unroll
-          for (int q = 0; q < NS; ++q) out32[q * (plane / 2) + idx] = code[q];
+          for (int q = 0; q < 4; ++q) out32[q * (plane / 2) + idx] = code[q];
         }
       }
       if (lane == 0) T.tc_e[0][static_cast<size_t>(y) * (T.nxp / KC) + xb] = static_cast<int8_t>(E);
@@ -1601,20 +1616,21 @@ k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   }
 }
 
-template <bool BF16, int STAGE>
+template <bool BF16, int STAGE, int NSL>
 cudaError_t set_attr() {
-  return cudaFuncSetAttribute(k_prec_tc<BF16, STAGE, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              TcGeom<NS>::kSmem);
+  return cudaFuncSetAttribute(k_prec_tc<BF16, STAGE, NSL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              TcGeom<NSL>::kSmem);
 }
 
-template <bool BF16>
+template <bool BF16, int NSL>
 void launch_all(const LaunchCfg& c, int stage, int mode, int* err) {
   const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
+  constexpr int smem = TcGeom<NSL>::kSmem;
   switch (stage) {
-    case 0: launch_cfg(c, k_prec_tc<BF16, 0, NS>, c.grid, kThreads, TcGeom<NS>::kSmem, c.slots, c.items, c.n_items, mode, err, wc); break;
-    case 1: launch_cfg(c, k_prec_tc<BF16, 1, NS>, c.grid, kThreads, TcGeom<NS>::kSmem, c.slots, c.items, c.n_items, mode, err, wc); break;
-    case 2: launch_cfg(c, k_prec_tc<BF16, 2, NS>, c.grid, kThreads, TcGeom<NS>::kSmem, c.slots, c.items, c.n_items, mode, err, wc); break;
-    default: launch_cfg(c, k_prec_tc<BF16, 3, NS>, c.grid, kThreads, TcGeom<NS>::kSmem, c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 0: launch_cfg(c, k_prec_tc<BF16, 0, NSL>, c.grid, kThreads, smem, c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 1: launch_cfg(c, k_prec_tc<BF16, 1, NSL>, c.grid, kThreads, smem, c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 2: launch_cfg(c, k_prec_tc<BF16, 2, NSL>, c.grid, kThreads, smem, c.slots, c.items, c.n_items, mode, err, wc); break;
+    default: launch_cfg(c, k_prec_tc<BF16, 3, NSL>, c.grid, kThreads, smem, c.slots, c.items, c.n_items, mode, err, wc); break;
   }
 }
 
@@ -1627,11 +1643,11 @@ bool tc_supported() {
     cudaGetLastError();
     return false;
   }
-  if (p.major != 10 || p.sharedMemPerBlockOptin < static_cast<size_t>(TcGeom<NS>::kSmem)) return false;
+  if (p.major != 10 || p.sharedMemPerBlockOptin < static_cast<size_t>(TcGeom<4>::kSmem)) return false;
   // one CTA of kThreads threads at kMaxRegs registers each must fit an SM
   int blocks = 0;
-  if (set_attr<true, 0>() != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_prec_tc<true, 0, NS>, kThreads, TcGeom<NS>::kSmem) !=
+  if (set_attr<true, 0, 4>() != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_prec_tc<true, 0, 4>, kThreads, TcGeom<4>::kSmem) !=
           cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -1639,7 +1655,8 @@ bool tc_supported() {
   return blocks >= 1;
 }
 
-int tc_planes(int) { return NS; }
+int tc_step_k(int ns) { return ns == 4 ? TcGeom<4>::BK : TcGeom<6>::BK; }
+int tc_tile_cols(int ns) { return ns == 4 ? TcGeom<4>::BN : TcGeom<6>::BN; }
 
 int tc_block() { return KC; }
 
@@ -1652,8 +1669,10 @@ static cudaError_t set_low_attr() {
 
 cudaError_t tc_init() {
   cudaError_t e = cudaSuccess;
-  const cudaError_t r[12] = {set_attr<false, 0>(), set_attr<false, 1>(), set_attr<false, 2>(), set_attr<false, 3>(),
-                             set_attr<true, 0>(),  set_attr<true, 1>(),  set_attr<true, 2>(),  set_attr<true, 3>(),
+  const cudaError_t r[16] = {set_attr<false, 0, 4>(), set_attr<false, 1, 4>(), set_attr<false, 2, 4>(),
+                             set_attr<false, 3, 4>(), set_attr<true, 0, 4>(),  set_attr<true, 1, 4>(),
+                             set_attr<true, 2, 4>(),  set_attr<true, 3, 4>(),  set_attr<true, 0, 6>(),
+                             set_attr<true, 1, 6>(),  set_attr<true, 2, 6>(),  set_attr<true, 3, 6>(),
                              set_low_attr<false, 0>(), set_low_attr<false, 1>(), set_low_attr<true, 0>(),
                              set_low_attr<true, 1>()};
   for (cudaError_t x : r)
@@ -1686,9 +1705,10 @@ void launch_unfold(const LaunchCfg& c, int mode) {
   launch_cfg(c, k_unfold, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
 }
 
-void launch_prec_tc(const LaunchCfg& c, int stage, int mode, int split_kind, int* err) {
-  if (split_kind == 0) launch_all<false>(c, stage, mode, err);
-  else launch_all<true>(c, stage, mode, err);
+void launch_prec_tc(const LaunchCfg& c, int stage, int mode, int split_kind, int ns, int* err) {
+  if (ns == 6) launch_all<true, 6>(c, stage, mode, err);
+  else if (split_kind == 0) launch_all<false, 4>(c, stage, mode, err);
+  else launch_all<true, 4>(c, stage, mode, err);
 }
 
 void launch_prec_tc_prepare(const LaunchCfg& c, int mode, int split_kind) {

@@ -659,7 +659,7 @@ void precondition(const Solve3Args& a, const State3& s, float wnorm, const float
       c.items = t.d_items[k];
       c.n_items = t.d_counts + k;
       c.grid = std::max(1, std::min(t.n_items[k], t.sm_count));
-      launch_prec_tc(c, kForm[k], 2, t.split, t.d_err);
+      launch_prec_tc(c, kForm[k], 2, t.split, t.ns, t.d_err);
       ++*a.launches;
     }
     if (with_dot) {
