@@ -54,14 +54,15 @@ thread_local std::string g_last_error;
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct PlanDev {
-  int n = 0, np = 0, bc = 0, ns = 0;
+  int n = 0, np = 0, bc = 0;
   int cls = -1;   // -1: the axis basis; 0 / 1: its even / odd mirror class (n = ceil(nfull / 2))
   int nfull = 0;  // nodes of the axis
   float* q = nullptr;   // [2][np][np]: hi plane, lo plane (3-D CUDA-core products only)
   float* qt = nullptr;  // [2][np][np]
   std::vector<double> lam;
-  void* tc = nullptr;   // tensor-core operand planes: [Q planes][Q^T planes], 2-byte elements
-  int tc_split = -1;
+  // tensor-core operand planes, [0] four slices, [1] six: [Q planes][Q^T planes], 2-byte elements,
+  // then the exponents
+  void* tc[2] = {nullptr, nullptr};
   // low-mode operands (six slices): Q^T rows k < 32 [6][32][np] with exponents [32][np/128];
   // Q columns k < 32 as rows [6][np][64] with exponents [np]; Q[:, :32] double-float [2][np][32]
   void* low = nullptr;
@@ -89,13 +90,16 @@ struct Workspace {
   SlotDesc* d_slots = nullptr;
   SlotScalars* d_sc = nullptr;
   SlotScalars* h_sc = nullptr;  // pinned
-  WorkItem *d_st = nullptr, *d_vec = nullptr, *d_gm = nullptr;
+  WorkItem *d_st = nullptr, *d_vec = nullptr;
+  WorkItem* d_gm[2] = {nullptr, nullptr};  // transform tiles of the problems with four, six slices
   WorkItem* d_sl = nullptr;     // one item per slot (tile 0), for the per-slot scalar kernels
-  int *d_counts = nullptr;      // [0] grid tiles, [1] vector items, [2] gemm items, [3] slots,
+  int *d_counts = nullptr;      // [0] grid tiles, [1] vector items, [2] transform tiles with four
+                                // slices, [11] with six, [3] slots,
                                 // [4] stencil tiles, [5] [6] low-mode tiles, [7] fold items,
                                 // [8] unfold tiles, [9] tensor-core problems, [10] grid tiles
                                 // of unfolded slots
-  int n_st = 0, n_vec = 0, n_gm = 0, n_sl = 0;
+  int n_st = 0, n_vec = 0, n_sl = 0;
+  int n_gm[2] = {0, 0};
   WorkItem* d_sten = nullptr;   // the stencil kernel's tiles (64 x sten_ty)
   int n_sten = 0;
   int sten_ty = 32;             // stencil tile height of this workspace (autotuned)
@@ -115,9 +119,12 @@ struct Workspace {
   float** d_outs = nullptr;
   int* d_dirs = nullptr;
   void* h_ptrs = nullptr;       // pinned staging for the pointer arrays
-  cudaGraphExec_t graph = nullptr;
-  int graph_iters = 0;
-  int64_t graph_nodes = 0;
+  // iteration graphs by graph_key (which kernels the lists need: a serving table meets several)
+  struct Graph {
+    cudaGraphExec_t exec = nullptr;
+    int64_t nodes = 0;
+  };
+  std::map<int, Graph> graphs;
   void* d_tmaps = nullptr;      // per slot 8 CUtensorMap (tensor-core modes)
   struct Ev { int kind; cudaEvent_t a, b; };
   std::vector<Ev> graph_events;  // profiling: event-record nodes of the graph
@@ -144,7 +151,8 @@ struct ext_ctx {
   std::map<int, PlanDev> plans;
   std::map<std::string, Workspace*> ws;
   std::mutex api_mu;  // serialises ext_solve* and the serving worker on the stream
-  int ns = 4;         // integer slices per transform operand: 4 (mixed modes) or 6 (FP32 mode)
+  int ns = 4;         // integer slices per transform operand: 6 in FP32 mode; 4 in mixed modes, where
+                      // build_slot may give a grid 6
   int split = 0;      // their type: 0 = FP16, 1 = BF16
   int* d_err = nullptr;   // device flag raised by a bounded wait that ran out
   int* h_err = nullptr;   // pinned copy
@@ -315,32 +323,24 @@ static void slice_plan_host(int n, int bc, int np, int split, std::vector<uint16
   slice_plan_basis(make_axis_basis(n, bc), np, split, 4, h, ex);
 }
 
-static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P) {
-  if (P->tc && P->tc_split == ctx->split) return EXT_OK;
-  if (P->tc) {
-    cudaFree(P->tc);
-    P->tc = nullptr;
-  }
+static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P, int ns) {
+  void*& tc = P->tc[ns == 6];
+  if (tc) return EXT_OK;
   std::vector<uint16_t> h;
   std::vector<int8_t> ex;
   const AxisBasis B = plan_basis(P->nfull, P->bc, P->cls);
-  slice_plan_basis(B, P->np, ctx->split, ctx->ns, h, ex);
+  slice_plan_basis(B, P->np, ctx->split, ns, h, ex);
   const size_t bytes = 2 * h.size() + ex.size();
-  if (cudaMalloc(&P->tc, bytes) != cudaSuccess) {
+  if (cudaMalloc(&tc, bytes) != cudaSuccess) {
     cudaGetLastError();
+    tc = nullptr;
     g_last_error = "cudaMalloc of tensor-core plan failed";
     return EXT_ENOMEM;
   }
-  BX_CUDA(cudaMemcpy(P->tc, h.data(), 2 * h.size(), cudaMemcpyHostToDevice));
-  BX_CUDA(cudaMemcpy((char*)P->tc + 2 * h.size(), ex.data(), ex.size(), cudaMemcpyHostToDevice));
-  P->tc_split = ctx->split;
-  P->ns = ctx->ns;
-  if (ctx->ns == 6) return EXT_OK;  // no low-mode correction in FP32 mode
+  BX_CUDA(cudaMemcpy(tc, h.data(), 2 * h.size(), cudaMemcpyHostToDevice));
+  BX_CUDA(cudaMemcpy((char*)tc + 2 * h.size(), ex.data(), ex.size(), cudaMemcpyHostToDevice));
+  if (ns == 6) return EXT_OK;  // no low-mode correction beside six slices
   // low-mode operands of the same basis
-  if (P->low) {
-    cudaFree(P->low);
-    P->low = nullptr;
-  }
   const int np = P->np, nkb = np / tc_block();
   const int m = std::min(kLowM, P->n);
   auto Qv = [&](int i, int k) { return (i < P->n && k < m) ? B.Q[(size_t)i * P->n + k] : 0.0; };
@@ -390,10 +390,10 @@ static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P) {
 }
 
 // Exponent arrays of a plan: t = 0 for Q rows, 1 for Q^T rows.
-static const int8_t* plan_exps(const PlanDev* P, int t) {
+static const int8_t* plan_exps(const PlanDev* P, int ns, int t) {
   const size_t plane = (size_t)P->np * P->np;
   const size_t nkb = P->np / tc_block();
-  return (const int8_t*)((const char*)P->tc + 2 * 2 * (size_t)P->ns * plane) +
+  return (const int8_t*)((const char*)P->tc[ns == 6] + 2 * 2 * (size_t)ns * plane) +
          t * (size_t)P->np * nkb;
 }
 
@@ -455,9 +455,22 @@ void bx::set_weights(SlotDesc& d, double hx, double hy) {
   d.aniso = (a != c) ? 1 : 0;
 }
 
+static void drop_graphs(Workspace* W) {
+  for (auto& g : W->graphs) cudaGraphExecDestroy(g.second.exec);
+  W->graphs.clear();
+}
+
+// The kernels an iteration of W launches: which lists hold work, and the scalar steps' place.
+static int graph_key(const Workspace* W) {
+  const int n[7] = {W->n_gm[0], W->n_gm[1], W->n_l1, W->n_fold, W->n_prep, W->aniso, W->fuse};
+  int k = 0;
+  for (int i = 0; i < 7; ++i) k |= (n[i] != 0) << i;
+  return k;
+}
+
 static void free_workspace(Workspace* W) {
   if (!W) return;
-  if (W->graph) cudaGraphExecDestroy(W->graph);
+  drop_graphs(W);
   for (auto& e : W->graph_events) {
     cudaEventDestroy(e.a);
     cudaEventDestroy(e.b);
@@ -468,7 +481,7 @@ static void free_workspace(Workspace* W) {
   cudaFree(W->d_st);
   cudaFree(W->d_sten);
   cudaFree(W->d_vec);
-  cudaFree(W->d_gm);
+  for (WorkItem* g : W->d_gm) cudaFree(g);
   cudaFree(W->d_sl);
   cudaFree(W->d_l1);
   cudaFree(W->d_l3);
@@ -524,9 +537,19 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   d.sten_ty = 32;
   d.n_sten_tiles = d.n_st_tiles;
   const size_t N = (size_t)nx * ny;
+  // slices per transform operand, and the low-mode correction of four-slice grids: always (1), never
+  // (0), or (2) for grids of side >= 2048 and for every grid of a call whose grids hold >= 2048^2 nodes
+  // together (large_call): there the correction's kernels run at throughput and the iterations
+  // they save outweigh their cost.  With 2, the other grids up to kSixNodes take six slices.
+  const bool automatic = ctx->ns == 4 && ctx->opt.low_modes == 2;
+  const bool low = ctx->ns == 4 && (ctx->opt.low_modes == 1 ||
+                                    (automatic && (std::max(nx, ny) >= kLowAutoSide || large_call)));
+  const int NS = ctx->ns == 6 || (automatic && !low && (long long)N <= kSixNodes) ? 6 : 4;
+  const int nr = low ? kLowNS : NS;  // slices of the residual
+  const int bn = tc_tile_cols(NS), bk = tc_step_k(NS);
+  d.tc_ns = NS;
   d.vec_chunk = vec_chunk_of((long long)N);
   d.n_vec_items = (int)((N + d.vec_chunk - 1) / d.vec_chunk);
-  const int bn = tc_tile_cols(ctx->ns), bk = tc_step_k(ctx->ns);
   const int n_gm = (d.nxp / 128) * (d.nyp / bn);
   d.n_gm_tiles = n_gm;
   set_weights(d, prob.hx, prob.hy);
@@ -568,15 +591,6 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     size_t o_g = 0, o_lh = 0, o_ljt = 0, o_ljte = 0, o_lz = 0, o_lmaps = 0;
   };
   std::vector<TcLay> tl;
-  const int NS = ctx->ns;
-  // the low-mode correction: always (1), never (0), or (2) for grids of side >= 2048 and for every
-  // grid of a call whose grids hold >= 2048^2 nodes together (large_call): there the correction's
-  // kernels run at throughput and the iterations they save outweigh their cost; on one smaller
-  // grid they are latency-bound and cost more than they save
-  const bool low = NS == 4 && (ctx->opt.low_modes == 1 ||
-                               (ctx->opt.low_modes == 2 &&
-                                (std::max(nx, ny) >= kLowAutoSide || large_call)));
-  const int nr = low ? kLowNS : NS;  // slices of the residual
   // transform problems: the slot itself or its classes
   {
     for (int cy = 0; cy < ((d.mir & 2) ? 2 : 1); ++cy)
@@ -685,8 +699,8 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     SlotDesc t = d;  // the slot's fields; a class problem overrides its domain and operands below
     PlanDev* qx = L.px;
     PlanDev* qy = L.py;
-    int rc2 = ensure_tc_plan(ctx, qx);
-    if (!rc2) rc2 = ensure_tc_plan(ctx, qy);
+    int rc2 = ensure_tc_plan(ctx, qx, NS);
+    if (!rc2) rc2 = ensure_tc_plan(ctx, qy, NS);
     if (rc2) return rc2;
     if (d.mir) {
       t.nx = qx->n;
@@ -722,16 +736,16 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     t.tc_t3 = A + L.o_tt3;
     t.tmaps = A + L.o_maps;
     for (int k = 0; k < 4; ++k) t.tc_e[k] = (int8_t*)(A + L.o_ex + k * nex);
-    t.tc_eb[0] = plan_exps(qx, 1);  // Qx^T rows
-    t.tc_eb[1] = plan_exps(qy, 1);  // Qy^T rows
-    t.tc_eb[2] = plan_exps(qx, 0);  // Qx rows
-    t.tc_eb[3] = plan_exps(qy, 0);  // Qy rows
+    t.tc_eb[0] = plan_exps(qx, NS, 1);  // Qx^T rows
+    t.tc_eb[1] = plan_exps(qy, NS, 1);  // Qy^T rows
+    t.tc_eb[2] = plan_exps(qx, NS, 0);  // Qx rows
+    t.tc_eb[3] = plan_exps(qy, NS, 0);  // Qy rows
     BX_CUDA(cudaMemset(t.tc_r, 0, 2 * nr * Npc));
     BX_CUDA(cudaMemset(A + L.o_ex, 0, 4 * nex));
     CUtensorMap maps[kTcMaps];
     const size_t pxp = (size_t)t.nxp * t.nxp, pyp = (size_t)t.nyp * t.nyp;
-    uint16_t* qxb = (uint16_t*)qx->tc;
-    uint16_t* qyb = (uint16_t*)qy->tc;
+    uint16_t* qxb = (uint16_t*)qx->tc[NS == 6];
+    uint16_t* qyb = (uint16_t*)qy->tc[NS == 6];
     // A operands: r planes [P][nyp][nxp], T1 [P][nxp][nyp], T2 [P][nyp][nxp], T3 [P][nxp][nyp]
     int rc3 = make_tmap(&maps[0], t.tc_r, bf, t.nxp, (uint64_t)NS * t.nyp, 128, bk);
     if (!rc3) rc3 = make_tmap(&maps[1], t.tc_t1, bf, t.nyp, (uint64_t)NS * t.nxp, 128, bk);
@@ -787,14 +801,14 @@ static void set_slot_scalars(SlotHost& s, SlotScalars* sc) {
 }
 
 // Work items of the tensor-core problems of slot i (problem index kMirClasses * i + c).
-static void tc_items(const SlotHost& s, int i, std::vector<WorkItem>& gm, std::vector<WorkItem>& l1,
+static void tc_items(const SlotHost& s, int i, std::vector<WorkItem> (&gm)[2], std::vector<WorkItem>& l1,
                      std::vector<WorkItem>& l3, std::vector<WorkItem>& tcl) {
   for (int c = 0; c < kMirClasses; ++c) {
     if (s.d.mir == 0 && c > 0) break;
     if (((c & 1) && !(s.d.mir & 1)) || ((c & 2) && !(s.d.mir & 2))) continue;
     const SlotDesc& t = s.tcp[c];
     const int k = kMirClasses * i + c;
-    for (int tt = 0; tt < t.n_gm_tiles; ++tt) gm.push_back({k, tt});
+    for (int tt = 0; tt < t.n_gm_tiles; ++tt) gm[t.tc_ns == 6].push_back({k, tt});
     if (t.lowm_x) {
       for (int tt = 0; tt < t.n_l1_tiles; ++tt) l1.push_back({k, tt});
       for (int tt = 0; tt < t.n_l3_tiles; ++tt) l3.push_back({k, tt});
@@ -822,13 +836,18 @@ static int upload(T** dst, const std::vector<T>& v) {
   return EXT_OK;
 }
 
+// Whether every block of a kernel may add up the slot's partial sums itself.
+static bool fuse_fits(const SlotDesc& d) {
+  return std::max(((d.ny + 15) / 16) * ((d.nx + kStTileX - 1) / kStTileX), d.n_prec_parts) <= kFuseParts;
+}
+
 static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bool host_io,
                            Workspace** out) {
   std::unique_ptr<Workspace> W(new Workspace());
   W->key = shape_key(count, probs, host_io);
   W->host_io = host_io;
   W->slots.resize(count);
-  std::vector<WorkItem> st, vec, gm, l1, l3, fold, unfold, tcl, prep;
+  std::vector<WorkItem> st, vec, gm[2], l1, l3, fold, unfold, tcl, prep;
   long long call_nodes = 0;
   for (int i = 0; i < count; ++i) call_nodes += (long long)probs[i].nx * probs[i].ny;
   for (int i = 0; i < count; ++i) {
@@ -849,13 +868,13 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
     if (!d.mir)
       for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
   }
-  longest_first_tc(gm, W->slots);
+  for (auto& g : gm) longest_first_tc(g, W->slots);
   std::vector<WorkItem> sl;
   for (int i = 0; i < count; ++i) sl.push_back({i, 0});
   W->n_sl = (int)sl.size();
   W->n_st = (int)st.size();
   W->n_vec = (int)vec.size();
-  W->n_gm = (int)gm.size();
+  for (int k = 0; k < 2; ++k) W->n_gm[k] = (int)gm[k].size();
   BX_CUDA(cudaMalloc(&W->d_sc, sizeof(SlotScalars) * count));
   BX_CUDA(cudaMemset(W->d_sc, 0, sizeof(SlotScalars) * count));
   BX_CUDA(cudaMallocHost(&W->h_sc, sizeof(SlotScalars) * count));
@@ -869,7 +888,8 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   if (!rc) rc = upload(&W->d_tcp, tcps);
   if (!rc) rc = upload(&W->d_st, st);
   if (!rc) rc = upload(&W->d_vec, vec);
-  if (!rc) rc = upload(&W->d_gm, gm);
+  if (!rc) rc = upload(&W->d_gm[0], gm[0]);
+  if (!rc) rc = upload(&W->d_gm[1], gm[1]);
   if (!rc) rc = upload(&W->d_sl, sl);
   if (!rc) rc = upload(&W->d_sten, st);
   if (!rc) rc = upload(&W->d_l1, l1);
@@ -884,18 +904,15 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   // saves two launches an iteration (1024^2 solve: 334 -> 328 ms); with many slots, each met by
   // every block in turn, the repeated sums cost as much as the launches.
   W->fuse = count <= kFuseSlots;
-  for (const SlotHost& h : W->slots) {
-    const int pq_parts = ((h.d.ny + 15) / 16) * ((h.d.nx + kStTileX - 1) / kStTileX);
-    if (std::max(pq_parts, h.d.n_prec_parts) > kFuseParts) W->fuse = false;
-  }
+  for (const SlotHost& h : W->slots) W->fuse = W->fuse && fuse_fits(h.d);
   W->n_l1 = (int)l1.size();
   W->n_l3 = (int)l3.size();
   W->n_fold = (int)fold.size();
   W->n_unfold = (int)unfold.size();
   W->n_tcl = (int)tcl.size();
   W->n_prep = (int)prep.size();
-  int counts[11] = {W->n_st, W->n_vec, W->n_gm, W->n_sl, W->n_sten, W->n_l1, W->n_l3,
-                    W->n_fold, W->n_unfold, W->n_tcl, W->n_prep};
+  int counts[12] = {W->n_st, W->n_vec, W->n_gm[0], W->n_sl, W->n_sten, W->n_l1, W->n_l3,
+                    W->n_fold, W->n_unfold, W->n_tcl, W->n_prep, W->n_gm[1]};
   BX_CUDA(cudaMalloc(&W->d_counts, sizeof(counts)));
   BX_CUDA(cudaMemcpy(W->d_counts, counts, sizeof(counts), cudaMemcpyHostToDevice));
   BX_CUDA(cudaMalloc(&W->d_phis, sizeof(void*) * count));
@@ -970,10 +987,12 @@ static LaunchCfg cfg_of(ext_ctx* ctx, Workspace* W, int which) {
     c.items = W->d_sten;
     c.n_items = W->d_counts + 4;
     c.grid = std::max(1, std::min(W->n_sten, ctx->sm_count * stencil_blocks_per_sm(W->sten_ty)));
-  } else {
-    c.items = W->d_gm;
-    c.n_items = W->d_counts + 2;
-    c.grid = std::max(1, std::min(W->n_gm, ctx->sm_count * 2));
+  } else {  // 2, 11: transform tiles with four and six slices, over the transform problems
+    const int k = which == 11;
+    c.slots = W->d_tcp;
+    c.items = W->d_gm[k];
+    c.n_items = W->d_counts + which;
+    c.grid = std::max(1, std::min(W->n_gm[k], ctx->sm_count));
   }
   return c;
 }
@@ -1039,15 +1058,12 @@ static void harvest(ext_ctx* ctx) {
 
 // with_finish = false: the next stencil forms rho and beta from the partials itself
 static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish = true) {
-  LaunchCfg g = cfg_of(ctx, W, 2);
+  const LaunchCfg g = cfg_of(ctx, W, 2), g6 = cfg_of(ctx, W, 11);
   // residual slices: unfolded slots directly, folded slots per mirror class
   if (W->n_prep > 0)
     timed(ctx, EXT_KERNEL_SPLIT, [&] { launch_prec_tc_prepare(cfg_of(ctx, W, 10), mode, ctx->split); }, g.stream);
   if (W->n_fold > 0)
     timed(ctx, EXT_KERNEL_FOLD, [&] { launch_tc_fold(cfg_of(ctx, W, 7), mode, ctx->split); }, g.stream);
-  // the transform kernels run over the tensor-core problems
-  g.slots = W->d_tcp;
-  g.grid = std::max(1, std::min(W->n_gm, ctx->sm_count));
   if (W->n_l1 > 0) {
     // the lowest modes in high precision: forward product, middle, inverse product
     LaunchCfg c1 = cfg_of(ctx, W, 5), cm = cfg_of(ctx, W, 6), c3 = cfg_of(ctx, W, 6);
@@ -1061,9 +1077,10 @@ static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish =
     timed(ctx, EXT_KERNEL_LOW_INV, [&] { launch_low_tc(c3, 1, mode, ctx->split, ctx->d_err); }, g.stream);
   }
   for (int s = 0; s < 4; ++s) {
-    timed(ctx, EXT_KERNEL_PREC0 + s, [&] {
-      launch_prec_tc(g, s, mode, ctx->split, ctx->ns, ctx->d_err);
-    }, g.stream);
+    if (W->n_gm[0] > 0)
+      timed(ctx, EXT_KERNEL_PREC0 + s, [&] { launch_prec_tc(g, s, mode, ctx->split, 4, ctx->d_err); }, g.stream);
+    if (W->n_gm[1] > 0)
+      timed(ctx, EXT_KERNEL_PREC0 + s, [&] { launch_prec_tc(g6, s, mode, ctx->split, 6, ctx->d_err); }, g.stream);
   }
   if (W->n_unfold > 0)
     timed(ctx, EXT_KERNEL_UNFOLD, [&] { launch_unfold(cfg_of(ctx, W, 8), mode); }, g.stream);
@@ -1092,11 +1109,9 @@ static void enqueue_iterations(ext_ctx* ctx, Workspace* W, int iters) {
 static int ensure_graph(ext_ctx* ctx, Workspace* W) {
   // with profiling on, the graph holds an event-record node before and after every kernel
   const int G = ctx->opt.iters_per_launch;
-  if (W->graph && W->graph_iters == G) return EXT_OK;
-  if (W->graph) {
-    cudaGraphExecDestroy(W->graph);
-    W->graph = nullptr;
-  }
+  const int key = graph_key(W);
+  if (W->graphs.count(key)) return EXT_OK;
+  Workspace::Graph made;
   cudaGraph_t g;
   if (ctx->opt.profile) {
     // events for the graph's timing nodes are created before capture begins
@@ -1112,7 +1127,7 @@ static int ensure_graph(ext_ctx* ctx, Workspace* W) {
   const int64_t before = ctx->launches.load();
   const size_t pend0 = ctx->pending.size();
   enqueue_iterations(ctx, W, G);
-  W->graph_nodes = ctx->launches - before;
+  made.nodes = ctx->launches - before;
   ctx->launches = before;  // captured, not launched
   W->graph_events.assign(ctx->pending.begin() + pend0, ctx->pending.end());
   ctx->pending.resize(pend0);
@@ -1121,13 +1136,13 @@ static int ensure_graph(ext_ctx* ctx, Workspace* W) {
     g_last_error = std::string("graph capture: ") + cudaGetErrorString(e);
     return EXT_ECUDA;
   }
-  e = cudaGraphInstantiate(&W->graph, g, 0);
+  e = cudaGraphInstantiate(&made.exec, g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) {
     g_last_error = std::string("graph instantiate: ") + cudaGetErrorString(e);
     return EXT_ECUDA;
   }
-  W->graph_iters = G;
+  W->graphs[key] = made;
   return EXT_OK;
 }
 
@@ -1162,10 +1177,7 @@ static int set_stencil_shape(ext_ctx* ctx, Workspace* W, int ty) {
   BX_CUDA(cudaMemcpy(W->d_counts + 4, &W->n_sten, sizeof(int), cudaMemcpyHostToDevice));
   BX_CUDA(cudaMemcpy(W->d_slots, descs.data(), sizeof(SlotDesc) * descs.size(), cudaMemcpyHostToDevice));
   W->sten_ty = ty;
-  if (W->graph) {
-    cudaGraphExecDestroy(W->graph);
-    W->graph = nullptr;
-  }
+  drop_graphs(W);
   return EXT_OK;
 }
 
@@ -1321,6 +1333,7 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
   ctx->last_tile_y = W->sten_ty;
   rc = ensure_graph(ctx, W);
   if (rc) return rc;
+  const Workspace::Graph graph = W->graphs[graph_key(W)];
   launch_prec(ctx, W, 1);
   BX_CUDA(cudaGetLastError());
   int max_blocks = 0;
@@ -1329,10 +1342,10 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
     const int mi = ctx->opt.maxit > 0 ? ctx->opt.maxit : 10 * std::max(p.nx, p.ny);
     max_blocks = std::max(max_blocks, mi);
   }
-  max_blocks = max_blocks / std::max(1, W->graph_iters) + 8;
+  max_blocks = max_blocks / std::max(1, ctx->opt.iters_per_launch) + 8;
   for (int blk = 0; blk < max_blocks; ++blk) {
-    BX_CUDA(cudaGraphLaunch(W->graph, s));
-    ctx->launches += W->graph_nodes;
+    BX_CUDA(cudaGraphLaunch(graph.exec, s));
+    ctx->launches += graph.nodes;
     BX_CUDA(cudaMemcpyAsync(W->h_sc, W->d_sc, sizeof(SlotScalars) * count, cudaMemcpyDeviceToHost, s));
     BX_CUDA(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
     BX_CUDA(cudaStreamSynchronize(s));
@@ -1513,7 +1526,8 @@ void ext_destroy(ext_ctx* ctx) {
   for (auto& kv : ctx->plans) {
     cudaFree(kv.second.q);
     cudaFree(kv.second.qt);
-    cudaFree(kv.second.tc);
+    cudaFree(kv.second.tc[0]);
+    cudaFree(kv.second.tc[1]);
     cudaFree(kv.second.low);
   }
   harvest(ctx);
@@ -1652,7 +1666,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
     const int n[3] = {X, Y, Z};
     for (int ax = 0; ax < 3; ++ax) {
       int rc = get_plan(ctx, n[ax], a.bc[ax], -1, &P[ax]);
-      if (!rc) rc = ensure_tc_plan(ctx, P[ax]);
+      if (!rc) rc = ensure_tc_plan(ctx, P[ax], NS);
       if (rc) return rc;
     }
   }
@@ -1717,7 +1731,8 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
     d[k] = SlotDesc{};
     d[k].sc = sc;
   }
-  const uint16_t* q[3] = {(const uint16_t*)P[0]->tc, (const uint16_t*)P[1]->tc, (const uint16_t*)P[2]->tc};
+  const uint16_t* q[3] = {(const uint16_t*)P[0]->tc[NS == 6], (const uint16_t*)P[1]->tc[NS == 6],
+                         (const uint16_t*)P[2]->tc[NS == 6]};
   const size_t pl[3] = {(size_t)X * X, (size_t)Y * Y, (size_t)Z * Z};
   auto QT = [&](int ax) { return (void*)(q[ax] + NS * pl[ax]); };  // Q^T planes follow the Q planes
   auto QQ = [&](int ax) { return (void*)q[ax]; };
@@ -1731,39 +1746,39 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   d[1].nyp = Z * Y; d[1].nxp = X; d[1].nx = X; d[1].ny = Z * Y;
   int rc = make_tmap(&m[0][0], S0, bf, X, (uint64_t)NS * Z * Y, 128, bk);
   if (!rc) rc = make_tmap(&m[0][4], QT(0), bf, X, (uint64_t)NS * X, bn, bk);
-  d[1].tc_e[0] = E0; d[1].tc_eb[0] = plan_exps(P[0], 1); d[1].tc_t1 = SA; d[1].tc_e[1] = EA;
+  d[1].tc_e[0] = E0; d[1].tc_eb[0] = plan_exps(P[0], NS, 1); d[1].tc_t1 = SA; d[1].tc_e[1] = EA;
   if (!rc) rc = make_tmap(&m[0][8], SA, bf, (uint64_t)Z * Y, (uint64_t)NS * X, 32);
   // [2] F2 (stage-0 form): A = SA as [X Z][Y], B = Qy^T -> SB [Y][X Z]
   d[2].nyp = X * Z; d[2].nxp = Y; d[2].nx = Y; d[2].ny = X * Z;
   if (!rc) rc = make_tmap(&m[1][0], SA, bf, Y, (uint64_t)NS * X * Z, 128, bk);
   if (!rc) rc = make_tmap(&m[1][4], QT(1), bf, Y, (uint64_t)NS * Y, bn, bk);
-  d[2].tc_e[0] = EA; d[2].tc_eb[0] = plan_exps(P[1], 1); d[2].tc_t1 = SB; d[2].tc_e[1] = EB;
+  d[2].tc_e[0] = EA; d[2].tc_eb[0] = plan_exps(P[1], NS, 1); d[2].tc_t1 = SB; d[2].tc_e[1] = EB;
   if (!rc) rc = make_tmap(&m[1][8], SB, bf, (uint64_t)X * Z, (uint64_t)NS * Y, 32);
   // [3] F3 (stage-1 form, weights): A = SB as [Y X][Z], B = Qz^T -> SA [Z][Y X]
   d[3].nxp = Y * X; d[3].nyp = Z; d[3].nx = Y * X; d[3].ny = Z;
   if (!rc) rc = make_tmap(&m[2][1], SB, bf, Z, (uint64_t)NS * Y * X, 128, bk);
   if (!rc) rc = make_tmap(&m[2][5], QT(2), bf, Z, (uint64_t)NS * Z, bn, bk);
-  d[3].tc_e[1] = EB; d[3].tc_eb[1] = plan_exps(P[2], 1); d[3].tc_t2 = SA; d[3].tc_e[2] = EA;
+  d[3].tc_e[1] = EB; d[3].tc_eb[1] = plan_exps(P[2], NS, 1); d[3].tc_t2 = SA; d[3].tc_e[2] = EA;
   d[3].lamx = lam; d[3].lamy = lam + (size_t)Y * X; d[3].wnorm = (float)(smin * smin);
   if (!rc) rc = make_tmap(&m[2][9], SA, bf, (uint64_t)Y * X, (uint64_t)NS * Z, 32);
   // [4] I1 (stage-2 form): A = SA as [Z Y][X], B = Qx -> SB [X][Z Y]
   d[4].nyp = Z * Y; d[4].nxp = X; d[4].nx = X; d[4].ny = Z * Y;
   if (!rc) rc = make_tmap(&m[3][2], SA, bf, X, (uint64_t)NS * Z * Y, 128, bk);
   if (!rc) rc = make_tmap(&m[3][6], QQ(0), bf, X, (uint64_t)NS * X, bn, bk);
-  d[4].tc_e[2] = EA; d[4].tc_eb[2] = plan_exps(P[0], 0); d[4].tc_t3 = SB; d[4].tc_e[3] = EB;
+  d[4].tc_e[2] = EA; d[4].tc_eb[2] = plan_exps(P[0], NS, 0); d[4].tc_t3 = SB; d[4].tc_e[3] = EB;
   if (!rc) rc = make_tmap(&m[3][10], SB, bf, (uint64_t)Z * Y, (uint64_t)NS * X, 32);
   // [5] I2 (stage-2 form): A = SB as [X Z][Y], B = Qy -> SA [Y][X Z]
   d[5].nyp = X * Z; d[5].nxp = Y; d[5].nx = Y; d[5].ny = X * Z;
   if (!rc) rc = make_tmap(&m[4][2], SB, bf, Y, (uint64_t)NS * X * Z, 128, bk);
   if (!rc) rc = make_tmap(&m[4][6], QQ(1), bf, Y, (uint64_t)NS * Y, bn, bk);
-  d[5].tc_e[2] = EB; d[5].tc_eb[2] = plan_exps(P[1], 0); d[5].tc_t3 = SA; d[5].tc_e[3] = EA;
+  d[5].tc_e[2] = EB; d[5].tc_eb[2] = plan_exps(P[1], NS, 0); d[5].tc_t3 = SA; d[5].tc_e[3] = EA;
   if (!rc) rc = make_tmap(&m[4][10], SA, bf, (uint64_t)X * Z, (uint64_t)NS * Y, 32);
   // [6] I3 (stage-3 form): A = SA as [Y X][Z], B = Qz -> z[Z][Y X] masked, r.z per tile
   d[6].nxp = Y * X; d[6].nyp = Z; d[6].nx = Y * X; d[6].ny = Z;
   if (!rc) rc = make_tmap(&m[5][3], SA, bf, Z, (uint64_t)NS * Y * X, 128, bk);
   if (!rc) rc = make_tmap(&m[5][7], QQ(2), bf, Z, (uint64_t)NS * Z, bn, bk);
   if (rc) return rc;
-  d[6].tc_e[3] = EA; d[6].tc_eb[3] = plan_exps(P[2], 0);
+  d[6].tc_e[3] = EA; d[6].tc_eb[3] = plan_exps(P[2], NS, 0);
   d[6].r = const_cast<float*>(io.rh); d[6].r_lo = const_cast<float*>(io.rl);
   d[6].q = const_cast<float*>(io.qh); d[6].q_lo = const_cast<float*>(io.ql);
   d[6].z = io.zh; d[6].z_lo = io.zl; d[6].mask = const_cast<uint8_t*>(io.mask); d[6].part = part;
@@ -2075,7 +2090,7 @@ static int serve_alloc_lists(ext_ctx::Serve* S, int cap) {
   cudaFree(W->d_st);
   cudaFree(W->d_sten);
   cudaFree(W->d_vec);
-  cudaFree(W->d_gm);
+  for (WorkItem* g : W->d_gm) cudaFree(g);
   cudaFree(W->d_l1);
   cudaFree(W->d_l3);
   cudaFree(W->d_fold);
@@ -2084,7 +2099,7 @@ static int serve_alloc_lists(ext_ctx::Serve* S, int cap) {
   cudaFree(W->d_prep);
   cudaFree(S->d_new);
   cudaFree(S->d_ret);
-  W->d_st = W->d_sten = W->d_vec = W->d_gm = W->d_l1 = W->d_l3 = S->d_new = S->d_ret = nullptr;
+  W->d_st = W->d_sten = W->d_vec = W->d_gm[0] = W->d_gm[1] = W->d_l1 = W->d_l3 = S->d_new = S->d_ret = nullptr;
   W->d_fold = W->d_unfold = W->d_tcl = W->d_prep = nullptr;
   BX_CUDA(cudaMalloc(&W->d_prep, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_fold, sizeof(WorkItem) * cap));
@@ -2095,17 +2110,14 @@ static int serve_alloc_lists(ext_ctx::Serve* S, int cap) {
   BX_CUDA(cudaMalloc(&W->d_l1, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_l3, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_vec, sizeof(WorkItem) * cap));
-  BX_CUDA(cudaMalloc(&W->d_gm, sizeof(WorkItem) * cap));
+  for (auto& g : W->d_gm) BX_CUDA(cudaMalloc(&g, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&S->d_new, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&S->d_ret, sizeof(WorkItem) * cap));
   S->cap_items = cap;
   // grids sized for the capacity
-  W->n_st = W->n_vec = W->n_gm = W->n_sten = W->n_l1 = W->n_l3 = cap;
+  W->n_st = W->n_vec = W->n_gm[0] = W->n_gm[1] = W->n_sten = W->n_l1 = W->n_l3 = cap;
   W->n_fold = W->n_unfold = W->n_tcl = W->n_prep = cap;
-  if (W->graph) {
-    cudaGraphExecDestroy(W->graph);
-    W->graph = nullptr;
-  }
+  drop_graphs(W);
   return EXT_OK;
 }
 
@@ -2123,8 +2135,8 @@ static int serve_init(ext_ctx* ctx) {
   BX_CUDA(cudaMemset(W->d_sc, 0, sizeof(SlotScalars) * cap));
   BX_CUDA(cudaMallocHost(&W->h_sc, sizeof(SlotScalars) * cap));
   memset(W->h_sc, 0, sizeof(SlotScalars) * cap);
-  BX_CUDA(cudaMalloc(&W->d_counts, 11 * sizeof(int)));
-  BX_CUDA(cudaMemset(W->d_counts, 0, 11 * sizeof(int)));
+  BX_CUDA(cudaMalloc(&W->d_counts, 12 * sizeof(int)));
+  BX_CUDA(cudaMemset(W->d_counts, 0, 12 * sizeof(int)));
   BX_CUDA(cudaMalloc(&W->d_sl, sizeof(WorkItem) * cap));
   W->n_sl = cap;  // the per-slot grid is sized for the slot table
   BX_CUDA(cudaMalloc(&W->d_phis, sizeof(void*) * cap));
@@ -2147,7 +2159,7 @@ static int serve_init(ext_ctx* ctx) {
 static int serve_rebuild_lists(ext_ctx* ctx) {
   ext_ctx::Serve* S = ctx->serve;
   Workspace* W = S->W;
-  std::vector<WorkItem> st, vec, gm, sl, l1, l3, fold, unfold, tcl, prep;
+  std::vector<WorkItem> st, vec, gm[2], sl, l1, l3, fold, unfold, tcl, prep;
   bool aniso = false;
   for (int i = 0; i < (int)S->slots.size(); ++i) {
     if (!S->slots[i].used) continue;
@@ -2163,9 +2175,9 @@ static int serve_rebuild_lists(ext_ctx* ctx) {
       for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
     sl.push_back({i, 0});
   }
-  longest_first_tc(gm, W->slots);
+  for (auto& g : gm) longest_first_tc(g, W->slots);
   size_t need = 0;
-  for (const auto* v : {&st, &vec, &gm, &l1, &l3, &fold, &unfold, &tcl, &prep}) need = std::max(need, v->size());
+  for (const auto* v : {&st, &vec, &gm[0], &gm[1], &l1, &l3, &fold, &unfold, &tcl, &prep}) need = std::max(need, v->size());
   if ((int)need > S->cap_items) {
     int cap = S->cap_items;
     while (cap < (int)need) cap *= 2;
@@ -2173,11 +2185,17 @@ static int serve_rebuild_lists(ext_ctx* ctx) {
     int rc = serve_alloc_lists(S, cap);
     if (rc) return rc;
   }
-  if (aniso != W->aniso && W->graph) {
-    cudaGraphExecDestroy(W->graph);
-    W->graph = nullptr;
-  }
   W->aniso = aniso;
+  // the launches: grids sized for the capacity, kernels without work left out (each mix of lists has
+  // its own graph), the scalar steps fused while few slots run
+  const int cap = S->cap_items;
+  W->n_gm[0] = gm[0].empty() ? 0 : cap;
+  W->n_gm[1] = gm[1].empty() ? 0 : cap;
+  W->n_l1 = W->n_l3 = l1.empty() ? 0 : cap;
+  W->n_fold = W->n_unfold = fold.empty() ? 0 : cap;
+  W->n_prep = prep.empty() ? 0 : cap;
+  W->fuse = sl.size() <= kFuseSlots;
+  for (const WorkItem& it : sl) W->fuse = W->fuse && fuse_fits(W->slots[it.slot].d);
   cudaStream_t s = W->stream;
   auto put = [&](WorkItem* dst, const std::vector<WorkItem>& v) -> int {
     if (!v.empty()) BX_CUDA(cudaMemcpyAsync(dst, v.data(), sizeof(WorkItem) * v.size(), cudaMemcpyHostToDevice, s));
@@ -2187,7 +2205,8 @@ static int serve_rebuild_lists(ext_ctx* ctx) {
   // the serving table keeps the 64 x 32 stencil tiles: its stencil list is the grid-tile list
   if (!rc) rc = put(W->d_sten, st);
   if (!rc) rc = put(W->d_vec, vec);
-  if (!rc) rc = put(W->d_gm, gm);
+  if (!rc) rc = put(W->d_gm[0], gm[0]);
+  if (!rc) rc = put(W->d_gm[1], gm[1]);
   if (!rc) rc = put(W->d_sl, sl);
   if (!rc) rc = put(W->d_l1, l1);
   if (!rc) rc = put(W->d_l3, l3);
@@ -2196,9 +2215,9 @@ static int serve_rebuild_lists(ext_ctx* ctx) {
   if (!rc) rc = put(W->d_tcl, tcl);
   if (!rc) rc = put(W->d_prep, prep);
   if (rc) return rc;
-  int counts[11] = {(int)st.size(), (int)vec.size(), (int)gm.size(), (int)sl.size(), (int)st.size(),
+  int counts[12] = {(int)st.size(), (int)vec.size(), (int)gm[0].size(), (int)sl.size(), (int)st.size(),
                     (int)l1.size(), (int)l3.size(), (int)fold.size(), (int)unfold.size(), (int)tcl.size(),
-                    (int)prep.size()};
+                    (int)prep.size(), (int)gm[1].size()};
   BX_CUDA(cudaMemcpyAsync(W->d_counts, counts, sizeof(counts), cudaMemcpyHostToDevice, s));
   // the host vectors die here: the copies above must finish first (pageable sources are staged)
   BX_CUDA(cudaStreamSynchronize(s));
@@ -2405,8 +2424,9 @@ static void serve_loop(ext_ctx* ctx) {
     if (!rc && active > 0) {
       rc = ensure_graph(ctx, W);
       if (!rc) {
-        if (cudaGraphLaunch(W->graph, W->stream) != cudaSuccess) rc = EXT_ECUDA;
-        ctx->launches += W->graph_nodes;
+        const Workspace::Graph& graph = W->graphs[graph_key(W)];
+        if (cudaGraphLaunch(graph.exec, W->stream) != cudaSuccess) rc = EXT_ECUDA;
+        ctx->launches += graph.nodes;
       }
     }
     if (!rc) {

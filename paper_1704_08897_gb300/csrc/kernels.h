@@ -72,8 +72,7 @@ void launch_apply(const SlotDesc* slot, int n_tiles, bool aniso, const float* p,
                   double* part, cudaStream_t s);
 
 // fast Poisson preconditioner (kernels_gemm_tc.cu): exact block-scaled integer slice planes stored
-// as FP16 (split_kind 0) or BF16 (split_kind 1), ns = 4 of them (mixed modes) or 6 (FP32 mode, BF16
-// only).  stage 0..3 = forward x, forward y (+ eigenvalue weights), inverse x, inverse y (+ mask,
+// as FP16 (split_kind 0) or BF16 (split_kind 1), ns = 4 or 6 of them per operand.  stage 0..3 = forward x, forward y (+ eigenvalue weights), inverse x, inverse y (+ mask,
 // dots).  mode 0: slots with active iterations; mode 1: slots with a pending preconditioner pass;
 // mode 2: every slot (verification entry point).  err receives 1 if a bounded wait ran out.
 void launch_prec_tc(const LaunchCfg& c, int stage, int mode, int split_kind, int ns, int* err);

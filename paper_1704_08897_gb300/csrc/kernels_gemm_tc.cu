@@ -31,9 +31,9 @@
 // 64-blocks (24 bits) cost this operator 30-80% more CG iterations than exact transforms; four on
 // 128-blocks come within 5-10% of them.
 //
-// FP32 mode runs the same kernels with six slices per operand (48 bits of each 128-block, orders
-// 0..5, 21 products), the accuracy of its double-float vectors: it takes the FP64 iteration's count
-// plus 10-20%.  Its tiles are 128 x 32 (six accumulators twice in TMEM) and its steps 32 deep.
+// FP32 mode, and the mixed modes' smaller grids, run the same kernels with six slices per operand
+// (48 bits of each 128-block, orders 0..5, 21 products), the accuracy of the double-float vectors:
+// they take the FP64 iteration's count plus 10-20%.  Its tiles are 128 x 32 (six accumulators twice in TMEM) and its steps 32 deep.
 //
 // Kernel structure (one CTA per SM, persistent over the (slot, tile) work list):
 //   warp 0      : TMA producer: 128B-swizzled K-major tiles of the slices of A and B, two 64-deep
@@ -1669,10 +1669,12 @@ static cudaError_t set_low_attr() {
 
 cudaError_t tc_init() {
   cudaError_t e = cudaSuccess;
-  const cudaError_t r[16] = {set_attr<false, 0, 4>(), set_attr<false, 1, 4>(), set_attr<false, 2, 4>(),
+  const cudaError_t r[20] = {set_attr<false, 0, 4>(), set_attr<false, 1, 4>(), set_attr<false, 2, 4>(),
                              set_attr<false, 3, 4>(), set_attr<true, 0, 4>(),  set_attr<true, 1, 4>(),
                              set_attr<true, 2, 4>(),  set_attr<true, 3, 4>(),  set_attr<true, 0, 6>(),
                              set_attr<true, 1, 6>(),  set_attr<true, 2, 6>(),  set_attr<true, 3, 6>(),
+                             set_attr<false, 0, 6>(), set_attr<false, 1, 6>(), set_attr<false, 2, 6>(),
+                             set_attr<false, 3, 6>(),
                              set_low_attr<false, 0>(), set_low_attr<false, 1>(), set_low_attr<true, 0>(),
                              set_low_attr<true, 1>()};
   for (cudaError_t x : r)
@@ -1706,9 +1708,8 @@ void launch_unfold(const LaunchCfg& c, int mode) {
 }
 
 void launch_prec_tc(const LaunchCfg& c, int stage, int mode, int split_kind, int ns, int* err) {
-  if (ns == 6) launch_all<true, 6>(c, stage, mode, err);
-  else if (split_kind == 0) launch_all<false, 4>(c, stage, mode, err);
-  else launch_all<true, 4>(c, stage, mode, err);
+  if (ns == 6) split_kind == 0 ? launch_all<false, 6>(c, stage, mode, err) : launch_all<true, 6>(c, stage, mode, err);
+  else split_kind == 0 ? launch_all<false, 4>(c, stage, mode, err) : launch_all<true, 4>(c, stage, mode, err);
 }
 
 void launch_prec_tc_prepare(const LaunchCfg& c, int mode, int split_kind) {
