@@ -1947,27 +1947,44 @@ static int single_setup(ext_ctx* ctx, const ext_problem* prob, const float* phi,
   return EXT_OK;
 }
 
+// Workspace and inputs of a single-stage call: the mask, the stage's input vector and the scalars of
+// an iterating slot at iteration 0 with beta = 0.
+static int stage_setup(ext_ctx* ctx, const ext_problem* prob, const float* phi, const float* v, bool op,
+                       Workspace** Wout) {
+  int rc = validate_problem(prob);
+  if (rc) return rc;
+  if (!is_device_ptr(phi) || !is_device_ptr(v)) return EXT_EINVAL;
+  Workspace* W = nullptr;
+  rc = get_workspace(ctx, 1, prob, false, &W);
+  if (rc) return rc;
+  if (!ctx->opt.autotune) rc = set_stencil_shape(ctx, W, ctx->opt.tile_y == 16 ? 16 : 32);
+  if (rc) return rc;
+  memset(W->h_sc, 0, sizeof(SlotScalars));
+  W->h_sc[0].active = 1;
+  W->h_sc[0].maxit = 1;
+  W->h_sc[0].status = ST_RUNNING;
+  BX_CUDA(cudaMemcpyAsync(W->d_sc, W->h_sc, sizeof(SlotScalars), cudaMemcpyHostToDevice, ctx->stream));
+  LaunchCfg c = cfg_of(ctx, W, 0);
+  c.grid = ctx->sm_count * 8;
+  timed(ctx, EXT_KERNEL_SETUP, [&] { launch_stage_setup(c, op, phi, v, prob->nx * prob->ny, prob->dir); });
+  BX_CUDA(cudaGetLastError());
+  *Wout = W;
+  return EXT_OK;
+}
+
 int ext_apply_biharmonic(ext_ctx* ctx, const ext_problem* prob, const float* phi, const float* p,
                          float* q, double* sum_pq) {
   if (!ctx || !is_device_ptr(p) || !is_device_ptr(q)) return EXT_EINVAL;
   std::lock_guard<std::mutex> lk(ctx->api_mu);
   Workspace* W = nullptr;
-  int rc = single_setup(ctx, prob, phi, p, &W);
+  // The solver's own stencil kernel at iteration 0 with beta = 0 and z = p: it forms
+  // p_new = z + 0 * p_old = p in its window (the set-up zeroed p_old), q = M L^2 p_new and the
+  // per-tile p.q partials, through the same tensor-copy or plain-load window path as in a solve.
+  int rc = stage_setup(ctx, prob, phi, p, true, &W);
   if (rc) return rc;
   SlotHost& sl = W->slots[0];
   cudaStream_t s = ctx->stream;
   const size_t N = (size_t)prob->nx * prob->ny;
-  // The solver's own stencil kernel at iteration 0 with beta = 0 and z = p: it forms
-  // p_new = z + 0 * p_old = p in its window (the set-up zeroed p_old), q = M L^2 p_new and the
-  // per-tile p.q partials, through the same tensor-copy or plain-load window path as in a solve.
-  BX_CUDA(cudaMemcpyAsync(sl.d.z, p, 4 * N, cudaMemcpyDeviceToDevice, s));
-  BX_CUDA(cudaMemsetAsync(sl.d.z_lo, 0, 4 * N, s));
-  const int it0 = 0, on = 1;
-  const float zero[2] = {0.f, 0.f};
-  char* dsc = reinterpret_cast<char*>(W->d_sc);
-  BX_CUDA(cudaMemcpyAsync(dsc + offsetof(SlotScalars, it), &it0, sizeof(int), cudaMemcpyHostToDevice, s));
-  BX_CUDA(cudaMemcpyAsync(dsc + offsetof(SlotScalars, active), &on, sizeof(int), cudaMemcpyHostToDevice, s));
-  BX_CUDA(cudaMemcpyAsync(dsc + offsetof(SlotScalars, beta_f), zero, sizeof(zero), cudaMemcpyHostToDevice, s));
   const LaunchCfg sc = cfg_of(ctx, W, 4);
   timed(ctx, EXT_KERNEL_STENCIL, [&] { launch_stencil(sc, W->aniso, W->sten_ty, ctx->d_err); });
   BX_CUDA(cudaGetLastError());
@@ -2007,14 +2024,10 @@ int ext_apply_preconditioner(ext_ctx* ctx, const ext_problem* prob, const float*
   if (!ctx || !r || !z) return EXT_EINVAL;
   std::lock_guard<std::mutex> lk(ctx->api_mu);
   Workspace* W = nullptr;
-  int rc = single_setup(ctx, prob, phi, r, &W);
+  int rc = stage_setup(ctx, prob, phi, r, false, &W);
   if (rc) return rc;
   SlotHost& sl = W->slots[0];
   const size_t N = (size_t)prob->nx * prob->ny;
-  BX_CUDA(cudaMemcpyAsync(sl.d.r, r, 4 * N, cudaMemcpyDefault, ctx->stream));
-  BX_CUDA(cudaMemsetAsync(sl.d.r_lo, 0, 4 * N, ctx->stream));
-  BX_CUDA(cudaMemsetAsync(sl.d.q, 0, 4 * N, ctx->stream));
-  BX_CUDA(cudaMemsetAsync(sl.d.q_lo, 0, 4 * N, ctx->stream));
   launch_prec(ctx, W, 2);
   BX_CUDA(cudaGetLastError());
   BX_CUDA(cudaMemcpyAsync(z, sl.d.z, 4 * N, cudaMemcpyDefault, ctx->stream));

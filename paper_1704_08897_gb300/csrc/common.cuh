@@ -512,7 +512,7 @@ __device__ __forceinline__ double warp_sum_strided(const double* p, int n, int s
 __device__ __forceinline__ double sum_pq(const SlotDesc& S) {
   return warp_sum_strided(S.pq_part, ((S.ny + 15) >> 4) * ((S.nx + kStTileX - 1) / kStTileX), 1);
 }
-// One warp: the sums of the slot's r.z and (for the flexible beta and mode 2) z.q partials.
+// One warp: the sums of the slot's r.z and (for the flexible beta) z.q partials.
 __device__ __forceinline__ void sum_rz(const SlotDesc& S, bool with_zq, double& rz, double& zq) {
   rz = warp_sum_strided(S.part + 2, S.n_prec_parts, 4);
   zq = with_zq ? warp_sum_strided(S.part + 3, S.n_prec_parts, 4) : 0.0;

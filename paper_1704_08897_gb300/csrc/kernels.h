@@ -53,6 +53,8 @@ bool is_device_ptr(const void* p);
 void launch_setup(const LaunchCfg& c, const float* const* phis, const float* const* fs,
                   const int* dirs);
 void launch_rhs_scale(const LaunchCfg& c);
+// set-up of a single-stage call on slot 0: mask and input vector v (n nodes; at most c.grid blocks)
+void launch_stage_setup(const LaunchCfg& c, bool op, const float* phi, const float* v, int n, int dir);
 // err receives 1 if a bounded wait for a tensor copy ran out; tile_y = 16 or 32 (tiles 64 wide)
 // fuse_prec: the blocks form rho and beta from the preconditioner's partials themselves
 void launch_stencil(const LaunchCfg& c, bool aniso, int tile_y, int* err, bool fuse_prec = false);
@@ -68,7 +70,12 @@ void launch_output(const LaunchCfg& c, const float* const* fs, float* const* out
 void launch_output64(const SlotDesc* slot, int n, const float* f, double* out, cudaStream_t s);
 // per-slot reduction of the last preconditioner stage's r.z, z.q partials -> rho, beta
 void launch_prec_finish(const LaunchCfg& c, int mode);
-void launch_apply(const SlotDesc* slot, int n_tiles, bool aniso, const float* p, float* q,
+// q = M L^2 p straight from the caller's arrays, the p.q partial of each tile of 64 x kApplyTileY
+constexpr int kApplyTileY = 16;
+inline int apply_tiles(int nx, int ny) {
+  return ((nx + kStTileX - 1) / kStTileX) * ((ny + kApplyTileY - 1) / kApplyTileY);
+}
+void launch_apply(const SlotDesc& slot, const float* phi, bool extend_out, const float* p, float* q,
                   double* part, cudaStream_t s);
 
 // fast Poisson preconditioner (kernels_gemm_tc.cu): exact block-scaled integer slice planes stored

@@ -706,7 +706,7 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         if (epi_vote(fail)) break;
         CompDotDF c_rz, c_zq;
         const bool mir_out = S.mir_out != 0;
-        const bool with_zq = !mir_out && (sc->flexible != 0 || mode == 2);
+        const bool with_zq = !mir_out && sc->flexible != 0;
         const int nx = S.nx, ny = S.ny;
         const size_t nn = static_cast<size_t>(nx) * ny;
         float* __restrict__ zh = S.z;
@@ -1014,7 +1014,7 @@ k_unfold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
     const int ntx = (S.mhx + 31) >> 5;
     const int x = (it.tile % ntx) * 32 + lane, y = (it.tile / ntx) * 8 + warp;
     CompDotDF c_rz, c_zq;
-    const bool with_zq = S.sc->flexible != 0 || mode == 2;  // z.q enters only the flexible beta
+    const bool with_zq = S.sc->flexible != 0;  // z.q enters only the flexible beta
     if (x < S.mhx && y < S.mhy) {
       const int xx = fx ? S.nx - 1 - x : x, yy = fy ? S.ny - 1 - y : y;
       // every load first: the classes' g at (y, x), then mask, r (and q) at the mirror nodes

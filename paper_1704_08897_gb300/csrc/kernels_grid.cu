@@ -7,6 +7,8 @@
 // matrix-free ("no need to form the 13-banded matrix", Sec. 2.2).
 //
 // CG vectors are double-float pairs of FP32 planes (hi, lo); see SlotDesc.
+#include <algorithm>
+
 #include "async.cuh"
 #include "common.cuh"
 #include "kernels.h"
@@ -77,11 +79,6 @@ __device__ __forceinline__ float stencil13_plain(const SlotDesc& S, const float*
   const float f = c[-2] + c[2], g = c[-2 * RS] + c[2 * RS];
   if (!ANISO) return 20.f * c[0] - 8.f * (e + n) + 2.f * d + (f + g);
   return S.wc * c[0] + S.wex * e + S.wey * n + S.wd * d + S.wfx * f + S.wfy * g;
-}
-
-template <bool ANISO, int RS = kHX>
-__device__ __forceinline__ float stencil13(const SlotDesc& S, const float* t, int ly, int lx) {
-  return stencil13_acc<ANISO, RS>(S, t, ly, lx).result();
 }
 
 // The isotropic 13-point stencil at two adjacent nodes (x, x+1) of a smem tile with an even row
@@ -270,6 +267,48 @@ k_rhs_scale(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ ite
       const f2 v = df_of(ldexp(S.b[g], e));
       S.r[g] = v.hi;
       S.r_lo[g] = v.lo;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Set-up of the single-stage entry points: the slot's mask from sign(phi) and the stage's input
+// vector v.  OPERATOR: z = v, z_lo = 0 and a zero direction p[0], as at iteration 0 of a solve;
+// otherwise the residual r = v, r_lo = 0.  25 (17) bytes a node, bound by HBM; the solve's full
+// set-up (FP64 right-hand side, thirteen planes) took 40% of these calls at 2048^2 nodes and more.
+// ---------------------------------------------------------------------------------------------
+template <bool OPERATOR>
+__global__ void __launch_bounds__(kVecThreads)
+k_stage_setup(const SlotDesc* __restrict__ slots, const float* __restrict__ phi, const float* __restrict__ v,
+              int extend_out) {
+  const SlotDesc& S = slots[0];
+  const int n = S.nx * S.ny;
+  uint8_t* __restrict__ mask = S.mask;
+  float* __restrict__ hi = OPERATOR ? S.z : S.r;
+  float* __restrict__ lo = OPERATOR ? S.z_lo : S.r_lo;
+  float* __restrict__ p = S.p[0];
+  float* __restrict__ p_lo = S.p_lo[0];
+  constexpr int U = 4;
+  for (int e0 = blockIdx.x * U * kVecThreads + threadIdx.x; e0 < n; e0 += gridDim.x * U * kVecThreads) {
+    float ph[U], x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * kVecThreads;
+      ph[u] = e < n ? __ldg(phi + e) : 0.f;
+      x[u] = e < n ? __ldg(v + e) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * kVecThreads;
+      if (e >= n) break;
+      const bool known = extend_out ? (ph[u] < 0.f) : (ph[u] > 0.f);
+      mask[e] = known ? 0 : 1;
+      hi[e] = x[u];
+      lo[e] = 0.f;
+      if (OPERATOR) {
+        p[e] = 0.f;
+        p_lo[e] = 0.f;
+      }
     }
   }
 }
@@ -902,7 +941,7 @@ k_prec_finish(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ i
     const int run = mode == 0 ? sc->active : (mode == 1 ? sc->need_prec : 1);
     if (!run) continue;
     double rz, zq;
-    sum_rz(S, sc->flexible != 0 || mode == 2, rz, zq);
+    sum_rz(S, sc->flexible != 0, rz, zq);
     __syncwarp();  // every lane has read the flags
     if (threadIdx.x == 0) finish_preconditioner(S, rz, zq, mode);
   }
@@ -941,42 +980,67 @@ k_output64(const SlotDesc* __restrict__ slots, const float* __restrict__ f, doub
 }
 
 // ---------------------------------------------------------------------------------------------
-// q = M L^2 p for a caller-supplied FP32 p (same compensated evaluation, one node per thread;
-// used by the entry point that allocates nothing).
+// q = M L^2 p for a caller-supplied FP32 p (the solver's compensated evaluation; used by the entry
+// point that allocates nothing): mask from phi's sign, 64 x 16 tiles, the window of p in shared
+// memory, p.q per tile in compensated FP32 (an FP64 product per node took longer than the rest of
+// the kernel).  12 bytes a node; a call on 1000 x 700 nodes is bound by its launches and the copy
+// of p.q back, so the descriptor travels as a kernel argument.
 // ---------------------------------------------------------------------------------------------
 template <bool ANISO>
 __global__ void __launch_bounds__(kStThreads)
-k_apply(const SlotDesc* __restrict__ slots, const float* __restrict__ p, float* __restrict__ q,
-        double* __restrict__ part) {
-  __shared__ float sp[kHalo];
-  __shared__ double red[64];
-  const SlotDesc& S = slots[0];
-  for (int tile = blockIdx.x; tile < S.n_st_tiles; tile += gridDim.x) {
-    int x0, y0;
-    tile_origin(S, tile, x0, y0);
-    for (int i = threadIdx.x; i < kHalo; i += blockDim.x) {
+k_apply(const __grid_constant__ SlotDesc S, const float* __restrict__ phi, int extend_out,
+        const float* __restrict__ p, float* __restrict__ q, double* __restrict__ part) {
+  constexpr int TY = kApplyTileY;
+  __shared__ __align__(16) float win[kWX * (TY + 4)];  // rows y0-2 .., columns x0-4 ..
+  __shared__ float2 red[kStThreads / 32];
+  const int ntx = (S.nx + kStTileX - 1) / kStTileX;
+  const int tile = blockIdx.x;
+  const int x0 = (tile % ntx) * kStTileX, y0 = (tile / ntx) * TY;
+  const bool interior = x0 >= 2 && y0 >= 2 && x0 + kStTileX + 2 <= S.nx && y0 + TY + 2 <= S.ny;
+  for (int i = threadIdx.x; i < kHX * (TY + 4); i += kStThreads) {
+    const int ly = i / kHX, lx = i - ly * kHX;
+    float v;
+    if (interior) {
+      v = __ldg(p + (size_t)(y0 - 2 + ly) * S.nx + x0 - 2 + lx);
+    } else {
       float s;
-      const int g = halo_src(S, x0, y0, i, s);
-      sp[i] = (s != 0.f) ? s * p[g] : 0.f;
+      const int g = halo_src_ty<TY>(S, x0, y0, i, s);
+      v = s != 0.f ? s * __ldg(p + g) : 0.f;
     }
-    __syncthreads();
-    double pq = 0.0;
-  bool run = false;
-    for (int k = threadIdx.x; k < kStTileX * kStTileY; k += blockDim.x) {
-      const int ly = k / kStTileX, lx = k - ly * kStTileX;
-      const int gx = x0 + lx, gy = y0 + ly;
-      if (gx >= S.nx || gy >= S.ny) continue;
-      const int g = gy * S.nx + gx;
-      float qv = 0.f;
-      if (S.mask[g]) qv = stencil13<ANISO>(S, sp, ly, lx);
-      q[g] = qv;
-      pq += (double)p[g] * (double)qv;
-    }
-    double d2 = 0.0;
-    block_sum2<kStThreads>(pq, d2, red);
-    if (threadIdx.x == 0) part[tile] = pq;
-    __syncthreads();
+    win[ly * kWX + lx + 2] = v;
   }
+  __syncthreads();
+  CompDot dot;
+#pragma unroll
+  for (int k = threadIdx.x; k < kStTileX * TY / 2; k += kStThreads) {
+    const int ly = k / (kStTileX / 2), lx = 2 * (k - ly * (kStTileX / 2));
+    const int gx = x0 + lx, gy = y0 + ly;
+    if (gx >= S.nx || gy >= S.ny) continue;
+    const size_t g = (size_t)gy * S.nx + gx;
+    const bool two = gx + 1 < S.nx;
+    const float f0 = __ldg(phi + g), f1 = two ? __ldg(phi + g + 1) : 0.f;
+    const bool u0 = !(extend_out ? f0 < 0.f : f0 > 0.f), u1 = two && !(extend_out ? f1 < 0.f : f1 > 0.f);
+    const float* c = win + (ly + 2) * kWX + lx + 4;
+    float2 r = make_float2(0.f, 0.f);
+    if (u0 || u1) {
+      if (!ANISO) {
+        const CompSum2 a = stencil13_pair_acc<kWX>(c);
+        r = a.result();
+      } else {
+        r.x = stencil13_acc<true, kWX>(S, win + 2, ly, lx).result();
+        r.y = two ? stencil13_acc<true, kWX>(S, win + 2, ly, lx + 1).result() : 0.f;
+      }
+    }
+    const float q0 = u0 ? r.x : 0.f, q1 = u1 ? r.y : 0.f;
+    q[g] = q0;
+    dot.add(c[0], q0);
+    if (two) {
+      q[g + 1] = q1;
+      dot.add(c[1], q1);
+    }
+  }
+  const double t = block_sum_comp<kStThreads>(dot, red);
+  if (threadIdx.x == 0) part[tile] = t;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -985,6 +1049,11 @@ k_apply(const SlotDesc* __restrict__ slots, const float* __restrict__ p, float* 
 void launch_setup(const LaunchCfg& c, const float* const* phis, const float* const* fs,
                   const int* dirs) {
   k_setup<<<c.grid, kStThreads, 0, c.stream>>>(c.slots, c.items, c.n_items, phis, fs, dirs);
+}
+void launch_stage_setup(const LaunchCfg& c, bool op, const float* phi, const float* v, int n, int dir) {
+  const int grid = std::max(1, std::min((n + 4 * kVecThreads - 1) / (4 * kVecThreads), c.grid));
+  if (op) k_stage_setup<true><<<grid, kVecThreads, 0, c.stream>>>(c.slots, phi, v, dir == 0);
+  else k_stage_setup<false><<<grid, kVecThreads, 0, c.stream>>>(c.slots, phi, v, dir == 0);
 }
 void launch_rhs_scale(const LaunchCfg& c) {
   k_rhs_scale<<<c.grid, kStThreads, 0, c.stream>>>(c.slots, c.items, c.n_items);
@@ -1051,11 +1120,11 @@ void launch_output64(const SlotDesc* slot, int n, const float* f, double* out, c
   grid = grid < 4096 ? grid : 4096;
   k_output64<<<grid, kVecThreads, 0, s>>>(slot, f, out);
 }
-void launch_apply(const SlotDesc* slot, int n_tiles, bool aniso, const float* p, float* q,
+void launch_apply(const SlotDesc& slot, const float* phi, bool extend_out, const float* p, float* q,
                   double* part, cudaStream_t s) {
-  const int grid = n_tiles < 4096 ? n_tiles : 4096;
-  if (aniso) k_apply<true><<<grid, kStThreads, 0, s>>>(slot, p, q, part);
-  else k_apply<false><<<grid, kStThreads, 0, s>>>(slot, p, q, part);
+  const int grid = apply_tiles(slot.nx, slot.ny);
+  if (slot.aniso) k_apply<true><<<grid, kStThreads, 0, s>>>(slot, phi, extend_out, p, q, part);
+  else k_apply<false><<<grid, kStThreads, 0, s>>>(slot, phi, extend_out, p, q, part);
 }
 
 }  // namespace bx
