@@ -156,6 +156,7 @@ struct ext_ctx {
   int split = 0;      // their type: 0 = FP16, 1 = BF16
   int* d_err = nullptr;   // device flag raised by a bounded wait that ran out
   int* h_err = nullptr;   // pinned copy
+  SlotScalars* h_sc3 = nullptr;  // pinned, two entries (3-D solves)
   // launch accounting and optional per-kernel timing (ext_options.profile)
   std::atomic<int64_t> launches{0};
   std::recursive_mutex plan_mu;  // plan cache: shared by user threads and the serving worker
@@ -1506,6 +1507,7 @@ int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out) {
   BX_CUDA(cudaMemset(ctx->d_err, 0, sizeof(int)));
   BX_CUDA(cudaMallocHost(&ctx->h_err, sizeof(int)));
   *ctx->h_err = 0;
+  BX_CUDA(cudaMallocHost(&ctx->h_sc3, 2 * sizeof(SlotScalars)));
   if (cuda_stream) {
     ctx->stream = (cudaStream_t)cuda_stream;
   } else {
@@ -1533,6 +1535,7 @@ void ext_destroy(ext_ctx* ctx) {
   harvest(ctx);
   cudaFree(ctx->d_err);
   cudaFreeHost(ctx->h_err);
+  cudaFreeHost(ctx->h_sc3);
   for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
   if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
@@ -1641,6 +1644,8 @@ static int args3(ext_ctx* ctx, const ext_problem3* p, Solve3Args& a) {
   a.true_res_every = ctx->opt.true_res_every;
   a.replace_factor = ctx->opt.replace_factor;
   a.stream = ctx->stream;
+  a.sm_count = ctx->sm_count;
+  a.h_sc = ctx->h_sc3;
   if (on_tc)
     a.tc_build = [ctx, &a](const Tc3Io& io, Tc3& t) { return tc3_build(ctx, a, io, t); };
   return EXT_OK;
@@ -1688,19 +1693,15 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   const int tiles3 = ((Y * X) / 128) * (Z / bn);
   double* part = (double*)take(sizeof(double) * 4 * (size_t)tiles3);
   float* lam = (float*)take(sizeof(float) * ((size_t)Y * X + Z));
-  SlotScalars* sc = (SlotScalars*)take(sizeof(SlotScalars));
+  SlotScalars* sc = io.sc;  // the solve's own (the passes run as its flags say)
   void* maps = take(6 * kTcMaps * sizeof(CUtensorMap));
   SlotDesc* descs = (SlotDesc*)take(7 * sizeof(SlotDesc));
-  if (!S0 || !SA || !SB || !E0 || !EA || !EB || !part || !lam || !sc || !maps || !descs) {
+  if (!S0 || !SA || !SB || !E0 || !EA || !EB || !part || !lam || !maps || !descs) {
     g_last_error = "cudaMalloc of the 3-D tensor-core workspace failed";
     return EXT_ENOMEM;
   }
   BX_CUDA(cudaMemset(S0, 0, 2 * (size_t)NS * N3));
   BX_CUDA(cudaMemset(E0, 0, N3 / 128));
-  SlotScalars hsc{};
-  hsc.active = 1;
-  hsc.need_prec = 1;
-  BX_CUDA(cudaMemcpy(sc, &hsc, sizeof(hsc), cudaMemcpyHostToDevice));
   // eigenvalues scaled like the stencil (largest 1/h^2 = 1): lam_y + lam_x per row of the
   // weighted product ([ky][kx] flattened), lam_z per column; wnorm = (smallest nonzero sum)^2
   const double c[3] = {1.0 / (a.h[0] * a.h[0]), 1.0 / (a.h[1] * a.h[1]), 1.0 / (a.h[2] * a.h[2])};

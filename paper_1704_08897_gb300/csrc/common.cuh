@@ -542,6 +542,39 @@ __device__ __forceinline__ void finish_pq(SlotScalars* sc, double pq) {
   sc->aro_n += 1;
 }
 
+// One thread, after an update with ||r||^2 = s: count the iteration and decide stop or residual
+// replacement.
+__device__ __forceinline__ void decide_update(SlotScalars* sc, double s) {
+  sc->rr = s;
+  const int itn = sc->it + 1;
+  sc->it = itn;
+  if (s <= sc->rtol2 * sc->bb || itn >= sc->maxit || !isfinite(s)) {
+    sc->active = 0;
+    sc->fold = 1;
+  } else if (s < sc->delta2 * sc->rr_ref || itn % sc->fold_every == 0) {
+    sc->fold = 1;
+  }
+}
+// One thread, after the true residual's ||r||^2 = s: converged, stopped, or continue with a fresh
+// preconditioner pass.
+__device__ __forceinline__ void decide_true(SlotScalars* sc, double s) {
+  sc->rr_true = s;
+  sc->rr = s;
+  sc->rr_ref = s;
+  sc->fold = 0;
+  sc->active = 0;
+  sc->need_prec = 0;
+  if (s <= sc->rtol2 * sc->bb) {
+    sc->status = ST_OK;
+  } else if (sc->status == ST_EBREAKDOWN) {
+  } else if (sc->it >= sc->maxit || !isfinite(s)) {
+    sc->status = ST_ENOTCONV;
+  } else {
+    sc->active = 1;
+    sc->need_prec = 1;
+  }
+}
+
 // beta of the next direction (flexible or Fletcher-Reeves); 0 before the first iteration.
 __device__ __forceinline__ double prec_beta(const SlotScalars* sc, double rz, double zq) {
   if (sc->it == 0) return 0.0;
@@ -557,9 +590,7 @@ __device__ __forceinline__ void record_preconditioner(SlotScalars* sc, double rz
 }
 // One thread: record rho and beta, or the breakdown.  Mode 1 (the pass after a residual
 // replacement) recomputes them for the same iteration.
-__device__ __forceinline__ void finish_preconditioner(const SlotDesc& S, double rz, double zq,
-                                                      int mode) {
-  SlotScalars* sc = S.sc;
+__device__ __forceinline__ void finish_preconditioner(SlotScalars* sc, double rz, double zq, int mode) {
   if (mode == 2) {
     sc->rho2[0] = rz;
     sc->zq = zq;

@@ -27,10 +27,10 @@ struct LaunchCfg {
 
 // Launch `kernel` under `c` (its stream and dependence form).
 template <class... KArgs, class... Args>
-inline void launch_cfg(const LaunchCfg& c, void (*kernel)(KArgs...), int grid, int threads, size_t smem,
+inline void launch_cfg(const LaunchCfg& c, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem,
                        Args... args) {
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3((unsigned)grid);
+  lc.gridDim = grid;
   lc.blockDim = dim3((unsigned)threads);
   lc.dynamicSmemBytes = smem;
   lc.stream = c.stream;
@@ -122,9 +122,10 @@ struct Tc3Io {
   const float *rh, *rl, *qh, *ql;
   float *zh, *zl;
   const uint8_t* mask;
+  SlotScalars* sc;
 };
 
-// three-dimensional extension (solve3d.cu): the CUDA-core double-float path, host-driven CG
+// three-dimensional extension (solve3d.cu)
 struct Solve3Args {
   int nx, ny, nz;
   int bc[3];               // ext_bc of x, y, z
@@ -140,6 +141,8 @@ struct Solve3Args {
   double replace_factor;
   cudaStream_t stream;
   long long* launches;     // incremented by every kernel launch (host counter)
+  int sm_count;
+  SlotScalars* h_sc;       // pinned, two entries: the scalars as blocks of iterations leave them
   // builds the tensor-core preconditioner for the given vectors (empty: CUDA-core transforms)
   std::function<int(const Tc3Io&, Tc3&)> tc_build;
 };

@@ -837,15 +837,7 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
       double s = 0.0;
       if (threadIdx.x < 32) s = warp_sum_strided(S.part, S.n_vec_items, 4);
       if (threadIdx.x == 0) {
-        sc->rr = s;
-        const int itn = sc->it + 1;
-        sc->it = itn;
-        if (s <= sc->rtol2 * sc->bb || itn >= sc->maxit || !isfinite(s)) {
-          sc->active = 0;
-          sc->fold = 1;
-        } else if (s < sc->delta2 * sc->rr_ref || itn % sc->fold_every == 0) {
-          sc->fold = 1;
-        }
+        decide_update(sc, s);
       }
     }
     __syncthreads();
@@ -898,27 +890,7 @@ k_true_residual(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__
       double sums[1];
       reduce_partials<kStThreads, 1>(S.part, S.n_st_tiles, sums, red);
       if (threadIdx.x == 0) {
-        const double s = sums[0];
-        sc->rr_true = s;
-        sc->rr = s;
-        sc->rr_ref = s;
-        sc->fold = 0;
-        if (sc->status == ST_EBREAKDOWN) {
-          sc->active = 0;
-          sc->need_prec = 0;
-          if (s <= sc->rtol2 * sc->bb) sc->status = ST_OK;
-        } else if (s <= sc->rtol2 * sc->bb) {
-          sc->status = ST_OK;
-          sc->active = 0;
-          sc->need_prec = 0;
-        } else if (sc->it >= sc->maxit || !isfinite(s)) {
-          sc->status = ST_ENOTCONV;
-          sc->active = 0;
-          sc->need_prec = 0;
-        } else {
-          sc->active = 1;
-          sc->need_prec = 1;
-        }
+        decide_true(sc, sums[0]);
       }
     }
     __syncthreads();
@@ -943,7 +915,7 @@ k_prec_finish(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ i
     double rz, zq;
     sum_rz(S, sc->flexible != 0, rz, zq);
     __syncwarp();  // every lane has read the flags
-    if (threadIdx.x == 0) finish_preconditioner(S, rz, zq, mode);
+    if (threadIdx.x == 0) finish_preconditioner(sc, rz, zq, mode);
   }
 }
 

@@ -16,11 +16,18 @@
 // that axis moved to the front, so that three products rotate the box through all three axes;
 // the eigenvalue weights come between the forward and the inverse three.
 //
-// The iteration is preconditioned CG from x = 0 with the Fletcher-Reeves beta, driven from the
-// host (one scalar read per reduction); every reduction sums per-block partials in a fixed
-// order, so results are reproducible bit for bit.
+// The iteration is preconditioned CG from x = 0 with the Fletcher-Reeves beta.  Its scalars live on
+// the device (the two-dimensional path's SlotScalars and its decisions: stop, residual
+// replacement, breakdown) and its kernels follow one another as dependent launches, in blocks of
+// kBlockIters iterations with the replacement work at the block's end; the host stays one block
+// ahead, reading the scalars that the block before left, so the device never waits for it.  (Read
+// after every reduction, three times an iteration, the scalars cost a 72 x 60 x 50 solve 80 of
+// its 330 us an iteration.)  Kernels whose flag is down return at once.  Every reduction sums
+// per-block partials in a fixed order, so results are reproducible bit for bit.
 #include <cmath>
+#include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -56,6 +63,13 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
   return s;
 }
 
+// Every kernel of the iteration first waits for the one before it (pdl_wait), then returns if the
+// flag that its pass runs under is down (no flag: always on).
+__device__ __forceinline__ bool gate_shut(const int* gate) {
+  pdl_wait();
+  return gate != nullptr && *static_cast<const volatile int*>(gate) == 0;
+}
+
 __device__ __forceinline__ int block_linear() {
   return (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
 }
@@ -84,7 +98,8 @@ __device__ __forceinline__ Taps7 taps7(const Grid3& G, int x, int y, int z) {
 }
 
 // Double-float Laplacian pass, marching along z.  A block of 32 x 8 threads owns 32 x kBy nodes of
-// (x, y) (two rows per thread, ty and ty + 8) and a chunk of kZc planes.  Each thread keeps its
+// (x, y) (two rows per thread, ty and ty + 8) and a chunk of zc planes (16, or fewer on boxes too small
+// to fill the device with such chunks).  Each thread keeps its
 // own two columns in registers (planes z - 1, z, z + 1 and the two in flight); the x and y
 // neighbours come from a shared-memory tile of the plane with its one-node halo, written once per
 // plane and double-buffered, so one barrier per plane suffices.  Global loads run two planes ahead
@@ -93,7 +108,6 @@ __device__ __forceinline__ Taps7 taps7(const Grid3& G, int x, int y, int z) {
 // FINAL = true: out = M L in (zero at known nodes), and the block's partial p.out (compensated).
 // The terms are added in the order centre, x-1, x+1, y-1, y+1, z-1, z+1, as the single-node form
 // would.
-constexpr int kZc = 16;                       // planes per block
 constexpr int kBy = 16;                       // rows per block
 constexpr int kTw = 34, kTh = kBy + 2;        // tile with halo
 constexpr int kHalo = 2 * kTw + 2 * kBy;      // halo cells of a tile
@@ -177,14 +191,15 @@ __device__ __forceinline__ f2 k3_node(const Grid3& G, const float* th, const flo
 
 template <bool FINAL>
 __global__ void __launch_bounds__(kT)
-k3_lap(Grid3 G, const float* __restrict__ ih, const float* __restrict__ il, float* __restrict__ oh,
-       float* __restrict__ ol, const uint8_t* __restrict__ mask, const float* __restrict__ ph,
-       const float* __restrict__ pl, double* __restrict__ part) {
+k3_lap(Grid3 G, int zc, const int* __restrict__ gate, const float* ih, const float* il,
+       float* __restrict__ oh, float* __restrict__ ol, const uint8_t* __restrict__ mask, const float* ph,
+       const float* pl, double* __restrict__ part) {
+  if (gate_shut(gate)) return;
   __shared__ double sh[kT / 32];
   __shared__ float tile[2][2][kTh * kTw];  // [buffer][hi, lo]
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * kBy, z0 = blockIdx.z * kZc;
-  const int z1 = min(z0 + kZc, G.nz);
+  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * kBy, z0 = blockIdx.z * zc;
+  const int z1 = min(z0 + zc, G.nz);
   const int x = x0 + tx;
   const int yr[2] = {y0 + ty, y0 + ty + 8};
   const bool in[2] = {x < G.nx && yr[0] < G.ny, x < G.nx && yr[1] < G.ny};
@@ -265,8 +280,10 @@ k3_lap(Grid3 G, const float* __restrict__ ih, const float* __restrict__ il, floa
 // double-float copy (rh, rl) of out when rh is given.
 template <int MODE>
 __global__ void __launch_bounds__(kT)
-k3_lap64(Grid3 G, const double* __restrict__ in, double* __restrict__ out, const uint8_t* __restrict__ mask,
-         const double* __restrict__ b, double* __restrict__ part, float* __restrict__ rh, float* __restrict__ rl) {
+k3_lap64(Grid3 G, const int* __restrict__ gate, const double* in, double* __restrict__ out,
+         const uint8_t* __restrict__ mask, const double* __restrict__ b, double* __restrict__ part,
+         float* __restrict__ rh, float* __restrict__ rl) {
+  if (gate_shut(gate)) return;
   __shared__ double sh[kT / 32];
   const int x = blockIdx.x * 32 + (threadIdx.x & 31);
   const int y = blockIdx.y * 8 + (threadIdx.x >> 5);
@@ -341,43 +358,90 @@ k3_init(size_t n, const double* __restrict__ b, double s, float* __restrict__ rh
   }
 }
 
-// x += alpha p, r -= alpha q (double-float), partial ||r||^2
-__global__ void __launch_bounds__(kT)
-k3_update(size_t n, f2 alpha, const float* __restrict__ ph, const float* __restrict__ pl,
-          const float* __restrict__ qh, const float* __restrict__ ql, float* __restrict__ xh,
-          float* __restrict__ xl, float* __restrict__ rh, float* __restrict__ rl, double* __restrict__ part) {
-  __shared__ double sh[kT / 32];
-  const f2 na{-alpha.hi, -alpha.lo};
+// x += alpha p, r -= alpha q (double-float), partial ||r||^2 per block
+__global__ void __launch_bounds__(kT, 4)
+k3_update(size_t n, const SlotScalars* sc, const float* ph, const float* pl, const float* qh,
+          const float* ql, float* xh, float* xl, float* rh, float* rl, double* __restrict__ part) {
+  __shared__ float2 sh[kT / 32];
+  if (gate_shut(&sc->active)) return;
+  const f2 alpha{sc->alpha_f[0], sc->alpha_f[1]}, na{-alpha.hi, -alpha.lo};
   CompDotDF rr;
-  for (size_t i = blockIdx.x * static_cast<size_t>(kT) + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * kT) {
-    float a = xh[i], al = xl[i];
-    df_axpy(a, al, alpha, ph[i], pl[i]);
-    xh[i] = a;
-    xl[i] = al;
-    float r = rh[i], rlo = rl[i];
-    df_axpy(r, rlo, na, qh[i], ql[i]);
-    rh[i] = r;
-    rl[i] = rlo;
-    rr.add(r, rlo, r, rlo);
+  const size_t n4 = n / 4;
+  for (size_t i = blockIdx.x * static_cast<size_t>(kT) + threadIdx.x; i < n4; i += static_cast<size_t>(gridDim.x) * kT) {
+    const float4 p = reinterpret_cast<const float4*>(ph)[i], po = reinterpret_cast<const float4*>(pl)[i];
+    const float4 q = reinterpret_cast<const float4*>(qh)[i], qo = reinterpret_cast<const float4*>(ql)[i];
+    float4 x = reinterpret_cast<float4*>(xh)[i], xo = reinterpret_cast<float4*>(xl)[i];
+    float4 r = reinterpret_cast<float4*>(rh)[i], ro = reinterpret_cast<float4*>(rl)[i];
+    df_axpy(x.x, xo.x, alpha, p.x, po.x);
+    df_axpy(x.y, xo.y, alpha, p.y, po.y);
+    df_axpy(x.z, xo.z, alpha, p.z, po.z);
+    df_axpy(x.w, xo.w, alpha, p.w, po.w);
+    df_axpy(r.x, ro.x, na, q.x, qo.x);
+    df_axpy(r.y, ro.y, na, q.y, qo.y);
+    df_axpy(r.z, ro.z, na, q.z, qo.z);
+    df_axpy(r.w, ro.w, na, q.w, qo.w);
+    reinterpret_cast<float4*>(xh)[i] = x;
+    reinterpret_cast<float4*>(xl)[i] = xo;
+    reinterpret_cast<float4*>(rh)[i] = r;
+    reinterpret_cast<float4*>(rl)[i] = ro;
+    rr.add(r.x, ro.x, r.x, ro.x);
+    rr.add(r.y, ro.y, r.y, ro.y);
+    rr.add(r.z, ro.z, r.z, ro.z);
+    rr.add(r.w, ro.w, r.w, ro.w);
   }
-  const double s = block_sum_d(rr.value(), sh);
+  if (blockIdx.x == 0)
+    for (size_t i = 4 * n4 + threadIdx.x; i < n; i += kT) {
+      df_axpy(xh[i], xl[i], alpha, ph[i], pl[i]);
+      df_axpy(rh[i], rl[i], na, qh[i], ql[i]);
+      rr.add(rh[i], rl[i], rh[i], rl[i]);
+    }
+  const double s = block_sum_comp<kT>(rr.as_comp(), sh);
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
 // p = z + beta p (double-float)
 __global__ void __launch_bounds__(kT)
-k3_direction(size_t n, f2 beta, const float* __restrict__ zh, const float* __restrict__ zl,
-             float* __restrict__ ph, float* __restrict__ pl) {
-  for (size_t i = blockIdx.x * static_cast<size_t>(kT) + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * kT) {
-    const f2 v = df_fma(beta, f2{ph[i], pl[i]}, f2{zh[i], zl[i]});
-    ph[i] = v.hi;
-    pl[i] = v.lo;
+k3_direction(size_t n, const SlotScalars* sc, const float* zh, const float* zl, float* ph, float* pl) {
+  if (gate_shut(&sc->active)) return;
+  const f2 beta{sc->beta_f[0], sc->beta_f[1]};
+  const size_t n4 = n / 4;
+  for (size_t i = blockIdx.x * static_cast<size_t>(kT) + threadIdx.x; i < n4; i += static_cast<size_t>(gridDim.x) * kT) {
+    const float4 z = reinterpret_cast<const float4*>(zh)[i], zo = reinterpret_cast<const float4*>(zl)[i];
+    const float4 p = reinterpret_cast<const float4*>(ph)[i], po = reinterpret_cast<const float4*>(pl)[i];
+    const f2 a = df_fma(beta, f2{p.x, po.x}, f2{z.x, zo.x}), b = df_fma(beta, f2{p.y, po.y}, f2{z.y, zo.y});
+    const f2 c = df_fma(beta, f2{p.z, po.z}, f2{z.z, zo.z}), d = df_fma(beta, f2{p.w, po.w}, f2{z.w, zo.w});
+    reinterpret_cast<float4*>(ph)[i] = make_float4(a.hi, b.hi, c.hi, d.hi);
+    reinterpret_cast<float4*>(pl)[i] = make_float4(a.lo, b.lo, c.lo, d.lo);
   }
+  if (blockIdx.x == 0)
+    for (size_t i = 4 * n4 + threadIdx.x; i < n; i += kT) {
+      const f2 v = df_fma(beta, f2{ph[i], pl[i]}, f2{zh[i], zl[i]});
+      ph[i] = v.hi;
+      pl[i] = v.lo;
+    }
+}
+
+// One warp: a scalar step from n partials (entry i at part[i * stride]).  KIND 0: p.q -> alpha;
+// 1: ||r||^2 after an update; 2: r.z -> rho, beta (mode 0 or 1); 3: ||b - A x||^2 of a replacement.
+template <int KIND>
+__global__ void __launch_bounds__(32)
+k3_finish(SlotScalars* sc, const double* part, int n, int stride, int mode) {
+  pdl_wait();
+  const int on = KIND == 3 ? sc->fold : (KIND == 2 && mode == 1) ? sc->need_prec : sc->active;
+  if (!on) return;
+  const double v = warp_sum_strided(part, n, stride);
+  __syncwarp();  // every lane has read its flag
+  if (threadIdx.x != 0) return;
+  if (KIND == 0) finish_pq(sc, v);
+  if (KIND == 1) decide_update(sc, v);
+  if (KIND == 2) finish_preconditioner(sc, v, 0.0, mode);
+  if (KIND == 3) decide_true(sc, v);
 }
 
 // the iterate as FP64 (for the true residual)
 __global__ void __launch_bounds__(kT)
-k3_to_double(size_t n, const float* __restrict__ h, const float* __restrict__ l, double* __restrict__ d) {
+k3_to_double(size_t n, const int* __restrict__ gate, const float* h, const float* l, double* __restrict__ d) {
+  if (gate_shut(gate)) return;
   for (size_t i = blockIdx.x * static_cast<size_t>(kT) + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * kT)
     d[i] = static_cast<double>(h[i]) + static_cast<double>(l[i]);
 }
@@ -412,104 +476,126 @@ k3_sum(const double* __restrict__ part, int n, double* __restrict__ out, int str
 }
 
 // ---------------------------------------------------------------------------------------------
-// Transform products.  D[m][n] = sum_k A[m][k] B[n][k] for double-float A ([M][K], row-major, lo
-// plane separate) and B (rows of length ldb, lo plane at + ldb * ldb), written with n first:
-// out[n * M + m].  Tiles of 64 x 64, k in steps of 16 through shared memory; each thread keeps
-// 4 x 4 compensated dot products (Ogita-Rump-Oishi Dot2 of double-float operands).
+// Transform products on the CUDA cores (boxes with a side that is no multiple of 128).
+// D[m][n] = sum_k A[m][k] B[n][k] for double-float A ([M][K], row-major, lo plane separate) and B
+// (rows of length ldb, lo plane at + ldb * ldb), written with n first: out[n * M + m].  Each thread
+// keeps 2 x 4 compensated dot products (Ogita-Rump-Oishi Dot2 of double-float operands, pairs of n on
+// packed FP32x2).
+//
+// FORM 0: a plain product.  FORM 1 (the third): times the weights wnorm / (lam_z + lam_y + lam_x)^2
+// of the modes [kz][ky][kx], zero for a zero sum (the constant mode when no axis is Dirichlet).
+// FORM 2 (the last): z = M Z, zero at known nodes, with the block's partial r.z.
+//
+// Bound by FP32 issue: twelve operations a multiply-add.  Tiles of 32 x 32 by 128 threads: a
+// 72 x 60 x 50 box then has about 280 blocks a product, two an SM, where 64 x 64 tiles left half the
+// SMs idle and the rest with eight warps (28-36 us a product); the next 16-deep slab is loaded into
+// registers while the current one multiplies.
 // ---------------------------------------------------------------------------------------------
-constexpr int GM = 64, GN = 64, GK = 16;
+constexpr int GM = 32, GN = 32, GK = 16, kGt = 128;
 
-__global__ void __launch_bounds__(kT)
-k3_gemm(const float* __restrict__ A, const float* __restrict__ Al, int M, int K,
-        const float* __restrict__ B, int ldb, int N, float* __restrict__ out, float* __restrict__ outl) {
-  __shared__ float As[2][GK][GM + 1];
-  __shared__ float Bs[2][GK][GN + 1];
-  const float* Bl = B + static_cast<size_t>(ldb) * ldb;
+struct Gemm3 {
+  const float *A, *Al, *B;
+  float *out, *outl;
+  int M, K, ldb, N;
+  const float *lx, *ly, *lz;  // FORM 1
+  int nx;
+  float wnorm;
+  const uint8_t* mask;        // FORM 2
+  const float *rh, *rl;
+  double* part;
+};
+
+template <int FORM>
+__global__ void __launch_bounds__(kGt)
+k3_gemm(Gemm3 g, const int* __restrict__ gate) {
+  __shared__ __align__(16) float As[2][2][GK][GM + 1];  // [buffer][hi, lo][k][m]
+  __shared__ __align__(16) float Bs[2][2][GK][GN + 4];
+  __shared__ float2 sh[kGt / 32];
+  if (gate_shut(gate)) return;
+  const float* Bl = g.B + static_cast<size_t>(g.ldb) * g.ldb;
   const int m0 = blockIdx.x * GM, n0 = blockIdx.y * GN;
   const int t = threadIdx.x, tm = t & 15, tn = t >> 4;
-  CompDotDF acc[4][4];
-  for (int k0 = 0; k0 < K; k0 += GK) {
-    for (int e = t; e < GM * GK; e += kT) {
-      const int mm = e / GK, kk = e - mm * GK;
-      const int m = m0 + mm, k = k0 + kk;
-      const bool ok = m < M && k < K;
-      const size_t a = static_cast<size_t>(m) * K + k;
-      As[0][kk][mm] = ok ? A[a] : 0.f;
-      As[1][kk][mm] = ok ? Al[a] : 0.f;
+  const int lk = t & 15, lr = t >> 4;  // loads: k and first row of the slab (rows lr + 8 i)
+  constexpr int kRows = GM * GK / kGt;
+  float ra[2][kRows], rb[2][kRows];
+  auto fetch = [&](int k0) {
+    const int k = k0 + lk;
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      const int m = m0 + lr + 8 * i, n = n0 + lr + 8 * i;
+      const size_t a = static_cast<size_t>(m) * g.K + k, b = static_cast<size_t>(n) * g.ldb + k;
+      const bool oa = m < g.M && k < g.K, ob = n < g.N && k < g.K;
+      ra[0][i] = oa ? g.A[a] : 0.f;
+      ra[1][i] = oa ? g.Al[a] : 0.f;
+      rb[0][i] = ob ? __ldg(g.B + b) : 0.f;
+      rb[1][i] = ob ? __ldg(Bl + b) : 0.f;
     }
-    for (int e = t; e < GN * GK; e += kT) {
-      const int nn = e / GK, kk = e - nn * GK;
-      const int n = n0 + nn, k = k0 + kk;
-      const bool ok = n < N && k < K;
-      const size_t a = static_cast<size_t>(n) * ldb + k;
-      Bs[0][kk][nn] = ok ? B[a] : 0.f;
-      Bs[1][kk][nn] = ok ? Bl[a] : 0.f;
+  };
+  auto put = [&](int b) {
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      As[b][0][lk][lr + 8 * i] = ra[0][i];
+      As[b][1][lk][lr + 8 * i] = ra[1][i];
+      Bs[b][0][lk][lr + 8 * i] = rb[0][i];
+      Bs[b][1][lk][lr + 8 * i] = rb[1][i];
     }
-    __syncthreads();
+  };
+  CompDotDF2 acc[2][2];  // [row tm + 16 i][pair of columns 4 tn + 2 j]
+  fetch(0);
+  put(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = 0; k0 < g.K; k0 += GK) {
+    const bool more = k0 + GK < g.K;
+    if (more) fetch(k0 + GK);
 #pragma unroll 4
     for (int kk = 0; kk < GK; ++kk) {
-      float ah[4], al[4], bh[4], bl[4];
+      const float4 bh = *reinterpret_cast<const float4*>(&Bs[buf][0][kk][4 * tn]);
+      const float4 bl = *reinterpret_cast<const float4*>(&Bs[buf][1][kk][4 * tn]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        ah[i] = As[0][kk][tm + 16 * i];
-        al[i] = As[1][kk][tm + 16 * i];
-        bh[i] = Bs[0][kk][tn + 16 * i];
-        bl[i] = Bs[1][kk][tn + 16 * i];
+      for (int i = 0; i < 2; ++i) {
+        const float ah = As[buf][0][kk][tm + 16 * i], al = As[buf][1][kk][tm + 16 * i];
+        const float2 a2 = make_float2(ah, ah), l2 = make_float2(al, al);
+        acc[i][0].add(a2, l2, make_float2(bh.x, bh.y), make_float2(bl.x, bl.y));
+        acc[i][1].add(a2, l2, make_float2(bh.z, bh.w), make_float2(bl.z, bl.w));
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j].add(ah[i], al[i], bh[j], bl[j]);
     }
+    if (more) put(buf ^ 1);
     __syncthreads();
+    buf ^= 1;
   }
+  CompDotDF dot;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int m = m0 + tm + 16 * i, n = n0 + tn + 16 * j;
-      if (m < M && n < N) {
-        const f2 v = df_norm(acc[i][j].s, acc[i][j].c);
-        out[static_cast<size_t>(n) * M + m] = v.hi;
-        outl[static_cast<size_t>(n) * M + m] = v.lo;
+    for (int i = 0; i < 2; ++i) {
+      const int m = m0 + tm + 16 * i, n = n0 + 4 * tn + j;
+      if (m >= g.M || n >= g.N) continue;
+      const CompDotDF2& c = acc[i][j >> 1];
+      f2 v = (j & 1) ? df_norm(c.s.y, c.c.y) : df_norm(c.s.x, c.c.x);
+      const size_t o = static_cast<size_t>(n) * g.M + m;
+      if (FORM == 1) {
+        const float s = g.lz[n] + g.ly[m / g.nx] + g.lx[m % g.nx];
+        v = s > 0.f ? df_mul(v, spectral_weight_of(g.wnorm, s)) : f2{0.f, 0.f};
       }
+      if (FORM == 2) {
+        if (!g.mask[o]) v = f2{0.f, 0.f};
+        dot.add(g.rh[o], g.rl[o], v.hi, v.lo);
+      }
+      g.out[o] = v.hi;
+      g.outl[o] = v.lo;
     }
-}
-
-// Weights of the modes [kz][ky][kx]: wnorm / (lam_z + lam_y + lam_x)^2, zero for a zero sum (the
-// constant mode when no axis is Dirichlet).
-__global__ void __launch_bounds__(kT)
-k3_weights(int nx, int ny, int nz, const float* __restrict__ lx, const float* __restrict__ ly,
-           const float* __restrict__ lz, float wnorm, float* __restrict__ h, float* __restrict__ l) {
-  const size_t n = static_cast<size_t>(nx) * ny * nz;
-  for (size_t i = blockIdx.x * static_cast<size_t>(kT) + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * kT) {
-    const int kx = static_cast<int>(i % nx);
-    const int ky = static_cast<int>((i / nx) % ny);
-    const int kz = static_cast<int>(i / (static_cast<size_t>(nx) * ny));
-    const float s = lz[kz] + ly[ky] + lx[kx];
-    f2 v{0.f, 0.f};
-    if (s > 0.f) v = df_mul(f2{h[i], l[i]}, spectral_weight_of(wnorm, s));
-    h[i] = v.hi;
-    l[i] = v.lo;
+  if (FORM == 2) {
+    group_sum_pair<32>(dot.s, dot.c);
+    if ((t & 31) == 0) sh[t >> 5] = make_float2(dot.s, dot.c);
+    __syncthreads();
+    if (t < 32) {
+      const float2 v = sh[t & 3];
+      float s = v.x, c = v.y;
+      group_sum_pair<4>(s, c);
+      if (t == 0) g.part[blockIdx.y * gridDim.x + blockIdx.x] = (double)s + (double)c;
+    }
   }
-}
-
-// z = M Z (zero at known nodes) and the block's partial r.z
-__global__ void __launch_bounds__(kT)
-k3_mask_dot(size_t n, const float* __restrict__ Zh, const float* __restrict__ Zl, const uint8_t* __restrict__ mask,
-            const float* __restrict__ rh, const float* __restrict__ rl, float* __restrict__ zh,
-            float* __restrict__ zl, double* __restrict__ part) {
-  __shared__ double sh[kT / 32];
-  CompDotDF d;
-  for (size_t i = blockIdx.x * static_cast<size_t>(kT) + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * kT) {
-    const bool u = mask[i] != 0;
-    const float a = u ? Zh[i] : 0.f, b = u ? Zl[i] : 0.f;
-    zh[i] = a;
-    zl[i] = b;
-    d.add(rh[i], rl[i], a, b);
-  }
-  const double s = block_sum_d(d.value(), sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -524,35 +610,27 @@ k3_mask_dot(size_t n, const float* __restrict__ Zh, const float* __restrict__ Zl
     }                                                                 \
   } while (0)
 
-// Device state of one 3-D solve (allocated per call, freed on every return path).
+// Device state of one 3-D call: one allocation, freed on every return path.
 struct State3 {
   size_t n = 0;
-  int vec_blocks = 0;
+  int vec_blocks = 0, zc = 16;
   dim3 grid3, gridz, block3;  // gridz: the z-marching double-float passes
-  int n_parts = 0, n_parts_z = 0;
+  int n_parts = 0, n_parts_z = 0, n_parts_g = 0;
   uint8_t* mask = nullptr;
   double *b = nullptr, *d0 = nullptr, *d1 = nullptr, *part = nullptr, *scal = nullptr;
   float *xh = nullptr, *xl = nullptr, *rh = nullptr, *rl = nullptr, *ph = nullptr, *pl = nullptr;
   float *qh = nullptr, *ql = nullptr, *zh = nullptr, *zl = nullptr, *uh = nullptr, *ul = nullptr;
   float *th = nullptr, *tl = nullptr, *lam = nullptr;
   unsigned long long* counts = nullptr;
-  std::vector<void*> owned;
+  SlotScalars* sc = nullptr;
+  char* arena = nullptr;
+  cudaEvent_t ev[2] = {nullptr, nullptr};
   Tc3 tc;  // the tensor-core preconditioner, when built
   ~State3() {
-    for (void* p : owned) cudaFree(p);
+    cudaFree(arena);
     for (void* p : tc.owned) cudaFree(p);
-  }
-  template <class T>
-  int take(T** p, size_t count, std::string* err) {
-    void* v = nullptr;
-    if (cudaMalloc(&v, sizeof(T) * (count ? count : 1)) != cudaSuccess) {
-      cudaGetLastError();
-      *err = "cudaMalloc of the 3-D workspace failed";
-      return EXT_ENOMEM;
-    }
-    owned.push_back(v);
-    *p = static_cast<T*>(v);
-    return EXT_OK;
+    for (cudaEvent_t e : ev)
+      if (e) cudaEventDestroy(e);
   }
 };
 
@@ -575,40 +653,58 @@ Grid3 grid_of(const Solve3Args& a) {
   return G;
 }
 
+dim3 gemm_grid(int M, int N) { return dim3((M + GM - 1) / GM, (N + GN - 1) / GN); }
+
 int alloc_state(const Solve3Args& a, State3& s, bool solve, std::string* err) {
   s.n = (size_t)a.nx * a.ny * a.nz;
   s.block3 = dim3(kT);
   s.grid3 = dim3((a.nx + 31) / 32, (a.ny + 7) / 8, a.nz);
   s.n_parts = (int)(s.grid3.x * s.grid3.y * s.grid3.z);
-  s.gridz = dim3(s.grid3.x, (a.ny + kBy - 1) / kBy, (a.nz + kZc - 1) / kZc);
+  // chunks of 16 planes, or of 8 or 4 while the blocks would not fill the device twice (the two
+  // planes a chunk reads beyond its own then cost less than the idle SMs)
+  const int xy = s.grid3.x * ((a.ny + kBy - 1) / kBy);
+  s.zc = 16;
+  while (s.zc > 4 && xy * ((a.nz + s.zc - 1) / s.zc) < 2 * a.sm_count) s.zc /= 2;
+  s.gridz = dim3(s.grid3.x, (a.ny + kBy - 1) / kBy, (a.nz + s.zc - 1) / s.zc);
   s.n_parts_z = (int)(s.gridz.x * s.gridz.y * s.gridz.z);
-  s.vec_blocks = (int)std::min<size_t>((s.n + kT - 1) / kT, 4096);
+  const dim3 gl = gemm_grid(a.ny * a.nx, a.nz);
+  s.n_parts_g = (int)(gl.x * gl.y);
+  s.vec_blocks = (int)std::max<size_t>(1, std::min<size_t>((s.n / 4 + kT - 1) / kT, (size_t)a.sm_count * 8));
   const size_t n = s.n;
-  int rc = s.take(&s.mask, n, err);
-  if (!rc) rc = s.take(&s.part, std::max(s.n_parts, s.vec_blocks), err);
-  if (!rc) rc = s.take(&s.scal, 8, err);
-  if (!rc) rc = s.take(&s.counts, 4, err);
-  if (!rc) rc = s.take(&s.d0, n, err);
-  if (!rc) rc = s.take(&s.zh, n, err);
-  if (!rc) rc = s.take(&s.zl, n, err);
-  if (!rc) rc = s.take(&s.th, n, err);
-  if (!rc) rc = s.take(&s.tl, n, err);
-  if (!rc) rc = s.take(&s.uh, n, err);
-  if (!rc) rc = s.take(&s.ul, n, err);
-  if (!rc) rc = s.take(&s.lam, (size_t)a.nx + a.ny + a.nz, err);
-  if (!rc && solve) {
-    rc = s.take(&s.b, n, err);
-    if (!rc) rc = s.take(&s.d1, n, err);
-    if (!rc) rc = s.take(&s.xh, n, err);
-    if (!rc) rc = s.take(&s.xl, n, err);
-    if (!rc) rc = s.take(&s.rh, n, err);
-    if (!rc) rc = s.take(&s.rl, n, err);
-    if (!rc) rc = s.take(&s.ph, n, err);
-    if (!rc) rc = s.take(&s.pl, n, err);
-    if (!rc) rc = s.take(&s.qh, n, err);
-    if (!rc) rc = s.take(&s.ql, n, err);
+  const bool simt = !a.tc_build;
+  size_t total = 0;
+  auto layout = [&](char* base) {
+    size_t off = 0;
+    auto take = [&](auto** p, size_t count) {
+      *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(base + off);
+      off = (off + sizeof(**p) * count + 255) / 256 * 256;
+    };
+    take(&s.mask, n);
+    take(&s.part, std::max(std::max(s.n_parts, s.n_parts_g), std::max(s.vec_blocks, s.n_parts_z)));
+    take(&s.scal, 8);
+    take(&s.counts, 4);
+    take(&s.sc, 1);
+    take(&s.d0, n);
+    for (float** v : {&s.zh, &s.zl, &s.uh, &s.ul}) take(v, n);
+    if (simt || !solve)
+      for (float** v : {&s.th, &s.tl}) take(v, n);
+    take(&s.lam, (size_t)a.nx + a.ny + a.nz);
+    if (solve) {
+      take(&s.b, n);
+      take(&s.d1, n);
+      for (float** v : {&s.xh, &s.xl, &s.rh, &s.rl, &s.ph, &s.pl, &s.qh, &s.ql}) take(v, n);
+    }
+    total = off;
+  };
+  layout(nullptr);
+  if (cudaMalloc(&s.arena, total) != cudaSuccess) {
+    cudaGetLastError();
+    s.arena = nullptr;
+    *err = "cudaMalloc of the 3-D workspace failed";
+    return EXT_ENOMEM;
   }
-  return rc;
+  layout(s.arena);
+  return EXT_OK;
 }
 
 // Eigenvalues of each axis scaled like the stencil weights, and the weight normaliser wnorm =
@@ -636,73 +732,93 @@ int upload_eigen(const Solve3Args& a, const Grid3& G, State3& s, float* wnorm, s
   return EXT_OK;
 }
 
-// z = M (L^2)^+ M r: six transform products with the weights between (r, z double-float; the
-// products alternate between (th, tl) and (uh, ul)).  r must be zero at known nodes.
+LaunchCfg dependent(const Solve3Args& a) {
+  LaunchCfg c{};
+  c.stream = a.stream;
+  c.pdl = true;
+  return c;
+}
+
+// z = M (L^2)^+ M r: six transform products with the weights in the third and the mask and the r.z
+// partials in the last (r, z double-float; the products alternate between (th, tl) and (uh, ul)).
+// r must be zero at known nodes.  mode as in launch_prec_tc; the CUDA-core kernels take its flag.
 void precondition(const Solve3Args& a, const State3& s, float wnorm, const float* rh, const float* rl,
-                  float* zh, float* zl, bool with_dot) {
+                  float* zh, float* zl, int mode) {
   const int nx = a.nx, ny = a.ny, nz = a.nz;
-  cudaStream_t st = a.stream;
+  LaunchCfg c = dependent(a);
   if (s.tc.on) {
     // the tensor-core path: its descriptors hold r, q, z and the mask of this solve
     const Tc3& t = s.tc;
-    LaunchCfg c;
     c.slots = t.d_descs;
-    c.stream = st;
     c.wait_cycles = t.wait_cycles;
     c.items = t.d_items[0];
     c.n_items = t.d_counts;
     c.grid = std::max(1, std::min(t.n_items[0], t.sm_count * 8));
-    launch_prec_tc_prepare(c, 2, t.split);
-    ++*a.launches;
+    launch_prec_tc_prepare(c, mode, t.split);
     static const int kForm[7] = {-1, 0, 0, 1, 2, 2, 3};
     for (int k = 1; k < 7; ++k) {
       c.items = t.d_items[k];
       c.n_items = t.d_counts + k;
       c.grid = std::max(1, std::min(t.n_items[k], t.sm_count));
-      launch_prec_tc(c, kForm[k], 2, t.split, t.ns, t.d_err);
-      ++*a.launches;
+      launch_prec_tc(c, kForm[k], mode, t.split, t.ns, t.d_err);
     }
-    if (with_dot) {
-      k3_sum<<<1, kT, 0, st>>>(t.part + 2, t.n_tiles3, s.scal + 1, 4);
-      ++*a.launches;
-    }
-    return;
+    *a.launches += 7;
+  } else {
+    const int* gate = mode == 0 ? &s.sc->active : mode == 1 ? &s.sc->need_prec : nullptr;
+    auto gemm = [&](auto kernel, const float* A, const float* Al, int M, int K, const float* B, int ldb, int N,
+                    float* o, float* ol) {
+      const Gemm3 g{A, Al, B, o, ol, M, K, ldb, N, s.lam, s.lam + nx, s.lam + nx + ny, nx, wnorm, s.mask, rh, rl,
+                    s.part};
+      launch_cfg(c, kernel, gemm_grid(M, N), kGt, 0, g, gate);
+    };
+    // forward: x, y, z (each contracts the contiguous axis and moves it to the front)
+    gemm(k3_gemm<0>, rh, rl, nz * ny, nx, a.qt[0], a.np[0], nx, s.th, s.tl);      // [kx][z][y]
+    gemm(k3_gemm<0>, s.th, s.tl, nx * nz, ny, a.qt[1], a.np[1], ny, s.uh, s.ul);  // [ky][kx][z]
+    gemm(k3_gemm<1>, s.uh, s.ul, ny * nx, nz, a.qt[2], a.np[2], nz, s.th, s.tl);  // [kz][ky][kx]
+    // inverse: x, y, z
+    gemm(k3_gemm<0>, s.th, s.tl, nz * ny, nx, a.q[0], a.np[0], nx, s.uh, s.ul);   // [x][kz][ky]
+    gemm(k3_gemm<0>, s.uh, s.ul, nx * nz, ny, a.q[1], a.np[1], ny, s.th, s.tl);   // [y][x][kz]
+    gemm(k3_gemm<2>, s.th, s.tl, ny * nx, nz, a.q[2], a.np[2], nz, zh, zl);       // [z][y][x]
+    *a.launches += 6;
   }
-  auto gemm = [&](const float* A, const float* Al, int M, int K, const float* B, int ldb, int N, float* o, float* ol) {
-    const dim3 grid((M + GM - 1) / GM, (N + GN - 1) / GN);
-    k3_gemm<<<grid, kT, 0, st>>>(A, Al, M, K, B, ldb, N, o, ol);
-    ++*a.launches;
-  };
-  // forward: x, y, z (each contracts the contiguous axis and moves it to the front)
-  gemm(rh, rl, nz * ny, nx, a.qt[0], a.np[0], nx, s.th, s.tl);   // [kx][z][y]
-  gemm(s.th, s.tl, nx * nz, ny, a.qt[1], a.np[1], ny, s.uh, s.ul);  // [ky][kx][z]
-  gemm(s.uh, s.ul, ny * nx, nz, a.qt[2], a.np[2], nz, s.th, s.tl);  // [kz][ky][kx]
-  k3_weights<<<s.vec_blocks, kT, 0, st>>>(nx, ny, nz, s.lam, s.lam + nx, s.lam + nx + ny, wnorm, s.th, s.tl);
-  ++*a.launches;
-  // inverse: x, y, z
-  gemm(s.th, s.tl, nz * ny, nx, a.q[0], a.np[0], nx, s.uh, s.ul);   // [x][kz][ky]
-  gemm(s.uh, s.ul, nx * nz, ny, a.q[1], a.np[1], ny, s.th, s.tl);   // [y][x][kz]
-  gemm(s.th, s.tl, ny * nx, nz, a.q[2], a.np[2], nz, s.uh, s.ul);   // [z][y][x]
-  k3_mask_dot<<<s.vec_blocks, kT, 0, st>>>(s.n, s.uh, s.ul, s.mask, rh, rl, zh, zl, s.part);
-  ++*a.launches;
-  if (with_dot) k3_sum<<<1, kT, 0, st>>>(s.part, s.vec_blocks, s.scal + 1);
-}
-
-// q = M L^2 p (p double-float, zero at known nodes), p.q into scal[0]
-void apply_operator(const Solve3Args& a, const Grid3& G, const State3& s, const float* ph, const float* pl,
-                    float* qh, float* ql) {
-  k3_lap<false><<<s.gridz, s.block3, 0, a.stream>>>(G, ph, pl, s.uh, s.ul, s.mask, nullptr, nullptr, nullptr);
-  ++*a.launches;
-  k3_lap<true><<<s.gridz, s.block3, 0, a.stream>>>(G, s.uh, s.ul, qh, ql, s.mask, ph, pl, s.part);
-  ++*a.launches;
-  k3_sum<<<1, kT, 0, a.stream>>>(s.part, s.n_parts_z, s.scal + 0);
+  if (mode == 2) return;
+  if (s.tc.on) launch_cfg(c, k3_finish<2>, 1, 32, 0, s.sc, s.tc.part + 2, s.tc.n_tiles3, 4, mode);
+  else launch_cfg(c, k3_finish<2>, 1, 32, 0, s.sc, s.part, s.n_parts_g, 1, mode);
   ++*a.launches;
 }
 
-int read_scalars(const Solve3Args& a, const State3& s, double* h, int count, std::string* err) {
-  BX3(cudaMemcpyAsync(h, s.scal, sizeof(double) * count, cudaMemcpyDeviceToHost, a.stream));
-  BX3(cudaStreamSynchronize(a.stream));
-  return EXT_OK;
+// q = M L^2 p (p double-float, zero at known nodes), p.q partials in part
+void apply_operator(const Solve3Args& a, const Grid3& G, const State3& s, const int* gate, const float* ph,
+                    const float* pl, float* qh, float* ql) {
+  const LaunchCfg c = dependent(a);
+  launch_cfg(c, k3_lap<false>, s.gridz, kT, 0, G, s.zc, gate, ph, pl, s.uh, s.ul, s.mask, nullptr, nullptr, nullptr);
+  launch_cfg(c, k3_lap<true>, s.gridz, kT, 0, G, s.zc, gate, s.uh, s.ul, qh, ql, s.mask, ph, pl, s.part);
+  *a.launches += 2;
+}
+
+// One CG iteration: p = z + beta p, q = A p, alpha, x, r, ||r||^2, z, rho and beta.
+void enqueue_iteration(const Solve3Args& a, const Grid3& G, const State3& s, float wnorm) {
+  const LaunchCfg c = dependent(a);
+  launch_cfg(c, k3_direction, s.vec_blocks, kT, 0, s.n, s.sc, s.zh, s.zl, s.ph, s.pl);
+  apply_operator(a, G, s, &s.sc->active, s.ph, s.pl, s.qh, s.ql);
+  launch_cfg(c, k3_finish<0>, 1, 32, 0, s.sc, s.part, s.n_parts_z, 1, 0);
+  launch_cfg(c, k3_update, s.vec_blocks, kT, 0, s.n, s.sc, s.ph, s.pl, s.qh, s.ql, s.xh, s.xl, s.rh, s.rl, s.part);
+  launch_cfg(c, k3_finish<1>, 1, 32, 0, s.sc, s.part, s.vec_blocks, 1, 0);
+  *a.launches += 4;
+  precondition(a, s, wnorm, s.rh, s.rl, s.zh, s.zl, 0);
+}
+
+// The end of a block: the FP64 true residual where one is due, the decision, and the fresh
+// preconditioner pass of a solve that continues.
+void enqueue_tail(const Solve3Args& a, const Grid3& G, const State3& s, float wnorm) {
+  const LaunchCfg c = dependent(a);
+  const int* gate = &s.sc->fold;
+  launch_cfg(c, k3_to_double, s.vec_blocks, kT, 0, s.n, gate, s.xh, s.xl, s.d0);
+  launch_cfg(c, k3_lap64<0>, s.grid3, kT, 0, G, gate, s.d0, s.d1, s.mask, nullptr, nullptr, nullptr, nullptr);
+  launch_cfg(c, k3_lap64<2>, s.grid3, kT, 0, G, gate, s.d1, s.d0, s.mask, s.b, s.part, s.rh, s.rl);
+  launch_cfg(c, k3_finish<3>, 1, 32, 0, s.sc, s.part, s.n_parts, 1, 0);
+  *a.launches += 4;
+  precondition(a, s, wnorm, s.rh, s.rl, s.zh, s.zl, 1);
 }
 
 // mask and known field; validation of the data
@@ -721,6 +837,8 @@ int setup_mask(const Solve3Args& a, State3& s, const float* phi, const float* f,
   return EXT_OK;
 }
 
+constexpr int kBlockIters = 8;  // iterations between two readings of the scalars
+
 }  // namespace
 
 int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* out, ext_result* res,
@@ -729,7 +847,7 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
   int rc = alloc_state(a, s, true, err);
   if (rc) return rc;
   if (a.tc_build) {
-    rc = a.tc_build(Tc3Io{s.rh, s.rl, s.qh, s.ql, s.zh, s.zl, s.mask}, s.tc);
+    rc = a.tc_build(Tc3Io{s.rh, s.rl, s.qh, s.ql, s.zh, s.zl, s.mask, s.sc}, s.tc);
     if (rc) return rc;
   }
   const Grid3 G = grid_of(a);
@@ -748,16 +866,16 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
   }
   cudaStream_t st = a.stream;
   // b = -M L^2 E_K f (FP64) and ||b||^2
-  k3_lap64<0><<<s.grid3, s.block3, 0, st>>>(G, s.d0, s.d1, s.mask, nullptr, nullptr, nullptr, nullptr);
+  k3_lap64<0><<<s.grid3, s.block3, 0, st>>>(G, nullptr, s.d0, s.d1, s.mask, nullptr, nullptr, nullptr, nullptr);
   ++*a.launches;
-  k3_lap64<1><<<s.grid3, s.block3, 0, st>>>(G, s.d1, s.b, s.mask, nullptr, s.part, nullptr, nullptr);
+  k3_lap64<1><<<s.grid3, s.block3, 0, st>>>(G, nullptr, s.d1, s.b, s.mask, nullptr, s.part, nullptr, nullptr);
   ++*a.launches;
-  k3_sum<<<1, kT, 0, st>>>(s.part, s.n_parts, s.scal + 2);
+  k3_sum<<<1, kT, 0, st>>>(s.part, s.n_parts, s.scal);
   ++*a.launches;
-  double sc[4];
-  rc = read_scalars(a, s, sc, 3, err);
-  if (rc) return rc;
-  const double bnorm = std::sqrt(sc[2]);
+  double bb = 0.0;
+  BX3(cudaMemcpyAsync(&bb, s.scal, sizeof(double), cudaMemcpyDeviceToHost, st));
+  BX3(cudaStreamSynchronize(st));
+  const double bnorm = std::sqrt(bb);
   res->iters = 0;
   res->relres_true = res->relres_rec = 0.0;
   res->err_est = 0.0;
@@ -778,108 +896,47 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
   k3_init<<<s.vec_blocks, kT, 0, st>>>(s.n, s.b, scale, s.rh, s.rl, s.xh, s.xl);
   ++*a.launches;
   // the scaled right-hand side for the true residual: b <- 2^-e b (exact)
-  k3_to_double<<<s.vec_blocks, kT, 0, st>>>(s.n, s.rh, s.rl, s.b);
+  k3_to_double<<<s.vec_blocks, kT, 0, st>>>(s.n, nullptr, s.rh, s.rl, s.b);
   ++*a.launches;
   const double bn = bnorm * scale;
-  const int maxit = a.maxit > 0 ? a.maxit : 10 * std::max(a.nx, std::max(a.ny, a.nz));
-  precondition(a, s, wnorm, s.rh, s.rl, s.zh, s.zl, true);
-  BX3(cudaMemcpyAsync(s.ph, s.zh, 4 * s.n, cudaMemcpyDeviceToDevice, st));
-  BX3(cudaMemcpyAsync(s.pl, s.zl, 4 * s.n, cudaMemcpyDeviceToDevice, st));
-  rc = read_scalars(a, s, sc, 2, err);
-  if (rc) return rc;
-  double rho = sc[1];
-  double rnorm_last_repl = bn;
-  int since_repl = 0;
-  int it = 0;
-  int status = EXT_ENOTCONV;
-  double rel_rec = 1.0, aro_total = 0.0;
-  std::vector<double> aro;
-  auto true_residual = [&](bool replace, double* rel) -> int {
-    k3_to_double<<<s.vec_blocks, kT, 0, st>>>(s.n, s.xh, s.xl, s.d0);
-    ++*a.launches;
-    k3_lap64<0><<<s.grid3, s.block3, 0, st>>>(G, s.d0, s.d1, s.mask, nullptr, nullptr, nullptr, nullptr);
-    ++*a.launches;
-    k3_lap64<2><<<s.grid3, s.block3, 0, st>>>(G, s.d1, s.d0, s.mask, s.b, s.part, replace ? s.rh : nullptr,
-                                             replace ? s.rl : nullptr);
-    ++*a.launches;
-    k3_sum<<<1, kT, 0, st>>>(s.part, s.n_parts, s.scal + 3);
-    ++*a.launches;
-    double v[4];
-    const int r2 = read_scalars(a, s, v, 4, err);
-    if (r2) return r2;
-    *rel = std::sqrt(v[3]) / bn;
-    return EXT_OK;
-  };
-  while (it < maxit) {
-    apply_operator(a, G, s, s.ph, s.pl, s.qh, s.ql);
-    rc = read_scalars(a, s, sc, 1, err);
-    if (rc) return rc;
-    const double pq = sc[0];
-    if (!(pq > 0.0) || !std::isfinite(pq) || !std::isfinite(rho)) {
-      status = EXT_EBREAKDOWN;
-      break;
-    }
-    const double alpha = rho / pq;
-    aro.push_back(alpha * rho);
-    aro_total += alpha * rho;
-    k3_update<<<s.vec_blocks, kT, 0, st>>>(s.n, df_of(alpha), s.ph, s.pl, s.qh, s.ql, s.xh, s.xl, s.rh, s.rl, s.part);
-    ++*a.launches;
-    k3_sum<<<1, kT, 0, st>>>(s.part, s.vec_blocks, s.scal + 2);
-    ++*a.launches;
-    rc = read_scalars(a, s, sc, 3, err);
-    if (rc) return rc;
-    ++it;
-    ++since_repl;
-    double rnorm = std::sqrt(sc[2]);
-    rel_rec = rnorm / bn;
-    bool replaced = false;
-    if (rel_rec <= a.rtol) {
-      // converged by the recursive residual: confirm with the FP64 true residual
-      double rel = 0.0;
-      rc = true_residual(true, &rel);
-      if (rc) return rc;
-      replaced = true;
-      if (rel <= a.rtol) {
-        status = EXT_OK;
-        res->relres_true = rel;
-        break;
-      }
-      rnorm = rel * bn;
-    } else if (rnorm < a.replace_factor * rnorm_last_repl || since_repl >= a.true_res_every) {
-      double rel = 0.0;
-      rc = true_residual(true, &rel);
-      if (rc) return rc;
-      replaced = true;
-      rnorm = rel * bn;
-    }
-    if (replaced) {
-      rnorm_last_repl = rnorm;
-      since_repl = 0;
-    }
-    precondition(a, s, wnorm, s.rh, s.rl, s.zh, s.zl, true);
-    rc = read_scalars(a, s, sc, 2, err);
-    if (rc) return rc;
-    const double rho_new = sc[1];
-    const double beta = rho_new / rho;
-    if (!std::isfinite(beta)) {
-      status = EXT_EBREAKDOWN;
-      break;
-    }
-    rho = rho_new;
-    k3_direction<<<s.vec_blocks, kT, 0, st>>>(s.n, df_of(beta), s.zh, s.zl, s.ph, s.pl);
-    ++*a.launches;
+  SlotScalars& h0 = a.h_sc[0];
+  h0 = SlotScalars{};
+  h0.bb = h0.rr = h0.rr_true = h0.rr_ref = bn * bn;
+  h0.rtol2 = a.rtol * a.rtol;
+  h0.delta2 = a.replace_factor * a.replace_factor;
+  h0.fold_every = a.true_res_every;
+  h0.maxit = a.maxit > 0 ? a.maxit : 10 * std::max(a.nx, std::max(a.ny, a.nz));
+  h0.status = ST_RUNNING;
+  h0.active = h0.need_prec = 1;
+  const int maxit = h0.maxit;
+  BX3(cudaMemcpyAsync(s.sc, &h0, sizeof(SlotScalars), cudaMemcpyHostToDevice, st));
+  // the first direction is z (beta = 0)
+  BX3(cudaMemsetAsync(s.ph, 0, 4 * s.n, st));
+  BX3(cudaMemsetAsync(s.pl, 0, 4 * s.n, st));
+  for (cudaEvent_t& v : s.ev) BX3(cudaEventCreateWithFlags(&v, cudaEventDisableTiming));
+  precondition(a, s, wnorm, s.rh, s.rl, s.zh, s.zl, 1);
+  SlotScalars last{};
+  const long long max_blocks = 2LL * (maxit / kBlockIters) + 8;
+  for (long long blk = 0; blk <= max_blocks; ++blk) {
+    for (int i = 0; i < kBlockIters; ++i) enqueue_iteration(a, G, s, wnorm);
+    enqueue_tail(a, G, s, wnorm);
+    BX3(cudaGetLastError());
+    BX3(cudaMemcpyAsync(&a.h_sc[blk & 1], s.sc, sizeof(SlotScalars), cudaMemcpyDeviceToHost, st));
+    BX3(cudaEventRecord(s.ev[blk & 1], st));
+    // one block stays ahead of the reading; with nothing left to do it passes by its flags
+    if (blk == 0 && blk < max_blocks) continue;
+    BX3(cudaEventSynchronize(s.ev[(blk & 1) ^ 1]));
+    last = a.h_sc[(blk & 1) ^ 1];
+    if (last.status != ST_RUNNING) break;
   }
-  if (status != EXT_OK) {
-    double rel = 0.0;
-    rc = true_residual(false, &rel);
-    if (rc) return rc;
-    res->relres_true = rel;
-  }
-  res->iters = it;
-  res->relres_rec = rel_rec;
+  BX3(cudaStreamSynchronize(st));
+  int status = last.status == ST_RUNNING ? EXT_ETIMEOUT : last.status;
+  res->iters = last.it;
+  res->relres_true = std::sqrt(last.rr_true) / bn;
+  res->relres_rec = std::sqrt(last.rr) / bn;
   double tail = 0.0;
-  for (size_t k = aro.size() > 8 ? aro.size() - 8 : 0; k < aro.size(); ++k) tail += aro[k];
-  res->err_est = aro_total > 0.0 ? std::sqrt(std::max(0.0, tail) / aro_total) : 0.0;
+  for (int k = 0; k < std::min(last.aro_n, kErrDelay); ++k) tail += last.aro_ring[k];
+  res->err_est = last.aro_total > 0.0 ? std::sqrt(std::max(0.0, tail) / last.aro_total) : 0.0;
   k3_output<<<s.vec_blocks, kT, 0, st>>>(s.n, s.xh, s.xl, e, s.mask, f, out);
   ++*a.launches;
   BX3(cudaGetLastError());
@@ -896,7 +953,7 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
     }
   }
   res->status = status;
-  return status == EXT_OK ? EXT_OK : status;
+  return status;
 }
 
 int apply3d_operator(const Solve3Args& a, const float* phi, const float* p, float* q, std::string* err) {
@@ -910,7 +967,7 @@ int apply3d_operator(const Solve3Args& a, const float* phi, const float* p, floa
   // p masked into (th, tl); q into (zh, zl); the hi plane is the result
   k3_load_masked<<<s.vec_blocks, kT, 0, a.stream>>>(s.n, p, s.mask, s.th, s.tl);
   ++*a.launches;
-  apply_operator(a, G, s, s.th, s.tl, s.zh, s.zl);
+  apply_operator(a, G, s, nullptr, s.th, s.tl, s.zh, s.zl);
   BX3(cudaMemcpyAsync(q, s.zh, 4 * s.n, cudaMemcpyDeviceToDevice, a.stream));
   BX3(cudaGetLastError());
   BX3(cudaStreamSynchronize(a.stream));
@@ -929,20 +986,18 @@ int apply3d_preconditioner(const Solve3Args& a, const float* phi, const float* r
   unsigned long long cnt[4];
   rc = setup_mask(a, s, phi, phi, cnt, err);
   if (rc) return rc;
-  // r masked into (th, tl) is consumed by the first product, so it is kept in (zh, zl)'s place:
-  // the masked copy goes to d0 reinterpreted as two float planes
+  // the masked copy of r: d0 reinterpreted as two float planes
   float* rh = reinterpret_cast<float*>(s.d0);
   float* rl = rh + s.n;
   if (a.tc_build) {
-    // z.q of the last product's epilogue is not used here: q = zeros
-    BX3(cudaMemsetAsync(s.uh, 0, 4 * s.n, a.stream));
-    BX3(cudaMemsetAsync(s.ul, 0, 4 * s.n, a.stream));
-    rc = a.tc_build(Tc3Io{rh, rl, s.uh, s.ul, s.zh, s.zl, s.mask}, s.tc);
+    SlotScalars h{};  // no flexible beta: the last product leaves z.q out
+    BX3(cudaMemcpyAsync(s.sc, &h, sizeof(h), cudaMemcpyHostToDevice, a.stream));
+    rc = a.tc_build(Tc3Io{rh, rl, s.uh, s.ul, s.zh, s.zl, s.mask, s.sc}, s.tc);
     if (rc) return rc;
   }
   k3_load_masked<<<s.vec_blocks, kT, 0, a.stream>>>(s.n, r, s.mask, rh, rl);
   ++*a.launches;
-  precondition(a, s, wnorm, rh, rl, s.zh, s.zl, false);
+  precondition(a, s, wnorm, rh, rl, s.zh, s.zl, 2);
   BX3(cudaMemcpyAsync(z, s.zh, 4 * s.n, cudaMemcpyDeviceToDevice, a.stream));
   BX3(cudaGetLastError());
   BX3(cudaStreamSynchronize(a.stream));
