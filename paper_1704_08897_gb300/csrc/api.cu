@@ -23,6 +23,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <deque>
+#include <functional>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -94,7 +95,7 @@ struct Workspace {
   WorkItem* d_gm[2] = {nullptr, nullptr};  // transform tiles of the problems with four, six slices
   WorkItem* d_sl = nullptr;     // one item per slot (tile 0), for the per-slot scalar kernels
   int *d_counts = nullptr;      // [0] grid tiles, [1] vector items, [2] transform tiles with four
-                                // slices, [11] with six, [3] slots,
+                                // slices, [11] with six, [12] the low-mode middle, [3] slots,
                                 // [4] stencil tiles, [5] [6] low-mode tiles, [7] fold items,
                                 // [8] unfold tiles, [9] tensor-core problems, [10] grid tiles
                                 // of unfolded slots
@@ -105,8 +106,8 @@ struct Workspace {
   int sten_ty = 32;             // stencil tile height of this workspace (autotuned)
   bool tuned = false;
   bool fuse = false;            // scalar steps inside the update and stencil (few slots)
-  WorkItem *d_l1 = nullptr, *d_l3 = nullptr;  // tiles of the low-mode products
-  int n_l1 = 0, n_l3 = 0;
+  WorkItem *d_l1 = nullptr, *d_l2 = nullptr, *d_l3 = nullptr;  // low-mode forward, middle, inverse
+  int n_l1 = 0, n_l2 = 0, n_l3 = 0;
   // tensor-core problems (mixed modes): kMirClasses entries per slot, the slot's own descriptor
   // or its mirror classes; items of the fold and unfold kernels; one item per problem
   SlotDesc* d_tcp = nullptr;
@@ -485,6 +486,7 @@ static void free_workspace(Workspace* W) {
   for (WorkItem* g : W->d_gm) cudaFree(g);
   cudaFree(W->d_sl);
   cudaFree(W->d_l1);
+  cudaFree(W->d_l2);
   cudaFree(W->d_l3);
   cudaFree(W->d_tcp);
   cudaFree(W->d_fold);
@@ -778,12 +780,13 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
       t.low_qxt_e = (const int8_t*)(lxp + qx->low_off_te);
       t.low_qy_e = (const int8_t*)(lyp + qy->low_off_qe);
       t.n_l1_tiles = t.nyp / 128;
-      t.n_l3_tiles = t.nxp / 128;  // inverse product: one item per 128 rows of x
+      t.n_l2_tiles = t.nxp / 32;
+      t.n_l3_tiles = (t.nxp / 128) * (t.nyp / 32);
       CUtensorMap lm[4];
-      int rc4 = make_tmap(&lm[0], t.tc_r, bf, t.nxp, (uint64_t)kLowNS * t.nyp, 128);
-      if (!rc4) rc4 = make_tmap(&lm[1], qx->low, bf, t.nxp, (uint64_t)kLowNS * kLowM, kLowM);
-      if (!rc4) rc4 = make_tmap(&lm[2], t.low_jt, bf, kLowK3, (uint64_t)kLowNS * t.nxp, 128);
-      if (!rc4) rc4 = make_tmap(&lm[3], (char*)qy->low + qy->low_off_q, bf, kLowK3, (uint64_t)kLowNS * t.nyp, kLowM);
+      int rc4 = make_tmap(&lm[0], t.tc_r, bf, t.nxp, (uint64_t)kLowNS * t.nyp, 128, 32);
+      if (!rc4) rc4 = make_tmap(&lm[1], qx->low, bf, t.nxp, (uint64_t)kLowNS * kLowM, kLowM, 32);
+      if (!rc4) rc4 = make_tmap(&lm[2], t.low_jt, bf, kLowK3, (uint64_t)kLowNS * t.nxp, 128, 32);
+      if (!rc4) rc4 = make_tmap(&lm[3], (char*)qy->low + qy->low_off_q, bf, kLowK3, (uint64_t)kLowNS * t.nyp, 32, 32);
       if (rc4) return rc4;
       BX_CUDA(cudaMemcpy(A + L.o_lmaps, lm, sizeof(lm), cudaMemcpyHostToDevice));
       t.low_maps = A + L.o_lmaps;
@@ -803,7 +806,7 @@ static void set_slot_scalars(SlotHost& s, SlotScalars* sc) {
 
 // Work items of the tensor-core problems of slot i (problem index kMirClasses * i + c).
 static void tc_items(const SlotHost& s, int i, std::vector<WorkItem> (&gm)[2], std::vector<WorkItem>& l1,
-                     std::vector<WorkItem>& l3, std::vector<WorkItem>& tcl) {
+                     std::vector<WorkItem>& l2, std::vector<WorkItem>& l3, std::vector<WorkItem>& tcl) {
   for (int c = 0; c < kMirClasses; ++c) {
     if (s.d.mir == 0 && c > 0) break;
     if (((c & 1) && !(s.d.mir & 1)) || ((c & 2) && !(s.d.mir & 2))) continue;
@@ -812,22 +815,47 @@ static void tc_items(const SlotHost& s, int i, std::vector<WorkItem> (&gm)[2], s
     for (int tt = 0; tt < t.n_gm_tiles; ++tt) gm[t.tc_ns == 6].push_back({k, tt});
     if (t.lowm_x) {
       for (int tt = 0; tt < t.n_l1_tiles; ++tt) l1.push_back({k, tt});
+      for (int tt = 0; tt < t.n_l2_tiles; ++tt) l2.push_back({k, tt});
       for (int tt = 0; tt < t.n_l3_tiles; ++tt) l3.push_back({k, tt});
     }
     tcl.push_back({k, 0});
   }
 }
 
-// Tensor-core work items in the order the persistent kernels take them: decreasing k extent of
-// their transform problem (a tile's cost is proportional to it), so that the persistent CTAs of a
-// launch end together; tiles of one problem keep their order.  Any order gives the same results:
-// tile partial sums are stored per tile and reduced in tile order.
-static void longest_first_tc(std::vector<WorkItem>& gm, const std::vector<SlotHost>& slots) {
-  std::stable_sort(gm.begin(), gm.end(), [&](const WorkItem& a, const WorkItem& b) {
-    const SlotDesc& da = slots[a.slot / kMirClasses].tcp[a.slot % kMirClasses];
-    const SlotDesc& db = slots[b.slot / kMirClasses].tcp[b.slot % kMirClasses];
-    return std::max(da.nxp, da.nyp) > std::max(db.nxp, db.nyp);
-  });
+// Work items of the tensor-core kernels, dealt to the launch's blocks so that the blocks end together:
+// longest first, each to the least loaded block (a block takes every grid-th item, so the list is
+// written row by row; a block with fewer items than others gets empty places, slot -1).  Any order
+// gives the same results: tile partial sums are stored per tile and reduced in tile order.
+template <class Cost>
+static void balance(std::vector<WorkItem>& items, int blocks, Cost cost) {
+  std::stable_sort(items.begin(), items.end(), [&](const WorkItem& a, const WorkItem& b) { return cost(a) > cost(b); });
+  if ((int)items.size() <= blocks) return;
+  std::vector<std::vector<WorkItem>> bin(blocks);
+  std::vector<std::pair<double, int>> heap;  // (load, block), least load on top
+  for (int b = 0; b < blocks; ++b) heap.push_back({0.0, b});
+  const auto more = std::greater<std::pair<double, int>>();
+  for (const WorkItem& it : items) {
+    std::pop_heap(heap.begin(), heap.end(), more);
+    bin[heap.back().second].push_back(it);
+    heap.back().first += cost(it);
+    std::push_heap(heap.begin(), heap.end(), more);
+  }
+  std::stable_sort(bin.begin(), bin.end(), [](const auto& a, const auto& b) { return a.size() > b.size(); });
+  items.clear();
+  for (size_t row = 0; row < bin[0].size(); ++row)
+    for (int b = 0; b < blocks; ++b) {
+      if (row < bin[b].size()) items.push_back(bin[b][row]);
+      else if (row + 1 < bin[0].size()) items.push_back({-1, 0});
+    }
+}
+// The stages' and the low-mode products' lists (costs in thousands of SM cycles, from clock stamps: a
+// transform tile's epilogue and its k-blocks; a forward tile's dot products and k-blocks).
+static void balance_lists(ext_ctx* ctx, const std::vector<SlotHost>& slots, std::vector<WorkItem> (&gm)[2],
+                          std::vector<WorkItem>& l1) {
+  auto prob = [&](const WorkItem& w) -> const SlotDesc& { return slots[w.slot / kMirClasses].tcp[w.slot % kMirClasses]; };
+  for (auto& g : gm)
+    balance(g, ctx->sm_count, [&](const WorkItem& w) { return 5.0 + 3.4 * (prob(w).nxp + prob(w).nyp) / 256; });
+  balance(l1, ctx->sm_count, [&](const WorkItem& w) { return 6.0 + 4.0 * prob(w).nxp / 128; });
 }
 
 template <class T>
@@ -848,7 +876,7 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   W->key = shape_key(count, probs, host_io);
   W->host_io = host_io;
   W->slots.resize(count);
-  std::vector<WorkItem> st, vec, gm[2], l1, l3, fold, unfold, tcl, prep;
+  std::vector<WorkItem> st, vec, gm[2], l1, l2, l3, fold, unfold, tcl, prep;
   long long call_nodes = 0;
   for (int i = 0; i < count; ++i) call_nodes += (long long)probs[i].nx * probs[i].ny;
   for (int i = 0; i < count; ++i) {
@@ -863,13 +891,13 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
     if (d.aniso) W->aniso = true;
     for (int t = 0; t < d.n_st_tiles; ++t) st.push_back({i, t});
     for (int t = 0; t < d.n_vec_items; ++t) vec.push_back({i, t});
-    tc_items(s, i, gm, l1, l3, tcl);
+    tc_items(s, i, gm, l1, l2, l3, tcl);
     for (int t = 0; t < d.n_fold_items; ++t) fold.push_back({i, t});
     for (int t = 0; t < d.n_unfold_tiles; ++t) unfold.push_back({i, t});
     if (!d.mir)
       for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
   }
-  for (auto& g : gm) longest_first_tc(g, W->slots);
+  balance_lists(ctx, W->slots, gm, l1);
   std::vector<WorkItem> sl;
   for (int i = 0; i < count; ++i) sl.push_back({i, 0});
   W->n_sl = (int)sl.size();
@@ -894,6 +922,7 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   if (!rc) rc = upload(&W->d_sl, sl);
   if (!rc) rc = upload(&W->d_sten, st);
   if (!rc) rc = upload(&W->d_l1, l1);
+  if (!rc) rc = upload(&W->d_l2, l2);
   if (!rc) rc = upload(&W->d_l3, l3);
   if (!rc) rc = upload(&W->d_fold, fold);
   if (!rc) rc = upload(&W->d_unfold, unfold);
@@ -907,13 +936,14 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   W->fuse = count <= kFuseSlots;
   for (const SlotHost& h : W->slots) W->fuse = W->fuse && fuse_fits(h.d);
   W->n_l1 = (int)l1.size();
+  W->n_l2 = (int)l2.size();
   W->n_l3 = (int)l3.size();
   W->n_fold = (int)fold.size();
   W->n_unfold = (int)unfold.size();
   W->n_tcl = (int)tcl.size();
   W->n_prep = (int)prep.size();
-  int counts[12] = {W->n_st, W->n_vec, W->n_gm[0], W->n_sl, W->n_sten, W->n_l1, W->n_l3,
-                    W->n_fold, W->n_unfold, W->n_tcl, W->n_prep, W->n_gm[1]};
+  int counts[13] = {W->n_st, W->n_vec, W->n_gm[0], W->n_sl, W->n_sten, W->n_l1, W->n_l3,
+                    W->n_fold, W->n_unfold, W->n_tcl, W->n_prep, W->n_gm[1], W->n_l2};
   BX_CUDA(cudaMalloc(&W->d_counts, sizeof(counts)));
   BX_CUDA(cudaMemcpy(W->d_counts, counts, sizeof(counts), cudaMemcpyHostToDevice));
   BX_CUDA(cudaMalloc(&W->d_phis, sizeof(void*) * count));
@@ -988,6 +1018,10 @@ static LaunchCfg cfg_of(ext_ctx* ctx, Workspace* W, int which) {
     c.items = W->d_sten;
     c.n_items = W->d_counts + 4;
     c.grid = std::max(1, std::min(W->n_sten, ctx->sm_count * stencil_blocks_per_sm(W->sten_ty)));
+  } else if (which == 12) {  // the low-mode middle: small blocks
+    c.items = W->d_l2;
+    c.n_items = W->d_counts + 12;
+    c.grid = std::max(1, std::min(W->n_l2, cap));
   } else {  // 2, 11: transform tiles with four and six slices, over the transform problems
     const int k = which == 11;
     c.slots = W->d_tcp;
@@ -1067,9 +1101,8 @@ static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish =
     timed(ctx, EXT_KERNEL_FOLD, [&] { launch_tc_fold(cfg_of(ctx, W, 7), mode, ctx->split); }, g.stream);
   if (W->n_l1 > 0) {
     // the lowest modes in high precision: forward product, middle, inverse product
-    LaunchCfg c1 = cfg_of(ctx, W, 5), cm = cfg_of(ctx, W, 6), c3 = cfg_of(ctx, W, 6);
+    LaunchCfg c1 = cfg_of(ctx, W, 5), cm = cfg_of(ctx, W, 12), c3 = cfg_of(ctx, W, 6);
     c1.slots = cm.slots = c3.slots = W->d_tcp;
-    cm.grid = std::max(1, std::min(W->n_l3, ctx->sm_count * 8));  // the middle: small blocks
     timed(ctx, EXT_KERNEL_LOW_FWD, [&] { launch_low_tc(c1, 0, mode, ctx->split, ctx->d_err); }, g.stream);
     // the middle starts on a free device: blocks placed as the forward product's leave would load
     // the SMs unevenly (15 us more per application on a batch of 48 grids)
@@ -2106,6 +2139,7 @@ static int serve_alloc_lists(ext_ctx::Serve* S, int cap) {
   cudaFree(W->d_vec);
   for (WorkItem* g : W->d_gm) cudaFree(g);
   cudaFree(W->d_l1);
+  cudaFree(W->d_l2);
   cudaFree(W->d_l3);
   cudaFree(W->d_fold);
   cudaFree(W->d_unfold);
@@ -2113,7 +2147,7 @@ static int serve_alloc_lists(ext_ctx::Serve* S, int cap) {
   cudaFree(W->d_prep);
   cudaFree(S->d_new);
   cudaFree(S->d_ret);
-  W->d_st = W->d_sten = W->d_vec = W->d_gm[0] = W->d_gm[1] = W->d_l1 = W->d_l3 = S->d_new = S->d_ret = nullptr;
+  W->d_st = W->d_sten = W->d_vec = W->d_gm[0] = W->d_gm[1] = W->d_l1 = W->d_l2 = W->d_l3 = S->d_new = S->d_ret = nullptr;
   W->d_fold = W->d_unfold = W->d_tcl = W->d_prep = nullptr;
   BX_CUDA(cudaMalloc(&W->d_prep, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_fold, sizeof(WorkItem) * cap));
@@ -2122,6 +2156,7 @@ static int serve_alloc_lists(ext_ctx::Serve* S, int cap) {
   BX_CUDA(cudaMalloc(&W->d_st, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_sten, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_l1, sizeof(WorkItem) * cap));
+  BX_CUDA(cudaMalloc(&W->d_l2, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_l3, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_vec, sizeof(WorkItem) * cap));
   for (auto& g : W->d_gm) BX_CUDA(cudaMalloc(&g, sizeof(WorkItem) * cap));
@@ -2129,7 +2164,7 @@ static int serve_alloc_lists(ext_ctx::Serve* S, int cap) {
   BX_CUDA(cudaMalloc(&S->d_ret, sizeof(WorkItem) * cap));
   S->cap_items = cap;
   // grids sized for the capacity
-  W->n_st = W->n_vec = W->n_gm[0] = W->n_gm[1] = W->n_sten = W->n_l1 = W->n_l3 = cap;
+  W->n_st = W->n_vec = W->n_gm[0] = W->n_gm[1] = W->n_sten = W->n_l1 = W->n_l2 = W->n_l3 = cap;
   W->n_fold = W->n_unfold = W->n_tcl = W->n_prep = cap;
   drop_graphs(W);
   return EXT_OK;
@@ -2149,8 +2184,8 @@ static int serve_init(ext_ctx* ctx) {
   BX_CUDA(cudaMemset(W->d_sc, 0, sizeof(SlotScalars) * cap));
   BX_CUDA(cudaMallocHost(&W->h_sc, sizeof(SlotScalars) * cap));
   memset(W->h_sc, 0, sizeof(SlotScalars) * cap);
-  BX_CUDA(cudaMalloc(&W->d_counts, 12 * sizeof(int)));
-  BX_CUDA(cudaMemset(W->d_counts, 0, 12 * sizeof(int)));
+  BX_CUDA(cudaMalloc(&W->d_counts, 13 * sizeof(int)));
+  BX_CUDA(cudaMemset(W->d_counts, 0, 13 * sizeof(int)));
   BX_CUDA(cudaMalloc(&W->d_sl, sizeof(WorkItem) * cap));
   W->n_sl = cap;  // the per-slot grid is sized for the slot table
   BX_CUDA(cudaMalloc(&W->d_phis, sizeof(void*) * cap));
@@ -2173,7 +2208,7 @@ static int serve_init(ext_ctx* ctx) {
 static int serve_rebuild_lists(ext_ctx* ctx) {
   ext_ctx::Serve* S = ctx->serve;
   Workspace* W = S->W;
-  std::vector<WorkItem> st, vec, gm[2], sl, l1, l3, fold, unfold, tcl, prep;
+  std::vector<WorkItem> st, vec, gm[2], sl, l1, l2, l3, fold, unfold, tcl, prep;
   bool aniso = false;
   for (int i = 0; i < (int)S->slots.size(); ++i) {
     if (!S->slots[i].used) continue;
@@ -2182,16 +2217,16 @@ static int serve_rebuild_lists(ext_ctx* ctx) {
     aniso |= d.aniso != 0;
     for (int t = 0; t < d.n_st_tiles; ++t) st.push_back({i, t});
     for (int t = 0; t < d.n_vec_items; ++t) vec.push_back({i, t});
-    tc_items(h, i, gm, l1, l3, tcl);
+    tc_items(h, i, gm, l1, l2, l3, tcl);
     for (int t = 0; t < d.n_fold_items; ++t) fold.push_back({i, t});
     for (int t = 0; t < d.n_unfold_tiles; ++t) unfold.push_back({i, t});
     if (!d.mir)
       for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
     sl.push_back({i, 0});
   }
-  for (auto& g : gm) longest_first_tc(g, W->slots);
+  balance_lists(ctx, W->slots, gm, l1);
   size_t need = 0;
-  for (const auto* v : {&st, &vec, &gm[0], &gm[1], &l1, &l3, &fold, &unfold, &tcl, &prep}) need = std::max(need, v->size());
+  for (const auto* v : {&st, &vec, &gm[0], &gm[1], &l1, &l2, &l3, &fold, &unfold, &tcl, &prep}) need = std::max(need, v->size());
   if ((int)need > S->cap_items) {
     int cap = S->cap_items;
     while (cap < (int)need) cap *= 2;
@@ -2205,7 +2240,7 @@ static int serve_rebuild_lists(ext_ctx* ctx) {
   const int cap = S->cap_items;
   W->n_gm[0] = gm[0].empty() ? 0 : cap;
   W->n_gm[1] = gm[1].empty() ? 0 : cap;
-  W->n_l1 = W->n_l3 = l1.empty() ? 0 : cap;
+  W->n_l1 = W->n_l2 = W->n_l3 = l1.empty() ? 0 : cap;
   W->n_fold = W->n_unfold = fold.empty() ? 0 : cap;
   W->n_prep = prep.empty() ? 0 : cap;
   W->fuse = sl.size() <= kFuseSlots;
@@ -2223,15 +2258,16 @@ static int serve_rebuild_lists(ext_ctx* ctx) {
   if (!rc) rc = put(W->d_gm[1], gm[1]);
   if (!rc) rc = put(W->d_sl, sl);
   if (!rc) rc = put(W->d_l1, l1);
+  if (!rc) rc = put(W->d_l2, l2);
   if (!rc) rc = put(W->d_l3, l3);
   if (!rc) rc = put(W->d_fold, fold);
   if (!rc) rc = put(W->d_unfold, unfold);
   if (!rc) rc = put(W->d_tcl, tcl);
   if (!rc) rc = put(W->d_prep, prep);
   if (rc) return rc;
-  int counts[12] = {(int)st.size(), (int)vec.size(), (int)gm[0].size(), (int)sl.size(), (int)st.size(),
+  int counts[13] = {(int)st.size(), (int)vec.size(), (int)gm[0].size(), (int)sl.size(), (int)st.size(),
                     (int)l1.size(), (int)l3.size(), (int)fold.size(), (int)unfold.size(), (int)tcl.size(),
-                    (int)prep.size(), (int)gm[1].size()};
+                    (int)prep.size(), (int)gm[1].size(), (int)l2.size()};
   BX_CUDA(cudaMemcpyAsync(W->d_counts, counts, sizeof(counts), cudaMemcpyHostToDevice, s));
   // the host vectors die here: the copies above must finish first (pageable sources are staged)
   BX_CUDA(cudaStreamSynchronize(s));

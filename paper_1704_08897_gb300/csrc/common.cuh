@@ -32,7 +32,7 @@ constexpr long long kLowAutoNodes = 2048LL * 2048;  // low_modes = 2: or calls w
 // 768^2, 520 / 604 at 1024^2, 187 / 174 for 16 grids of 128..512 together, 525 / 537 for 48.
 constexpr long long kSixNodes = 768LL * 768;
 constexpr int kLowNS = 6;           // integer slices per operand of the low-mode products
-constexpr int kLowK3 = 64;          // k extent of the inverse low-mode product (32 modes, zero-padded)
+constexpr int kLowK3 = 32;          // k extent of the inverse low-mode product
 constexpr int kVecThreads = 256;
 constexpr int kVecStep = 4 * kVecThreads;  // elements a block moves with one vector per thread
 // Elements per work item of the vector kernels (a function of the grid alone, so that the partial
@@ -144,7 +144,8 @@ struct SlotDesc {
   const int8_t* low_qy_e;   // exponents of the inverse product's B operand: [nyp]
   const void* low_maps;     // 4 CUtensorMap: r slices, Qx_low^T slices, J^T slices, Qy_low slices
   int n_l1_tiles;           // tiles of the forward product: nyp / 128
-  int n_l3_tiles;           // items of the inverse product: nxp / 128 (each walks every y-tile)
+  int n_l2_tiles;           // blocks of the middle: nxp / 32
+  int n_l3_tiles;           // tiles of the inverse product: (nxp / 128) * (nyp / 32)
   // Mirror fold of the tensor-core transforms (i -> n-1-i on an axis; even and odd classes of
   // ceil(n/2) nodes each): a slot with a folded axis runs its four stages as two or four
   // half-size problems, the slot's classes, held in the tensor-core problem list at

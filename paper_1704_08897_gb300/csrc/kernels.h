@@ -89,8 +89,8 @@ void launch_prec_tc_prepare(const LaunchCfg& c, int mode, int split_kind);
 int tc_tile_cols(int ns);  // columns of a stage's output tile
 int tc_step_k(int ns);     // k per pipeline step of a stage (the copies' box width)
 // low-mode correction of the tensor-core preconditioner: kind 0 = forward product with the tiles'
-// shares of G (one CTA per 128 rows of y), kind 1 = inverse product (one CTA per 128 rows of x,
-// walking the y-tiles); the middle step one block per (problem, 128 rows of x)
+// shares of G (tiles of 128 rows of y), kind 1 = inverse product (tiles of 128 x 32); the middle
+// step one block per (problem, 32 rows of x)
 void launch_low_tc(const LaunchCfg& c, int kind, int mode, int split_kind, int* err);
 void launch_low_mid(const LaunchCfg& c, int mode, int split_kind);
 // mirror fold: residual -> slices of each class's first operand (c.slots = slots, items of the

@@ -80,30 +80,40 @@ constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kMaxRegs = (16384 / (32 * ((kThreads / 32 + 3) / 4))) & ~7;
 constexpr int kChunks = 2;                       // TMEM ring of k-block accumulator sets
 constexpr int kTmemCols = 512;                   // power of two >= kChunks * sets
-constexpr int STAGES = 2;
+constexpr int kMaxSteps = 3;                     // pipeline steps in flight
+
+// The products a launch can be: the preconditioner's four stages, and the low-mode correction's
+// forward and inverse products (six slices).
+constexpr int kLowFwd = 4, kLowInv = 5;
 
 // Tile geometry by the number of slices: shared memory holds two steps of both operands and the
 // staging tile of the outgoing slices; six slices of a 64-deep step would not fit twice.
-template <int NSL>
+template <int STAGE, int NSL>
 struct TcGeom {
+  static constexpr bool kLow = STAGE == kLowFwd || STAGE == kLowInv;
   static constexpr int BN = NSL == 4 ? 64 : 32;   // tile columns
   static constexpr int BK = NSL == 4 ? 64 : 32;   // one swizzle atom (128 or 64 bytes) per pipeline step
-  static constexpr int KPC = KC / BK;             // pipeline steps per accumulation block
+  static constexpr int KPC = STAGE == kLowInv ? 1 : KC / BK;  // pipeline steps per accumulation block
   static constexpr int A_PLANE = BM * BK * 2;
   static constexpr int kCb = BN / 32;             // 8-column blocks per epilogue warp
   static constexpr int kEpiCols = 8 * kCb;        // tile columns per epilogue warp
   static constexpr int kBPlane = BN * BK * 2;
-  static constexpr int kStageBytes = NSL * (A_PLANE + kBPlane);  // one 64-deep step of both operands
-  static constexpr int kStage = NSL * 32 * BM * 2;  // staging: [slice][64-row half][column] 128 B rows
+  static constexpr int kStageBytes = NSL * (A_PLANE + kBPlane);  // one step of both operands
+  // staging of the epilogue: the outgoing slices [slice][64-row half][column] as 128-byte rows; the
+  // forward low-mode product's H tile and Qy rows; nothing for the inverse one
+  static constexpr int kStage = STAGE == kLowInv ? 0 : STAGE == kLowFwd ? 8 * BM * 33 + 8 * BM * kLowM
+                                                                       : NSL * 32 * BM * 2;
+  static constexpr int kSteps = STAGE == kLowInv ? 3 : 2;
   static constexpr int kSetCols = NSL * BN;       // one accumulator per slice order
-  static constexpr int kSmem = STAGES * kStageBytes + kStage + 1024 + 2048;
+  static constexpr int kSmem = kSteps * kStageBytes + kStage + 1024 + 2048;
+  static_assert(!kLow || NSL == kLowNS, "six slices in the low-mode products");
   static_assert(kChunks * kSetCols <= kTmemCols, "TMEM columns");
-  static_assert(kSmem <= 232448, "shared memory of an SM's block");
+  static_assert(kSmem <= 232448 && kStage % 8 == 0, "shared memory of an SM's block");
 };
 
 struct Ctl {
-  uint64_t full[STAGES];
-  uint64_t empty[STAGES];
+  uint64_t full[kMaxSteps];
+  uint64_t empty[kMaxSteps];
   uint64_t tfull[kChunks];
   uint64_t tempty[kChunks];
   uint64_t drain;
@@ -156,11 +166,6 @@ __device__ __forceinline__ bool elect_one() {
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-               : "r"(taddr));
-}
 // Sixteen TMEM lanes by eight columns as a matrix fragment: lane l of the warp gets columns
 // 2 (l % 4), 2 (l % 4) + 1 of rows l / 4 (v[0], v[1]) and l / 4 + 8 (v[2], v[3]).
 __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&v)[4]) {
@@ -284,15 +289,26 @@ __device__ __forceinline__ bool epi_vote(bool fail) {
 
 struct TcStage {
   int M, N, K;
-  int8_t* eout;     // next stage's block exponents [N][M/128]
+  const unsigned char *ma, *mb;  // tensor maps of A and B
+  const int8_t *ea, *eb;         // block exponents: A rows [M][K / KC], B rows [N][K / KC]
+  int8_t* eout;                  // next stage's block exponents [N][M/128]
 };
 
-__device__ __forceinline__ TcStage tc_stage(const SlotDesc& S, int stage) {
-  switch (stage) {
-    case 0: return {S.nyp, S.nxp, S.nxp, S.tc_e[1]};
-    case 1: return {S.nxp, S.nyp, S.nyp, S.tc_e[2]};
-    case 2: return {S.nyp, S.nxp, S.nxp, S.tc_e[3]};
-    default: return {S.nxp, S.nyp, S.nyp, nullptr};
+template <int STAGE>
+__device__ __forceinline__ TcStage tc_stage(const SlotDesc& S) {
+  const unsigned char* maps = static_cast<const unsigned char*>(S.tmaps);
+  const unsigned char* low = static_cast<const unsigned char*>(S.low_maps);
+  if constexpr (STAGE == kLowFwd)  // H = r Qx_low
+    return {S.nyp, kLowM, S.nxp, low, low + 128, S.tc_e[0], S.low_qxt_e, nullptr};
+  else if constexpr (STAGE == kLowInv)  // zl^T = J^T Qy_low^T, one block of 32 k
+    return {S.nxp, S.nyp, kLowM, low + 256, low + 384, S.low_jt_e, S.low_qy_e, nullptr};
+  else {
+    const int8_t *ea = S.tc_e[STAGE], *eb = S.tc_eb[STAGE];
+    int8_t* eo = STAGE < 3 ? S.tc_e[(STAGE + 1) & 3] : nullptr;
+    if constexpr (STAGE == 0 || STAGE == 2)
+      return {S.nyp, S.nxp, S.nxp, maps + 128 * STAGE, maps + 128 * (4 + STAGE), ea, eb, eo};
+    else
+      return {S.nxp, S.nyp, S.nyp, maps + 128 * STAGE, maps + 128 * (4 + STAGE), ea, eb, eo};
   }
 }
 
@@ -326,9 +342,9 @@ template <bool BF16, int STAGE, int NSL>
 __global__ void __maxnreg__(kMaxRegs)
 k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
           const int* __restrict__ n_items, int mode, int* __restrict__ err, long long wait_cycles) {
-  using G = TcGeom<NSL>;
+  using G = TcGeom<STAGE, NSL>;
   constexpr int BN = G::BN, kCb = G::kCb, kEpiCols = G::kEpiCols, BK = G::BK, KPC = G::KPC;
-  constexpr int A_PLANE = G::A_PLANE;
+  constexpr int A_PLANE = G::A_PLANE, STAGES = G::kSteps;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -373,14 +389,13 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         const unsigned char *ma, *mb;
         int M, N, steps, m0, n0;
       };
-      auto tile_of = [&](int w) {
+      auto tile_of = [&](int w) -> Tile {
         const WorkItem it = items[w];
+        if (it.slot < 0) return {};
         const SlotDesc& S = slots[it.slot];
-        const TcStage v = tc_stage(S, STAGE);
+        const TcStage v = tc_stage<STAGE>(S);
         const int mt = v.M / BM;
-        Tile t = {S.sc, static_cast<const unsigned char*>(S.tmaps) + 128 * STAGE,
-                  static_cast<const unsigned char*>(S.tmaps) + 128 * (4 + STAGE), v.M, v.N, v.K / BK,
-                  (it.tile % mt) * BM, (it.tile / mt) * BN};
+        Tile t = {S.sc, v.ma, v.mb, v.M, v.N, v.K / BK, (it.tile % mt) * BM, (it.tile / mt) * BN};
         tmap_acquire(t.ma);
         tmap_acquire(t.mb);
         return t;
@@ -391,7 +406,7 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
       int n = 0;  // steps issued
       for (int w = blockIdx.x; w < total && !*abort_flag; w += gridDim.x) {
         if (w != blockIdx.x) t = tile_of(w);
-        if (!slot_runs(t.sc, mode)) continue;
+        if (t.sc == nullptr || !slot_runs(t.sc, mode)) continue;
         for (int kb = 0; kb < t.steps; ++kb) {
           const int st = n % STAGES;
           unsigned char* sa = smem + st * G::kStageBytes;
@@ -429,15 +444,15 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     const SlotScalars* sc = nullptr;
     int k_tile = 0;
     auto tile_of = [&](int w) {
-      const SlotDesc& S = slots[items[w].slot];
-      sc = S.sc;
-      k_tile = tc_stage(S, STAGE).K;
+      const int slot = items[w].slot;
+      sc = slot < 0 ? nullptr : slots[slot].sc;
+      k_tile = slot < 0 ? 0 : tc_stage<STAGE>(slots[slot]).K;
     };
     if (blockIdx.x < total) tile_of(blockIdx.x);
     pdl_wait();
     for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
       if (w != blockIdx.x) tile_of(w);
-      if (!__any_sync(0xffffffffu, slot_runs(sc, mode))) continue;
+      if (!__any_sync(0xffffffffu, sc != nullptr && slot_runs(sc, mode))) continue;
       const int steps = __reduce_max_sync(0xffffffffu, k_tile / BK);
       for (int kb = 0; kb < steps; ++kb) {
         const int half_kb = kb % KPC;  // position inside the accumulation block
@@ -486,7 +501,7 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     const int t4 = lane >> 2, tc = lane & 3;
     const bool col_lane = lane < kEpiCols;   // lanes that own one of the warp's columns
     int chunk = 0;
-    if (blockIdx.x < total) {
+    if (blockIdx.x < total && items[blockIdx.x].slot >= 0) {
       // the first tile's descriptor into this SM's L1
       const SlotDesc& S = slots[items[blockIdx.x].slot];
       if (lane < static_cast<int>((sizeof(SlotDesc) + 127) / 128)) {
@@ -498,16 +513,17 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     // the epilogue warps leave the list only together, at a vote: after an abort their waits fail
     for (int w = blockIdx.x; w < total; w += gridDim.x) {
       const WorkItem it = items[w];
+      if (it.slot < 0) continue;  // an empty place of the balanced list
       const SlotDesc& S = slots[it.slot];
       SlotScalars* sc = S.sc;
       if (!slot_runs(sc, mode)) continue;
-      const TcStage v = tc_stage(S, STAGE);
+      const TcStage v = tc_stage<STAGE>(S);
       const int mt = v.M / BM;
       const int m0 = (it.tile % mt) * BM, n0 = (it.tile / mt) * BN;
       const int mq = m0 + 32 * quarter;          // first row of the quarter
       const int ng = n0 + 8 * group;             // first column of the group (block cb: + 32 cb)
       const int n_mine = ng + 32 * (lane >> 3) + (lane & 7);  // a column lane's column
-      const int kblocks = v.K / KC;
+      const int kblocks = STAGE == kLowInv ? 1 : v.K / KC;
       if (STAGE == 3 && col_lane && !S.mir_out) {
         // the r, q and mask entries read after the last k-block: start them towards L2 now
         const int n = n_mine;
@@ -537,8 +553,20 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         }
         wnorm = ld_early(&S.wnorm);
       }
-      const int8_t* ea_row = S.tc_e[STAGE] + static_cast<size_t>(mq + lane) * kblocks;
-      const int8_t* eb_col = S.tc_eb[STAGE] + static_cast<size_t>(col_lane ? n_mine : ng) * kblocks;
+      const int8_t* ea_row = v.ea + static_cast<size_t>(mq + lane) * kblocks;
+      const int8_t* eb_col = v.eb + static_cast<size_t>(col_lane ? n_mine : ng) * kblocks;
+      // the thread's share of the tile's Qy_low rows (the G share's operand), loaded now so that
+      // their latency hides behind the k-blocks
+      constexpr int kYq = STAGE == kLowFwd ? BM * kLowM / (32 * kEpiWarps) : 1;
+      float yq[2 * kYq];
+      if (STAGE == kLowFwd) {
+#pragma unroll
+        for (int i = 0; i < kYq; ++i) {
+          const size_t a = static_cast<size_t>(m0) * kLowM + 32 * ew + lane + i * 32 * kEpiWarps;
+          yq[i] = ld_early(S.low_qyd + a);
+          yq[kYq + i] = ld_early(S.low_qyd + static_cast<size_t>(S.nyp) * kLowM + a);
+        }
+      }
       // compensated (hi, lo) pairs, one packed register pair per (rb, cb)
       float2 hi[kCb][4], lo[kCb][4];
 #pragma unroll
@@ -623,7 +651,63 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
             lo[cb][rb] = t.lo;
           }
       }
-      if (STAGE <= 2) {
+      if (STAGE == kLowFwd) {
+        // the tile's share of G = Qy_low^T H (its 128 rows of y), by compensated dot products of
+        // double-float operands staged in shared memory; H itself is not stored
+        if (epi_vote(fail)) break;  // (also: the previous tile's dot products have read the staging)
+        float* hs = reinterpret_cast<float*>(sO);  // H tile [128][33]: hi, then lo
+        float* ys = hs + 2 * BM * 33;              // Qy_low rows m0 .. m0+127 [128][32]: hi, lo
+#pragma unroll
+        for (int rb = 0; rb < 4; ++rb) {
+          float* h = hs + (32 * quarter + 8 * rb + t4) * 33 + 8 * group + 2 * tc;
+          h[0] = hi[0][rb].x;
+          h[1] = hi[0][rb].y;
+          h[BM * 33] = lo[0][rb].x;
+          h[BM * 33 + 1] = lo[0][rb].y;
+        }
+#pragma unroll
+        for (int i = 0; i < kYq; ++i) {
+          ys[32 * ew + lane + i * 32 * kEpiWarps] = yq[i];
+          ys[BM * kLowM + 32 * ew + lane + i * 32 * kEpiWarps] = yq[kYq + i];
+        }
+        epi_bar();
+        // thread: kx = lane, ky = 2 ew and 2 ew + 1, the two dot products on packed FP32x2 (one
+        // 8-byte broadcast load of each plane's Qy_low pair per row)
+        CompDotDF2 g;
+        const int ky0 = 2 * ew;
+#pragma unroll 4
+        for (int rr = 0; rr < BM; ++rr) {
+          const float bh = hs[rr * 33 + lane], bl = hs[BM * 33 + rr * 33 + lane];
+          const float2 ah = *reinterpret_cast<const float2*>(ys + rr * kLowM + ky0);
+          const float2 al = *reinterpret_cast<const float2*>(ys + BM * kLowM + rr * kLowM + ky0);
+          g.add(ah, al, make_float2(bh, bh), make_float2(bl, bl));
+        }
+        float* gp = S.low_gp + static_cast<size_t>(it.tile) * 2 * kLowM * kLowM;
+        const f2 a0 = df_norm(g.s.x, g.c.x), a1 = df_norm(g.s.y, g.c.y);
+        gp[ky0 * kLowM + lane] = a0.hi;
+        gp[kLowM * kLowM + ky0 * kLowM + lane] = a0.lo;
+        gp[(ky0 + 1) * kLowM + lane] = a1.hi;
+        gp[kLowM * kLowM + (ky0 + 1) * kLowM + lane] = a1.lo;
+      } else if (STAGE == kLowInv) {
+        // zl[y][x] at rows n = y of the tile's columns
+        if (epi_vote(fail)) break;
+        const int nx = S.nx, ny = S.ny;
+        float* zl = S.low_z;
+        const size_t nn = static_cast<size_t>(nx) * ny;
+#pragma unroll
+        for (int rb = 0; rb < 4; ++rb) {
+          const int m = mq + 8 * rb + t4, n = ng + 2 * tc;
+          if (m < nx && n < ny) {
+            const size_t g = static_cast<size_t>(n) * nx + m;
+            zl[g] = hi[0][rb].x;
+            zl[nn + g] = lo[0][rb].x;
+            if (n + 1 < ny) {
+              zl[g + nx] = hi[0][rb].y;
+              zl[nn + g + nx] = lo[0][rb].y;
+            }
+          }
+        }
+      } else if (STAGE <= 2) {
         // block exponents of the next operand: row n, k-block of the tile's 128 m.  The largest
         // magnitude of each column: over the thread's rows, then by halving exchanges over the
         // lanes of equal tc, after which the lane holds one column
@@ -1097,432 +1181,12 @@ k_unfold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
 // exact integer of at most 2^24.  Orders 0..2 are merged into the double-float result with TwoSum,
 // orders 3..5 (below 2^-24 of it) in plain FP32.
 //
-// The forward product: one CTA per 128 rows of y, sixteen warps (four per TMEM lane quarter, eight
-// of the 32 columns each); thread 0 issues the tensor copies and the MMAs one 64-wide k step at a
-// time (the products are thin, so a simple serial pipeline suffices), every thread drains its own
-// TMEM lane after each exponent block, and after the last block the CTA forms its share of G.
+// Both products are launches of the stage kernel (forms kLowFwd and kLowInv): 128 x 32 tiles, 32-deep
+// steps copied ahead, MMAs of one accumulation block running while the sixteen warps merge the one
+// before.  (As kernels of their own, each tile copying, multiplying and merging in turn and the
+// inverse one item per 128 rows of x, the two took 45 + 47 us per application on a batch of 48 grids.)
 // ---------------------------------------------------------------------------------------------
-constexpr int LBN = kLowM;                   // N tile (columns)
-constexpr int LBK = 64;                      // k per tensor copy
-constexpr int LA_PLANE = BM * LBK * 2;       // 16 KB
-constexpr int LB_PLANE = LBN * LBK * 2;      // 4 KB
-constexpr int kLowThreads = 512;              // 16 warps: four per TMEM lane quarter
-constexpr int kLowCols = LBN / 4;             // columns per warp in the merge
-constexpr int kLowTmemCols = 256;            // >= kLowNS * LBN
-constexpr int kLowSmem = kLowNS * (LA_PLANE + LB_PLANE) + 1024 + 256;
-static_assert(kLowNS * LBN <= kLowTmemCols, "low-mode TMEM columns");
-static_assert(kLowK3 == LBK, "the inverse product's k fits one copy");
-static_assert(kLowThreads == 16 * 32 && 2 * BM * 33 * 4 + 2 * BM * kLowM * 4 <= kLowNS * (LA_PLANE + LB_PLANE),
-              "the G stage: sixteen warps (ky = 2 warp, 2 warp + 1) and its staging in the operand buffers");
-static_assert((2 * BM * 33) % 2 == 0 && kLowM % 2 == 0, "8-byte aligned Qy_low pairs in the G stage");
-static_assert((BM * kLowM) % kLowThreads == 0, "the tile's Qy_low rows in equal shares per thread");
-
-struct LowCtl {
-  uint64_t full, done;
-  uint32_t tmem;
-  int abort_flag;
-};
-
-template <bool BF16>
-__global__ void __launch_bounds__(kLowThreads, 1)
-k_low_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
-         const int* __restrict__ n_items, int mode, int* __restrict__ err, long long wait_cycles) {
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char* smem = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  LowCtl* ctl = reinterpret_cast<LowCtl*>(smem + kLowNS * (LA_PLANE + LB_PLANE));
-  volatile int* abort_flag = &ctl->abort_flag;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int total = *n_items;
-  if (threadIdx.x == 0) {
-    mbar_init(&ctl->full, 1);
-    mbar_init(&ctl->done, 1);
-    ctl->abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem)),
-                 "r"(kLowTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = ctl->tmem;
-  pdl_wait();
-  uint32_t ph_full = 0, ph_done = 0;
-  int inflight = 0;     // thread 0: tensor copies issued and not yet waited for (0 or 1)
-  int mma_pending = 0;  // thread 0: MMAs committed and not yet waited for (0 or 1)
-  const int quarter = warp & 3, cg = warp >> 2;  // TMEM lane quarter, column group
-  const int row = quarter * 32 + lane;          // TMEM lane of this thread = tile row
-  bool failed = false;
-  for (int w = blockIdx.x; w < total && !failed; w += gridDim.x) {
-    const WorkItem it = items[w];
-    const SlotDesc& S = slots[it.slot];
-    if (!slot_runs(S.sc, mode) || S.lowm_x == 0) continue;
-    // geometry: A = the residual's six slice planes (rows y), B = Qx_low^T's (rows kx)
-    const unsigned char* maps = static_cast<const unsigned char*>(S.low_maps);
-    const void* ma = maps;
-    const void* mb = maps + 128;
-    const int m0 = it.tile * BM, n0 = 0, K = S.nxp, KC = 128, rowsA = S.nyp, rowsB = kLowM;
-    if (threadIdx.x == 0) {
-      tmap_acquire(ma);
-      tmap_acquire(mb);
-    }
-    const int m = m0 + row;
-    // the thread's share of the tile's Qy_low rows (the G stage's operand), loaded now so that
-    // their latency hides behind the k-blocks
-    constexpr int kYq = BM * kLowM / kLowThreads;
-    float yq[2 * kYq];
-#pragma unroll
-    for (int i = 0; i < kYq; ++i) {
-      const size_t a = static_cast<size_t>(m0) * kLowM + threadIdx.x + i * kLowThreads;
-      yq[i] = ld_early(S.low_qyd + a);
-      yq[kYq + i] = ld_early(S.low_qyd + static_cast<size_t>(S.nyp) * kLowM + a);
-    }
-    // double-float result of the thread's row, one per column of its group
-    float hi[kLowCols], lo[kLowCols];
-#pragma unroll
-    for (int c = 0; c < kLowCols; ++c) {
-      hi[c] = 0.f;
-      lo[c] = 0.f;
-    }
-    for (int kb = 0; kb < K / KC && !failed; ++kb) {
-      if (threadIdx.x == 0) {
-        for (int sub = 0; sub < KC / LBK; ++sub) {
-          const int k0 = kb * KC + sub * LBK;
-          unsigned char* sa = smem;
-          unsigned char* sb = smem + kLowNS * LA_PLANE;
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          mbar_expect_tx(&ctl->full, kLowNS * (LA_PLANE + LB_PLANE));
-#pragma unroll
-          for (int p = 0; p < kLowNS; ++p) tma_load_2d(sa + p * LA_PLANE, ma, &ctl->full, k0, p * rowsA + m0);
-#pragma unroll
-          for (int p = 0; p < kLowNS; ++p) tma_load_2d(sb + p * LB_PLANE, mb, &ctl->full, k0, p * rowsB + n0);
-          inflight = 1;
-          if (!mbar_wait(&ctl->full, ph_full, abort_flag, wait_cycles)) break;
-          inflight = 0;
-          ph_full ^= 1;
-          tc_fence_after();
-          const uint32_t a0 = smem_u32(sa), b0 = smem_u32(sb);
-#pragma unroll
-          for (int j = 0; j < LBK / 16; ++j) {
-#pragma unroll
-            for (int i = 0; i < kLowNS; ++i) {
-              // slice i of A against the B slices 0 .. kLowNS-1-i stacked along N: order i + j'
-              // lands in the accumulator at column (i + j') * LBN
-              umma(tmem_base + i * LBN, sdesc(a0 + i * LA_PLANE) + 2 * j, sdesc(b0) + 2 * j,
-                   idesc_f16(BF16, BM, (kLowNS - i) * LBN), (sub > 0 || j > 0 || i > 0) ? 1u : 0u);
-            }
-          }
-          umma_commit(&ctl->done);
-          // the next copy reuses the shared memory, and the block's sums must be complete
-          mma_pending = 1;
-          if (!mbar_wait(&ctl->done, ph_done, abort_flag, wait_cycles)) break;
-          mma_pending = 0;
-          ph_done ^= 1;
-        }
-      }
-      __syncthreads();
-      if (*abort_flag) {
-        failed = true;
-        break;
-      }
-      tc_fence_after();
-      // exponents of the block: the thread's row (A) and every column (B)
-      const int ea = S.tc_e[0][static_cast<size_t>(min(m, S.nyp - 1)) * (S.nxp / 128) + kb];
-      // 2^(E_A + E_B - 16) of every column (exact products of powers of two)
-      float scl[kLowCols];
-#pragma unroll
-      for (int c = 0; c < kLowCols; ++c) {
-        const int cc = cg * kLowCols + c;
-        const int eb = S.low_qxt_e[static_cast<size_t>(cc) * (S.nxp / 128) + kb];
-        scl[c] = pow2f(ea - 16) * pow2f(eb);
-      }
-      // the six order sums of the warp's columns, loaded together
-      uint32_t v[kLowNS][kLowCols];
-#pragma unroll
-      for (int d = 0; d < kLowNS; ++d)
-        tmem_ld8(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + d * LBN + cg * kLowCols, v[d]);
-      tmem_wait_ld();
-#pragma unroll
-      for (int d = 0; d < kLowNS; ++d) {
-        const float od = pow2f(-8 * d);
-#pragma unroll
-        for (int c = 0; c < kLowCols; ++c) {
-          const float t = __uint_as_float(v[d][c]) * scl[c] * od;
-          if (d <= 2) {
-            float e;
-            two_sum(hi[c], t, hi[c], e);
-            lo[c] = __fadd_rn(lo[c], e);
-          } else {
-            lo[c] = __fadd_rn(lo[c], t);
-          }
-        }
-      }
-      tc_fence_before();
-      __syncthreads();  // the next block's MMAs overwrite the accumulators
-    }
-    if (failed) break;
-    {
-      // the tile's share of G = Qy_low^T H (its 128 rows of y), by compensated dot products of
-      // double-float operands staged in shared memory (the operand buffers are free: the last
-      // MMAs completed before the block's TMEM reads); H itself is not stored
-      float* hs = reinterpret_cast<float*>(smem);  // H tile [128][33]: hi, then lo
-      float* ys = hs + 2 * BM * 33;                 // Qy_low rows m0 .. m0+127 [128][32]: hi, lo
-#pragma unroll
-      for (int c = 0; c < kLowCols; ++c) {
-        const f2 hv = df_norm(hi[c], lo[c]);
-        hs[row * 33 + cg * kLowCols + c] = hv.hi;
-        hs[BM * 33 + row * 33 + cg * kLowCols + c] = hv.lo;
-      }
-#pragma unroll
-      for (int i = 0; i < kYq; ++i) {
-        ys[threadIdx.x + i * kLowThreads] = yq[i];
-        ys[BM * kLowM + threadIdx.x + i * kLowThreads] = yq[kYq + i];
-      }
-      __syncthreads();
-      // thread: kx = lane, ky = 2 warp and 2 warp + 1, the two dot products on packed FP32x2
-      // (one 8-byte broadcast load of each plane's Qy_low pair per row)
-      CompDotDF2 g;
-      const int ky0 = 2 * warp;
-#pragma unroll 4
-      for (int rr = 0; rr < BM; ++rr) {
-        const float bh = hs[rr * 33 + lane], bl = hs[BM * 33 + rr * 33 + lane];
-        const float2 ah = *reinterpret_cast<const float2*>(ys + rr * kLowM + ky0);
-        const float2 al = *reinterpret_cast<const float2*>(ys + BM * kLowM + rr * kLowM + ky0);
-        g.add(ah, al, make_float2(bh, bh), make_float2(bl, bl));
-      }
-      float* gp = S.low_gp + static_cast<size_t>(it.tile) * 2 * kLowM * kLowM;
-      const f2 a0 = df_norm(g.s.x, g.c.x), a1 = df_norm(g.s.y, g.c.y);
-      gp[ky0 * kLowM + lane] = a0.hi;
-      gp[kLowM * kLowM + ky0 * kLowM + lane] = a0.lo;
-      gp[(ky0 + 1) * kLowM + lane] = a1.hi;
-      gp[kLowM * kLowM + (ky0 + 1) * kLowM + lane] = a1.lo;
-      __syncthreads();  // the next item's tensor copies overwrite the staging
-    }
-  }
-  if (threadIdx.x == 0) {
-    // after an abort: a copy still in flight lands, and committed MMAs complete, before the CTA
-    // frees its TMEM and leaves
-    if (inflight) {
-      const long long t0 = clock64();
-      while (!mbar_try(&ctl->full, ph_full) && clock64() - t0 < kWaitCycles / 4) {
-      }
-    }
-    if (mma_pending) {
-      const long long t0 = clock64();
-      while (!mbar_try(&ctl->done, ph_done) && clock64() - t0 < kWaitCycles / 4) {
-      }
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kLowTmemCols)
-                 : "memory");
-  }
-  if (threadIdx.x == 0 && ctl->abort_flag) atomicExch(err, 1);
-}
-
-// Inverse low-mode product, zl[y][x] = sum_ky Qy[y][ky] J[ky][x], one item per (slot, 128-row
-// tile of x).  The tile's six J^T slice planes (its A operand, k = ky padded to 64; the products
-// use the 32 real k) are copied once; the B operand (Qy_low's slices for 32 values of y) is
-// double-buffered, each copy issued two y-tiles ahead (as soon as the products that read its
-// buffer are complete), and the products of consecutive y-tiles go to two TMEM sets, so that the
-// MMAs of one y-tile run while the sixteen warps merge and store the previous one.
-struct LowInvCtl {
-  uint64_t fa, fb[2], md[2];
-  uint32_t tmem;
-  int abort_flag;
-};
-constexpr int kLowInvSmem = kLowNS * LA_PLANE + 2 * kLowNS * LB_PLANE + 1024 + 256;
-constexpr int kLowInvThreads = 512;            // 16 warps: four per TMEM lane quarter
-constexpr int kLowInvCols = LBN / 4;           // columns per warp
-constexpr int kLowInvTmemCols = 512;  // two sets of kLowNS * LBN columns, at 0 and 256
-static_assert(kLowNS * LBN <= 256, "low-mode TMEM set");
-
-template <bool BF16>
-__global__ void __launch_bounds__(kLowInvThreads, 1)
-k_low_inv(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
-          const int* __restrict__ n_items, int mode, int* __restrict__ err, long long wait_cycles) {
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char* smem = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  unsigned char* sA = smem;
-  unsigned char* sB = smem + kLowNS * LA_PLANE;  // two buffers of kLowNS * LB_PLANE
-  LowInvCtl* ctl = reinterpret_cast<LowInvCtl*>(sB + 2 * kLowNS * LB_PLANE);
-  volatile int* abort_flag = &ctl->abort_flag;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int total = *n_items;
-  if (threadIdx.x == 0) {
-    mbar_init(&ctl->fa, 1);
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&ctl->fb[b], 1);
-      mbar_init(&ctl->md[b], 1);
-    }
-    ctl->abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem)),
-                 "r"(kLowInvTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = ctl->tmem;
-  pdl_wait();
-  // thread 0's barrier bookkeeping: phases and the waits still owed
-  uint32_t ph_fa = 0, ph_fb[2] = {0, 0}, ph_md[2] = {0, 0};
-  int owe_fa = 0, owe_fb[2] = {0, 0}, owe_md[2] = {0, 0};
-  const int quarter = warp & 3, cg = warp >> 2;   // TMEM lane quarter, column group
-  const int row = quarter * 32 + lane;
-  bool failed = false;
-  for (int w = blockIdx.x; w < total && !failed; w += gridDim.x) {
-    const WorkItem it = items[w];
-    const SlotDesc& S = slots[it.slot];
-    if (!slot_runs(S.sc, mode) || S.lowm_x == 0) continue;
-    const unsigned char* maps = static_cast<const unsigned char*>(S.low_maps);
-    const void* ma = maps + 128 * 2;
-    const void* mb = maps + 128 * 3;
-    const int m0 = it.tile * BM;
-    const int nt = S.nyp / LBN;
-    auto issue_b = [&](int j) {  // thread 0: B slices of y-tile j into buffer j & 1
-      const int b = j & 1;
-      unsigned char* dst = sB + b * kLowNS * LB_PLANE;
-      mbar_expect_tx(&ctl->fb[b], kLowNS * LB_PLANE);
-#pragma unroll
-      for (int p = 0; p < kLowNS; ++p) tma_load_2d(dst + p * LB_PLANE, mb, &ctl->fb[b], 0, p * S.nyp + j * LBN);
-      owe_fb[b] = 1;
-    };
-    auto issue_mma = [&](int j) -> bool {  // thread 0: wait for B(j), products into set j & 1
-      const int b = j & 1;
-      if (!mbar_wait(&ctl->fb[b], ph_fb[b], abort_flag, wait_cycles)) return false;
-      owe_fb[b] = 0;
-      ph_fb[b] ^= 1;
-      tc_fence_after();
-      const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB + b * kLowNS * LB_PLANE);
-      const uint32_t dset = tmem_base + b * 256;
-      // only the first kLowM of the copy's LBK k are modes; the rest is zero padding
-#pragma unroll
-      for (int jj = 0; jj < kLowM / 16; ++jj) {
-#pragma unroll
-        for (int i = 0; i < kLowNS; ++i)
-          umma(dset + i * LBN, sdesc(a0 + i * LA_PLANE) + 2 * jj, sdesc(b0) + 2 * jj,
-               idesc_f16(BF16, BM, (kLowNS - i) * LBN), (jj > 0 || i > 0) ? 1u : 0u);
-      }
-      umma_commit(&ctl->md[b]);
-      owe_md[b] = 1;
-      return true;
-    };
-    if (threadIdx.x == 0) {
-      tmap_acquire(ma);
-      tmap_acquire(mb);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_expect_tx(&ctl->fa, kLowNS * LA_PLANE);
-#pragma unroll
-      for (int p = 0; p < kLowNS; ++p) tma_load_2d(sA + p * LA_PLANE, ma, &ctl->fa, 0, p * S.nxp + m0);
-      owe_fa = 1;
-      issue_b(0);
-      bool ok = mbar_wait(&ctl->fa, ph_fa, abort_flag, wait_cycles);
-      if (ok) {
-        owe_fa = 0;
-        ph_fa ^= 1;
-        ok = issue_mma(0);
-      }
-      if (ok && nt > 1) issue_b(1);
-    }
-    const int m = m0 + row;
-    const float sa = pow2f(static_cast<int>(S.low_jt_e[min(m, S.nxp - 1)]) - 16);
-    const size_t nn = static_cast<size_t>(S.nx) * S.ny;
-    for (int j = 0; j < nt; ++j) {
-      const int b = j & 1;
-      if (threadIdx.x == 0 && !*abort_flag) {
-        // B(j + 1) was copied a step ago; once y-tile j's products are complete its B buffer
-        // takes the copy of y-tile j + 2, which lands while this step's sums are merged
-        if (mbar_wait(&ctl->md[b], ph_md[b], abort_flag, wait_cycles)) {
-          owe_md[b] = 0;
-          ph_md[b] ^= 1;
-          if (j + 1 < nt && issue_mma(j + 1) && j + 2 < nt) issue_b(j + 2);
-        }
-      }
-      __syncthreads();
-      if (*abort_flag) {
-        failed = true;
-        break;
-      }
-      tc_fence_after();
-      const int n0 = j * LBN + cg * kLowInvCols;  // the warp's columns
-      float hi[kLowInvCols], lo[kLowInvCols], scl[kLowInvCols];
-#pragma unroll
-      for (int c = 0; c < kLowInvCols; ++c) {
-        hi[c] = 0.f;
-        lo[c] = 0.f;
-        scl[c] = sa * pow2f(S.low_qy_e[n0 + c]);
-      }
-      uint32_t v[kLowNS][kLowInvCols];  // the six order sums, loaded together
-#pragma unroll
-      for (int d = 0; d < kLowNS; ++d)
-        tmem_ld8(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + b * 256 + d * LBN +
-                     cg * kLowInvCols, v[d]);
-      tmem_wait_ld();
-#pragma unroll
-      for (int d = 0; d < kLowNS; ++d) {
-        const float od = pow2f(-8 * d);
-#pragma unroll
-        for (int c = 0; c < kLowInvCols; ++c) {
-          const float t = __uint_as_float(v[d][c]) * scl[c] * od;
-          if (d <= 2) {
-            float e;
-            two_sum(hi[c], t, hi[c], e);
-            lo[c] = __fadd_rn(lo[c], e);
-          } else {
-            lo[c] = __fadd_rn(lo[c], t);
-          }
-        }
-      }
-      tc_fence_before();
-      if (m < S.nx) {
-#pragma unroll
-        for (int c = 0; c < kLowInvCols; ++c) {
-          const int y = n0 + c;
-          if (y < S.ny) {
-            const f2 v = df_norm(hi[c], lo[c]);
-            const size_t g = static_cast<size_t>(y) * S.nx + m;
-            S.low_z[g] = v.hi;
-            S.low_z[nn + g] = v.lo;
-          }
-        }
-      }
-      __syncthreads();  // TMEM set b and B buffer b are free for y-tile j + 2
-    }
-  }
-  if (threadIdx.x == 0) {
-    // after an abort: copies still in flight land and committed MMAs complete before the CTA
-    // frees its TMEM and leaves
-    const long long t0 = clock64();
-    if (owe_fa) while (!mbar_try(&ctl->fa, ph_fa) && clock64() - t0 < kWaitCycles / 4) {}
-    for (int b = 0; b < 2; ++b) {
-      if (owe_fb[b]) while (!mbar_try(&ctl->fb[b], ph_fb[b]) && clock64() - t0 < kWaitCycles / 4) {}
-      if (owe_md[b]) while (!mbar_try(&ctl->md[b], ph_md[b]) && clock64() - t0 < kWaitCycles / 4) {}
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kLowInvTmemCols)
-                 : "memory");
-  }
-  if (threadIdx.x == 0 && ctl->abort_flag) atomicExch(err, 1);
-}
+static_assert(kLowM == 32 && kLowK3 == kLowM, "the inverse product's k is one step");
 
 // The slices of one double-float value on a single lane (the packed routine on lane x).
 template <bool BF16>
@@ -1535,15 +1199,16 @@ __device__ __forceinline__ void slice_codes_df(float vh, float vl, float up, flo
   for (int k = 0; k < kLowNS; ++k) code[k] = static_cast<uint16_t>(c2[k] & 0xffffu);
 }
 
-// Middle of the low-mode correction, one block per (problem, 128 rows of x) (the inverse
-// product's items): G = the forward tiles' shares summed in tile order, G' = w o G, and the
-// block's rows of J^T, J^T[x][ky] = sum_kx G'[ky][kx] Qx[x][kx], by compensated dot products of
-// double-float operands (Ogita-Rump-Oishi), each row then cut into six slices with its block
-// exponent (the inverse product's A operand).  Lane ky reads its row of G' from shared memory;
-// the block's rows of Qx_low are staged there transposed, so that a warp takes the values of two
-// adjacent rows at one kx by one 8-byte broadcast load, and eight rows run as four packed
-// chains.
-constexpr int kQsStride = BM + 2;  // [kx][row] stride: even (8-byte pairs), 2-way staging conflicts
+// Middle of the low-mode correction, one block per (problem, 32 rows of x): G = the forward tiles'
+// shares summed in tile order, G' = w o G, and the block's rows of J^T,
+// J^T[x][ky] = sum_kx G'[ky][kx] Qx[x][kx], by compensated dot products of double-float operands
+// (Ogita-Rump-Oishi), each row then cut into six slices with its block exponent (the inverse
+// product's A operand).  Lane ky reads its row of G' from shared memory; the block's rows of Qx_low
+// are staged there transposed, so that a warp takes the values of two adjacent rows at one kx by one
+// 8-byte broadcast load; each warp runs four rows as two packed chains.  Bound by FP32 issue, so the
+// blocks are small (128 rows a block left some SMs two blocks and others one).
+constexpr int kMidRows = 32;
+constexpr int kQsStride = kMidRows + 2;  // [kx][row] stride: even (8-byte pairs), 2-way staging conflicts
 template <bool BF16>
 __global__ void __launch_bounds__(256)
 k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
@@ -1559,8 +1224,8 @@ k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     if (!slot_runs(S.sc, mode) || S.lowm_x == 0) continue;
     const float* qx_h = S.low_qxd;
     const float* qx_l = S.low_qxd + static_cast<size_t>(S.nxp) * kLowM;
-    const int xb = it.tile * BM;
-    for (int e = t; e < BM * kLowM; e += 256) {
+    const int xb = it.tile * kMidRows;
+    for (int e = t; e < kMidRows * kLowM; e += 256) {
       const int r = e / kLowM, kx = e - r * kLowM;
       const size_t a = static_cast<size_t>(xb + r) * kLowM + kx;
       qs[0][kx][r] = __ldg(qx_h + a);
@@ -1582,35 +1247,30 @@ k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     __syncthreads();
     uint16_t* jt = static_cast<uint16_t*>(S.low_jt);
     const size_t plane = static_cast<size_t>(S.nxp) * kLowK3;
-    // the warp's 16 rows of the block, eight at a time: four packed pairs of independent chains
-    constexpr int kRowsPerGroup = 8;
-    for (int rb = warp * (BM / 8); rb < (warp + 1) * (BM / 8); rb += kRowsPerGroup) {
-      CompDotDF2 acc[kRowsPerGroup / 2];
+    constexpr int kRows = kMidRows / 8;  // per warp
+    const int rb = warp * kRows;
+    CompDotDF2 acc[kRows / 2];
 #pragma unroll 4
-      for (int kx = 0; kx < kLowM; ++kx) {
-        const float ah = gh[lane][kx], al = gl[lane][kx];
+    for (int kx = 0; kx < kLowM; ++kx) {
+      const float ah = gh[lane][kx], al = gl[lane][kx];
 #pragma unroll
-        for (int q = 0; q < kRowsPerGroup / 2; ++q) {
-          const float2 bh = *reinterpret_cast<const float2*>(&qs[0][kx][rb + 2 * q]);
-          const float2 bl = *reinterpret_cast<const float2*>(&qs[1][kx][rb + 2 * q]);
-          acc[q].add(make_float2(ah, ah), make_float2(al, al), bh, bl);
-        }
+      for (int q = 0; q < kRows / 2; ++q) {
+        const float2 bh = *reinterpret_cast<const float2*>(&qs[0][kx][rb + 2 * q]);
+        const float2 bl = *reinterpret_cast<const float2*>(&qs[1][kx][rb + 2 * q]);
+        acc[q].add(make_float2(ah, ah), make_float2(al, al), bh, bl);
       }
+    }
 #pragma unroll
-      for (int r = 0; r < kRowsPerGroup; ++r) {
-        const int x = xb + rb + r;
-        const CompDotDF2& d = acc[r / 2];
-        const f2 j = (r & 1) ? df_norm(d.s.y, d.c.y) : df_norm(d.s.x, d.c.x);
-        const int E = block_exp(warp_max(fabsf(j.hi)));
-        uint16_t code[kLowNS];
-        slice_codes_df<BF16>(j.hi, j.lo, pow2f(16 - E), -pow2f(E - 16), code);
+    for (int r = 0; r < kRows; ++r) {
+      const int x = xb + rb + r;
+      const CompDotDF2& d = acc[r / 2];
+      const f2 j = (r & 1) ? df_norm(d.s.y, d.c.y) : df_norm(d.s.x, d.c.x);
+      const int E = block_exp(warp_max(fabsf(j.hi)));
+      uint16_t code[kLowNS];
+      slice_codes_df<BF16>(j.hi, j.lo, pow2f(16 - E), -pow2f(E - 16), code);
 #pragma unroll
-        for (int p = 0; p < kLowNS; ++p) {
-          jt[p * plane + static_cast<size_t>(x) * kLowK3 + lane] = code[p];
-          jt[p * plane + static_cast<size_t>(x) * kLowK3 + kLowM + lane] = 0;  // padding columns
-        }
-        if (lane == 0) S.low_jt_e[x] = static_cast<int8_t>(E);
-      }
+      for (int p = 0; p < kLowNS; ++p) jt[p * plane + static_cast<size_t>(x) * kLowK3 + lane] = code[p];
+      if (lane == 0) S.low_jt_e[x] = static_cast<int8_t>(E);
     }
     __syncthreads();  // gh, gl and qs are rewritten by the next item
   }
@@ -1619,18 +1279,23 @@ k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
 template <bool BF16, int STAGE, int NSL>
 cudaError_t set_attr() {
   return cudaFuncSetAttribute(k_prec_tc<BF16, STAGE, NSL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              TcGeom<NSL>::kSmem);
+                              TcGeom<STAGE, NSL>::kSmem);
+}
+
+template <bool BF16, int STAGE, int NSL>
+void launch_one(const LaunchCfg& c, int mode, int* err) {
+  const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
+  launch_cfg(c, k_prec_tc<BF16, STAGE, NSL>, c.grid, kThreads, TcGeom<STAGE, NSL>::kSmem, c.slots, c.items,
+             c.n_items, mode, err, wc);
 }
 
 template <bool BF16, int NSL>
 void launch_all(const LaunchCfg& c, int stage, int mode, int* err) {
-  const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
-  constexpr int smem = TcGeom<NSL>::kSmem;
   switch (stage) {
-    case 0: launch_cfg(c, k_prec_tc<BF16, 0, NSL>, c.grid, kThreads, smem, c.slots, c.items, c.n_items, mode, err, wc); break;
-    case 1: launch_cfg(c, k_prec_tc<BF16, 1, NSL>, c.grid, kThreads, smem, c.slots, c.items, c.n_items, mode, err, wc); break;
-    case 2: launch_cfg(c, k_prec_tc<BF16, 2, NSL>, c.grid, kThreads, smem, c.slots, c.items, c.n_items, mode, err, wc); break;
-    default: launch_cfg(c, k_prec_tc<BF16, 3, NSL>, c.grid, kThreads, smem, c.slots, c.items, c.n_items, mode, err, wc); break;
+    case 0: launch_one<BF16, 0, NSL>(c, mode, err); break;
+    case 1: launch_one<BF16, 1, NSL>(c, mode, err); break;
+    case 2: launch_one<BF16, 2, NSL>(c, mode, err); break;
+    default: launch_one<BF16, 3, NSL>(c, mode, err); break;
   }
 }
 
@@ -1643,11 +1308,11 @@ bool tc_supported() {
     cudaGetLastError();
     return false;
   }
-  if (p.major != 10 || p.sharedMemPerBlockOptin < static_cast<size_t>(TcGeom<4>::kSmem)) return false;
+  if (p.major != 10 || p.sharedMemPerBlockOptin < static_cast<size_t>(TcGeom<0, 4>::kSmem)) return false;
   // one CTA of kThreads threads at kMaxRegs registers each must fit an SM
   int blocks = 0;
   if (set_attr<true, 0, 4>() != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_prec_tc<true, 0, 4>, kThreads, TcGeom<4>::kSmem) !=
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_prec_tc<true, 0, 4>, kThreads, TcGeom<0, 4>::kSmem) !=
           cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -1655,17 +1320,10 @@ bool tc_supported() {
   return blocks >= 1;
 }
 
-int tc_step_k(int ns) { return ns == 4 ? TcGeom<4>::BK : TcGeom<6>::BK; }
-int tc_tile_cols(int ns) { return ns == 4 ? TcGeom<4>::BN : TcGeom<6>::BN; }
+int tc_step_k(int ns) { return ns == 4 ? TcGeom<0, 4>::BK : TcGeom<0, 6>::BK; }
+int tc_tile_cols(int ns) { return ns == 4 ? TcGeom<0, 4>::BN : TcGeom<0, 6>::BN; }
 
 int tc_block() { return KC; }
-
-template <bool BF16, int KIND>
-static cudaError_t set_low_attr() {
-  if (KIND == 0)
-    return cudaFuncSetAttribute(k_low_tc<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLowSmem);
-  return cudaFuncSetAttribute(k_low_inv<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLowInvSmem);
-}
 
 cudaError_t tc_init() {
   cudaError_t e = cudaSuccess;
@@ -1675,22 +1333,16 @@ cudaError_t tc_init() {
                              set_attr<true, 1, 6>(),  set_attr<true, 2, 6>(),  set_attr<true, 3, 6>(),
                              set_attr<false, 0, 6>(), set_attr<false, 1, 6>(), set_attr<false, 2, 6>(),
                              set_attr<false, 3, 6>(),
-                             set_low_attr<false, 0>(), set_low_attr<false, 1>(), set_low_attr<true, 0>(),
-                             set_low_attr<true, 1>()};
+                             set_attr<false, kLowFwd, 6>(), set_attr<false, kLowInv, 6>(),
+                             set_attr<true, kLowFwd, 6>(), set_attr<true, kLowInv, 6>()};
   for (cudaError_t x : r)
     if (x != cudaSuccess) e = x;
   return e;
 }
 
 void launch_low_tc(const LaunchCfg& c, int kind, int mode, int split_kind, int* err) {
-  const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
-  if (split_kind == 0) {
-    if (kind == 0) launch_cfg(c, k_low_tc<false>, c.grid, kLowThreads, kLowSmem, c.slots, c.items, c.n_items, mode, err, wc);
-    else launch_cfg(c, k_low_inv<false>, c.grid, kLowInvThreads, kLowInvSmem, c.slots, c.items, c.n_items, mode, err, wc);
-  } else {
-    if (kind == 0) launch_cfg(c, k_low_tc<true>, c.grid, kLowThreads, kLowSmem, c.slots, c.items, c.n_items, mode, err, wc);
-    else launch_cfg(c, k_low_inv<true>, c.grid, kLowInvThreads, kLowInvSmem, c.slots, c.items, c.n_items, mode, err, wc);
-  }
+  if (kind == 0) split_kind == 0 ? launch_one<false, kLowFwd, 6>(c, mode, err) : launch_one<true, kLowFwd, 6>(c, mode, err);
+  else split_kind == 0 ? launch_one<false, kLowInv, 6>(c, mode, err) : launch_one<true, kLowInv, 6>(c, mode, err);
 }
 
 void launch_low_mid(const LaunchCfg& c, int mode, int split_kind) {
