@@ -37,9 +37,10 @@ __device__ __forceinline__ int halo_src(const SlotDesc& S, int x0, int y0, int i
   return my * S.nx + mx;
 }
 
-// 13-point masked biharmonic of a smem tile (row stride RS) at local (ly+2, lx+2), as a
-// compensated FP32 sum (s, c): s + c carries the exact sum of the 13 terms to about 48 bits.
-template <bool ANISO, int RS = kHX>
+// The operator on unequal spacings: the 13-point sum of a smem tile (row stride RS) at local
+// (ly+2, lx+2), as a compensated FP32 sum (s, c) that carries the exact sum of the 13 products to about
+// 48 bits.
+template <int RS>
 __device__ __forceinline__ CompSum stencil13_acc(const SlotDesc& S, const float* t, int ly, int lx) {
   const float* c = t + (ly + 2) * RS + (lx + 2);
   const float C = c[0];
@@ -47,78 +48,66 @@ __device__ __forceinline__ CompSum stencil13_acc(const SlotDesc& S, const float*
   const float D0 = c[-RS - 1], D1 = c[-RS + 1], D2 = c[RS - 1], D3 = c[RS + 1];
   const float F0 = c[-2], F1 = c[2], G0 = c[-2 * RS], G1 = c[2 * RS];
   CompSum acc;
-  if (!ANISO) {
-    // 20 C - 8 (edges) + 2 (diagonals) + (distance 2); every term is an exact FP32 value
-    acc.add(16.f * C);
-    acc.add(4.f * C);
-    acc.add(-8.f * E0); acc.add(-8.f * E1); acc.add(-8.f * N0); acc.add(-8.f * N1);
-    acc.add(2.f * D0); acc.add(2.f * D1); acc.add(2.f * D2); acc.add(2.f * D3);
-    acc.add(F0); acc.add(F1); acc.add(G0); acc.add(G1);
-  } else {
-    acc.add_prod(S.wc, C);
-    acc.add_prod(S.wex, E0); acc.add_prod(S.wex, E1);
-    acc.add_prod(S.wey, N0); acc.add_prod(S.wey, N1);
-    acc.add_prod(S.wd, D0); acc.add_prod(S.wd, D1); acc.add_prod(S.wd, D2); acc.add_prod(S.wd, D3);
-    acc.add_prod(S.wfx, F0); acc.add_prod(S.wfx, F1);
-    acc.add_prod(S.wfy, G0); acc.add_prod(S.wfy, G1);
-    // low parts of the weights: products far below the result's ulp, plain FP32 suffices
-    float lo = S.wc_l * C + S.wex_l * (E0 + E1) + S.wey_l * (N0 + N1) +
-               S.wd_l * ((D0 + D1) + (D2 + D3)) + S.wfx_l * (F0 + F1) + S.wfy_l * (G0 + G1);
-    acc.c = __fadd_rn(acc.c, lo);
-  }
+  acc.add_prod(S.wc, C);
+  acc.add_prod(S.wex, E0); acc.add_prod(S.wex, E1);
+  acc.add_prod(S.wey, N0); acc.add_prod(S.wey, N1);
+  acc.add_prod(S.wd, D0); acc.add_prod(S.wd, D1); acc.add_prod(S.wd, D2); acc.add_prod(S.wd, D3);
+  acc.add_prod(S.wfx, F0); acc.add_prod(S.wfx, F1);
+  acc.add_prod(S.wfy, G0); acc.add_prod(S.wfy, G1);
+  // low parts of the weights: products far below the result's ulp, plain FP32 suffices
+  float lo = S.wc_l * C + S.wex_l * (E0 + E1) + S.wey_l * (N0 + N1) +
+             S.wd_l * ((D0 + D1) + (D2 + D3)) + S.wfx_l * (F0 + F1) + S.wfy_l * (G0 + G1);
+  acc.c = __fadd_rn(acc.c, lo);
   return acc;
 }
 
 // The same stencil applied in plain FP32 (for the lo plane of a double-float vector, whose
 // contribution is 2^-24 of the hi plane's: its own rounding is far below the result's ulp).
-template <bool ANISO, int RS>
+template <int RS>
 __device__ __forceinline__ float stencil13_plain(const SlotDesc& S, const float* t, int ly, int lx) {
   const float* c = t + (ly + 2) * RS + (lx + 2);
   const float e = (c[-1] + c[1]), n = (c[-RS] + c[RS]);
   const float d = (c[-RS - 1] + c[-RS + 1]) + (c[RS - 1] + c[RS + 1]);
   const float f = c[-2] + c[2], g = c[-2 * RS] + c[2 * RS];
-  if (!ANISO) return 20.f * c[0] - 8.f * (e + n) + 2.f * d + (f + g);
   return S.wc * c[0] + S.wex * e + S.wey * n + S.wd * d + S.wfx * f + S.wfy * g;
 }
 
-// The isotropic 13-point stencil at two adjacent nodes (x, x+1) of a smem tile with an even row
-// stride RS; c points at node x, an even index.  Eleven aligned 8-byte loads cover both
-// neighbourhoods, and each lane runs the scalar stencil13_acc's operations in the same order
-// (bit-identical results).
+// The operator on equal spacings is the five-point g(u) = (sum of the four neighbours) - 4 u taken
+// twice (M g(g(p)); the boundary rules make g at a ghost node the reflected, wrapped or zero one).
+// One application at two adjacent nodes (x, x+1) of the smem planes h (hi) and l (lo) with an even
+// row stride RS, h and l pointing at node x, an even index: error-free TwoSums of the hi plane
+// (4 u is exact), the errors and the lo plane's five points in plain FP32.  33 packed operations;
+// the 13-point sum of fourteen TwoSums that this replaced took 124 for the two planes, the two
+// applications take 66 (and one node of w's ring per tile edge).
 __device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
-template <int RS>
-__device__ __forceinline__ CompSum2 stencil13_pair_acc(const float* c) {
+template <int RS, bool LO = true>
+__device__ __forceinline__ f2x2 lap_pair(const float* h, const float* l) {
   static_assert(RS % 2 == 0, "pairs of nodes start on 8-byte boundaries");
-  const float2 Cm = ld2(c - 2), C = ld2(c), Cp = ld2(c + 2);                  // row y
-  const float2 Nm = ld2(c - RS - 2), N = ld2(c - RS), Np = ld2(c - RS + 2);   // row y-1
-  const float2 Sm = ld2(c + RS - 2), Sv = ld2(c + RS), Sp = ld2(c + RS + 2);  // row y+1
-  const float2 NN = ld2(c - 2 * RS), SS = ld2(c + 2 * RS);                    // rows y-2, y+2
-  const float2 E0 = make_float2(Cm.y, C.x), E1 = make_float2(C.y, Cp.x);
-  const float2 D0 = make_float2(Nm.y, N.x), D1 = make_float2(N.y, Np.x);
-  const float2 D2 = make_float2(Sm.y, Sv.x), D3 = make_float2(Sv.y, Sp.x);
-  CompSum2 acc;
-  acc.add(mul2(16.f, C));
-  acc.add(mul2(4.f, C));
-  acc.add(mul2(-8.f, E0)); acc.add(mul2(-8.f, E1)); acc.add(mul2(-8.f, N)); acc.add(mul2(-8.f, Sv));
-  acc.add(mul2(2.f, D0)); acc.add(mul2(2.f, D1)); acc.add(mul2(2.f, D2)); acc.add(mul2(2.f, D3));
-  acc.add(Cm); acc.add(Cp); acc.add(NN); acc.add(SS);
-  return acc;
+  const float2 C = ld2(h), Cm = ld2(h - 2), Cp = ld2(h + 2);
+  float2 a, ea, b, eb, t, et, s, es;
+  two_sum2(make_float2(Cm.y, C.x), make_float2(C.y, Cp.x), a, ea);
+  two_sum2(ld2(h - RS), ld2(h + RS), b, eb);
+  two_sum2(a, b, t, et);
+  two_sum2(t, mul2(-4.f, C), s, es);
+  float2 e = add2(es, add2(et, add2(ea, eb)));
+  if (LO) {
+    const float2 c = ld2(l), cm = ld2(l - 2), cp = ld2(l + 2);
+    const float2 n = add2(add2(make_float2(cm.y, c.x), make_float2(c.y, cp.x)), add2(ld2(l - RS), ld2(l + RS)));
+    e = add2(e, fma2(make_float2(-4.f, -4.f), c, n));
+  }
+  return {s, e};
 }
-// plain FP32 stencil of the lo plane at two adjacent nodes
-template <int RS>
-__device__ __forceinline__ float2 stencil13_pair_plain(const float* c) {
-  const float2 Cm = ld2(c - 2), C = ld2(c), Cp = ld2(c + 2);
-  const float2 Nm = ld2(c - RS - 2), N = ld2(c - RS), Np = ld2(c - RS + 2);
-  const float2 Sm = ld2(c + RS - 2), Sv = ld2(c + RS), Sp = ld2(c + RS + 2);
-  const float2 NN = ld2(c - 2 * RS), SS = ld2(c + 2 * RS);
-  const float2 E = add2(make_float2(Cm.y, C.x), make_float2(C.y, Cp.x));
-  const float2 D = add2(add2(make_float2(Nm.y, N.x), make_float2(N.y, Np.x)),
-                        add2(make_float2(Sm.y, Sv.x), make_float2(Sv.y, Sp.x)));
-  const float2 F = add2(add2(Cm, Cp), add2(NN, SS));
-  float2 v = mul2(20.f, C);
-  v = fma2(make_float2(-8.f, -8.f), add2(E, add2(N, Sv)), v);
-  v = fma2(make_float2(2.f, 2.f), D, v);
-  return add2(v, F);
+// The first application over a tile's nodes and their ring of one: rows 1 .. TY + 2 and columns
+// 2 .. 69 of the windows h, l into the same places of sh, sl.
+template <int TY, int RS, bool LO = true>
+__device__ __forceinline__ void lap_tile(const float* h, const float* l, float* sh, float* sl) {
+  constexpr int kPairs = kStTileX / 2 + 2;
+  for (int k = threadIdx.x; k < kPairs * (TY + 2); k += kStThreads) {
+    const int r = k / kPairs, c = (1 + r) * RS + 2 + 2 * (k - r * kPairs);
+    const f2x2 w = lap_pair<RS, LO>(h + c, l + c);
+    *reinterpret_cast<float2*>(sh + c) = w.hi;
+    *reinterpret_cast<float2*>(sl + c) = w.lo;
+  }
 }
 
 __device__ __forceinline__ double stencil13_f64(const SlotDesc& S, const double* t, int ly, int lx) {
@@ -318,8 +307,10 @@ k_stage_setup(const SlotDesc* __restrict__ slots, const float* __restrict__ phi,
 // double-float), q = M L^2 p (Algorithm 1, matvec, with the mask in the epilogue), and p.q as
 // partial sums over fixed 64 x 16 node blocks; k_pq_finish then forms alpha = rho / p.q.
 //
-// q is the double-float pair of the exact 13-point sum of p's hi plane (compensated FP32) plus
-// the same stencil of p's lo plane in plain FP32.
+// q is a double-float pair: on equal spacings the five-point g of p's pair taken twice (lap_pair: the
+// first application into the p_old windows, a barrier, the second at the tile's nodes; tiles with
+// no unknown node skip both), on unequal ones the exact 13-point sum of p's hi plane (compensated
+// FP32) plus the same stencil of its lo plane in plain FP32.
 //
 // Tiles are 64 nodes wide and TY rows high (TY = 16 or 32, chosen per workspace by the
 // autotuner).  Each block walks its share of the (slot, tile) list with two shared-memory window
@@ -433,6 +424,17 @@ __device__ __forceinline__ void stencil_issue_next(const SlotDesc* __restrict__ 
   }
 }
 
+// Whether any of the calling thread's share of a tile's mask bytes is set (all threads: the tile).
+template <int BYTES>
+__device__ __forceinline__ int mask_any(const unsigned char* m) {
+  static_assert(BYTES % (4 * kStThreads) == 0, "whole words per thread");
+  unsigned v = 0;
+#pragma unroll
+  for (int i = 0; i < BYTES / (4 * kStThreads); ++i)
+    v |= reinterpret_cast<const unsigned*>(m)[threadIdx.x + i * kStThreads];
+  return v != 0;
+}
+
 template <bool ANISO, int TY, bool FUSE>
 __global__ void __launch_bounds__(kStThreads, StGeom<TY>::kBlocksPerSm)
 k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
@@ -497,6 +499,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     // a tile whose halo lies inside the grid has no ghost cell
     const bool interior = x0 >= 2 && y0 >= 2 && x0 + kStTileX + 2 <= S.nx && y0 + TY + 2 <= S.ny;
     unsigned char* buf;
+    int unknown;  // whether the tile has an unknown node
     if (S.st_maps != nullptr) {
       const int b = n_used & 1;
       buf = sbuf + b * G::kBufBytes;
@@ -525,6 +528,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         }
       }
       mbar_wait(&full[b], (n_used >> 1) & 1, abort_flag, wait_cycles);
+      unknown = mask_any<G::kMaskBytes>(buf + 4 * G::kWinBytes);
       // p = z + beta p_old over the whole window, in place of z
       float4* zh = reinterpret_cast<float4*>(buf);
       float4* zl = reinterpret_cast<float4*>(buf + G::kWinBytes);
@@ -539,7 +543,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         zh[v] = make_float4(u.hi.x, u.hi.y, t.hi.x, t.hi.y);
         zl[v] = make_float4(u.lo.x, u.lo.y, t.lo.x, t.lo.y);
       }
-      __syncthreads();
+      unknown = __syncthreads_or(unknown);
       if (*abort_flag) break;  // every thread reads the flag after the barrier: uniform
       ++n_used;
       if (!interior) {
@@ -565,6 +569,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         const int gx = x0 + lx, gy = y0 + ly;
         mt[e] = (gx < S.nx && gy < S.ny) ? S.mask[gy * S.nx + gx] : 0;
       }
+      unknown = 1;
       constexpr int kChunk = 4;
 #pragma unroll 1
       for (int i0 = 0; i0 < G::kHalo; i0 += kChunk * kStThreads) {
@@ -607,6 +612,12 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     // warp its lanes in a fixed butterfly, and one thread the eight warps in order
     CompDotDF dot;
     if (!ANISO) {
+      float* sh = reinterpret_cast<float*>(buf + 2 * G::kWinBytes);  // g(p), in place of p_old
+      float* sl = reinterpret_cast<float*>(buf + 3 * G::kWinBytes);
+      if (unknown) {  // uniform
+        lap_tile<TY, kWX>(wh, wl, sh, sl);
+        __syncthreads();
+      }
       // node pairs (x, x+1): the window's row stride is even and x - x0 is even.  In step j the
       // warp covers one tile row; lanes 0-15 its first 32 nodes, lanes 16-31 the next 32.  Two
       // steps (eight rows each) make a 16-row block.
@@ -622,9 +633,8 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
           const unsigned m2 = *reinterpret_cast<const uint16_t*>(mt + ly * kStTileX + lx);
           f2x2 q2 = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
           if (m2) {
-            const CompSum2 a = stencil13_pair_acc<kWX>(wh + wc);
-            const float2 l = stencil13_pair_plain<kWX>(wl + wc);
-            q2 = df_norm2(a.s, add2(a.c, l));
+            const f2x2 a = lap_pair<kWX>(sh + wc, sl + wc);
+            q2 = df_norm2(a.hi, a.lo);
           }
           const bool m0 = (m2 & 0xffu) != 0, m1 = (m2 >> 8) != 0;
           const f2 q0 = m0 ? f2{q2.hi.x, q2.lo.x} : f2{0.f, 0.f};
@@ -673,8 +683,8 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
           const float pvh = wh[(ly + 2) * kWX + lx + 4], pvl = wl[(ly + 2) * kWX + lx + 4];
           f2 qv = {0.f, 0.f};
           if (mt[ly * kStTileX + lx]) {
-            const CompSum a = stencil13_acc<ANISO, kWX>(S, wh + 2, ly, lx);
-            const float l = stencil13_plain<ANISO, kWX>(S, wl + 2, ly, lx);
+            const CompSum a = stencil13_acc<kWX>(S, wh + 2, ly, lx);
+            const float l = stencil13_plain<kWX>(S, wl + 2, ly, lx);
             qv = df_norm(a.s, __fadd_rn(a.c, l));
           }
           pnew[g] = pvh;
@@ -964,6 +974,7 @@ k_apply(const __grid_constant__ SlotDesc S, const float* __restrict__ phi, int e
         const float* __restrict__ p, float* __restrict__ q, double* __restrict__ part) {
   constexpr int TY = kApplyTileY;
   __shared__ __align__(16) float win[kWX * (TY + 4)];  // rows y0-2 .., columns x0-4 ..
+  __shared__ __align__(16) float lap[ANISO ? 1 : 2][ANISO ? 4 : kWX * (TY + 4)];  // g(p), hi and lo
   __shared__ float2 red[kStThreads / 32];
   const int ntx = (S.nx + kStTileX - 1) / kStTileX;
   const int tile = blockIdx.x;
@@ -982,6 +993,10 @@ k_apply(const __grid_constant__ SlotDesc S, const float* __restrict__ phi, int e
     win[ly * kWX + lx + 2] = v;
   }
   __syncthreads();
+  if (!ANISO) {
+    lap_tile<TY, kWX, false>(win, nullptr, lap[0], lap[ANISO ? 0 : 1]);
+    __syncthreads();
+  }
   CompDot dot;
 #pragma unroll
   for (int k = threadIdx.x; k < kStTileX * TY / 2; k += kStThreads) {
@@ -996,11 +1011,12 @@ k_apply(const __grid_constant__ SlotDesc S, const float* __restrict__ phi, int e
     float2 r = make_float2(0.f, 0.f);
     if (u0 || u1) {
       if (!ANISO) {
-        const CompSum2 a = stencil13_pair_acc<kWX>(c);
-        r = a.result();
+        const int o = (ly + 2) * kWX + lx + 4;
+        const f2x2 a = lap_pair<kWX>(lap[0] + o, lap[ANISO ? 0 : 1] + o);
+        r = add2(a.hi, a.lo);
       } else {
-        r.x = stencil13_acc<true, kWX>(S, win + 2, ly, lx).result();
-        r.y = two ? stencil13_acc<true, kWX>(S, win + 2, ly, lx + 1).result() : 0.f;
+        r.x = stencil13_acc<kWX>(S, win + 2, ly, lx).result();
+        r.y = two ? stencil13_acc<kWX>(S, win + 2, ly, lx + 1).result() : 0.f;
       }
     }
     const float q0 = u0 ? r.x : 0.f, q1 = u1 ? r.y : 0.f;
