@@ -345,7 +345,7 @@ struct StGeom {
   static_assert(kWinBytes % 128 == 0 && kBufBytes % 128 == 0, "tensor copy destinations");
   static_assert(kGhostSlots <= 2 * kStThreads, "two ghost candidates per thread");
   static_assert(kOwn * kStThreads == kStTileX * TY && kOwn % 2 == 0, "tile / block size");
-  static_assert(kBlocksPerSm * (kSmemBytes + 1024) <= 228 * 1024, "window sets per SM");
+  static_assert(kBlocksPerSm * (kSmemBytes + 1280) <= 228 * 1024, "window sets per SM");
 };
 
 __device__ __forceinline__ void tile_origin_ty(const SlotDesc& S, int tile, int ty, int& x0, int& y0) {
@@ -391,36 +391,121 @@ __device__ __forceinline__ int halo_src_ty(const SlotDesc& S, int x0, int y0, in
   return my * S.nx + mx;
 }
 
-// Thread 0: start the tensor copies of the block's next copied tile (the next item at or after
-// w_issue whose slot iterates and has stencil maps) into window set n_issued % 2.
-template <int TY>
-__device__ __forceinline__ void stencil_issue_next(const SlotDesc* __restrict__ slots,
-                                                   const WorkItem* __restrict__ items, int total,
-                                                   unsigned char* sbuf, uint64_t* full,
-                                                   int& w_issue, int& n_issued) {
+// A tile as the block's producer warp hands it to the eight that compute: what they need of the item,
+// its slot and the slot's scalars, and whether its windows were copied.
+struct StTile {
+  const SlotDesc* S;  // null: the end of the list
+  int x0, y0, par, copied;
+  float beta_hi, beta_lo;
+};
+constexpr int kStBlock = kStThreads + 32;  // the computing warps and the producer
+
+__device__ __forceinline__ void st_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kStThreads) : "memory"); }
+// the same barrier, telling whether v is set in any of the computing threads
+__device__ __forceinline__ bool st_bar_or(bool v) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, 1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(any)
+      : "r"(v ? 1u : 0u), "n"(kStThreads)
+      : "memory");
+  return any != 0;
+}
+
+// The producer warp: for each of the block's tiles (those whose slot iterates) it waits for a free
+// window set, starts the tensor copies (lane 0), forms beta (FUSE: from the preconditioner's partials,
+// once per slot) and hands the tile over.  Done by a computing thread between two tiles, these dependent
+// loads, tensor-map fences and copies took 3.5 K of a tile's 11.5 K cycles.
+template <int TY, bool FUSE>
+__device__ __forceinline__ void stencil_producer(const SlotDesc* __restrict__ slots,
+                                                 const WorkItem* __restrict__ items, int total, unsigned char* sbuf,
+                                                 uint64_t* full, uint64_t* empty, StTile* info,
+                                                 volatile int* abort_flag, long long wait_cycles) {
   using G = StGeom<TY>;
-  while (w_issue < total) {
-    const WorkItem it = items[w_issue];
-    w_issue += gridDim.x;
+  const int lane = threadIdx.x & 31;
+  int n = 0, slot = -1;
+  f2 beta = {0.f, 0.f};
+  auto acquire = [&](const SlotDesc& S) {
+    if (lane < kStMaps && S.st_maps != nullptr)
+      tmap_acquire(static_cast<const unsigned char*>(S.st_maps) + 128 * lane);
+    __syncwarp();
+  };
+  if (static_cast<int>(blockIdx.x) < total) {  // what no kernel writes, before the wait
+    slot = items[blockIdx.x].slot;
+    acquire(slots[slot]);
+  }
+  int beta_slot = -1;
+  pdl_wait();
+  bool ok = true;
+  for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+    const WorkItem it = items[w];
     const SlotDesc& S = slots[it.slot];
-    if (S.st_maps == nullptr || !S.sc->active) continue;
+    SlotScalars* sc = S.sc;
+    if (!sc->active) continue;
+    if (it.slot != slot) {
+      slot = it.slot;
+      acquire(S);
+    }
+    const int b = n & 1, par = sc->it & 1;
     int x0, y0;
     tile_origin_ty(S, it.tile, TY, x0, y0);
     const unsigned char* maps = static_cast<const unsigned char*>(S.st_maps);
-    const int par = S.sc->it & 1;
-    const void* src[5] = {maps, maps + 128, maps + 128 * (2 + 2 * par), maps + 128 * (3 + 2 * par),
-                          maps + 128 * 6};
-#pragma unroll
-    for (int k = 0; k < 5; ++k) tmap_acquire(src[k]);
-    const int b = n_issued & 1;
-    unsigned char* dst = sbuf + b * G::kBufBytes;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(&full[b], G::kBufBytes);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) tma_load_2d(dst + k * G::kWinBytes, src[k], &full[b], x0 - 4, y0 - 2);
-    tma_load_2d(dst + 4 * G::kWinBytes, src[4], &full[b], x0, y0);
-    ++n_issued;
-    return;
+    if (lane == 0) {
+      ok = mbar_wait(&empty[b], ((n >> 1) & 1) ^ 1, abort_flag, wait_cycles);
+      if (ok && maps != nullptr) {
+        unsigned char* dst = sbuf + b * G::kBufBytes;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_expect_tx_only(&full[b], G::kBufBytes);
+        tma_load_2d(dst, maps, &full[b], x0 - 4, y0 - 2);
+        tma_load_2d(dst + G::kWinBytes, maps + 128, &full[b], x0 - 4, y0 - 2);
+        tma_load_2d(dst + 2 * G::kWinBytes, maps + 128 * (2 + 2 * par), &full[b], x0 - 4, y0 - 2);
+        tma_load_2d(dst + 3 * G::kWinBytes, maps + 128 * (3 + 2 * par), &full[b], x0 - 4, y0 - 2);
+        tma_load_2d(dst + 4 * G::kWinBytes, maps + 128 * 6, &full[b], x0, y0);
+      }
+    }
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    if (!ok) break;
+    if (it.slot != beta_slot) {
+      beta_slot = it.slot;
+      if (FUSE) {
+        // r.z, z.q -> beta in every block; the tile-0 block records the scalars.  A breakdown (a
+        // non-finite r.z or beta) reaches p.q and rho, where the update finds it.
+        double rz, zq;
+        sum_rz(S, sc->flexible != 0, rz, zq);
+        if (lane == 0) {
+          const double bd = prec_beta(sc, rz, zq);
+          beta = df_of(bd);
+          if (it.tile == 0) record_preconditioner(sc, rz, zq, bd);
+        }
+      } else {
+        beta = f2{sc->beta_f[0], sc->beta_f[1]};
+      }
+    }
+    if (lane == 0) {
+      info[b] = StTile{&S, x0, y0, par, maps != nullptr, beta.hi, beta.lo};
+      mbar_arrive(&full[b]);
+    }
+    ++n;
+  }
+  if (lane == 0) {
+    if (ok && mbar_wait(&empty[n & 1], ((n >> 1) & 1) ^ 1, abort_flag, wait_cycles)) {
+      info[n & 1].S = nullptr;
+      mbar_arrive(&full[n & 1]);
+    }
+    // after an abort: the copies already issued (the last into each set) land before the block's
+    // memory is released
+    if (*abort_flag) {
+      const long long t0 = clock64();
+      for (int b = 0; b < 2; ++b) {
+        const int k = (n - b + 1) / 2;  // tiles handed over in set b
+        if (k > 0)
+          while (!mbar_try(&full[b], (k - 1) & 1) && clock64() - t0 < kWaitCycles / 4) {
+          }
+      }
+    }
   }
 }
 
@@ -436,77 +521,54 @@ __device__ __forceinline__ int mask_any(const unsigned char* m) {
 }
 
 template <bool ANISO, int TY, bool FUSE>
-__global__ void __launch_bounds__(kStThreads, StGeom<TY>::kBlocksPerSm)
+__global__ void __launch_bounds__(kStBlock, StGeom<TY>::kBlocksPerSm)
 k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
           const int* __restrict__ n_items, int* __restrict__ err, long long wait_cycles) {
   using G = StGeom<TY>;
   extern __shared__ unsigned char st_smem_raw[];
   unsigned char* sbuf = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(st_smem_raw) + 127) & ~static_cast<uintptr_t>(127));
-  __shared__ __align__(8) uint64_t full[2];
+  __shared__ __align__(8) uint64_t full[2], empty[2];
+  __shared__ StTile info[2];
   __shared__ int s_abort;
   __shared__ float2 blk_sm[TY / 16][kStThreads / 32];  // p.q of each warp in each 16-row block
-  __shared__ float2 s_beta;                            // FUSE: beta of slot beta_slot
-  int beta_slot = -1;
-  f2 beta_fused = {0.f, 0.f};
   const int total = *n_items;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
-    mbar_init(&full[0], 1);
-    mbar_init(&full[1], 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&full[b], 1);
+      mbar_init(&empty[b], 1);
+    }
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
-  pdl_wait();
   volatile int* abort_flag = &s_abort;
-  int w_issue = blockIdx.x, n_issued = 0;  // thread 0: the tensor-copy cursor
-  int n_used = 0;                          // copied windows consumed (uniform over the block)
-  if (threadIdx.x == 0) stencil_issue_next<TY>(slots, items, total, sbuf, full, w_issue, n_issued);
-  for (int w = blockIdx.x; w < total; w += gridDim.x) {
-    const WorkItem it = items[w];
-    const SlotDesc& S = slots[it.slot];
-    SlotScalars* sc = S.sc;
-    if (!sc->active) continue;
-    if (FUSE && it.slot != beta_slot) {
-      // r.z, z.q -> beta in this block; the tile-0 block records the scalars.  A breakdown (a
-      // non-finite r.z or beta) reaches p.q and rho, where the update finds it.
-      if (threadIdx.x < 32) {
-        double rz, zq;
-        sum_rz(S, sc->flexible != 0, rz, zq);
-        if (threadIdx.x == 0) {
-          const double b = prec_beta(sc, rz, zq);
-          const f2 bf = df_of(b);
-          s_beta = make_float2(bf.hi, bf.lo);
-          if (it.tile == 0) record_preconditioner(sc, rz, zq, b);
-        }
-      }
-      __syncthreads();
-      beta_fused = f2{s_beta.x, s_beta.y};
-      beta_slot = it.slot;
-    }
-    const f2 beta = FUSE ? beta_fused : f2{sc->beta_f[0], sc->beta_f[1]};
-    const int par = sc->it & 1;
+  if (warp == kStThreads / 32) {
+    stencil_producer<TY, FUSE>(slots, items, total, sbuf, full, empty, info, abort_flag, wait_cycles);
+  } else {
+  pdl_wait();
+  for (int n = 0;; ++n) {
+    const int b = n & 1;
+    if (st_bar_or(!mbar_wait(&full[b], (n >> 1) & 1, abort_flag, wait_cycles))) break;
+    const StTile tile = info[b];
+    if (tile.S == nullptr) break;
+    const SlotDesc& S = *tile.S;
+    const f2 beta = {tile.beta_hi, tile.beta_lo};
+    const int par = tile.par, x0 = tile.x0, y0 = tile.y0;
     const float* __restrict__ pold = S.p[par];
     const float* __restrict__ pold_lo = S.p_lo[par];
     float* __restrict__ pnew = S.p[par ^ 1];
     float* __restrict__ pnew_lo = S.p_lo[par ^ 1];
     const float* __restrict__ z = S.z;
     const float* __restrict__ z_lo = S.z_lo;
-    int x0, y0;
-    tile_origin_ty(S, it.tile, TY, x0, y0);
     // a tile whose halo lies inside the grid has no ghost cell
     const bool interior = x0 >= 2 && y0 >= 2 && x0 + kStTileX + 2 <= S.nx && y0 + TY + 2 <= S.ny;
-    unsigned char* buf;
-    int unknown;  // whether the tile has an unknown node
-    if (S.st_maps != nullptr) {
-      const int b = n_used & 1;
-      buf = sbuf + b * G::kBufBytes;
-      // the other window set finished with the previous tile: start the next tile's copies
-      if (threadIdx.x == 0 && n_issued == n_used + 1)
-        stencil_issue_next<TY>(slots, items, total, sbuf, full, w_issue, n_issued);
-      // ghost cells by plain loads, issued before the wait so that both latencies overlap
+    unsigned char* buf = sbuf + b * G::kBufBytes;
+    bool unknown;  // whether the tile has an unknown node
+    if (tile.copied) {
+      // ghost cells by plain loads, whose latency passes under the window's p
       int gcell[2] = {-1, -1};
       float gs[2] = {0.f, 0.f};
       f2 gz[2] = {{0.f, 0.f}, {0.f, 0.f}}, gp[2] = {{0.f, 0.f}, {0.f, 0.f}};
@@ -527,7 +589,6 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
           }
         }
       }
-      mbar_wait(&full[b], (n_used >> 1) & 1, abort_flag, wait_cycles);
       unknown = mask_any<G::kMaskBytes>(buf + 4 * G::kWinBytes);
       // p = z + beta p_old over the whole window, in place of z
       float4* zh = reinterpret_cast<float4*>(buf);
@@ -543,9 +604,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         zh[v] = make_float4(u.hi.x, u.hi.y, t.hi.x, t.hi.y);
         zl[v] = make_float4(u.lo.x, u.lo.y, t.lo.x, t.lo.y);
       }
-      unknown = __syncthreads_or(unknown);
-      if (*abort_flag) break;  // every thread reads the flag after the barrier: uniform
-      ++n_used;
+      unknown = st_bar_or(unknown);
       if (!interior) {
         float* wh = reinterpret_cast<float*>(buf);
         float* wl = reinterpret_cast<float*>(buf + G::kWinBytes);
@@ -556,11 +615,10 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
             wh[gcell[h]] = gs[h] * v.hi;
             wl[gcell[h]] = gs[h] * v.lo;
           }
-        __syncthreads();
+        st_bar();
       }
     } else {
-      // plain loads into the free window set, kChunk cells per thread in flight at a time
-      buf = sbuf + ((n_used + 1) & 1) * G::kBufBytes;
+      // plain loads into the window set, kChunk cells per thread in flight at a time
       float* wh = reinterpret_cast<float*>(buf);
       float* wl = reinterpret_cast<float*>(buf + G::kWinBytes);
       uint8_t* mt = buf + 4 * G::kWinBytes;
@@ -569,7 +627,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         const int gx = x0 + lx, gy = y0 + ly;
         mt[e] = (gx < S.nx && gy < S.ny) ? S.mask[gy * S.nx + gx] : 0;
       }
-      unknown = 1;
+      unknown = true;
       constexpr int kChunk = 4;
 #pragma unroll 1
       for (int i0 = 0; i0 < G::kHalo; i0 += kChunk * kStThreads) {
@@ -600,7 +658,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
           }
         }
       }
-      __syncthreads();
+      st_bar();
     }
     const float* wh = reinterpret_cast<const float*>(buf);
     const float* wl = reinterpret_cast<const float*>(buf + G::kWinBytes);
@@ -616,59 +674,57 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
       float* sl = reinterpret_cast<float*>(buf + 3 * G::kWinBytes);
       if (unknown) {  // uniform
         lap_tile<TY, kWX>(wh, wl, sh, sl);
-        __syncthreads();
+        st_bar();
       }
-      // node pairs (x, x+1): the window's row stride is even and x - x0 is even.  In step j the
-      // warp covers one tile row; lanes 0-15 its first 32 nodes, lanes 16-31 the next 32.  Two
-      // steps (eight rows each) make a 16-row block.
+      // node pairs (x, x+1): the window's row stride is even and x - x0 is even.  In a step the warp
+      // covers one tile row; two steps (eight rows each) make a 16-row block, unrolled so that their
+      // dependent chains overlap.
+      const int gx = x0 + 2 * lane;
+      const bool in0 = gx < S.nx, in1 = gx + 1 < S.nx;
+      const int nx = S.nx, rows = S.ny - y0;
+      const int wc0 = (warp + 2) * kWX + 2 * lane + 4;
 #pragma unroll 1
-      for (int j = 0; j < G::kOwn / 2; ++j) {
-        const int k = threadIdx.x + j * kStThreads;
-        const int ly = k / (kStTileX / 2), lx = 2 * (k - ly * (kStTileX / 2));
-        const int gx = x0 + lx, gy = y0 + ly;
-        if (gx < S.nx && gy < S.ny) {
-          const int g = gy * S.nx + gx;
-          const int wc = (ly + 2) * kWX + lx + 4;
+      for (int j = 0; j < TY / 16; ++j) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int ly = warp + 8 * (2 * j + h);
+          if (ly >= rows || !in0) continue;
+          const int g = (y0 + ly) * nx + gx;
+          const int wc = wc0 + 8 * (2 * j + h) * kWX;
           const float2 pvh = ld2(wh + wc), pvl = ld2(wl + wc);
-          const unsigned m2 = *reinterpret_cast<const uint16_t*>(mt + ly * kStTileX + lx);
+          const unsigned m2 = *reinterpret_cast<const uint16_t*>(mt + ly * kStTileX + 2 * lane);
           f2x2 q2 = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
           if (m2) {
             const f2x2 a = lap_pair<kWX>(sh + wc, sl + wc);
             q2 = df_norm2(a.hi, a.lo);
           }
           const bool m0 = (m2 & 0xffu) != 0, m1 = (m2 >> 8) != 0;
-          const f2 q0 = m0 ? f2{q2.hi.x, q2.lo.x} : f2{0.f, 0.f};
-          const f2 q1 = m1 ? f2{q2.hi.y, q2.lo.y} : f2{0.f, 0.f};
-          dot.add(pvh.x, pvl.x, q0.hi, q0.lo);
-          if (gx + 1 < S.nx) {
-            dot.add(pvh.y, pvl.y, q1.hi, q1.lo);
-            if ((g & 1) == 0) {
-              *reinterpret_cast<float2*>(pnew + g) = pvh;
-              *reinterpret_cast<float2*>(pnew_lo + g) = pvl;
-              *reinterpret_cast<float2*>(qh + g) = make_float2(q0.hi, q1.hi);
-              *reinterpret_cast<float2*>(ql + g) = make_float2(q0.lo, q1.lo);
-            } else {
-              pnew[g] = pvh.x;
-              pnew[g + 1] = pvh.y;
-              pnew_lo[g] = pvl.x;
-              pnew_lo[g + 1] = pvl.y;
-              qh[g] = q0.hi;
-              qh[g + 1] = q1.hi;
-              ql[g] = q0.lo;
-              ql[g + 1] = q1.lo;
-            }
+          q2.hi = make_float2(m0 ? q2.hi.x : 0.f, m1 ? q2.hi.y : 0.f);
+          q2.lo = make_float2(m0 ? q2.lo.x : 0.f, m1 ? q2.lo.y : 0.f);
+          if (m0) dot.add(pvh.x, pvl.x, q2.hi.x, q2.lo.x);
+          if (in1 && m1) dot.add(pvh.y, pvl.y, q2.hi.y, q2.lo.y);
+          if (in1 && (g & 1) == 0) {
+            *reinterpret_cast<float2*>(pnew + g) = pvh;
+            *reinterpret_cast<float2*>(pnew_lo + g) = pvl;
+            *reinterpret_cast<float2*>(qh + g) = q2.hi;
+            *reinterpret_cast<float2*>(ql + g) = q2.lo;
           } else {
             pnew[g] = pvh.x;
             pnew_lo[g] = pvl.x;
-            qh[g] = q0.hi;
-            ql[g] = q0.lo;
+            qh[g] = q2.hi.x;
+            ql[g] = q2.lo.x;
+            if (in1) {
+              pnew[g + 1] = pvh.y;
+              pnew_lo[g + 1] = pvl.y;
+              qh[g + 1] = q2.hi.y;
+              ql[g + 1] = q2.lo.y;
+            }
           }
         }
-        if (j & 1) {  // the end of a 16-row block: every lane joins the butterfly
-          group_sum_pair<32>(dot.s, dot.c);
-          if (lane == 0) blk_sm[j >> 1][threadIdx.x >> 5] = make_float2(dot.s, dot.c);
-          dot = CompDotDF{};
-        }
+        // the end of a 16-row block: every lane joins the butterfly
+        group_sum_pair<32>(dot.s, dot.c);
+        if (lane == 0) blk_sm[j][warp] = make_float2(dot.s, dot.c);
+        dot = CompDotDF{};
       }
     } else {
       // one node per lane; in step j the warp covers 32 consecutive nodes of one tile row; four
@@ -700,7 +756,8 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         }
       }
     }
-    __syncthreads();  // the window set is free for the copies started at the next copied tile
+    st_bar();
+    if (threadIdx.x == 0) mbar_arrive(&empty[b]);  // the window set and the tile's entry are free
     // the 16-row blocks of the tile (TY / 16 of them, so the partials do not depend on TY); the
     // next tile writes blk_sm only after its own block barriers, which these threads join later
     if (threadIdx.x < 32) {
@@ -713,15 +770,9 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         S.pq_part[by * nbx + x0 / kStTileX] = (double)sv + (double)cv;
     }
   }
-  if (threadIdx.x == 0) {
-    // copies still in flight (only after an abort) land before the block's memory is released
-    for (int o = n_used; o < n_issued; ++o) {
-      const long long t0 = clock64();
-      while (!mbar_try(&full[o & 1], (o >> 1) & 1) && clock64() - t0 < kWaitCycles / 4) {
-      }
-    }
-    if (s_abort) atomicExch(err, 1);
   }
+  __syncthreads();
+  if (threadIdx.x == 0 && s_abort) atomicExch(err, 1);
 }
 
 // One block per slot (the slot's tile-0 item of the per-slot list): p.q from the stencil's
@@ -1050,9 +1101,9 @@ template <int TY, bool FUSE>
 static void launch_stencil_ty(const LaunchCfg& c, bool aniso, int* err, long long wc) {
   constexpr int smem = StGeom<TY>::kSmemBytes;
   if (aniso)
-    launch_cfg(c, k_stencil<true, TY, FUSE>, c.grid, kStThreads, smem, c.slots, c.items, c.n_items, err, wc);
+    launch_cfg(c, k_stencil<true, TY, FUSE>, c.grid, kStBlock, smem, c.slots, c.items, c.n_items, err, wc);
   else
-    launch_cfg(c, k_stencil<false, TY, FUSE>, c.grid, kStThreads, smem, c.slots, c.items, c.n_items, err, wc);
+    launch_cfg(c, k_stencil<false, TY, FUSE>, c.grid, kStBlock, smem, c.slots, c.items, c.n_items, err, wc);
 }
 void launch_stencil(const LaunchCfg& c, bool aniso, int tile_y, int* err, bool fuse_prec) {
   const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
