@@ -90,7 +90,7 @@ struct Workspace {
   std::vector<SlotHost> slots;
   SlotDesc* d_slots = nullptr;
   SlotScalars* d_sc = nullptr;
-  SlotScalars* h_sc = nullptr;  // pinned
+  SlotScalars* h_sc = nullptr;  // pinned; solve workspaces: two sets, one per block of iterations in flight
   WorkItem *d_st = nullptr, *d_vec = nullptr;
   WorkItem* d_gm[2] = {nullptr, nullptr};  // transform tiles of the problems with four, six slices
   WorkItem* d_sl = nullptr;     // one item per slot (tile 0), for the per-slot scalar kernels
@@ -156,7 +156,8 @@ struct ext_ctx {
                       // build_slot may give a grid 6
   int split = 0;      // their type: 0 = FP16, 1 = BF16
   int* d_err = nullptr;   // device flag raised by a bounded wait that ran out
-  int* h_err = nullptr;   // pinned copy
+  int* h_err = nullptr;   // pinned copies, two
+  cudaEvent_t blk_ev[2] = {nullptr, nullptr};  // the ends of a solve's blocks of iterations
   SlotScalars* h_sc3 = nullptr;  // pinned, two entries (3-D solves)
   // launch accounting and optional per-kernel timing (ext_options.profile)
   std::atomic<int64_t> launches{0};
@@ -906,7 +907,7 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   for (int k = 0; k < 2; ++k) W->n_gm[k] = (int)gm[k].size();
   BX_CUDA(cudaMalloc(&W->d_sc, sizeof(SlotScalars) * count));
   BX_CUDA(cudaMemset(W->d_sc, 0, sizeof(SlotScalars) * count));
-  BX_CUDA(cudaMallocHost(&W->h_sc, sizeof(SlotScalars) * count));
+  BX_CUDA(cudaMallocHost(&W->h_sc, 2 * sizeof(SlotScalars) * count));
   for (int i = 0; i < count; ++i) set_slot_scalars(W->slots[i], W->d_sc + i);
   std::vector<SlotDesc> descs(count), tcps(kMirClasses * count);
   for (int i = 0; i < count; ++i) {
@@ -1377,23 +1378,36 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
     max_blocks = std::max(max_blocks, mi);
   }
   max_blocks = max_blocks / std::max(1, ctx->opt.iters_per_launch) + 8;
+  // The host stays one block ahead: block k + 1 is launched before the scalars that block k left are
+  // read, so the device never waits for the host; with nothing left to do a block passes by the slots'
+  // flags.  (A profiled solve reads each block's events before the next one records over them.)
+  const int ahead = ctx->opt.profile ? 0 : 1;
+  const SlotScalars* end = W->h_sc;  // the scalars last read
   for (int blk = 0; blk < max_blocks; ++blk) {
     BX_CUDA(cudaGraphLaunch(graph.exec, s));
     ctx->launches += graph.nodes;
-    BX_CUDA(cudaMemcpyAsync(W->h_sc, W->d_sc, sizeof(SlotScalars) * count, cudaMemcpyDeviceToHost, s));
-    BX_CUDA(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BX_CUDA(cudaStreamSynchronize(s));
-    harvest(ctx);
-    if (ctx->opt.profile) harvest_graph(ctx, W->graph_events);
-    if (*ctx->h_err) {
+    BX_CUDA(cudaMemcpyAsync(W->h_sc + (blk & 1) * count, W->d_sc, sizeof(SlotScalars) * count, cudaMemcpyDeviceToHost, s));
+    BX_CUDA(cudaMemcpyAsync(ctx->h_err + (blk & 1), ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    BX_CUDA(cudaEventRecord(ctx->blk_ev[blk & 1], s));
+    if (blk < ahead && blk + 1 < max_blocks) continue;
+    const int seen = (blk & 1) ^ ahead;
+    BX_CUDA(cudaEventSynchronize(ctx->blk_ev[seen]));
+    if (ctx->opt.profile) {
+      BX_CUDA(cudaStreamSynchronize(s));
+      harvest(ctx);
+      harvest_graph(ctx, W->graph_events);
+    }
+    if (ctx->h_err[seen]) {
+      BX_CUDA(cudaStreamSynchronize(s));
       BX_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), s));
       BX_CUDA(cudaStreamSynchronize(s));
       g_last_error = "a bounded device wait (tensor copy or tensor-core pipeline) ran out";
       return EXT_ETIMEOUT;
     }
+    end = W->h_sc + seen * count;
     bool running = false;
     for (int i = 0; i < count; ++i)
-      if (W->h_sc[i].status == ST_RUNNING) running = true;
+      if (end[i].status == ST_RUNNING) running = true;
     if (!running) break;
   }
   if (out64) {
@@ -1418,7 +1432,7 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
       std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   int worst = EXT_OK;
   for (int i = 0; i < count; ++i) {
-    const SlotScalars& sc = W->h_sc[i];
+    const SlotScalars& sc = end[i];
     const ext_problem& p = W->slots[i].prob;
     int st = sc.status == ST_RUNNING ? EXT_ETIMEOUT : map_status(sc.status, sc.n_known, p);
     if (results) {
@@ -1538,8 +1552,9 @@ int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out) {
   BX_CUDA(stencil_init());
   BX_CUDA(cudaMalloc(&ctx->d_err, sizeof(int)));
   BX_CUDA(cudaMemset(ctx->d_err, 0, sizeof(int)));
-  BX_CUDA(cudaMallocHost(&ctx->h_err, sizeof(int)));
-  *ctx->h_err = 0;
+  BX_CUDA(cudaMallocHost(&ctx->h_err, 2 * sizeof(int)));
+  for (cudaEvent_t& e : ctx->blk_ev) BX_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  ctx->h_err[0] = ctx->h_err[1] = 0;
   BX_CUDA(cudaMallocHost(&ctx->h_sc3, 2 * sizeof(SlotScalars)));
   if (cuda_stream) {
     ctx->stream = (cudaStream_t)cuda_stream;
@@ -1568,6 +1583,8 @@ void ext_destroy(ext_ctx* ctx) {
   harvest(ctx);
   cudaFree(ctx->d_err);
   cudaFreeHost(ctx->h_err);
+  for (cudaEvent_t e : ctx->blk_ev)
+    if (e) cudaEventDestroy(e);
   cudaFreeHost(ctx->h_sc3);
   for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
   if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
