@@ -99,11 +99,14 @@ struct TcGeom {
   static constexpr int kEpiCols = 8 * kCb;        // tile columns per epilogue warp
   static constexpr int kBPlane = BN * BK * 2;
   static constexpr int kStageBytes = NSL * (A_PLANE + kBPlane);  // one step of both operands
-  // staging of the epilogue: the outgoing slices [slice][64-row half][column] as 128-byte rows; the
-  // forward low-mode product's H tile and Qy rows; nothing for the inverse one
-  static constexpr int kStage = STAGE == kLowInv ? 0 : STAGE == kLowFwd ? 8 * BM * 33 + 8 * BM * kLowM
-                                                                       : NSL * 32 * BM * 2;
-  static constexpr int kSteps = STAGE == kLowInv ? 3 : 2;
+  // staging of the epilogue: a group of the outgoing slices [slice][64-row half][column] as 128-byte
+  // rows (six slices leave in two groups, which makes room for a third step in flight: with two, a
+  // 32-deep step waited for its copies); the forward low-mode product's H tile and Qy rows; nothing
+  // where the results go straight to memory
+  static constexpr int kGroup = NSL == 4 ? 4 : 3;
+  static constexpr int kStage = STAGE == kLowFwd ? 8 * BM * 33 + 8 * BM * kLowM
+                                                 : STAGE <= 2 ? kGroup * 32 * BM * 2 : 0;
+  static constexpr int kSteps = NSL == 6 && STAGE != kLowFwd ? 3 : 2;
   static constexpr int kSetCols = NSL * BN;       // one accumulator per slice order
   static constexpr int kSmem = kSteps * kStageBytes + kStage + 1024 + 2048;
   static_assert(!kLow || NSL == kLowNS, "six slices in the low-mode products");
@@ -763,25 +766,28 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
           uint32_t code[4][NSL];
 #pragma unroll
           for (int rb = 0; rb < 4; ++rb) slice_codes2_df<BF16, NSL>(hi[cb][rb], lo[cb][rb], up, dn, code[rb]);
-          if (cb > 0) {
-            // the previous column block's stores have read the staging tile
-            if (ew == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+#pragma unroll
+          for (int q0 = 0; q0 < NSL; q0 += G::kGroup) {
+            if (cb > 0 || q0 > 0) {
+              // the previous group's stores have read the staging tile
+              if (ew == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+              epi_bar();
+            }
+#pragma unroll
+            for (int q = 0; q < G::kGroup; ++q) {
+              const uint32_t f[4] = {code[0][q0 + q], code[1][q0 + q], code[2][q0 + q], code[3][q0 + q]};
+              stmatrix4_t(so + (q * 2 * 32 << 7), f);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             epi_bar();
-          }
+            if (ew == 0 && lane == 0) {
 #pragma unroll
-          for (int q = 0; q < NSL; ++q) {
-            const uint32_t f[4] = {code[0][q], code[1][q], code[2][q], code[3][q]};
-            stmatrix4_t(so + (q * 2 * 32 << 7), f);
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          epi_bar();
-          if (ew == 0 && lane == 0) {
+              for (int q = 0; q < G::kGroup; ++q)
 #pragma unroll
-            for (int q = 0; q < NSL; ++q)
-#pragma unroll
-              for (int h = 0; h < 2; ++h)
-                tma_store_2d(mo, smem_u32(sO) + ((q * 2 + h) * 32 << 7), m0 + 64 * h, q * v.N + n0 + 32 * cb);
-            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                for (int h = 0; h < 2; ++h)
+                  tma_store_2d(mo, smem_u32(sO) + ((q * 2 + h) * 32 << 7), m0 + 64 * h, (q0 + q) * v.N + n0 + 32 * cb);
+              asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
           }
         }
         if (quarter == 0 && col_lane)
@@ -993,14 +999,41 @@ k_tc_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
           const WorkItem* __restrict__ items, const int* __restrict__ n_items, int mode) {
   const int total = *n_items;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // The item, its slot and its classes' operands.  The first item's are read before the wait for
+  // the previous kernel (no kernel writes them), the others' ahead of the residual's loads: read where
+  // the slices are stored, they were four dependent misses in a row.
+  // The classes of a slot have equal sizes and lie at equal distances in its arena.
+  struct Fold {
+    const SlotDesc* S = nullptr;
+    int tile = 0;
+    char *out = nullptr, *e = nullptr;  // class 0's operand and exponents
+    ptrdiff_t step = 0;                 // bytes from one class to the next
+    int nxp = 0, nyp = 0, nr = 4;
+  };
+  auto item = [&](int w) {
+    Fold t;
+    const WorkItem it = items[w];
+    t.S = slots + it.slot;
+    t.tile = it.tile;
+    const SlotDesc &T = tcp[kMirClasses * it.slot], &U = tcp[kMirClasses * it.slot + ((t.S->mir & 1) ? 1 : 2)];
+    t.out = static_cast<char*>(T.tc_r);
+    t.e = reinterpret_cast<char*>(T.tc_e[0]);
+    t.step = static_cast<char*>(U.tc_r) - t.out;
+    t.nxp = T.nxp;
+    t.nyp = T.nyp;
+    t.nr = T.tc_nr;
+    return t;
+  };
+  Fold t;
+  if (static_cast<int>(blockIdx.x) < total) t = item(blockIdx.x);
   pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
-    const WorkItem it = items[w];
-    const SlotDesc& S = slots[it.slot];
+    if (w != static_cast<int>(blockIdx.x)) t = item(w);
+    const SlotDesc& S = *t.S;
     if (!slot_runs(S.sc, mode)) continue;
     const bool fx = (S.mir & 1) != 0, fy = (S.mir & 2) != 0;
     const int nxb = (S.mhx + KC - 1) / KC;
-    const int y = (it.tile / nxb) * 8 + warp, xb = it.tile % nxb;
+    const int y = (t.tile / nxb) * 8 + warp, xb = t.tile % nxb;
     if (y >= S.mhy) continue;
     const int yy = fy ? S.ny - 1 - y : y;  // the mirrored row (y itself on an unfolded axis)
     const bool ymid = yy == y;
@@ -1053,18 +1086,18 @@ k_tc_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
     for (int c = 0; c < 4; ++c) {
       if ((c & 1) && !fx) continue;
       if ((c & 2) && !fy) continue;
-      const SlotDesc& T = tcp[kMirClasses * it.slot + c];
       float amax = 0.f;
 #pragma unroll
       for (int k = 0; k < 2; ++k) amax = fmaxf(amax, fmaxf(fabsf(ch[c][k].x), fabsf(ch[c][k].y)));
       const int E = block_exp(warp_max(amax));
       const float up = pow2f(16 - E), is = -pow2f(E - 16);
-      const size_t plane = static_cast<size_t>(T.nyp) * T.nxp;
-      uint32_t* out32 = static_cast<uint32_t*>(T.tc_r);
+      const size_t plane = static_cast<size_t>(t.nyp) * t.nxp;
+      const ptrdiff_t off = t.step * (fx ? c : c >> 1);
+      uint32_t* out32 = reinterpret_cast<uint32_t*>(t.out + off);
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const size_t idx = (static_cast<size_t>(y) * T.nxp + xb * KC + 64 * k + 2 * lane) / 2;
-        if (T.tc_nr == kLowNS) {
+        const size_t idx = (static_cast<size_t>(y) * t.nxp + xb * KC + 64 * k + 2 * lane) / 2;
+        if (t.nr == kLowNS) {
           uint32_t code[kLowNS];
           slice_codes2_df<BF16, kLowNS>(ch[c][k], cl[c][k], make_float2(up, up), make_float2(is, is), code);
 #pragma unroll
@@ -1076,7 +1109,7 @@ k_tc_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
           for (int q = 0; q < 4; ++q) out32[q * (plane / 2) + idx] = code[q];
         }
       }
-      if (lane == 0) T.tc_e[0][static_cast<size_t>(y) * (T.nxp / KC) + xb] = static_cast<int8_t>(E);
+      if (lane == 0) t.e[off + static_cast<ptrdiff_t>(y) * (t.nxp / KC) + xb] = static_cast<int8_t>(E);
     }
   }
 }

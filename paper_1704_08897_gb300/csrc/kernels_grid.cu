@@ -618,7 +618,8 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         st_bar();
       }
     } else {
-      // plain loads into the window set, kChunk cells per thread in flight at a time
+      // plain loads into the window set, kChunk cells per thread in flight at a time (a round is one
+      // memory latency)
       float* wh = reinterpret_cast<float*>(buf);
       float* wl = reinterpret_cast<float*>(buf + G::kWinBytes);
       uint8_t* mt = buf + 4 * G::kWinBytes;
@@ -628,7 +629,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         mt[e] = (gx < S.nx && gy < S.ny) ? S.mask[gy * S.nx + gx] : 0;
       }
       unknown = true;
-      constexpr int kChunk = 4;
+      constexpr int kChunk = TY == 16 ? 6 : 5;  // one round of loads or two
 #pragma unroll 1
       for (int i0 = 0; i0 < G::kHalo; i0 += kChunk * kStThreads) {
         int gi[kChunk];
