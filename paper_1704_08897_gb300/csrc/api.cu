@@ -554,7 +554,12 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   d.tc_ns = NS;
   d.vec_chunk = vec_chunk_of((long long)N);
   d.n_vec_items = (int)((N + d.vec_chunk - 1) / d.vec_chunk);
-  const int n_gm = (d.nxp / 128) * (d.nyp / bn);
+  // output tiles of a stage: 128 rows by bn columns, without those that hold only padding (the list
+  // is the longer of the two orientations; the kernel passes over the other's surplus)
+  auto gm_tiles = [bn](const SlotDesc& t) {
+    return std::max((t.nxp / 128) * ((t.ny + bn - 1) / bn), (t.nyp / 128) * ((t.nx + bn - 1) / bn));
+  };
+  const int n_gm = gm_tiles(d);
   d.n_gm_tiles = n_gm;
   set_weights(d, prob.hx, prob.hy);
   // the tensor-core transforms fold an axis by its mirror symmetry where both classes, padded,
@@ -570,7 +575,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   d.n_fold_items = !d.mir ? 0 : ((d.mhy + 7) / 8) * ((d.mhx + 127) / 128);
   d.n_prep_items = !d.mir ? ((ny + kStTileY - 1) / kStTileY) * ((nx + 127) / 128) : 0;
   d.n_unfold_tiles = d.mir ? ((d.mhx + 31) / 32) * ((d.mhy + 7) / 8) : 0;
-  d.n_prec_parts = d.mir ? d.n_unfold_tiles : n_gm;
+  d.n_prec_parts = d.mir ? d.n_unfold_tiles : (d.nxp / 128) * ((ny + bn - 1) / bn);
   const int n_part = std::max(std::max(d.n_st_tiles, d.n_vec_items), std::max(n_gm, d.n_unfold_tiles));
   // arena layout
   size_t off = 0;
@@ -711,7 +716,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
       t.ny = qy->n;
       t.nxp = qx->np;
       t.nyp = qy->np;
-      t.n_gm_tiles = (t.nxp / 128) * (t.nyp / bn);
+      t.n_gm_tiles = gm_tiles(t);
       t.mir = 0;
       t.mir_out = 1;
       // only the transform fields are live: grid vectors of the slot stay out of reach
@@ -744,7 +749,8 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
     t.tc_eb[1] = plan_exps(qy, NS, 1);  // Qy^T rows
     t.tc_eb[2] = plan_exps(qx, NS, 0);  // Qx rows
     t.tc_eb[3] = plan_exps(qy, NS, 0);  // Qy rows
-    BX_CUDA(cudaMemset(t.tc_r, 0, 2 * nr * Npc));
+    // the operands' padding is never written: zero it once (T1..T3 follow the residual in the arena)
+    BX_CUDA(cudaMemset(t.tc_r, 0, L.o_tt3 + 2 * NS * Npc - L.o_tr));
     BX_CUDA(cudaMemset(A + L.o_ex, 0, 4 * nex));
     CUtensorMap maps[kTcMaps];
     const size_t pxp = (size_t)t.nxp * t.nxp, pyp = (size_t)t.nyp * t.nyp;
@@ -782,7 +788,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
       t.low_qy_e = (const int8_t*)(lyp + qy->low_off_qe);
       t.n_l1_tiles = t.nyp / 128;
       t.n_l2_tiles = t.nxp / 32;
-      t.n_l3_tiles = (t.nxp / 128) * (t.nyp / 32);
+      t.n_l3_tiles = (t.nxp / 128) * ((t.ny + 31) / 32);
       CUtensorMap lm[4];
       int rc4 = make_tmap(&lm[0], t.tc_r, bf, t.nxp, (uint64_t)kLowNS * t.nyp, 128, 32);
       if (!rc4) rc4 = make_tmap(&lm[1], qx->low, bf, t.nxp, (uint64_t)kLowNS * kLowM, kLowM, 32);
@@ -855,7 +861,7 @@ static void balance_lists(ext_ctx* ctx, const std::vector<SlotHost>& slots, std:
                           std::vector<WorkItem>& l1) {
   auto prob = [&](const WorkItem& w) -> const SlotDesc& { return slots[w.slot / kMirClasses].tcp[w.slot % kMirClasses]; };
   for (auto& g : gm)
-    balance(g, ctx->sm_count, [&](const WorkItem& w) { return 5.0 + 3.4 * (prob(w).nxp + prob(w).nyp) / 256; });
+    balance(g, ctx->sm_count, [&](const WorkItem& w) { return 5.0 + 3.4 * (prob(w).nx + prob(w).ny) / 256; });
   balance(l1, ctx->sm_count, [&](const WorkItem& w) { return 6.0 + 4.0 * prob(w).nxp / 128; });
 }
 

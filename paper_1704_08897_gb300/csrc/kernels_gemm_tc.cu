@@ -291,7 +291,8 @@ __device__ __forceinline__ bool epi_vote(bool fail) {
 }
 
 struct TcStage {
-  int M, N, K;
+  int M, N, K;                   // padded extents (K: the exponents' row length)
+  int n, k;                      // real columns of the result and real k: beyond them all is zero
   const unsigned char *ma, *mb;  // tensor maps of A and B
   const int8_t *ea, *eb;         // block exponents: A rows [M][K / KC], B rows [N][K / KC]
   int8_t* eout;                  // next stage's block exponents [N][M/128]
@@ -302,16 +303,16 @@ __device__ __forceinline__ TcStage tc_stage(const SlotDesc& S) {
   const unsigned char* maps = static_cast<const unsigned char*>(S.tmaps);
   const unsigned char* low = static_cast<const unsigned char*>(S.low_maps);
   if constexpr (STAGE == kLowFwd)  // H = r Qx_low
-    return {S.nyp, kLowM, S.nxp, low, low + 128, S.tc_e[0], S.low_qxt_e, nullptr};
+    return {S.nyp, kLowM, S.nxp, kLowM, S.nx, low, low + 128, S.tc_e[0], S.low_qxt_e, nullptr};
   else if constexpr (STAGE == kLowInv)  // zl^T = J^T Qy_low^T, one block of 32 k
-    return {S.nxp, S.nyp, kLowM, low + 256, low + 384, S.low_jt_e, S.low_qy_e, nullptr};
+    return {S.nxp, S.nyp, kLowM, S.ny, kLowM, low + 256, low + 384, S.low_jt_e, S.low_qy_e, nullptr};
   else {
     const int8_t *ea = S.tc_e[STAGE], *eb = S.tc_eb[STAGE];
     int8_t* eo = STAGE < 3 ? S.tc_e[(STAGE + 1) & 3] : nullptr;
     if constexpr (STAGE == 0 || STAGE == 2)
-      return {S.nyp, S.nxp, S.nxp, maps + 128 * STAGE, maps + 128 * (4 + STAGE), ea, eb, eo};
+      return {S.nyp, S.nxp, S.nxp, S.nx, S.nx, maps + 128 * STAGE, maps + 128 * (4 + STAGE), ea, eb, eo};
     else
-      return {S.nxp, S.nyp, S.nyp, maps + 128 * STAGE, maps + 128 * (4 + STAGE), ea, eb, eo};
+      return {S.nxp, S.nyp, S.nyp, S.ny, S.ny, maps + 128 * STAGE, maps + 128 * (4 + STAGE), ea, eb, eo};
   }
 }
 
@@ -398,7 +399,8 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         const SlotDesc& S = slots[it.slot];
         const TcStage v = tc_stage<STAGE>(S);
         const int mt = v.M / BM;
-        Tile t = {S.sc, v.ma, v.mb, v.M, v.N, v.K / BK, (it.tile % mt) * BM, (it.tile / mt) * BN};
+        Tile t = {S.sc, v.ma, v.mb, v.M, v.N, (v.k + BK - 1) / BK, (it.tile % mt) * BM, (it.tile / mt) * BN};
+        if (t.n0 >= v.n) t.steps = 0;  // nothing but padding
         tmap_acquire(t.ma);
         tmap_acquire(t.mb);
         return t;
@@ -449,14 +451,18 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     auto tile_of = [&](int w) {
       const int slot = items[w].slot;
       sc = slot < 0 ? nullptr : slots[slot].sc;
-      k_tile = slot < 0 ? 0 : tc_stage<STAGE>(slots[slot]).K;
+      k_tile = 0;
+      if (slot >= 0) {
+        const TcStage v = tc_stage<STAGE>(slots[slot]);
+        if (items[w].tile / (v.M / BM) * BN < v.n) k_tile = v.k;
+      }
     };
     if (blockIdx.x < total) tile_of(blockIdx.x);
     pdl_wait();
     for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
       if (w != blockIdx.x) tile_of(w);
       if (!__any_sync(0xffffffffu, sc != nullptr && slot_runs(sc, mode))) continue;
-      const int steps = __reduce_max_sync(0xffffffffu, k_tile / BK);
+      const int steps = __reduce_max_sync(0xffffffffu, (k_tile + BK - 1) / BK);
       for (int kb = 0; kb < steps; ++kb) {
         const int half_kb = kb % KPC;  // position inside the accumulation block
         const int cb = chunk % kChunks, st = n % STAGES;
@@ -480,10 +486,10 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
                 umma(dset + pa * BN, ad + ((pa * A_PLANE) >> 4) + 2 * j, bd + 2 * j, idesc_f16(BF16, BM, (NSL - pa) * BN),
                      (half_kb > 0 || j > 0 || pa > 0) ? 1u : 0u);
           umma_commit(&ctl->empty[st]);
-          if (half_kb == KPC - 1) umma_commit(&ctl->tfull[cb]);
+          if (half_kb == KPC - 1 || kb == steps - 1) umma_commit(&ctl->tfull[cb]);
         }
         ++n;
-        if (half_kb == KPC - 1) ++chunk;
+        if (half_kb == KPC - 1 || kb == steps - 1) ++chunk;
       }
     }
     if (elected) {
@@ -526,7 +532,9 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
       const int mq = m0 + 32 * quarter;          // first row of the quarter
       const int ng = n0 + 8 * group;             // first column of the group (block cb: + 32 cb)
       const int n_mine = ng + 32 * (lane >> 3) + (lane & 7);  // a column lane's column
-      const int kblocks = STAGE == kLowInv ? 1 : v.K / KC;
+      if (n0 >= v.n) continue;                   // nothing but padding
+      const int kblocks = STAGE == kLowInv ? 1 : (v.k + KC - 1) / KC;
+      const int erow = STAGE == kLowInv ? 1 : v.K / KC;  // the exponents' row length
       if (STAGE == 3 && col_lane && !S.mir_out) {
         // the r, q and mask entries read after the last k-block: start them towards L2 now
         const int n = n_mine;
@@ -556,8 +564,8 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         }
         wnorm = ld_early(&S.wnorm);
       }
-      const int8_t* ea_row = v.ea + static_cast<size_t>(mq + lane) * kblocks;
-      const int8_t* eb_col = v.eb + static_cast<size_t>(col_lane ? n_mine : ng) * kblocks;
+      const int8_t* ea_row = v.ea + static_cast<size_t>(mq + lane) * erow;
+      const int8_t* eb_col = v.eb + static_cast<size_t>(col_lane ? n_mine : ng) * erow;
       // the thread's share of the tile's Qy_low rows (the G share's operand), loaded now so that
       // their latency hides behind the k-blocks
       constexpr int kYq = STAGE == kLowFwd ? BM * kLowM / (32 * kEpiWarps) : 1;

@@ -812,11 +812,37 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
   f2 alpha = {0.f, 0.f};
   bool run = false;
   const int total = *n_items;
+  // the first item and its descriptor ahead of the wait for the previous kernel
+  WorkItem it = {0, 0};
+  if (static_cast<int>(blockIdx.x) < total) it = items[blockIdx.x];
   pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
-    const WorkItem it = items[w];
+    if (w != static_cast<int>(blockIdx.x)) it = items[w];
     const SlotDesc& S = slots[it.slot];
     SlotScalars* sc = S.sc;
+    if (!FUSE && !sc->active) continue;
+    const int pi = (sc->it & 1) ^ 1;
+    const float* __restrict__ p = S.p[pi];
+    const float* __restrict__ p_lo = S.p_lo[pi];
+    const int n = S.nx * S.ny;
+    const int chunk = S.vec_chunk;
+    const int e0 = it.tile * chunk;
+    const int e1 = min(n, e0 + chunk);
+    const bool full = e0 + chunk <= n;
+    // one 16-byte vector of every plane per thread and step; the first step's loads pass under the sum
+    // of the p.q partials
+    float4 ph, pl, qh, ql, rh, rl, xh, xl;
+    auto load = [&](int e) {
+      ph = __ldg(reinterpret_cast<const float4*>(p + e));
+      pl = __ldg(reinterpret_cast<const float4*>(p_lo + e));
+      qh = __ldg(reinterpret_cast<const float4*>(S.q + e));
+      ql = __ldg(reinterpret_cast<const float4*>(S.q_lo + e));
+      rh = *reinterpret_cast<const float4*>(S.r + e);
+      rl = *reinterpret_cast<const float4*>(S.r_lo + e);
+      xh = *reinterpret_cast<const float4*>(S.xhi + e);
+      xl = *reinterpret_cast<const float4*>(S.xlo + e);
+    };
+    if (full) load(e0 + 4 * threadIdx.x);
     if (FUSE) {
       if (it.slot != pq_slot) {
         if (threadIdx.x < 32) {
@@ -839,30 +865,14 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
       // a breakdown: every block finds the same one, the tile-0 block records it
       if (!run) continue;
     } else {
-      if (!sc->active) continue;
       alpha = f2{sc->alpha_f[0], sc->alpha_f[1]};
     }
     const f2 nalpha = {-alpha.hi, -alpha.lo};
-    const int pi = (sc->it & 1) ^ 1;
-    const float* __restrict__ p = S.p[pi];
-    const float* __restrict__ p_lo = S.p_lo[pi];
-    const int n = S.nx * S.ny;
-    const int chunk = S.vec_chunk;
-    const int e0 = it.tile * chunk;
-    const int e1 = min(n, e0 + chunk);
     CompDotDF dot;
-    if (e0 + chunk <= n) {
-      // one 16-byte vector of every plane per thread and step, every load before any use
+    if (full) {
 #pragma unroll 1
       for (int e = e0 + 4 * threadIdx.x; e < e1; e += kVecStep) {
-        const float4 ph = __ldg(reinterpret_cast<const float4*>(p + e));
-        const float4 pl = __ldg(reinterpret_cast<const float4*>(p_lo + e));
-        const float4 qh = __ldg(reinterpret_cast<const float4*>(S.q + e));
-        const float4 ql = __ldg(reinterpret_cast<const float4*>(S.q_lo + e));
-        float4 rh = *reinterpret_cast<const float4*>(S.r + e);
-        float4 rl = *reinterpret_cast<const float4*>(S.r_lo + e);
-        float4 xh = *reinterpret_cast<const float4*>(S.xhi + e);
-        float4 xl = *reinterpret_cast<const float4*>(S.xlo + e);
+        if (e >= e0 + kVecStep) load(e);
         df_axpy(xh.x, xl.x, alpha, ph.x, pl.x);
         df_axpy(xh.y, xl.y, alpha, ph.y, pl.y);
         df_axpy(xh.z, xl.z, alpha, ph.z, pl.z);
