@@ -97,8 +97,8 @@ struct Workspace {
   int *d_counts = nullptr;      // [0] grid tiles, [1] vector items, [2] transform tiles with four
                                 // slices, [11] with six, [12] the low-mode middle, [3] slots,
                                 // [4] stencil tiles, [5] [6] low-mode tiles, [7] fold items,
-                                // [8] unfold tiles, [9] tensor-core problems, [10] grid tiles
-                                // of unfolded slots
+                                // [8] unfold tiles, [9] items of the update, [10] grid
+                                // tiles of unfolded slots
   int n_st = 0, n_vec = 0, n_sl = 0;
   int n_gm[2] = {0, 0};
   WorkItem* d_sten = nullptr;   // the stencil kernel's tiles (64 x sten_ty)
@@ -109,10 +109,11 @@ struct Workspace {
   WorkItem *d_l1 = nullptr, *d_l2 = nullptr, *d_l3 = nullptr;  // low-mode forward, middle, inverse
   int n_l1 = 0, n_l2 = 0, n_l3 = 0;
   // tensor-core problems (mixed modes): kMirClasses entries per slot, the slot's own descriptor
-  // or its mirror classes; items of the fold and unfold kernels; one item per problem
+  // or its mirror classes; items of the fold and unfold kernels and of the slicing update
   SlotDesc* d_tcp = nullptr;
-  WorkItem *d_fold = nullptr, *d_unfold = nullptr, *d_tcl = nullptr;
-  int n_fold = 0, n_unfold = 0, n_tcl = 0;
+  WorkItem *d_fold = nullptr, *d_unfold = nullptr, *d_upd = nullptr;
+  int n_fold = 0, n_unfold = 0, n_upd = 0;
+  bool slice = false;           // the updates slice the residuals (no slot above kSliceNodes)
   WorkItem* d_prep = nullptr;  // residual slicing of the unfolded slots (32 rows x 128 columns)
   int n_prep = 0;
   const float** d_phis = nullptr;
@@ -465,9 +466,9 @@ static void drop_graphs(Workspace* W) {
 
 // The kernels an iteration of W launches: which lists hold work, and the scalar steps' place.
 static int graph_key(const Workspace* W) {
-  const int n[7] = {W->n_gm[0], W->n_gm[1], W->n_l1, W->n_fold, W->n_prep, W->aniso, W->fuse};
+  const int n[8] = {W->n_gm[0], W->n_gm[1], W->n_l1, W->n_fold, W->n_prep, W->aniso, W->fuse, W->slice};
   int k = 0;
-  for (int i = 0; i < 7; ++i) k |= (n[i] != 0) << i;
+  for (int i = 0; i < 8; ++i) k |= (n[i] != 0) << i;
   return k;
 }
 
@@ -492,7 +493,7 @@ static void free_workspace(Workspace* W) {
   cudaFree(W->d_tcp);
   cudaFree(W->d_fold);
   cudaFree(W->d_unfold);
-  cudaFree(W->d_tcl);
+  cudaFree(W->d_upd);
   cudaFree(W->d_prep);
   cudaFree(W->d_counts);
   cudaFree(W->d_phis);
@@ -576,7 +577,10 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   d.n_prep_items = !d.mir ? ((ny + kStTileY - 1) / kStTileY) * ((nx + 127) / 128) : 0;
   d.n_unfold_tiles = d.mir ? ((d.mhx + 31) / 32) * ((d.mhy + 7) / 8) : 0;
   d.n_prec_parts = d.mir ? d.n_unfold_tiles : (d.nxp / 128) * ((ny + bn - 1) / bn);
-  const int n_part = std::max(std::max(d.n_st_tiles, d.n_vec_items), std::max(n_gm, d.n_unfold_tiles));
+  const int upd_rows = 8 >> ((d.mir & 1) + (d.mir >> 1));  // class rows of an update item: eight segments
+  d.upd_seg = (long long)N <= kSliceNodes;
+  d.n_upd_items = d.upd_seg ? ((d.mhy + upd_rows - 1) / upd_rows) * ((d.mhx + 127) / 128) : d.n_vec_items;
+  const int n_part = std::max({d.n_st_tiles, d.n_vec_items, d.n_upd_items, n_gm, d.n_unfold_tiles});
   // arena layout
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
@@ -813,7 +817,7 @@ static void set_slot_scalars(SlotHost& s, SlotScalars* sc) {
 
 // Work items of the tensor-core problems of slot i (problem index kMirClasses * i + c).
 static void tc_items(const SlotHost& s, int i, std::vector<WorkItem> (&gm)[2], std::vector<WorkItem>& l1,
-                     std::vector<WorkItem>& l2, std::vector<WorkItem>& l3, std::vector<WorkItem>& tcl) {
+                     std::vector<WorkItem>& l2, std::vector<WorkItem>& l3) {
   for (int c = 0; c < kMirClasses; ++c) {
     if (s.d.mir == 0 && c > 0) break;
     if (((c & 1) && !(s.d.mir & 1)) || ((c & 2) && !(s.d.mir & 2))) continue;
@@ -825,7 +829,6 @@ static void tc_items(const SlotHost& s, int i, std::vector<WorkItem> (&gm)[2], s
       for (int tt = 0; tt < t.n_l2_tiles; ++tt) l2.push_back({k, tt});
       for (int tt = 0; tt < t.n_l3_tiles; ++tt) l3.push_back({k, tt});
     }
-    tcl.push_back({k, 0});
   }
 }
 
@@ -883,7 +886,8 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   W->key = shape_key(count, probs, host_io);
   W->host_io = host_io;
   W->slots.resize(count);
-  std::vector<WorkItem> st, vec, gm[2], l1, l2, l3, fold, unfold, tcl, prep;
+  std::vector<WorkItem> st, vec, gm[2], l1, l2, l3, fold, unfold, upd, prep;
+  bool slice = true;
   long long call_nodes = 0;
   for (int i = 0; i < count; ++i) call_nodes += (long long)probs[i].nx * probs[i].ny;
   for (int i = 0; i < count; ++i) {
@@ -897,13 +901,15 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
     SlotDesc& d = s.d;
     if (d.aniso) W->aniso = true;
     for (int t = 0; t < d.n_st_tiles; ++t) st.push_back({i, t});
-    for (int t = 0; t < d.n_vec_items; ++t) vec.push_back({i, t});
-    tc_items(s, i, gm, l1, l2, l3, tcl);
-    for (int t = 0; t < d.n_fold_items; ++t) fold.push_back({i, t});
+    tc_items(s, i, gm, l1, l2, l3);
     for (int t = 0; t < d.n_unfold_tiles; ++t) unfold.push_back({i, t});
-    if (!d.mir)
-      for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
+    for (int t = 0; t < d.n_upd_items; ++t) upd.push_back({i, t});
+    for (int t = 0; t < d.n_vec_items; ++t) vec.push_back({i, t});
+    for (int t = 0; t < d.n_fold_items; ++t) fold.push_back({i, t});
+    for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
+    slice = slice && d.upd_seg;
   }
+  W->slice = slice;
   balance_lists(ctx, W->slots, gm, l1);
   std::vector<WorkItem> sl;
   for (int i = 0; i < count; ++i) sl.push_back({i, 0});
@@ -933,7 +939,7 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   if (!rc) rc = upload(&W->d_l3, l3);
   if (!rc) rc = upload(&W->d_fold, fold);
   if (!rc) rc = upload(&W->d_unfold, unfold);
-  if (!rc) rc = upload(&W->d_tcl, tcl);
+  if (!rc) rc = upload(&W->d_upd, upd);
   if (!rc) rc = upload(&W->d_prep, prep);
   if (rc) return rc;
   W->n_sten = W->n_st;
@@ -947,10 +953,10 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   W->n_l3 = (int)l3.size();
   W->n_fold = (int)fold.size();
   W->n_unfold = (int)unfold.size();
-  W->n_tcl = (int)tcl.size();
+  W->n_upd = (int)upd.size();
   W->n_prep = (int)prep.size();
   int counts[13] = {W->n_st, W->n_vec, W->n_gm[0], W->n_sl, W->n_sten, W->n_l1, W->n_l3,
-                    W->n_fold, W->n_unfold, W->n_tcl, W->n_prep, W->n_gm[1], W->n_l2};
+                    W->n_fold, W->n_unfold, W->n_upd, W->n_prep, W->n_gm[1], W->n_l2};
   BX_CUDA(cudaMalloc(&W->d_counts, sizeof(counts)));
   BX_CUDA(cudaMemcpy(W->d_counts, counts, sizeof(counts), cudaMemcpyHostToDevice));
   BX_CUDA(cudaMalloc(&W->d_phis, sizeof(void*) * count));
@@ -997,9 +1003,9 @@ static LaunchCfg cfg_of(ext_ctx* ctx, Workspace* W, int which) {
     c.n_items = W->d_counts + which;
     c.grid = std::max(1, std::min(which == 7 ? W->n_fold : W->n_unfold, cap));
   } else if (which == 9) {
-    c.items = W->d_tcl;
+    c.items = W->d_upd;
     c.n_items = W->d_counts + 9;
-    c.grid = std::max(1, std::min(W->n_tcl, cap));
+    c.grid = std::max(1, std::min(W->n_upd, cap));
   } else if (which == 10) {
     c.items = W->d_prep;
     c.n_items = W->d_counts + 10;
@@ -1099,12 +1105,13 @@ static void harvest(ext_ctx* ctx) {
 }
 
 // with_finish = false: the next stencil forms rho and beta from the partials itself
-static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish = true) {
+// sliced: the update has left the residuals' slices
+static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish = true, bool sliced = false) {
   const LaunchCfg g = cfg_of(ctx, W, 2), g6 = cfg_of(ctx, W, 11);
   // residual slices: unfolded slots directly, folded slots per mirror class
-  if (W->n_prep > 0)
+  if (W->n_prep > 0 && !sliced)
     timed(ctx, EXT_KERNEL_SPLIT, [&] { launch_prec_tc_prepare(cfg_of(ctx, W, 10), mode, ctx->split); }, g.stream);
-  if (W->n_fold > 0)
+  if (W->n_fold > 0 && !sliced)
     timed(ctx, EXT_KERNEL_FOLD, [&] { launch_tc_fold(cfg_of(ctx, W, 7), mode, ctx->split); }, g.stream);
   if (W->n_l1 > 0) {
     // the lowest modes in high precision: forward product, middle, inverse product
@@ -1131,7 +1138,7 @@ static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish =
 }
 
 static void enqueue_iterations(ext_ctx* ctx, Workspace* W, int iters) {
-  const LaunchCfg st = cfg_of(ctx, W, 0), vc = cfg_of(ctx, W, 1);
+  const LaunchCfg st = cfg_of(ctx, W, 0), up = cfg_of(ctx, W, 9);
   const LaunchCfg sc = cfg_of(ctx, W, 4);
   const bool fuse = W->fuse;
   for (int i = 0; i < iters; ++i) {
@@ -1140,8 +1147,11 @@ static void enqueue_iterations(ext_ctx* ctx, Workspace* W, int iters) {
     timed(ctx, EXT_KERNEL_STENCIL, [&] { launch_stencil(sc, W->aniso, W->sten_ty, ctx->d_err, fz); }, st.stream);
     const LaunchCfg pf = cfg_of(ctx, W, 3);  // one block per slot
     if (!fuse) timed(ctx, EXT_KERNEL_PQ_FINISH, [&] { launch_pq_finish(pf); }, st.stream);
-    timed(ctx, EXT_KERNEL_UPDATE, [&] { launch_update(vc, fuse); }, st.stream);
-    launch_prec(ctx, W, 0, !fuse || i + 1 == iters);
+    timed(ctx, EXT_KERNEL_UPDATE, [&] {
+      if (W->slice) launch_update_slice(up, ctx->split, fuse);
+      else launch_update(up, fuse);
+    }, st.stream);
+    launch_prec(ctx, W, 0, !fuse || i + 1 == iters, W->slice);
   }
   timed(ctx, EXT_KERNEL_TRUE_RESIDUAL, [&] { launch_true_residual(st); }, st.stream);
   launch_prec(ctx, W, 1);
@@ -1156,7 +1166,7 @@ static int ensure_graph(ext_ctx* ctx, Workspace* W) {
   cudaGraph_t g;
   if (ctx->opt.profile) {
     // events for the graph's timing nodes are created before capture begins
-    const size_t need = 2 * (size_t)(8 * G + 16);
+    const size_t need = 2 * (size_t)(20 * G + 40);
     while (ctx->ev_pool.size() < need) {
       cudaEvent_t e = nullptr;
       BX_CUDA(cudaEventCreate(&e));
@@ -2166,16 +2176,16 @@ static int serve_alloc_lists(ext_ctx::Serve* S, int cap) {
   cudaFree(W->d_l3);
   cudaFree(W->d_fold);
   cudaFree(W->d_unfold);
-  cudaFree(W->d_tcl);
+  cudaFree(W->d_upd);
   cudaFree(W->d_prep);
   cudaFree(S->d_new);
   cudaFree(S->d_ret);
   W->d_st = W->d_sten = W->d_vec = W->d_gm[0] = W->d_gm[1] = W->d_l1 = W->d_l2 = W->d_l3 = S->d_new = S->d_ret = nullptr;
-  W->d_fold = W->d_unfold = W->d_tcl = W->d_prep = nullptr;
+  W->d_fold = W->d_unfold = W->d_upd = W->d_prep = nullptr;
   BX_CUDA(cudaMalloc(&W->d_prep, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_fold, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_unfold, sizeof(WorkItem) * cap));
-  BX_CUDA(cudaMalloc(&W->d_tcl, sizeof(WorkItem) * cap));
+  BX_CUDA(cudaMalloc(&W->d_upd, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_st, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_sten, sizeof(WorkItem) * cap));
   BX_CUDA(cudaMalloc(&W->d_l1, sizeof(WorkItem) * cap));
@@ -2188,7 +2198,7 @@ static int serve_alloc_lists(ext_ctx::Serve* S, int cap) {
   S->cap_items = cap;
   // grids sized for the capacity
   W->n_st = W->n_vec = W->n_gm[0] = W->n_gm[1] = W->n_sten = W->n_l1 = W->n_l2 = W->n_l3 = cap;
-  W->n_fold = W->n_unfold = W->n_tcl = W->n_prep = cap;
+  W->n_fold = W->n_unfold = W->n_upd = W->n_prep = cap;
   drop_graphs(W);
   return EXT_OK;
 }
@@ -2231,25 +2241,27 @@ static int serve_init(ext_ctx* ctx) {
 static int serve_rebuild_lists(ext_ctx* ctx) {
   ext_ctx::Serve* S = ctx->serve;
   Workspace* W = S->W;
-  std::vector<WorkItem> st, vec, gm[2], sl, l1, l2, l3, fold, unfold, tcl, prep;
-  bool aniso = false;
+  std::vector<WorkItem> st, vec, gm[2], sl, l1, l2, l3, fold, unfold, upd, prep;
+  bool aniso = false, slice = true;
   for (int i = 0; i < (int)S->slots.size(); ++i) {
     if (!S->slots[i].used) continue;
     const SlotHost& h = W->slots[i];
     const SlotDesc& d = h.d;
     aniso |= d.aniso != 0;
     for (int t = 0; t < d.n_st_tiles; ++t) st.push_back({i, t});
-    for (int t = 0; t < d.n_vec_items; ++t) vec.push_back({i, t});
-    tc_items(h, i, gm, l1, l2, l3, tcl);
-    for (int t = 0; t < d.n_fold_items; ++t) fold.push_back({i, t});
+    tc_items(h, i, gm, l1, l2, l3);
     for (int t = 0; t < d.n_unfold_tiles; ++t) unfold.push_back({i, t});
-    if (!d.mir)
-      for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
+    for (int t = 0; t < d.n_upd_items; ++t) upd.push_back({i, t});
+    for (int t = 0; t < d.n_vec_items; ++t) vec.push_back({i, t});
+    for (int t = 0; t < d.n_fold_items; ++t) fold.push_back({i, t});
+    for (int t = 0; t < d.n_prep_items; ++t) prep.push_back({i, t});
+    slice = slice && d.upd_seg;
     sl.push_back({i, 0});
   }
+  W->slice = slice;
   balance_lists(ctx, W->slots, gm, l1);
   size_t need = 0;
-  for (const auto* v : {&st, &vec, &gm[0], &gm[1], &l1, &l2, &l3, &fold, &unfold, &tcl, &prep}) need = std::max(need, v->size());
+  for (const auto* v : {&st, &vec, &gm[0], &gm[1], &l1, &l2, &l3, &fold, &unfold, &upd, &prep}) need = std::max(need, v->size());
   if ((int)need > S->cap_items) {
     int cap = S->cap_items;
     while (cap < (int)need) cap *= 2;
@@ -2285,11 +2297,11 @@ static int serve_rebuild_lists(ext_ctx* ctx) {
   if (!rc) rc = put(W->d_l3, l3);
   if (!rc) rc = put(W->d_fold, fold);
   if (!rc) rc = put(W->d_unfold, unfold);
-  if (!rc) rc = put(W->d_tcl, tcl);
+  if (!rc) rc = put(W->d_upd, upd);
   if (!rc) rc = put(W->d_prep, prep);
   if (rc) return rc;
   int counts[13] = {(int)st.size(), (int)vec.size(), (int)gm[0].size(), (int)sl.size(), (int)st.size(),
-                    (int)l1.size(), (int)l3.size(), (int)fold.size(), (int)unfold.size(), (int)tcl.size(),
+                    (int)l1.size(), (int)l3.size(), (int)fold.size(), (int)unfold.size(), (int)upd.size(),
                     (int)prep.size(), (int)gm[1].size(), (int)l2.size()};
   BX_CUDA(cudaMemcpyAsync(W->d_counts, counts, sizeof(counts), cudaMemcpyHostToDevice, s));
   // the host vectors die here: the copies above must finish first (pageable sources are staged)

@@ -40,6 +40,12 @@ constexpr int kVecStep = 4 * kVecThreads;  // elements a block moves with one ve
 // once: the update of a 389 x 251 grid, 24 blocks of four steps before, went from about 13 to 7 us,
 // that of a 1024^2 grid from 14 to 12 us), four beyond (less per-item overhead: 43 us a launch on 48
 // grids of 5.1 M nodes against 61 with one step everywhere).
+// Calls whose grids are all of up to this size have the residuals sliced by the update itself
+// (k_update_slice): one launch less in the chain of an iteration (320 x 256, three fields: 69.7 -> 64 us;
+// 64^2: 50.5 -> 46).  Above, a pass of its own is as fast: the joint kernel holds a segment's planes
+// across a barrier, so that fewer loads are in flight (1024^2: 28 us either way; 48 grids of up to
+// 512^2: 76 us against 62).
+constexpr long long kSliceNodes = 1LL << 17;
 constexpr int vec_chunk_of(long long nodes) {
   return kVecStep * (nodes <= 1LL << 17 ? 1 : nodes <= 1LL << 21 ? 2 : 4);
 }
@@ -153,6 +159,8 @@ struct SlotDesc {
   int mir;           // slot: bit 0 = x folded, bit 1 = y folded (0: the slot is its own problem)
   int mhx, mhy;      // slot: class nodes along x, y (ceil(n/2) on a folded axis, else n)
   int n_fold_items;  // slot: items of the fold kernel (8 class rows x 128 columns)
+  int upd_seg;       // slot of at most kSliceNodes nodes: its update items are segments (seg_of), not chunks
+  int n_upd_items;   // slot: items of the update kernels
   int n_prep_items;  // slot with no folded axis: items of its residual slicing (32 rows x 128)
   int n_unfold_tiles;// slot: tiles of the unfold kernel (32 x 8 class nodes)
   int n_prec_parts;  // slot: r.z, z.q partials the preconditioner leaves (stage-3 or unfold tiles)
@@ -506,6 +514,67 @@ __device__ __forceinline__ double sum_pq(const SlotDesc& S) {
 __device__ __forceinline__ void sum_rz(const SlotDesc& S, bool with_zq, double& rz, double& zq) {
   rz = warp_sum_strided(S.part + 2, S.n_prec_parts, 4);
   zq = with_zq ? warp_sum_strided(S.part + 3, S.n_prec_parts, 4) : 0.0;
+}
+
+// A warp's part of an update item in segments (slots of up to kSliceNodes): an item is 8, 4 or 2 class rows
+// by 128 class columns, and its eight warps hold the rows' segments at the node and its mirrors.  With
+// rows of whole 16-byte vectors a lane holds one vector of each plane (reversed class columns on the
+// mirrored side), else nodes 32 apart.
+struct Seg {
+  int lseg, seg;     // log2 of a class row's segments, and the warp's (bits: mirrored in x, in y, folded ones only)
+  bool qx, qy, vec;  // mirrored side along x, along y; rows of whole vectors
+  bool whole;        // all four nodes exist and form a vector
+  int y, xb;         // class row, block of 128 class columns
+  int g0, gs;        // node indices g0 + i gs
+  unsigned have;     // which nodes exist (a middle row or column belongs to the unmirrored side)
+  __device__ __forceinline__ int col(int i) const {
+    const int lane = threadIdx.x & 31;
+    return vec ? 4 * lane + (qx ? 3 - i : i) : 32 * i + lane;
+  }
+  __device__ __forceinline__ float4 load(const float* a) const {
+    if (whole) return *reinterpret_cast<const float4*>(a + g0);
+    float4 v;
+    v.x = (have & 1u) ? a[g0] : 0.f;
+    v.y = (have & 2u) ? a[g0 + gs] : 0.f;
+    v.z = (have & 4u) ? a[g0 + 2 * gs] : 0.f;
+    v.w = (have & 8u) ? a[g0 + 3 * gs] : 0.f;
+    return v;
+  }
+  __device__ __forceinline__ void store(float* a, const float4 v) const {
+    if (whole) {
+      *reinterpret_cast<float4*>(a + g0) = v;
+      return;
+    }
+    if (have & 1u) a[g0] = v.x;
+    if (have & 2u) a[g0 + gs] = v.y;
+    if (have & 4u) a[g0 + 2 * gs] = v.z;
+    if (have & 8u) a[g0 + 3 * gs] = v.w;
+  }
+};
+__device__ __forceinline__ Seg seg_of(const SlotDesc& S, int tile) {
+  Seg g;
+  const int warp = threadIdx.x >> 5;
+  const bool fx = (S.mir & 1) != 0, fy = (S.mir & 2) != 0;
+  g.lseg = (fx ? 1 : 0) + (fy ? 1 : 0);
+  g.seg = warp & ((1 << g.lseg) - 1);
+  g.qx = fx && (g.seg & 1);
+  g.qy = fy && (g.seg >> (g.lseg - 1));
+  g.vec = (S.nx & 3) == 0;
+  const int nxb = (S.mhx + 127) / 128;
+  g.y = (tile / nxb) * (8 >> g.lseg) + (warp >> g.lseg);
+  g.xb = tile % nxb;
+  const int yy = g.qy ? S.ny - 1 - g.y : g.y;
+  g.have = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int x = g.xb * 128 + g.col(i);
+    if (g.y < S.mhy && !(g.qy && yy == g.y) && x < S.mhx && !(g.qx && S.nx - 1 - x == x)) g.have |= 1u << i;
+  }
+  const int x = g.xb * 128 + g.col(0);
+  g.g0 = yy * S.nx + (g.qx ? S.nx - 1 - x : x);
+  g.gs = g.vec ? 1 : g.qx ? -32 : 32;
+  g.whole = g.vec && g.have == 15u;
+  return g;
 }
 
 // alpha = rho / p.q is usable (p.q > 0, everything finite)

@@ -65,6 +65,8 @@ cudaError_t stencil_init();
 void launch_pq_finish(const LaunchCfg& c);
 // fuse_pq: the blocks form alpha from the stencil's partials themselves
 void launch_update(const LaunchCfg& c, bool fuse_pq = false);
+// the same with the new residuals' slices, where every slot is of up to kSliceNodes
+void launch_update_slice(const LaunchCfg& c, int split_kind, bool fuse_pq);
 void launch_true_residual(const LaunchCfg& c);
 void launch_output(const LaunchCfg& c, const float* const* fs, float* const* outs);
 void launch_output64(const SlotDesc* slot, int n, const float* f, double* out, cudaStream_t s);

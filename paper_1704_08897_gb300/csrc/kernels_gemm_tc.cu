@@ -916,6 +916,35 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   if (threadIdx.x == 0 && ctl->abort_flag) atomicExch(err, 1);
 }
 
+// One row of a transform operand: the warp's 128 columns (lane pairs 64 k + 2 lane) under their common
+// exponent, both codes of a slice in one 4-byte store.  `idx`: the lane's first pair in a plane of
+// `half` pairs.  With six slices in a mixed mode the first four are stage 0's operand, all six the
+// low-mode product's.
+template <bool BF16>
+__device__ __forceinline__ void slice_row(const float2 (&vh)[2], const float2 (&vl)[2], uint32_t* out32, size_t idx,
+                                          size_t half, int nr, int8_t* e, int lane) {
+  float amax = 0.f;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) amax = fmaxf(amax, fmaxf(fabsf(vh[k].x), fabsf(vh[k].y)));
+  const int E = block_exp(warp_max(amax));
+  const float2 up = make_float2(pow2f(16 - E), pow2f(16 - E)), dn = make_float2(-pow2f(E - 16), -pow2f(E - 16));
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (nr == kLowNS) {
+      uint32_t code[kLowNS];
+      slice_codes2_df<BF16, kLowNS>(vh[k], vl[k], up, dn, code);
+#pragma unroll
+      for (int q = 0; q < kLowNS; ++q) out32[q * half + idx + 32 * k] = code[q];
+    } else {
+      uint32_t code[4];
+      slice_codes2_df<BF16, 4>(vh[k], vl[k], up, dn, code);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) out32[q * half + idx + 32 * k] = code[q];
+    }
+  }
+  if (lane == 0) *e = static_cast<int8_t>(E);
+}
+
 // Residual -> slices of the first stage's A operand (slots with no folded axis).  One item per
 // 32 rows and KC columns; one warp per four of the rows, all four loaded before any is sliced.
 template <bool BF16>
@@ -938,7 +967,7 @@ k_tc_prepare(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ it
     uint16_t* out = static_cast<uint16_t*>(S.tc_r);
     // every row of the warp loaded before any is sliced
     constexpr int kRows = kStTileY / 8;
-    static_assert(kRows * 8 == kStTileY, "rows per warp");
+    static_assert(kRows * 8 == kStTileY && KC == 128, "rows per warp");
     // each lane takes adjacent pairs (x, x+1) and writes both codes of a slice in one 4-byte
     // store (x even, rows of nxp even: aligned)
     constexpr int kPairs = KC / 64;
@@ -962,28 +991,8 @@ k_tc_prepare(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ it
     for (int j = 0; j < kRows; ++j) {
       const int y = y0 + warp + 8 * j;
       if (y >= S.ny) break;
-      float amax = 0.f;
-#pragma unroll
-      for (int k = 0; k < kPairs; ++k) amax = fmaxf(amax, fmaxf(fabsf(v[j][k].x), fabsf(v[j][k].y)));
-      const int E = block_exp(warp_max(amax));
-      const float s = pow2f(16 - E), is = -pow2f(E - 16);
-#pragma unroll
-      for (int k = 0; k < kPairs; ++k) {
-        const size_t idx = (static_cast<size_t>(y) * S.nxp + x0 + 64 * k + 2 * lane) / 2;
-        if (S.tc_nr == kLowNS) {
-          // six slices (mixed modes: the first four are stage 0's operand, all six the low-mode product's)
-          uint32_t code[kLowNS];
-          slice_codes2_df<BF16, kLowNS>(v[j][k], vl[j][k], make_float2(s, s), make_float2(is, is), code);
-#pragma unroll
-          for (int q = 0; q < kLowNS; ++q) out32[q * (plane / 2) + idx] = code[q];
-        } else {
-          uint32_t code[4];
-          slice_codes2_df<BF16, 4>(v[j][k], vl[j][k], make_float2(s, s), make_float2(is, is), code);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) out32[q * (plane / 2) + idx] = code[q];
-        }
-      }
-      if (lane == 0) S.tc_e[0][static_cast<size_t>(y) * kblocks + x0 / KC] = static_cast<int8_t>(E);
+      slice_row<BF16>(v[j], vl[j], out32, (static_cast<size_t>(y) * S.nxp + x0 + 2 * lane) / 2, plane / 2, S.tc_nr,
+                      S.tc_e[0] + static_cast<size_t>(y) * kblocks + x0 / KC, lane);
     }
   }
 }
@@ -1000,6 +1009,32 @@ k_tc_prepare(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ it
 // partials that stage 3 leaves for an unfolded slot.
 // ---------------------------------------------------------------------------------------------
 
+// An item, its slot and its classes' operands.  The first item's are read before the wait for
+// the previous kernel (no kernel writes them), the others' ahead of the residual's loads: read where
+// the slices are stored, they were four dependent misses in a row.
+// The classes of a slot have equal sizes and lie at equal distances in its arena.
+struct FoldItem {
+  const SlotDesc* S = nullptr;
+  int tile = 0;
+  char *out = nullptr, *e = nullptr;  // class 0's operand and exponents
+  ptrdiff_t step = 0;                 // bytes from one class to the next
+  int nxp = 0, nyp = 0, nr = 4;
+};
+__device__ __forceinline__ FoldItem fold_item(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
+                                              const WorkItem it) {
+  FoldItem t;
+  t.S = slots + it.slot;
+  t.tile = it.tile;
+  const SlotDesc &T = tcp[kMirClasses * it.slot], &U = tcp[kMirClasses * it.slot + ((t.S->mir & 1) ? 1 : 2)];
+  t.out = static_cast<char*>(T.tc_r);
+  t.e = reinterpret_cast<char*>(T.tc_e[0]);
+  t.step = static_cast<char*>(U.tc_r) - t.out;
+  t.nxp = T.nxp;
+  t.nyp = T.nyp;
+  t.nr = T.tc_nr;
+  return t;
+}
+
 // One warp per (class row y, 128 class columns); lane pairs (x, x+1) at x = 64 k + 2 lane.
 template <bool BF16>
 __global__ void __launch_bounds__(256, 4)
@@ -1007,36 +1042,11 @@ k_tc_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
           const WorkItem* __restrict__ items, const int* __restrict__ n_items, int mode) {
   const int total = *n_items;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // The item, its slot and its classes' operands.  The first item's are read before the wait for
-  // the previous kernel (no kernel writes them), the others' ahead of the residual's loads: read where
-  // the slices are stored, they were four dependent misses in a row.
-  // The classes of a slot have equal sizes and lie at equal distances in its arena.
-  struct Fold {
-    const SlotDesc* S = nullptr;
-    int tile = 0;
-    char *out = nullptr, *e = nullptr;  // class 0's operand and exponents
-    ptrdiff_t step = 0;                 // bytes from one class to the next
-    int nxp = 0, nyp = 0, nr = 4;
-  };
-  auto item = [&](int w) {
-    Fold t;
-    const WorkItem it = items[w];
-    t.S = slots + it.slot;
-    t.tile = it.tile;
-    const SlotDesc &T = tcp[kMirClasses * it.slot], &U = tcp[kMirClasses * it.slot + ((t.S->mir & 1) ? 1 : 2)];
-    t.out = static_cast<char*>(T.tc_r);
-    t.e = reinterpret_cast<char*>(T.tc_e[0]);
-    t.step = static_cast<char*>(U.tc_r) - t.out;
-    t.nxp = T.nxp;
-    t.nyp = T.nyp;
-    t.nr = T.tc_nr;
-    return t;
-  };
-  Fold t;
-  if (static_cast<int>(blockIdx.x) < total) t = item(blockIdx.x);
+  FoldItem t;
+  if (static_cast<int>(blockIdx.x) < total) t = fold_item(slots, tcp, items[blockIdx.x]);
   pdl_wait();
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
-    if (w != static_cast<int>(blockIdx.x)) t = item(w);
+    if (w != static_cast<int>(blockIdx.x)) t = fold_item(slots, tcp, items[w]);
     const SlotDesc& S = *t.S;
     if (!slot_runs(S.sc, mode)) continue;
     const bool fx = (S.mir & 1) != 0, fy = (S.mir & 2) != 0;
@@ -1094,31 +1104,155 @@ k_tc_fold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
     for (int c = 0; c < 4; ++c) {
       if ((c & 1) && !fx) continue;
       if ((c & 2) && !fy) continue;
-      float amax = 0.f;
-#pragma unroll
-      for (int k = 0; k < 2; ++k) amax = fmaxf(amax, fmaxf(fabsf(ch[c][k].x), fabsf(ch[c][k].y)));
-      const int E = block_exp(warp_max(amax));
-      const float up = pow2f(16 - E), is = -pow2f(E - 16);
       const size_t plane = static_cast<size_t>(t.nyp) * t.nxp;
       const ptrdiff_t off = t.step * (fx ? c : c >> 1);
-      uint32_t* out32 = reinterpret_cast<uint32_t*>(t.out + off);
+      slice_row<BF16>(ch[c], cl[c], reinterpret_cast<uint32_t*>(t.out + off),
+                      (static_cast<size_t>(y) * t.nxp + xb * KC + 2 * lane) / 2, plane / 2, t.nr,
+                      reinterpret_cast<int8_t*>(t.e + off + static_cast<ptrdiff_t>(y) * (t.nxp / KC) + xb), lane);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Iteration, stage 2, for slots of up to kSliceNodes: what k_update does (x += alpha p, r -= alpha q,
+// partial ||r||^2, the last item's decision), and the new residual's slices, folded by class where an
+// axis is folded (what k_tc_prepare and k_tc_fold form from a stored residual).  Bound by the chain
+// of dependent loads and reductions: 7 us at 64^2, 10 at 320 x 256, where the two kernels took 8 and 3,
+// 9 and 5.  The block's eight warps hold an item's segments (seg_of), leave the new residual in shared
+// memory, and then slice one (class row, class) each.
+// ---------------------------------------------------------------------------------------------
+template <bool BF16, bool FUSE>
+__global__ void __launch_bounds__(kVecThreads, 2)
+k_update_slice(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
+               const WorkItem* __restrict__ items, const int* __restrict__ n_items) {
+  constexpr int kWarps = kVecThreads / 32;
+  __shared__ __align__(16) float sh[kWarps][KC], sl[kWarps][KC];  // the new residual by segment
+  __shared__ float2 red[kWarps];
+  __shared__ float2 s_alpha;  // FUSE: alpha of slot pq_slot, and whether the slot runs
+  __shared__ int s_run, s_last;
+  int pq_slot = -1;
+  f2 alpha = {0.f, 0.f};
+  bool run = false;
+  const int total = *n_items;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  WorkItem it = {0, 0};
+  FoldItem t;
+  if (static_cast<int>(blockIdx.x) < total) {
+    it = items[blockIdx.x];
+    t = fold_item(slots, tcp, it);
+  }
+  pdl_wait();
+  for (int w = blockIdx.x; w < total; w += gridDim.x) {
+    if (w != static_cast<int>(blockIdx.x)) {
+      it = items[w];
+      t = fold_item(slots, tcp, it);
+    }
+    const SlotDesc& S = *t.S;
+    SlotScalars* sc = S.sc;
+    if (!FUSE && !sc->active) continue;
+    const int pi = (sc->it & 1) ^ 1;
+    const Seg g = seg_of(S, t.tile);
+    // all loads pass under the sum of the p.q partials
+    const float4 ph = g.load(S.p[pi]), pl = g.load(S.p_lo[pi]), qh = g.load(S.q), ql = g.load(S.q_lo);
+    float4 rh = g.load(S.r), rl = g.load(S.r_lo), xh = g.load(S.xhi), xl = g.load(S.xlo);
+    if (FUSE) {
+      if (it.slot != pq_slot) {
+        if (threadIdx.x < 32) {
+          const bool act = sc->active != 0;  // one reading for the whole block
+          const double pq = sum_pq(S);
+          if (threadIdx.x == 0) {
+            const bool ok = act && pq_ok(sc, pq);
+            const f2 af = ok ? df_of(sc->rho2[sc->it & 1] / pq) : f2{0.f, 0.f};
+            s_alpha = make_float2(af.hi, af.lo);
+            s_run = ok;
+            if (act && it.tile == 0) finish_pq(sc, pq);
+          }
+        }
+        __syncthreads();
+        alpha = f2{s_alpha.x, s_alpha.y};
+        run = s_run != 0;
+        pq_slot = it.slot;
+        __syncthreads();  // s_alpha and s_run are written again for the next slot
+      }
+      // a breakdown: every block finds the same one, the tile-0 block records it
+      if (!run) continue;
+    } else {
+      alpha = f2{sc->alpha_f[0], sc->alpha_f[1]};
+    }
+    const f2 nalpha = {-alpha.hi, -alpha.lo};
+    df_axpy(rh.x, rl.x, nalpha, qh.x, ql.x);
+    df_axpy(rh.y, rl.y, nalpha, qh.y, ql.y);
+    df_axpy(rh.z, rl.z, nalpha, qh.z, ql.z);
+    df_axpy(rh.w, rl.w, nalpha, qh.w, ql.w);
+    auto stage = [&](float* a, const float4 v) {
+      if (!g.vec) {
+        a[lane] = v.x;
+        a[lane + 32] = v.y;
+        a[lane + 64] = v.z;
+        a[lane + 96] = v.w;
+      } else {
+        *reinterpret_cast<float4*>(a + 4 * lane) = g.qx ? make_float4(v.w, v.z, v.y, v.x) : v;
+      }
+    };
+    stage(sh[warp], rh);
+    stage(sl[warp], rl);
+    __syncthreads();
+    g.store(S.r, rh);
+    g.store(S.r_lo, rl);
+    CompDotDF dot;
+    dot.add(rh.x, rl.x, rh.x, rl.x);
+    dot.add(rh.y, rl.y, rh.y, rl.y);
+    dot.add(rh.z, rl.z, rh.z, rl.z);
+    dot.add(rh.w, rl.w, rh.w, rl.w);
+    df_axpy(xh.x, xl.x, alpha, ph.x, pl.x);
+    df_axpy(xh.y, xl.y, alpha, ph.y, pl.y);
+    df_axpy(xh.z, xl.z, alpha, ph.z, pl.z);
+    df_axpy(xh.w, xl.w, alpha, ph.w, pl.w);
+    g.store(S.xhi, xh);
+    g.store(S.xlo, xl);
+    if (g.y < S.mhy) {
+      // the warp's class row again, its class cls_y, cls_x = qy, qx
+      const int s0 = warp & ~((1 << g.lseg) - 1);
+      const bool fx = (S.mir & 1) != 0, fy = (S.mir & 2) != 0;
+      const bool xodd = (S.nx & 1) != 0, ymid = fy && S.ny - 1 - g.y == g.y;
+      float2 vh[2], vl[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const size_t idx = (static_cast<size_t>(y) * t.nxp + xb * KC + 64 * k + 2 * lane) / 2;
-        if (t.nr == kLowNS) {
-          uint32_t code[kLowNS];
-          slice_codes2_df<BF16, kLowNS>(ch[c][k], cl[c][k], make_float2(up, up), make_float2(is, is), code);
+        f2 v[2];
 #pragma unroll
-          for (int q = 0; q < kLowNS; ++q) out32[q * (plane / 2) + idx] = code[q];
-        } else {
-          uint32_t code[4];
-          slice_codes2_df<BF16, 4>(ch[c][k], cl[c][k], make_float2(up, up), make_float2(is, is), code);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) out32[q * (plane / 2) + idx] = code[q];
+        for (int e = 0; e < 2; ++e) {
+          const int c = 64 * k + 2 * lane + e;
+          auto at = [&](int s) { return f2{sh[s0 + s][c], sl[s0 + s][c]}; };
+          f2 u = at(0);
+          if (fx) u = df_add(u, g.qx ? df_neg(at(1)) : at(1));
+          if (fy) {
+            f2 m = at(fx ? 2 : 1);
+            if (fx) m = df_add(m, g.qx ? df_neg(at(3)) : at(3));
+            u = df_add(u, g.qy ? df_neg(m) : m);
+          }
+          // the odd classes vanish at the middle column, row
+          const int x = g.xb * KC + c;
+          if ((g.qx && xodd && S.nx - 1 - x == x) || (g.qy && ymid)) u = f2{0.f, 0.f};
+          v[e] = u;
         }
+        vh[k] = make_float2(v[0].hi, v[1].hi);
+        vl[k] = make_float2(v[0].lo, v[1].lo);
       }
-      if (lane == 0) t.e[off + static_cast<ptrdiff_t>(y) * (t.nxp / KC) + xb] = static_cast<int8_t>(E);
+      const ptrdiff_t off = t.step * g.seg;
+      slice_row<BF16>(vh, vl, reinterpret_cast<uint32_t*>(t.out + off),
+                      (static_cast<size_t>(g.y) * t.nxp + g.xb * KC + 2 * lane) / 2, static_cast<size_t>(t.nyp) * t.nxp / 2,
+                      t.nr, reinterpret_cast<int8_t*>(t.e + off + static_cast<ptrdiff_t>(g.y) * (t.nxp / KC) + g.xb), lane);
     }
+    const double rr = block_sum_comp<kVecThreads>(dot.as_comp(), red);
+    if (threadIdx.x == 0) S.part[it.tile * 4 + 0] = rr;
+    if (last_item_block(&sc->cnt[2], S.n_upd_items, &s_last)) {
+      double s = 0.0;
+      if (threadIdx.x < 32) s = warp_sum_strided(S.part, S.n_upd_items, 4);
+      if (threadIdx.x == 0) {
+        decide_update(sc, s);
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -1394,6 +1528,16 @@ void launch_low_mid(const LaunchCfg& c, int mode, int split_kind) {
 void launch_tc_fold(const LaunchCfg& c, int mode, int split_kind) {
   if (split_kind == 0) launch_cfg(c, k_tc_fold<false>, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
   else launch_cfg(c, k_tc_fold<true>, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
+}
+
+template <bool BF16>
+static void launch_update_slice_t(const LaunchCfg& c, bool fuse_pq) {
+  if (fuse_pq) launch_cfg(c, k_update_slice<BF16, true>, c.grid, kVecThreads, 0, c.slots, c.tcp, c.items, c.n_items);
+  else launch_cfg(c, k_update_slice<BF16, false>, c.grid, kVecThreads, 0, c.slots, c.tcp, c.items, c.n_items);
+}
+void launch_update_slice(const LaunchCfg& c, int split_kind, bool fuse_pq) {
+  if (split_kind == 0) launch_update_slice_t<false>(c, fuse_pq);
+  else launch_update_slice_t<true>(c, fuse_pq);
 }
 
 void launch_unfold(const LaunchCfg& c, int mode) {

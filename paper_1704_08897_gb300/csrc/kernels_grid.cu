@@ -828,7 +828,7 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
     const int chunk = S.vec_chunk;
     const int e0 = it.tile * chunk;
     const int e1 = min(n, e0 + chunk);
-    const bool full = e0 + chunk <= n;
+    const bool full = !S.upd_seg && e0 + chunk <= n;
     // one 16-byte vector of every plane per thread and step; the first step's loads pass under the sum
     // of the p.q partials
     float4 ph, pl, qh, ql, rh, rl, xh, xl;
@@ -890,6 +890,33 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
         dot.add(rh.z, rl.z, rh.z, rl.z);
         dot.add(rh.w, rl.w, rh.w, rl.w);
       }
+    } else if (S.upd_seg) {
+      // a small slot among larger ones: the segments, and so the partial sums, of k_update_slice
+      const Seg g = seg_of(S, it.tile);
+      ph = g.load(p);
+      pl = g.load(p_lo);
+      xh = g.load(S.xhi);
+      xl = g.load(S.xlo);
+      df_axpy(xh.x, xl.x, alpha, ph.x, pl.x);
+      df_axpy(xh.y, xl.y, alpha, ph.y, pl.y);
+      df_axpy(xh.z, xl.z, alpha, ph.z, pl.z);
+      df_axpy(xh.w, xl.w, alpha, ph.w, pl.w);
+      qh = g.load(S.q);
+      ql = g.load(S.q_lo);
+      rh = g.load(S.r);
+      rl = g.load(S.r_lo);
+      g.store(S.xhi, xh);
+      g.store(S.xlo, xl);
+      df_axpy(rh.x, rl.x, nalpha, qh.x, ql.x);
+      df_axpy(rh.y, rl.y, nalpha, qh.y, ql.y);
+      df_axpy(rh.z, rl.z, nalpha, qh.z, ql.z);
+      df_axpy(rh.w, rl.w, nalpha, qh.w, ql.w);
+      g.store(S.r, rh);
+      g.store(S.r_lo, rl);
+      dot.add(rh.x, rl.x, rh.x, rl.x);
+      dot.add(rh.y, rl.y, rh.y, rl.y);
+      dot.add(rh.z, rl.z, rh.z, rl.z);
+      dot.add(rh.w, rl.w, rh.w, rl.w);
     } else {
       for (int k = e0 + threadIdx.x; k < e1; k += blockDim.x) {
         float xh = S.xhi[k], xl = S.xlo[k];
@@ -905,9 +932,9 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
     }
     const double rr = block_sum_comp<kVecThreads>(dot.as_comp(), red);
     if (threadIdx.x == 0) S.part[it.tile * 4 + 0] = rr;
-    if (last_item_block(&sc->cnt[2], S.n_vec_items, &s_last)) {
+    if (last_item_block(&sc->cnt[2], S.n_upd_items, &s_last)) {
       double s = 0.0;
-      if (threadIdx.x < 32) s = warp_sum_strided(S.part, S.n_vec_items, 4);
+      if (threadIdx.x < 32) s = warp_sum_strided(S.part, S.n_upd_items, 4);
       if (threadIdx.x == 0) {
         decide_update(sc, s);
       }
