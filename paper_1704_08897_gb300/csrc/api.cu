@@ -3,8 +3,8 @@
 //
 // One solve (Algorithm 1): set-up kernel (mask from sign(phi), b = -M L^2 E_K f), one
 // preconditioner pass, then graph replays of G iterations
-//   [stencil (p = z + beta p, q = M L^2 p, p.q) -> update (x += alpha p in FP64, r, r.r) ->
-//    4 transform stages (z = M (L^2)^+ M r, r.z, z.q)] x G  +  tail [FP64 true residual for slots
+//   [stencil (p = z + beta p, q = M L^2 p, p.q) -> update (x += alpha p, r -= alpha q, r.r) ->
+//    residual slices (or by the update) -> 4 transform stages (z = M (L^2)^+ M r, r.z, z.q)] x G  +  tail [FP64 true residual for slots
 //    due a replacement -> 4 transform stages for slots that continue]
 // until every slot reports a final status.  Batches and the serving loop use the same kernels
 // over work lists that span all slots.
@@ -701,7 +701,6 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   smin = mx0 + my0;
   if (!(smin > 0)) smin = std::min(mx0 + my1, mx1 + my0);
   d.wnorm = (float)(smin * smin);
-  d.zero_mode = (prob.bc_x != EXT_BC_DIRICHLET && prob.bc_y != EXT_BC_DIRICHLET);
   d.lamx = (const float*)(A + o_lx);
   d.lamy = (const float*)(A + o_ly);
   BX_CUDA(cudaMemcpy(A + o_lx, lx.data(), 4 * lx.size(), cudaMemcpyHostToDevice));
@@ -1005,7 +1004,8 @@ static LaunchCfg cfg_of(ext_ctx* ctx, Workspace* W, int which) {
   } else if (which == 9) {
     c.items = W->d_upd;
     c.n_items = W->d_counts + 9;
-    c.grid = std::max(1, std::min(W->n_upd, cap));
+    // in batches the update runs over contiguous ranges of items, one for each resident block
+    c.grid = std::max(1, std::min(W->n_upd, W->slice || W->fuse ? cap : 3 * ctx->sm_count));
   } else if (which == 10) {
     c.items = W->d_prep;
     c.n_items = W->d_counts + 10;
@@ -1104,23 +1104,30 @@ static void harvest(ext_ctx* ctx) {
   cudaGetLastError();
 }
 
+// In batches (more than kFuseSlots grids) the memory-bound kernels and the low-mode middle start on a free
+// device: blocks placed as the previous kernel's leave would load the SMs unevenly (update, fold, slicing
+// and unfold so: 134.7 -> 144.3 solves/s on 256 grids; low-mode middle: 15 us an application on 48).
+static LaunchCfg settled(const Workspace* W, LaunchCfg c) {
+  c.pdl = c.pdl && W->fuse;
+  return c;
+}
+
 // with_finish = false: the next stencil forms rho and beta from the partials itself
 // sliced: the update has left the residuals' slices
 static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish = true, bool sliced = false) {
   const LaunchCfg g = cfg_of(ctx, W, 2), g6 = cfg_of(ctx, W, 11);
   // residual slices: unfolded slots directly, folded slots per mirror class
   if (W->n_prep > 0 && !sliced)
-    timed(ctx, EXT_KERNEL_SPLIT, [&] { launch_prec_tc_prepare(cfg_of(ctx, W, 10), mode, ctx->split); }, g.stream);
+    timed(ctx, EXT_KERNEL_SPLIT, [&] { launch_prec_tc_prepare(settled(W, cfg_of(ctx, W, 10)), mode, ctx->split); },
+          g.stream);
   if (W->n_fold > 0 && !sliced)
-    timed(ctx, EXT_KERNEL_FOLD, [&] { launch_tc_fold(cfg_of(ctx, W, 7), mode, ctx->split); }, g.stream);
+    timed(ctx, EXT_KERNEL_FOLD, [&] { launch_tc_fold(settled(W, cfg_of(ctx, W, 7)), mode, ctx->split); }, g.stream);
   if (W->n_l1 > 0) {
     // the lowest modes in high precision: forward product, middle, inverse product
     LaunchCfg c1 = cfg_of(ctx, W, 5), cm = cfg_of(ctx, W, 12), c3 = cfg_of(ctx, W, 6);
     c1.slots = cm.slots = c3.slots = W->d_tcp;
     timed(ctx, EXT_KERNEL_LOW_FWD, [&] { launch_low_tc(c1, 0, mode, ctx->split, ctx->d_err); }, g.stream);
-    // the middle starts on a free device: blocks placed as the forward product's leave would load
-    // the SMs unevenly (15 us more per application on a batch of 48 grids)
-    cm.pdl = false;
+    cm.pdl = false;  // see settled(): in a call of few grids too
     timed(ctx, EXT_KERNEL_LOW_MID, [&] { launch_low_mid(cm, mode, ctx->split); }, g.stream);
     timed(ctx, EXT_KERNEL_LOW_INV, [&] { launch_low_tc(c3, 1, mode, ctx->split, ctx->d_err); }, g.stream);
   }
@@ -1131,14 +1138,15 @@ static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish =
       timed(ctx, EXT_KERNEL_PREC0 + s, [&] { launch_prec_tc(g6, s, mode, ctx->split, 6, ctx->d_err); }, g.stream);
   }
   if (W->n_unfold > 0)
-    timed(ctx, EXT_KERNEL_UNFOLD, [&] { launch_unfold(cfg_of(ctx, W, 8), mode); }, g.stream);
+    timed(ctx, EXT_KERNEL_UNFOLD, [&] { launch_unfold(settled(W, cfg_of(ctx, W, 8)), mode); }, g.stream);
   if (!with_finish) return;
   const LaunchCfg f = cfg_of(ctx, W, 3);  // one block per slot
   timed(ctx, EXT_KERNEL_PREC_FINISH, [&] { launch_prec_finish(f, mode); }, f.stream);
 }
 
 static void enqueue_iterations(ext_ctx* ctx, Workspace* W, int iters) {
-  const LaunchCfg st = cfg_of(ctx, W, 0), up = cfg_of(ctx, W, 9);
+  const LaunchCfg st = cfg_of(ctx, W, 0);
+  const LaunchCfg up = settled(W, cfg_of(ctx, W, 9));
   const LaunchCfg sc = cfg_of(ctx, W, 4);
   const bool fuse = W->fuse;
   for (int i = 0; i < iters; ++i) {

@@ -36,19 +36,20 @@ constexpr int kLowK3 = 32;          // k extent of the inverse low-mode product
 constexpr int kVecThreads = 256;
 constexpr int kVecStep = 4 * kVecThreads;  // elements a block moves with one vector per thread
 // Elements per work item of the vector kernels (a function of the grid alone, so that the partial
-// sums do not depend on the call): one step up to 2^17 nodes and two up to 2^21 (more blocks at
-// once: the update of a 389 x 251 grid, 24 blocks of four steps before, went from about 13 to 7 us,
-// that of a 1024^2 grid from 14 to 12 us), four beyond (less per-item overhead: 43 us a launch on 48
-// grids of 5.1 M nodes against 61 with one step everywhere).
+// sums do not depend on the call): one step up to 2^17 nodes (the output only: their updates work in
+// segments, seg_of) and two up to 2^21 (more blocks at once: the update of a 1024^2 grid went from 14 to
+// 12 us), four beyond (less per-item overhead: 43 us a launch on 48 grids of 5.1 M nodes against 61
+// with one step everywhere).
+constexpr int vec_chunk_of(long long nodes) {
+  return kVecStep * (nodes <= 1LL << 17 ? 1 : nodes <= 1LL << 21 ? 2 : 4);
+}
+
 // Calls whose grids are all of up to this size have the residuals sliced by the update itself
 // (k_update_slice): one launch less in the chain of an iteration (320 x 256, three fields: 69.7 -> 64 us;
 // 64^2: 50.5 -> 46).  Above, a pass of its own is as fast: the joint kernel holds a segment's planes
 // across a barrier, so that fewer loads are in flight (1024^2: 28 us either way; 48 grids of up to
 // 512^2: 76 us against 62).
 constexpr long long kSliceNodes = 1LL << 17;
-constexpr int vec_chunk_of(long long nodes) {
-  return kVecStep * (nodes <= 1LL << 17 ? 1 : nodes <= 1LL << 21 ? 2 : 4);
-}
 
 enum Bc : int { BC_SYM = 0, BC_PER = 1, BC_DIR = 2 };
 
@@ -120,7 +121,6 @@ struct SlotDesc {
   const float* lamx; // [nxp] eigenvalues of T_x (scaled), padding entries never read
   const float* lamy;
   float wnorm;       // 1 / w_max, so that the scaled weights are <= 1
-  int zero_mode;     // 1: drop the (0,0) mode (both axes symmetric/periodic)
   // transforms: block-scaled integer slices (NS = 4 or 6 16-bit planes) and their TMA descriptors
   void* tc_r;        // [tc_nr][nyp][nxp]  residual
   int tc_ns;         // slices per transform operand: 4 or 6
@@ -216,14 +216,14 @@ __device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
   __syncthreads();
 }
 
-// Last-item protocol, called by every thread of the block after thread 0 has written the item's
-// partials.  Returns true in all threads of the item that completes the slot.
-__device__ __forceinline__ bool last_item_block(unsigned* counter, unsigned total, int* sflag) {
+// Last-item protocol, called by every thread of the block after thread 0 has written the partials of
+// its `items` items.  Returns true in all threads of the block that completes the slot.
+__device__ __forceinline__ bool last_item_block(unsigned* counter, unsigned total, int* sflag, unsigned items = 1) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    const unsigned prev = atomicAdd(counter, 1u);
-    const int last = (prev == total - 1) ? 1 : 0;
+    const unsigned prev = atomicAdd(counter, items);
+    const int last = (prev + items == total) ? 1 : 0;
     if (last) {
       __threadfence();
       *counter = 0u;
@@ -497,6 +497,13 @@ __device__ __forceinline__ double warp_sum_strided(const double* p, int n, int s
   const int l = threadIdx.x & 31;
   double a[4] = {0.0, 0.0, 0.0, 0.0};
   int i = l;
+  for (; i + 224 < n; i += 256) {  // eight loads in flight: the sum of 1024 partials in four trips, not eight
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = __ldcg(p + (size_t)(i + 32 * k) * stride);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) a[k & 3] += v[k];
+  }
   for (; i + 96 < n; i += 128) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) a[k] += __ldcg(p + (size_t)(i + 32 * k) * stride);

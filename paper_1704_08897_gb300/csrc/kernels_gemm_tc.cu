@@ -1345,11 +1345,11 @@ k_unfold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
 // to |r|, is amplified in exactly these modes and costs CG iterations.  The modes kx < 32,
 // ky < 32 (of each transform problem) are therefore left out of stage 1's weights and computed
 // here to about 48 bits:
-//   forward (k_low_tc):  H[y][kx] = sum_x r[y][x] Qx[x][kx], six slices each side, and each
+//   forward (kLowFwd):   H[y][kx] = sum_x r[y][x] Qx[x][kx], six slices each side, and each
 //                        128-row tile's share of G = Qy_low^T H (double-float dot products)
 //   middle (k_low_mid):  G = the shares in tile order, G' = w o G,
 //                        J[ky][x] = sum_kx G'[ky][kx] Qx[x][kx] (double-float), J^T in six slices
-//   inverse (k_low_inv): zl[y][x] = sum_ky Qy[y][ky] J[ky][x], six slices each side
+//   inverse (kLowInv):   zl[y][x] = sum_ky Qy[y][ky] J[ky][x], six slices each side
 // and stage 3 adds zl to its result.  With six 8-bit slices per operand the products of orders
 // 0..5 (21 of them) are kept, each order in its own TMEM accumulator; per k, the products of one
 // order add up to at most 2^17 in magnitude, so over a 128-wide block every partial sum is an

@@ -792,45 +792,78 @@ k_pq_finish(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ ite
   }
 }
 
+// An update item of a small slot among larger ones: the segments, and so the partial sums, of
+// k_update_slice.
+__device__ __forceinline__ CompDotDF update_segment(const SlotDesc& S, int tile, int pi, f2 alpha) {
+  const Seg g = seg_of(S, tile);
+  const f2 nalpha = {-alpha.hi, -alpha.lo};
+  CompDotDF dot;
+  const float4 ph = g.load(S.p[pi]), pl = g.load(S.p_lo[pi]), qh = g.load(S.q), ql = g.load(S.q_lo);
+  float4 rh = g.load(S.r), rl = g.load(S.r_lo), xh = g.load(S.xhi), xl = g.load(S.xlo);
+  df_axpy(xh.x, xl.x, alpha, ph.x, pl.x);
+  df_axpy(xh.y, xl.y, alpha, ph.y, pl.y);
+  df_axpy(xh.z, xl.z, alpha, ph.z, pl.z);
+  df_axpy(xh.w, xl.w, alpha, ph.w, pl.w);
+  g.store(S.xhi, xh);
+  g.store(S.xlo, xl);
+  df_axpy(rh.x, rl.x, nalpha, qh.x, ql.x);
+  df_axpy(rh.y, rl.y, nalpha, qh.y, ql.y);
+  df_axpy(rh.z, rl.z, nalpha, qh.z, ql.z);
+  df_axpy(rh.w, rl.w, nalpha, qh.w, ql.w);
+  g.store(S.r, rh);
+  g.store(S.r_lo, rl);
+  dot.add(rh.x, rl.x, rh.x, rl.x);
+  dot.add(rh.y, rl.y, rh.y, rl.y);
+  dot.add(rh.z, rl.z, rh.z, rl.z);
+  dot.add(rh.w, rl.w, rh.w, rl.w);
+  return dot;
+}
+
 // ---------------------------------------------------------------------------------------------
 // Iteration, stage 2: x += alpha p, r -= alpha q (all double-float), partial ||r||^2.  The last
 // item advances the iteration count and decides stop / residual replacement.  Bound by HBM on large
-// batches (48 B a node; 43 us on 5.1 M nodes, 84% of the measured copy rate) and by the chain of
-// dependent loads and reductions on one grid.  Each thread moves one 16-byte vector of every plane
-// per step, four blocks per SM (64 registers): 128 KB of loads in flight per SM.  alpha arrives as
-// a double-float pair: an FP64 division or conversion repeated by every thread costs more than a
-// step's loads.
+// batches (48 B a node) and by the chain of dependent loads and reductions on one grid.  Each thread
+// moves one 16-byte vector of every plane per step: 96 KB of loads in flight per SM with three blocks
+// (batches), 128 KB with four (few grids, where a slot's items then fit one wave).  alpha arrives as a
+// double-float pair: an FP64 division or conversion repeated by every thread costs more than a
+// step's loads.  A block takes a contiguous range of items, counts its items of a slot at once, and
+// has the next item's first loads in flight under an item's sum: 27.3 M nodes in 215 us (6.1 TB/s, 90% of
+// the measured copy rate); with items strided over the blocks, a fence and a counter update for
+// each, 290.
 // ---------------------------------------------------------------------------------------------
 template <bool FUSE>
-__global__ void __launch_bounds__(kVecThreads, 4)
+__global__ void __launch_bounds__(kVecThreads, FUSE ? 4 : 3)
 k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
          const int* __restrict__ n_items) {
-  __shared__ float2 red[kVecThreads / 32];
-  __shared__ float2 s_alpha;  // FUSE: alpha of slot pq_slot, and whether the slot runs
+  __shared__ float2 red[2][kVecThreads / 32];
+  __shared__ float2 s_alpha;  // FUSE: alpha of the slot, and whether it runs
   __shared__ int s_run, s_last;
-  int pq_slot = -1;
-  f2 alpha = {0.f, 0.f};
-  bool run = false;
   const int total = *n_items;
+  // the block's items: a contiguous range, so that most share a slot
+  const int w0 = static_cast<int>(static_cast<long long>(blockIdx.x) * total / gridDim.x);
+  const int w1 = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * total / gridDim.x);
   // the first item and its descriptor ahead of the wait for the previous kernel
   WorkItem it = {0, 0};
-  if (static_cast<int>(blockIdx.x) < total) it = items[blockIdx.x];
+  if (w0 < w1) it = items[w0];
   pdl_wait();
-  for (int w = blockIdx.x; w < total; w += gridDim.x) {
-    if (w != static_cast<int>(blockIdx.x)) it = items[w];
+  for (int w = w0; w < w1;) {
+    // the items w .. we - 1 of one slot (tiles it.tile, it.tile + 1, ...)
+    if (w != w0) it = items[w];
     const SlotDesc& S = slots[it.slot];
     SlotScalars* sc = S.sc;
+    const int we = min(w1, w + S.n_upd_items - it.tile);
+    const int count = we - w;
+    w = we;
     if (!FUSE && !sc->active) continue;
     const int pi = (sc->it & 1) ^ 1;
     const float* __restrict__ p = S.p[pi];
     const float* __restrict__ p_lo = S.p_lo[pi];
     const int n = S.nx * S.ny;
     const int chunk = S.vec_chunk;
-    const int e0 = it.tile * chunk;
-    const int e1 = min(n, e0 + chunk);
-    const bool full = !S.upd_seg && e0 + chunk <= n;
-    // one 16-byte vector of every plane per thread and step; the first step's loads pass under the sum
-    // of the p.q partials
+    const bool flat = !S.upd_seg;
+    // nodes of the run that lie in whole chunks: one 16-byte vector of every plane per thread and step
+    const int e_run = it.tile * chunk;
+    const int e_whole = flat ? min(e_run + count * chunk, n / chunk * chunk) : 0;
     float4 ph, pl, qh, ql, rh, rl, xh, xl;
     auto load = [&](int e) {
       ph = __ldg(reinterpret_cast<const float4*>(p + e));
@@ -842,97 +875,77 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
       xh = *reinterpret_cast<const float4*>(S.xhi + e);
       xl = *reinterpret_cast<const float4*>(S.xlo + e);
     };
-    if (full) load(e0 + 4 * threadIdx.x);
+    // the first step's loads pass under the sum of the p.q partials
+    if (e_run < e_whole) load(e_run + 4 * threadIdx.x);
+    f2 alpha;
     if (FUSE) {
-      if (it.slot != pq_slot) {
-        if (threadIdx.x < 32) {
-          const bool act = sc->active != 0;  // one reading for the whole block
-          const double pq = sum_pq(S);
-          if (threadIdx.x == 0) {
-            const bool ok = act && pq_ok(sc, pq);
-            const f2 af = ok ? df_of(sc->rho2[sc->it & 1] / pq) : f2{0.f, 0.f};
-            s_alpha = make_float2(af.hi, af.lo);
-            s_run = ok;
-            if (act && it.tile == 0) finish_pq(sc, pq);
-          }
+      if (threadIdx.x < 32) {
+        const bool act = sc->active != 0;  // one reading for the whole block
+        const double pq = sum_pq(S);
+        if (threadIdx.x == 0) {
+          const bool ok = act && pq_ok(sc, pq);
+          const f2 af = ok ? df_of(sc->rho2[sc->it & 1] / pq) : f2{0.f, 0.f};
+          s_alpha = make_float2(af.hi, af.lo);
+          s_run = ok;
+          if (act && it.tile == 0) finish_pq(sc, pq);
         }
-        __syncthreads();
-        alpha = f2{s_alpha.x, s_alpha.y};
-        run = s_run != 0;
-        pq_slot = it.slot;
-        __syncthreads();  // s_alpha and s_run are written again for the next slot
       }
+      __syncthreads();
+      alpha = f2{s_alpha.x, s_alpha.y};
+      const bool run = s_run != 0;
+      __syncthreads();  // s_alpha and s_run are written again for the next slot
       // a breakdown: every block finds the same one, the tile-0 block records it
       if (!run) continue;
     } else {
       alpha = f2{sc->alpha_f[0], sc->alpha_f[1]};
     }
     const f2 nalpha = {-alpha.hi, -alpha.lo};
-    CompDotDF dot;
-    if (full) {
 #pragma unroll 1
-      for (int e = e0 + 4 * threadIdx.x; e < e1; e += kVecStep) {
-        if (e >= e0 + kVecStep) load(e);
-        df_axpy(xh.x, xl.x, alpha, ph.x, pl.x);
-        df_axpy(xh.y, xl.y, alpha, ph.y, pl.y);
-        df_axpy(xh.z, xl.z, alpha, ph.z, pl.z);
-        df_axpy(xh.w, xl.w, alpha, ph.w, pl.w);
-        df_axpy(rh.x, rl.x, nalpha, qh.x, ql.x);
-        df_axpy(rh.y, rl.y, nalpha, qh.y, ql.y);
-        df_axpy(rh.z, rl.z, nalpha, qh.z, ql.z);
-        df_axpy(rh.w, rl.w, nalpha, qh.w, ql.w);
-        *reinterpret_cast<float4*>(S.xhi + e) = xh;
-        *reinterpret_cast<float4*>(S.xlo + e) = xl;
-        *reinterpret_cast<float4*>(S.r + e) = rh;
-        *reinterpret_cast<float4*>(S.r_lo + e) = rl;
-        dot.add(rh.x, rl.x, rh.x, rl.x);
-        dot.add(rh.y, rl.y, rh.y, rl.y);
-        dot.add(rh.z, rl.z, rh.z, rl.z);
-        dot.add(rh.w, rl.w, rh.w, rl.w);
+    for (int k = 0; k < count; ++k) {
+      const int e0 = e_run + k * chunk;
+      CompDotDF dot;
+      if (e0 < e_whole) {
+#pragma unroll 1
+        for (int e = e0 + 4 * threadIdx.x; e < e0 + chunk; e += kVecStep) {
+          df_axpy(xh.x, xl.x, alpha, ph.x, pl.x);
+          df_axpy(xh.y, xl.y, alpha, ph.y, pl.y);
+          df_axpy(xh.z, xl.z, alpha, ph.z, pl.z);
+          df_axpy(xh.w, xl.w, alpha, ph.w, pl.w);
+          df_axpy(rh.x, rl.x, nalpha, qh.x, ql.x);
+          df_axpy(rh.y, rl.y, nalpha, qh.y, ql.y);
+          df_axpy(rh.z, rl.z, nalpha, qh.z, ql.z);
+          df_axpy(rh.w, rl.w, nalpha, qh.w, ql.w);
+          *reinterpret_cast<float4*>(S.xhi + e) = xh;
+          *reinterpret_cast<float4*>(S.xlo + e) = xl;
+          *reinterpret_cast<float4*>(S.r + e) = rh;
+          *reinterpret_cast<float4*>(S.r_lo + e) = rl;
+          dot.add(rh.x, rl.x, rh.x, rl.x);
+          dot.add(rh.y, rl.y, rh.y, rl.y);
+          dot.add(rh.z, rl.z, rh.z, rl.z);
+          dot.add(rh.w, rl.w, rh.w, rl.w);
+          // the next step's loads, the next item's too, pass under the item's sum
+          if (e + kVecStep < e_whole) load(e + kVecStep);
+        }
+      } else if (!flat) {
+        dot = update_segment(S, it.tile + k, pi, alpha);
+      } else {
+        for (int e = e0 + threadIdx.x; e < n; e += blockDim.x) {  // the ragged last chunk
+          float xh = S.xhi[e], xl = S.xlo[e];
+          df_axpy(xh, xl, alpha, p[e], p_lo[e]);
+          S.xhi[e] = xh;
+          S.xlo[e] = xl;
+          float rh = S.r[e], rl = S.r_lo[e];
+          df_axpy(rh, rl, nalpha, S.q[e], S.q_lo[e]);
+          S.r[e] = rh;
+          S.r_lo[e] = rl;
+          dot.add(rh, rl, rh, rl);
+        }
       }
-    } else if (S.upd_seg) {
-      // a small slot among larger ones: the segments, and so the partial sums, of k_update_slice
-      const Seg g = seg_of(S, it.tile);
-      ph = g.load(p);
-      pl = g.load(p_lo);
-      xh = g.load(S.xhi);
-      xl = g.load(S.xlo);
-      df_axpy(xh.x, xl.x, alpha, ph.x, pl.x);
-      df_axpy(xh.y, xl.y, alpha, ph.y, pl.y);
-      df_axpy(xh.z, xl.z, alpha, ph.z, pl.z);
-      df_axpy(xh.w, xl.w, alpha, ph.w, pl.w);
-      qh = g.load(S.q);
-      ql = g.load(S.q_lo);
-      rh = g.load(S.r);
-      rl = g.load(S.r_lo);
-      g.store(S.xhi, xh);
-      g.store(S.xlo, xl);
-      df_axpy(rh.x, rl.x, nalpha, qh.x, ql.x);
-      df_axpy(rh.y, rl.y, nalpha, qh.y, ql.y);
-      df_axpy(rh.z, rl.z, nalpha, qh.z, ql.z);
-      df_axpy(rh.w, rl.w, nalpha, qh.w, ql.w);
-      g.store(S.r, rh);
-      g.store(S.r_lo, rl);
-      dot.add(rh.x, rl.x, rh.x, rl.x);
-      dot.add(rh.y, rl.y, rh.y, rl.y);
-      dot.add(rh.z, rl.z, rh.z, rl.z);
-      dot.add(rh.w, rl.w, rh.w, rl.w);
-    } else {
-      for (int k = e0 + threadIdx.x; k < e1; k += blockDim.x) {
-        float xh = S.xhi[k], xl = S.xlo[k];
-        df_axpy(xh, xl, alpha, p[k], p_lo[k]);
-        S.xhi[k] = xh;
-        S.xlo[k] = xl;
-        float rh = S.r[k], rl = S.r_lo[k];
-        df_axpy(rh, rl, nalpha, S.q[k], S.q_lo[k]);
-        S.r[k] = rh;
-        S.r_lo[k] = rl;
-        dot.add(rh, rl, rh, rl);
-      }
+      // double-buffered: an item's sum is read before the barrier of the next one's
+      const double rr = block_sum_comp<kVecThreads>(dot.as_comp(), red[k & 1]);
+      if (threadIdx.x == 0) S.part[(it.tile + k) * 4 + 0] = rr;
     }
-    const double rr = block_sum_comp<kVecThreads>(dot.as_comp(), red);
-    if (threadIdx.x == 0) S.part[it.tile * 4 + 0] = rr;
-    if (last_item_block(&sc->cnt[2], S.n_upd_items, &s_last)) {
+    if (last_item_block(&sc->cnt[2], S.n_upd_items, &s_last, count)) {
       double s = 0.0;
       if (threadIdx.x < 32) s = warp_sum_strided(S.part, S.n_upd_items, 4);
       if (threadIdx.x == 0) {

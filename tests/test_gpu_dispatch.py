@@ -60,7 +60,8 @@ def _problem(ext, nx, ny, seed):
     [(500, 500)] * 3 + [(260, 300)] * 5 + [(128, 128)],
 ], ids=["one-large", "edge-2^17", "ten-small", "many-tiles"])
 def test_a_grid_solves_the_same_in_any_company(ext, prec, sides):
-    c = ext.ext_create(ext.options(prec, rtol=1e-5, maxit=60, low_modes=0))
+    # bf16: six slices up to 768^2 nodes (automatic); fp16: four everywhere
+    c = ext.ext_create(ext.options(prec, rtol=1e-5, maxit=60, low_modes=0 if prec == "mixed_fp16" else 2))
     try:
         cases = [_problem(ext, nx, ny, i) for i, (nx, ny) in enumerate(sides)]
         single = []
@@ -79,7 +80,7 @@ def test_a_grid_solves_the_same_in_any_company(ext, prec, sides):
 
 def test_slices_by_grid_size_do_not_depend_on_company(ext):
     """768 x 768 nodes (six slices), one row more (four), and a small grid, alone and together."""
-    c = ext.ext_create(ext.options("mixed_bf16", rtol=1e-5, maxit=20, low_modes=0))
+    c = ext.ext_create(ext.options("mixed_bf16", rtol=1e-5, maxit=20))
     try:
         cases = [_problem(ext, nx, ny, i) for i, (nx, ny) in enumerate([(768, 768), (768, 769), (100, 100)])]
         single = []
