@@ -40,10 +40,6 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
 CSRC = os.path.join(ROOT, "paper_1704_08897_gb300", "csrc")
 
-# FP32 CUDA-core peak of a GB300 derived from unit counts and clock:
-# 152 SMs x 128 FP32 lanes x 2 flop (FMA) x 2.07 GHz.
-FP32_ALU_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
-
 
 def parse():
     ap = argparse.ArgumentParser()
@@ -129,9 +125,19 @@ def mirror_classes(n, fold=True):
     return [h, h] if fold and 2 * pad(h) <= pad(n) else [n]
 
 
-def issued_tensor_flop(probs, kind, fold=None):
-    """Flops the tensor cores execute in one launch of transform stage `kind` (mixed modes), over
-    the transform problems (mirror classes) of every instance."""
+def stage_products(p, prec, low):
+    """Slice products per useful product of a grid's transform stages: six slices (21) on the FP32
+    path, and in the mixed modes' automatic setting on grids of at most 768^2 nodes when the low-mode
+    correction is off; else four (10)."""
+    auto = _OPTION_OVERRIDES.get("low_modes", 2) == 2
+    return TC_LOW_PRODUCTS if prec == "fp32" or (auto and not low and p.nx * p.ny <= 768 ** 2) else TC_PRODUCTS
+
+
+def issued_tensor_flop(probs, kind, fold=None, products=lambda p: TC_PRODUCTS):
+    """Flops of one launch of transform stage `kind` on padded tiles, over the transform problems
+    (mirror classes) of every instance; products(p): slice products per useful product.  (Tiles of
+    nothing but padding, and steps of nothing but padding along k, are passed over: an upper bound
+    where a class's sides are not multiples of 64.)"""
     fold = _fold_default() if fold is None else fold
     pad = lambda n: -(-n // TC_PAD) * TC_PAD
     fl = 0
@@ -144,7 +150,7 @@ def issued_tensor_flop(probs, kind, fold=None):
                     fl += 2 * TC_LOW_PRODUCTS * pad(cx) * pad(cy) * 64
                 else:
                     s = int(kind[-1])
-                    fl += 2 * TC_PRODUCTS * pad(cx) * pad(cy) * pad(cx if s in (0, 2) else cy)
+                    fl += 2 * products(p) * pad(cx) * pad(cy) * pad(cx if s in (0, 2) else cy)
     return fl
 
 
@@ -168,7 +174,7 @@ def algorithmic_cost(probs, kind, low=False):
     # CG vectors are double-float pairs of FP32 planes: 8 bytes per node each
     if kind == "stencil":   # read z, p_old (8 + 8), mask (1); write p, q (8 + 8)
         return sum(33 * p.nx * p.ny for p in probs), "byte"
-    if kind == "update":    # read x, p, q, r; write x, r (8 bytes each)
+    if kind == "update":    # read x, p, q, r; write x, r (8 bytes each); slices it leaves not counted
         return sum(48 * p.nx * p.ny for p in probs), "byte"
     if kind in ("split", "fold"):  # read r (8); write four (six) 16-bit slices: unfolded / folded
         f = kind == "fold"
@@ -426,19 +432,15 @@ def run_ours(args, rank, world):
         amount, unit = algorithmic_cost(probs, dom, low="low_fwd" in kernels)
         if amount is not None and n:
             per_launch_s = ms / n / 1e3
-            if unit == "flop" and prec != "fp32":
+            if unit == "flop":
                 # tensor-core stage: algorithmic flops (2 n^3-type, unpadded) against the measured
-                # sustained dense BF16 peak; the MMAs actually issued (ten slice products over
+                # sustained dense BF16 peak; the MMAs actually issued (ten or 21 slice products over
                 # padded tiles) are reported beside it
                 achieved = amount / per_launch_s / 1e12
                 with open(PEAKS_FILE) as fh:
                     peak = json.load(fh)["bf16_tflops_sustained"]
                 bound, u = "tensor", "TFLOP/s"
                 peak_src = "measured bf16_tflops_sustained"
-            elif unit == "flop":
-                achieved = amount / per_launch_s / 1e12
-                peak, bound, u = FP32_ALU_PEAK_TFLOPS, "alu", "TFLOP/s"
-                peak_src = "derived: 152 SM x 128 FP32 lanes x 2 x 2.07 GHz"
             else:
                 achieved = amount / per_launch_s / 1e9
                 with open(PEAKS_FILE) as fh:
@@ -468,10 +470,13 @@ def run_ours(args, rank, world):
             kernels_hbm = hbm
             if bound == "tensor":
                 # what the tensor pipe actually executes: the exact slice products on padded tiles
-                issued = issued_tensor_flop(probs, dom) / per_launch_s / 1e12
+                low = "low_fwd" in kernels
+                issued = issued_tensor_flop(probs, dom, products=lambda p: stage_products(p, prec, low))
+                issued = issued / per_launch_s / 1e12
                 roofline["issued"] = {"achieved": round(issued, 3), "frac": round(issued / peak, 4),
                                       "products_per_useful_product":
-                                          TC_LOW_PRODUCTS if dom.startswith("low") else TC_PRODUCTS,
+                                          TC_LOW_PRODUCTS if dom.startswith("low") else
+                                          sorted({stage_products(p, prec, low) for p in probs}),
                                       "pad": TC_PAD}
 
     ext.ext_destroy(ctx)
@@ -546,8 +551,8 @@ PAPER_EXAMPLE2 = {32: (21, 1.08e-01), 64: (46, 3.42e-02), 128: (112, 1.07e-02), 
 
 def peanut3d_leg(sides=(64, 128, 256)):
     """The three-dimensional extension (Sec. 3 Example 2): the peanut on [-pi, pi]^3, periodic,
-    extend out, through ext_solve3d, on the FP32 path (CUDA-core transforms) and, for sides that
-    are multiples of 128, the mixed path (tensor-core transforms).  Per side and path: time and
+    extend out, through ext_solve3d, on the FP32 path (transforms on the CUDA cores, or with six slices
+    on the tensor cores for sides that are multiples of 128) and, for such sides, the mixed path.  Per side and path: time and
     iterations at rel-res 1e-8 and at the paper's 1e-6 (beside the printed iterations), and the
     max error within one grid cell of the interface against the analytic field."""
     import numpy as np

@@ -46,10 +46,11 @@ typedef enum { EXT_EXTEND_OUT = 0, EXT_EXTEND_IN = 1 } ext_dir;
  * updated in FP64 every iteration, and the recursive residual is replaced by the FP64 true
  * residual b - A x whenever it has fallen by replace_factor since the last replacement, at
  * least every true_res_every iterations, and before convergence is declared.
- *   FP32        : FP32 vectors, compensated FP32 stencil, FP32 CUDA-core transform products.
- *   MIXED_FP16  : as FP32, transforms on the tcgen05 tensor cores: every operand as four exact
- *                 8-bit integer slices per 128-wide exponent block, stored as FP16, products
- *                 summed exactly per slice order in FP32 accumulators.
+ *   FP32        : double-float vectors (pairs of FP32), compensated stencil, transforms on the tcgen05
+ *                 tensor cores with every operand as six exact 8-bit integer slices per 128-wide
+ *                 exponent block (48 bits, the accuracy of the vectors).
+ *   MIXED_FP16  : as FP32 with four slices per operand (32 bits) on larger grids (see low_modes),
+ *                 stored as FP16, products summed exactly per slice order in FP32 accumulators.
  *   MIXED_BF16  : the same slices stored as BF16 (results identical to MIXED_FP16).
  * The iteration runs on 2^e b with e chosen from ||b||; the answer is scaled back exactly.    */
 typedef enum {
@@ -94,14 +95,16 @@ typedef struct {
                               0 = all modes from the four-slice stages; 2 = on for grids with a
                               side of at least 2048 nodes and for every grid of an ext_solve /
                               ext_solve_batch / ext_solve_multi call whose grids hold at least
-                              2048^2 nodes together, off otherwise (default; served requests
-                              take the per-grid rule).  With 2, a grid's iterates therefore
-                              depend on the call it is solved in; 0 or 1 fix them.            */
+                              2048^2 nodes together; of the others, grids of at most 768^2
+                              nodes take six slices in every stage and larger ones four
+                              (default; served requests take the per-grid rule).  With 2, a
+                              grid's iterates therefore depend on the call it is solved in; 0
+                              or 1 fix them.                                                   */
   int64_t wait_cycles;     /* bound, in SM clock cycles, of every wait of a kernel for its own
                               tensor copies and tensor-core pipeline; a wait that runs out makes
                               the kernel drain what it issued and return, and the call returns
                               EXT_ETIMEOUT; 0 = 4e9 (about two seconds)                       */
-  int32_t fold;            /* mixed modes: 1 = an axis whose two mirror classes (ceil(n/2) nodes
+  int32_t fold;            /* 1 = an axis whose two mirror classes (ceil(n/2) nodes
                               each), padded to 128, fit in the axis padded to 128 runs its
                               transforms per class (even and odd vectors under i -> n-1-i: half
                               the products per stage) (default); 0 = full-size transforms      */
@@ -111,14 +114,15 @@ typedef struct {
 enum {
   EXT_KERNEL_SETUP = 0,          /* mask, right-hand side, CG state                          */
   EXT_KERNEL_STENCIL = 1,        /* p = z + beta p, q = M L^2 p, p.q                         */
-  EXT_KERNEL_UPDATE = 2,         /* x += alpha p, r -= alpha q, r.r                          */
+  EXT_KERNEL_UPDATE = 2,         /* x += alpha p, r -= alpha q, r.r; with only grids of up to 2^17
+                                    nodes in the call also SPLIT's and FOLD's work             */
   EXT_KERNEL_TRUE_RESIDUAL = 3,  /* FP64 b - A x and residual replacement                    */
   EXT_KERNEL_PREC0 = 4,          /* transform stages 0..3 of the fast Poisson preconditioner */
   EXT_KERNEL_PREC1 = 5,
   EXT_KERNEL_PREC2 = 6,
   EXT_KERNEL_PREC3 = 7,
   EXT_KERNEL_OUTPUT = 8,         /* out = f on Omega, x elsewhere                            */
-  EXT_KERNEL_SPLIT = 9,          /* residual -> 16-bit integer slices (mixed modes, unfolded)  */
+  EXT_KERNEL_SPLIT = 9,          /* residual -> 16-bit integer slices (unfolded slots)          */
   EXT_KERNEL_PREC_FINISH = 10,   /* per-slot r.z, z.q -> rho, beta                            */
   EXT_KERNEL_PQ_FINISH = 11,     /* per-slot p.q -> alpha                                     */
   EXT_KERNEL_LOW_FWD = 12,       /* low-mode correction: forward product, middle, inverse    */
@@ -268,9 +272,10 @@ int ext_axis_basis(int32_t n, ext_bc bc, double* Q, double* lam);
 /* Three-dimensional extension (Sec. 3 Example 2).  Solves the masked biharmonic system on the
  * nz x ny x nx box by preconditioned CG from x = 0 to the context's rtol (relative FP64 residual on
  * the unknowns), the preconditioner being the fast Poisson solve on the box by separable
- * transforms along the three axes.  It runs the CUDA-core double-float path in every precision
- * mode (double-float CG vectors, compensated products in the transforms, FP64 right-hand side and
- * residual replacements), one problem per call, the iteration driven from the host.  phi, f and
+ * transforms along the three axes (double-float CG vectors, FP64 right-hand side and residual
+ * replacements): with every side a multiple of 128 the transforms run as exact slice products on the
+ * tensor cores, as in two dimensions, else as compensated double-float products on the CUDA cores.
+ * One problem per call; the host enqueues blocks of iterations ahead of the scalars it reads.  phi, f and
  * out are device pointers ([nz][ny][nx] float32; host pointers return EXT_EINVAL); out = f at
  * known nodes (bit copy), the extension elsewhere; out may alias f.  res (may be NULL) receives
  * status, iterations, the true and recursive relative residuals, counts and err_est.  Returns
