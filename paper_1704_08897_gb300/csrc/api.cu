@@ -516,6 +516,14 @@ static std::string shape_key(int count, const ext_problem* probs, bool host_io) 
   return k;
 }
 
+// The memsets and copies of a set-up run on the legacy stream, the kernels on streams that do not wait
+// for it, and a memset (or a small copy from pageable memory) may still be in flight when its call
+// returns: wait for them once, at the end.
+static int set_up_done() {
+  BX_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+  return EXT_OK;
+}
+
 // Device state of one problem: plans, arena layout (allocated here unless `arena` is given), slot
 // descriptor, its tensor-core problems and their tensor maps.  With size_only, only s.bytes is
 // computed.
@@ -805,7 +813,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   }
   s.n_tcp = (int)tl.size();
   if (!d.mir) d = s.tcp[0];  // the slot is its own problem (k_tc_prepare reads it)
-  return EXT_OK;
+  return set_up_done();
 }
 
 // The slot's scalars, in the slot descriptor and in each of its tensor-core problems.
@@ -963,6 +971,8 @@ static int build_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bo
   BX_CUDA(cudaMalloc(&W->d_outs, sizeof(void*) * count));
   BX_CUDA(cudaMalloc(&W->d_dirs, sizeof(int) * count));
   BX_CUDA(cudaMallocHost(&W->h_ptrs, (3 * sizeof(void*) + sizeof(int)) * count));
+  rc = set_up_done();
+  if (rc) return rc;
   *out = W.release();
   return EXT_OK;
 }
@@ -1893,7 +1903,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   t.part = part;
   t.n_tiles3 = counts[6];
   t.on = true;
-  return EXT_OK;
+  return set_up_done();
 }
 
 int ext_solve3d(ext_ctx* ctx, const ext_problem3* prob, const float* phi, const float* f, float* out,

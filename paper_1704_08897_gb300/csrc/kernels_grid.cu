@@ -827,9 +827,9 @@ __device__ __forceinline__ CompDotDF update_segment(const SlotDesc& S, int tile,
 // (batches), 128 KB with four (few grids, where a slot's items then fit one wave).  alpha arrives as a
 // double-float pair: an FP64 division or conversion repeated by every thread costs more than a
 // step's loads.  A block takes a contiguous range of items, counts its items of a slot at once, and
-// has the next item's first loads in flight under an item's sum: 27.3 M nodes in 215 us (6.1 TB/s, 90% of
+// has the next item's first loads in flight under an item's sum: 27.3 M nodes in 222 us (5.9 TB/s, 87% of
 // the measured copy rate); with items strided over the blocks, a fence and a counter update for
-// each, 290.
+// each, 295.
 // ---------------------------------------------------------------------------------------------
 template <bool FUSE>
 __global__ void __launch_bounds__(kVecThreads, FUSE ? 4 : 3)
