@@ -198,6 +198,15 @@ bool bx::is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// The memsets and copies of a set-up run on the legacy stream, the kernels on streams that do not wait
+// for it, and a memset (or a small copy from pageable memory) may still be in flight when its call
+// returns: every set-up waits for its own
+// once, at its end.
+static int set_up_done() {
+  BX_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+  return EXT_OK;
+}
+
 // ---- tensor-core operands --------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
@@ -436,7 +445,7 @@ static int ensure_df_plan(PlanDev* P) {
   }
   BX_CUDA(cudaMemcpy(P->q, q.data(), bytes, cudaMemcpyHostToDevice));
   BX_CUDA(cudaMemcpy(P->qt, qt.data(), bytes, cudaMemcpyHostToDevice));
-  return EXT_OK;
+  return set_up_done();
 }
 
 // Stencil weights of (L_y (+) L_x)^2 scaled by 1/max(a, c)^2, a = 1/hx^2, c = 1/hy^2
@@ -514,14 +523,6 @@ static std::string shape_key(int count, const ext_problem* probs, bool host_io) 
     k += buf;
   }
   return k;
-}
-
-// The memsets and copies of a set-up run on the legacy stream, the kernels on streams that do not wait
-// for it, and a memset (or a small copy from pageable memory) may still be in flight when its call
-// returns: wait for them once, at the end.
-static int set_up_done() {
-  BX_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
-  return EXT_OK;
 }
 
 // Device state of one problem: plans, arena layout (allocated here unless `arena` is given), slot
@@ -1247,7 +1248,7 @@ static int set_stencil_shape(ext_ctx* ctx, Workspace* W, int ty) {
   BX_CUDA(cudaMemcpy(W->d_slots, descs.data(), sizeof(SlotDesc) * descs.size(), cudaMemcpyHostToDevice));
   W->sten_ty = ty;
   drop_graphs(W);
-  return EXT_OK;
+  return set_up_done();
 }
 
 // Tuning results by workspace shape, shared by the contexts of the process and, when the
@@ -1596,6 +1597,8 @@ int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out) {
     BX_CUDA(cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking));
     ctx->own_stream = true;
   }
+  const int rc = set_up_done();
+  if (rc) return rc;
   *out = ctx.release();
   return EXT_OK;
 }
@@ -2247,6 +2250,7 @@ static int serve_init(ext_ctx* ctx) {
   BX_CUDA(cudaMalloc(&S->d_aux, 2 * sizeof(int)));
   BX_CUDA(cudaMallocHost(&S->h_aux, 2 * sizeof(int)));
   int rc = serve_alloc_lists(S.get(), 1 << 16);
+  if (!rc) rc = set_up_done();
   if (rc) return rc;
   size_t fr = 0, tot = 0;
   BX_CUDA(cudaMemGetInfo(&fr, &tot));

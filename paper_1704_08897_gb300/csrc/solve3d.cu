@@ -946,7 +946,8 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
     int flag = 0;
     BX3(cudaMemcpy(&flag, s.tc.d_err, sizeof(int), cudaMemcpyDeviceToHost));
     if (flag) {
-      BX3(cudaMemset(s.tc.d_err, 0, sizeof(int)));
+      BX3(cudaMemsetAsync(s.tc.d_err, 0, sizeof(int), st));
+      BX3(cudaStreamSynchronize(st));
       *err = "a bounded device wait (tensor-core pipeline) ran out";
       res->status = EXT_ETIMEOUT;
       return EXT_ETIMEOUT;

@@ -1,0 +1,61 @@
+// The few kernels that the runtime without a device models: the end of a block of iterations
+// (k_true_residual; in three dimensions k3_finish<3>), which counts fake_model's iterations and decides;
+// the 3-D set-up's counts and norm; and the transform products, which raise the time-out flag on demand.
+#include "model.h"
+
+#include "../../paper_1704_08897_gb300/csrc/common.cuh"
+
+static struct Model {
+  int its = 1;           // iterations a block makes
+  int ok_after = 0;      // blocks until convergence (0: never)
+  int err_after = 0;     // transform products until one raises the time-out flag (0: none)
+  int blocks = 0, products = 0;
+} model;
+
+// what the kernel does, with its arguments read now
+std::function<void()> body(const std::string& k, void** a) {
+  using bx::SlotScalars;
+  auto block_end = [](SlotScalars* sc) {
+    if (sc->status != bx::ST_RUNNING) return;
+    ++model.blocks;
+    sc->it += model.its;
+    sc->rr = sc->rr_true = sc->bb * 1e-4 / model.blocks;
+    if (model.ok_after && model.blocks >= model.ok_after) sc->status = bx::ST_OK;
+    else if (sc->it >= sc->maxit) sc->status = bx::ST_ENOTCONV;
+  };
+  if (k.find("k_true_residual") != std::string::npos) {
+    auto slots = *(const bx::SlotDesc**)a[0];
+    auto items = *(const bx::WorkItem**)a[1];
+    auto n = *(const int**)a[2];
+    return [=] {
+      for (int i = 0; i < *n; ++i)
+        if (items[i].tile == 0) block_end(slots[items[i].slot].sc);
+    };
+  }
+  if (k.find("k3_finishILi3E") != std::string::npos) {
+    auto sc = *(SlotScalars**)a[0];
+    return [=] { block_end(sc); };
+  }
+  if (k.find("k3_setup") != std::string::npos) {
+    const size_t n = *(size_t*)a[0];
+    auto c = *(unsigned long long**)a[6];
+    return [=] { c[0] = n / 2, c[1] = n - n / 2; };
+  }
+  if (k.find("k3_sum") != std::string::npos) {
+    auto out = *(double**)a[2];
+    return [=] { *out = 1.0; };
+  }
+  if (k.find("k_prec_tc") != std::string::npos) {
+    auto err = *(int**)a[4];
+    return [=] {
+      if (++model.products == model.err_after) *err = 1;
+    };
+  }
+  return [] {};
+}
+
+extern "C" {
+void fake_model(int its, int ok_after, int err_after) { model = Model{its, ok_after, err_after, 0, 0}; }
+int fake_blocks() { return model.blocks; }
+int fake_products() { return model.products; }
+}

@@ -1,0 +1,97 @@
+"""The library's host code on the CPU, over a CUDA runtime without a device (fake_cuda/cudart.cu): what
+the host does around the kernels, which no result on a GPU shows reliably."""
+
+import os
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes as C, itertools, sys
+import numpy as np
+sys.path.insert(0, {root!r})
+from paper_1704_08897_gb300 import ext
+fake = C.CDLL({fake!r})
+fake.fake_fail_malloc.argtypes = [C.c_long]
+fake.fake_mallocs.restype = C.c_long
+fake.fake_live_bytes.restype = C.c_size_t
+rt = C.CDLL({fake!r})
+class Dev:  # an array in "device" memory
+    def __init__(self, n, itemsize=4):
+        p = C.c_void_p()
+        rt.cudaMalloc(C.byref(p), C.c_size_t(n * itemsize))
+        C.memset(p, 0, n * itemsize)
+        self.p = p.value
+    def is_contiguous(self): return True
+    def data_ptr(self): return self.p
+def faults():
+    b = C.create_string_buffer(1 << 16)
+    fake.fake_faults(b, len(b))
+    return b.value.decode()
+"""
+
+
+@pytest.fixture(scope="session")
+def fake_cuda(tmp_path_factory):
+    """Runs a script with the fake runtime in front; returns what it printed."""
+    from paper_1704_08897_gb300 import build_ext, ext
+    build_ext.build()
+    so = str(tmp_path_factory.mktemp("fake") / "libfakecudart.so")
+    subprocess.run([build_ext._nvcc(), "-std=c++17", "-O1", *build_ext.ARCH, "--cudart", "none", "-shared",
+                    "-Xcompiler", "-fPIC", "-diag-suppress", "177", os.path.join(HERE, "fake_cuda", "model.cu"),
+                    os.path.join(HERE, "fake_cuda", "cudart.cpp"),
+                    "-o", so], check=True, capture_output=True)
+
+    def run(script):
+        env = dict(os.environ, LD_PRELOAD=so)
+        env.pop("EXT_TUNE_CACHE", None)
+        p = subprocess.run([sys.executable, "-c", PRELUDE.format(root=ROOT, fake=so) + script], env=env,
+                           capture_output=True, text=True, timeout=300)
+        assert p.returncode == 0, p.stdout + p.stderr
+        return p.stdout
+    return run
+
+
+# Every way into the library that sets something up for kernels on a stream of its own.
+CALLS = """
+def calls():
+    phi, f, out = Dev(96 * 80), Dev(96 * 80), Dev(96 * 80)
+    prob = ext.problem(96, 80, "symmetric", "periodic")
+    for prec in ("fp32", "mixed_bf16"):
+        for kw in (dict(), dict(autotune=0, tile_y=16), dict(low_modes=1)):
+            c = ext.ext_create(ext.options(prec, **kw))
+            yield "solve", lambda: ext.ext_solve(c, prob, phi, f, out, check=False)
+            yield "batch", lambda: ext.ext_solve_batch(c, [prob] * 2, [phi] * 2, [f] * 2, [out] * 2, check=False)
+            yield "served", lambda: (ext.ext_submit(c, prob, phi, f, out), ext.ext_drain(c))
+            ext.ext_destroy(c)
+            c = ext.ext_create(ext.options(prec, **kw))
+            yield "operator", lambda: ext.ext_apply_biharmonic(c, prob, phi, f, out)
+            ext.ext_destroy(c)
+            c = ext.ext_create(ext.options(prec, **kw))
+            yield "preconditioner", lambda: ext.ext_apply_preconditioner(c, prob, phi, f, out)
+            ext.ext_destroy(c)
+        for n in (12, 128):
+            v = [Dev(n * n * 128) for _ in range(3)]
+            p3 = ext.problem3(n, n, 128)
+            for call in (ext.ext_apply_biharmonic3d, ext.ext_apply_preconditioner3d, ext.ext_solve3d):
+                c = ext.ext_create(ext.options(prec))
+                yield call.__name__, lambda: call(c, p3, *v)
+                ext.ext_destroy(c)
+"""
+
+
+def test_set_up_is_complete_before_kernels_on_other_streams(fake_cuda):
+    """Copies and memsets of the legacy stream may be in flight when their calls return, and the kernels'
+    streams do not wait for that stream: each set-up has to wait before the first operation of another
+    stream follows."""
+    out = fake_cuda(CALLS + """
+fake.fake_model(5, 3, 0)
+for name, call in calls():
+    call()
+print(faults())
+""")
+    assert out.strip() == ""
