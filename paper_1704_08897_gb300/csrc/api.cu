@@ -337,22 +337,24 @@ static void slice_plan_host(int n, int bc, int np, int split, std::vector<uint16
 }
 
 static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P, int ns) {
-  void*& tc = P->tc[ns == 6];
-  if (tc) return EXT_OK;
+  if (P->tc[ns == 6]) return EXT_OK;
   std::vector<uint16_t> h;
   std::vector<int8_t> ex;
   const AxisBasis B = plan_basis(P->nfull, P->bc, P->cls);
   slice_plan_basis(B, P->np, ctx->split, ns, h, ex);
   const size_t bytes = 2 * h.size() + ex.size();
+  void* tc = nullptr;
   if (cudaMalloc(&tc, bytes) != cudaSuccess) {
     cudaGetLastError();
-    tc = nullptr;
     g_last_error = "cudaMalloc of tensor-core plan failed";
     return EXT_ENOMEM;
   }
   BX_CUDA(cudaMemcpy(tc, h.data(), 2 * h.size(), cudaMemcpyHostToDevice));
   BX_CUDA(cudaMemcpy((char*)tc + 2 * h.size(), ex.data(), ex.size(), cudaMemcpyHostToDevice));
-  if (ns == 6) return EXT_OK;  // no low-mode correction beside six slices
+  if (ns == 6) {  // no low-mode correction beside six slices
+    P->tc[1] = tc;
+    return EXT_OK;
+  }
   // low-mode operands of the same basis
   const int np = P->np, nkb = np / tc_block();
   const int m = std::min(kLowM, P->n);
@@ -390,6 +392,7 @@ static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P, int ns) {
   if (cudaMalloc(&P->low, lbytes) != cudaSuccess) {
     cudaGetLastError();
     P->low = nullptr;
+    cudaFree(tc);  // a plan is kept whole or not at all
     g_last_error = "cudaMalloc of low-mode plan failed";
     return EXT_ENOMEM;
   }
@@ -399,6 +402,7 @@ static int ensure_tc_plan(ext_ctx* ctx, PlanDev* P, int ns) {
   BX_CUDA(cudaMemcpy(L + P->low_off_q, lq.data(), 2 * lq.size(), cudaMemcpyHostToDevice));
   BX_CUDA(cudaMemcpy(L + P->low_off_qe, lqe.data(), lqe.size(), cudaMemcpyHostToDevice));
   BX_CUDA(cudaMemcpy(L + P->low_off_d, ld.data(), 4 * ld.size(), cudaMemcpyHostToDevice));
+  P->tc[0] = tc;
   return EXT_OK;
 }
 

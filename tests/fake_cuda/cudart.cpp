@@ -6,7 +6,7 @@
 //    pageable memory, of the legacy stream may still be in flight (both may return before the device has
 //    done them, and a non-blocking stream does not wait for the legacy one): only a synchronisation of the
 //    legacy stream or a copy back ends that;
-//  * a copy, a memset or a tensor map outside a live allocation.
+//  * a copy, a memset, a tensor map or a work list outside a live allocation.
 #include <cuda.h>
 #include <cuda_runtime_api.h>
 
@@ -38,6 +38,10 @@ std::map<cudaStream_t, Graph*> capturing;
 
 using Lock = std::lock_guard<std::recursive_mutex>;
 
+}  // namespace
+void fault(const std::string& what) { faults.push_back(what); }
+namespace {
+
 bool legacy(cudaStream_t s) { return s == nullptr || s == cudaStreamLegacy; }
 bool inside(const void* p, size_t n) {
   auto it = live.upper_bound((char*)p);
@@ -46,7 +50,6 @@ bool inside(const void* p, size_t n) {
   return (const char*)p + n <= it->first + it->second;
 }
 bool device(const void* p) { return inside(p, 0); }
-void fault(const std::string& what) { faults.push_back(what); }
 void on_stream(cudaStream_t s, const std::string& what) {
   if (legacy(s) || !pending) return;
   fault(what + " with legacy-stream work possibly in flight");
@@ -84,6 +87,8 @@ CUresult encode(CUtensorMap* m, CUtensorMapDataType t, cuuint32_t rank, void* ba
 char symbol[1 << 21];
 
 }  // namespace
+
+bool in_device_memory(const void* p) { return device(p); }
 
 extern "C" {
 

@@ -23,6 +23,12 @@ std::function<void()> body(const std::string& k, void** a) {
     if (model.ok_after && model.blocks >= model.ok_after) sc->status = bx::ST_OK;
     else if (sc->it >= sc->maxit) sc->status = bx::ST_ENOTCONV;
   };
+  if (k.find("PKNS_8SlotDescEPKNS_8WorkItemEPKi") != std::string::npos)  // descriptors, work list, its length
+    for (int i = 0; i < 3; ++i)
+      if (!in_device_memory(*(const void**)a[i])) {
+        fault(k + ": argument outside a live allocation");
+        return [] {};
+      }
   if (k.find("k_true_residual") != std::string::npos) {
     auto slots = *(const bx::SlotDesc**)a[0];
     auto items = *(const bx::WorkItem**)a[1];

@@ -95,3 +95,45 @@ for name, call in calls():
 print(faults())
 """)
     assert out.strip() == ""
+
+
+@pytest.mark.parametrize("kw", ['dict(prec="mixed_bf16", low_modes=1, autotune=0)'])
+def test_a_failed_allocation_leaves_nothing_half_made(fake_cuda, kw):
+    """Each allocation of a first call fails in turn: the call reports it, and the same call on the same
+    context then works on complete plans and work lists (tensor maps, copies and lists inside live
+    allocations)."""
+    out = fake_cuda("""
+phi, f, out = [Dev(160 * 256) for _ in range(3)]
+v = [Dev(12 * 12 * 128) for _ in range(3)]
+CALLS = [lambda c: ext.ext_solve(c, prob, phi, f, out, check=False)["rc"],
+         lambda c: ext.load().ext_apply_preconditioner(c, C.byref(prob), phi.p, f.p, out.p, None),
+         lambda c: ext.ext_solve3d(c, ext.problem3(12, 12, 128), *v, check=False)["rc"]]
+told, kw = 0, """ + kw + """
+for i, call in enumerate(CALLS):
+    n = 0
+    while True:
+        fake.fake_fail_malloc(-1)
+        c = ext.ext_create(ext.options(**kw))
+        fake.fake_model(5, 2, 0)
+        prob = ext.problem(160, 96 + n, "symmetric", "dirichlet")  # another height each time: none is tuned yet
+        before = fake.fake_mallocs()
+        fake.fake_fail_malloc(n)
+        rc = call(c)
+        failed = fake.fake_mallocs() - before > n
+        fake.fake_fail_malloc(-1)
+        fake.fake_model(5, 2, 0)
+        if failed and rc not in (ext.EXT_ENOMEM, ext.EXT_ECUDA):
+            print(kw, i, n, "failed allocation gave", rc)
+        again = call(c)
+        if len(faults()) != told:
+            print(kw, i, n, rc, faults()[told:])
+            told = len(faults())
+        if again != ext.EXT_OK:
+            print(kw, i, n, "the next call gave", again)
+        ext.ext_destroy(c)
+        if not failed:
+            break
+        n += 1
+    assert n > 3, n
+""")
+    assert out.strip() == ""
