@@ -1229,12 +1229,20 @@ static int set_stencil_shape(ext_ctx* ctx, Workspace* W, int ty) {
   cudaStream_t s = W->stream ? W->stream : ctx->stream;
   BX_CUDA(cudaStreamSynchronize(s));
   std::vector<WorkItem> sten;
+  for (int i = 0; i < (int)W->slots.size(); ++i) {
+    const SlotDesc& d = W->slots[i].d;
+    const int n = ((d.nx + kStTileX - 1) / kStTileX) * ((d.ny + ty - 1) / ty);
+    for (int t = 0; t < n; ++t) sten.push_back({i, t});
+  }
+  WorkItem* list = nullptr;  // without it the present shape stays
+  BX_CUDA(cudaMalloc(&list, sizeof(WorkItem) * sten.size()));
+  cudaFree(W->d_sten);
+  W->d_sten = list;
   std::vector<SlotDesc> descs;
   for (int i = 0; i < (int)W->slots.size(); ++i) {
     SlotDesc& d = W->slots[i].d;
     d.sten_ty = ty;
     d.n_sten_tiles = ((d.nx + kStTileX - 1) / kStTileX) * ((d.ny + ty - 1) / ty);
-    for (int t = 0; t < d.n_sten_tiles; ++t) sten.push_back({i, t});
     if (d.st_maps) {
       CUtensorMap m[kStMaps];
       const int rc = make_stencil_maps(m, d, ty);
@@ -1243,9 +1251,6 @@ static int set_stencil_shape(ext_ctx* ctx, Workspace* W, int ty) {
     }
     descs.push_back(d);
   }
-  cudaFree(W->d_sten);
-  W->d_sten = nullptr;
-  BX_CUDA(cudaMalloc(&W->d_sten, sizeof(WorkItem) * sten.size()));
   BX_CUDA(cudaMemcpy(W->d_sten, sten.data(), sizeof(WorkItem) * sten.size(), cudaMemcpyHostToDevice));
   W->n_sten = (int)sten.size();
   BX_CUDA(cudaMemcpy(W->d_counts + 4, &W->n_sten, sizeof(int), cudaMemcpyHostToDevice));

@@ -97,7 +97,8 @@ print(faults())
     assert out.strip() == ""
 
 
-@pytest.mark.parametrize("kw", ['dict(prec="mixed_bf16", low_modes=1, autotune=0)'])
+@pytest.mark.parametrize("kw", ['dict(prec="mixed_bf16", low_modes=1, autotune=0)',
+                                'dict(prec="mixed_bf16")', 'dict(prec="fp32", autotune=0, tile_y=16)'])
 def test_a_failed_allocation_leaves_nothing_half_made(fake_cuda, kw):
     """Each allocation of a first call fails in turn: the call reports it, and the same call on the same
     context then works on complete plans and work lists (tensor maps, copies and lists inside live
