@@ -557,12 +557,14 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     const SlotDesc& S = *tile.S;
     const f2 beta = {tile.beta_hi, tile.beta_lo};
     const int par = tile.par, x0 = tile.x0, y0 = tile.y0;
-    const float* __restrict__ pold = S.p[par];
-    const float* __restrict__ pold_lo = S.p_lo[par];
+    // plain loads of what the kernels before wrote: their lifetimes overlap this one's, so nothing here
+    // may be read as read-only data (__ldg, const __restrict__)
+    const float* pold = S.p[par];
+    const float* pold_lo = S.p_lo[par];
     float* __restrict__ pnew = S.p[par ^ 1];
     float* __restrict__ pnew_lo = S.p_lo[par ^ 1];
-    const float* __restrict__ z = S.z;
-    const float* __restrict__ z_lo = S.z_lo;
+    const float* z = S.z;
+    const float* z_lo = S.z_lo;
     // a tile whose halo lies inside the grid has no ghost cell
     const bool interior = x0 >= 2 && y0 >= 2 && x0 + kStTileX + 2 <= S.nx && y0 + TY + 2 <= S.ny;
     unsigned char* buf = sbuf + b * G::kBufBytes;
@@ -583,8 +585,8 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
             if (s != 0.f) {  // zero-sign ghosts stay the zeros the copy filled in
               gcell[h] = wy * kWX + wx;
               gs[h] = s;
-              gz[h] = f2{__ldg(z + g), __ldg(z_lo + g)};
-              gp[h] = f2{__ldg(pold + g), __ldg(pold_lo + g)};
+              gz[h] = f2{z[g], z_lo[g]};
+              gp[h] = f2{pold[g], pold_lo[g]};
             }
           }
         }
@@ -645,8 +647,8 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
 #pragma unroll
         for (int j = 0; j < kChunk; ++j) {
           const bool on = gsg[j] != 0.f;
-          zv[j] = on ? f2{__ldg(z + gi[j]), __ldg(z_lo + gi[j])} : f2{0.f, 0.f};
-          pv[j] = on ? f2{__ldg(pold + gi[j]), __ldg(pold_lo + gi[j])} : f2{0.f, 0.f};
+          zv[j] = on ? f2{z[gi[j]], z_lo[gi[j]]} : f2{0.f, 0.f};
+          pv[j] = on ? f2{pold[gi[j]], pold_lo[gi[j]]} : f2{0.f, 0.f};
         }
 #pragma unroll
         for (int j = 0; j < kChunk; ++j) {
@@ -856,8 +858,8 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
     w = we;
     if (!FUSE && !sc->active) continue;
     const int pi = (sc->it & 1) ^ 1;
-    const float* __restrict__ p = S.p[pi];
-    const float* __restrict__ p_lo = S.p_lo[pi];
+    const float* p = S.p[pi];
+    const float* p_lo = S.p_lo[pi];
     const int n = S.nx * S.ny;
     const int chunk = S.vec_chunk;
     const bool flat = !S.upd_seg;
@@ -865,11 +867,11 @@ k_update(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
     const int e_run = it.tile * chunk;
     const int e_whole = flat ? min(e_run + count * chunk, n / chunk * chunk) : 0;
     float4 ph, pl, qh, ql, rh, rl, xh, xl;
-    auto load = [&](int e) {
-      ph = __ldg(reinterpret_cast<const float4*>(p + e));
-      pl = __ldg(reinterpret_cast<const float4*>(p_lo + e));
-      qh = __ldg(reinterpret_cast<const float4*>(S.q + e));
-      ql = __ldg(reinterpret_cast<const float4*>(S.q_lo + e));
+    auto load = [&](int e) {  // plain loads: the stencil, whose lifetime overlaps this kernel's, writes p and q
+      ph = *reinterpret_cast<const float4*>(p + e);
+      pl = *reinterpret_cast<const float4*>(p_lo + e);
+      qh = *reinterpret_cast<const float4*>(S.q + e);
+      ql = *reinterpret_cast<const float4*>(S.q_lo + e);
       rh = *reinterpret_cast<const float4*>(S.r + e);
       rl = *reinterpret_cast<const float4*>(S.r_lo + e);
       xh = *reinterpret_cast<const float4*>(S.xhi + e);

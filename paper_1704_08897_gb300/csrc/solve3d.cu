@@ -143,8 +143,8 @@ __device__ __forceinline__ int halo_pos(int k) {
 struct Plane3 {
   float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f};
 };
-__device__ __forceinline__ Plane3 k3_fetch(const Grid3& G, const float* __restrict__ ih,
-                                           const float* __restrict__ il, const Cell3 (&cl)[3], int zz) {
+__device__ __forceinline__ Plane3 k3_fetch(const Grid3& G, const float* ih, const float* il,
+                                           const Cell3 (&cl)[3], int zz) {
   Plane3 p;
   float sz;
   const int mz = ghost(zz, G.nz, G.bcz, sz);
