@@ -157,7 +157,7 @@ struct ext_ctx {
                       // build_slot may give a grid 6
   int split = 0;      // their type: 0 = FP16, 1 = BF16
   int* d_err = nullptr;   // device flag raised by a bounded wait that ran out
-  int* h_err = nullptr;   // pinned copies, two
+  int* h_err = nullptr;   // pinned copies: two of a solve, two of a 3-D solve, the serving worker's
   cudaEvent_t blk_ev[2] = {nullptr, nullptr};  // the ends of a solve's blocks of iterations
   SlotScalars* h_sc3 = nullptr;  // pinned, two entries (3-D solves)
   // launch accounting and optional per-kernel timing (ext_options.profile)
@@ -1356,6 +1356,15 @@ static int map_status(int st, int n_known, const ext_problem& p) {
   return st;
 }
 
+// A bounded wait ran out: the flag goes down once the stream has finished, so the next call starts afresh.
+static int timed_out(ext_ctx* ctx) {
+  BX_CUDA(cudaStreamSynchronize(ctx->stream));
+  BX_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
+  BX_CUDA(cudaStreamSynchronize(ctx->stream));
+  g_last_error = "a bounded device wait (tensor copy or tensor-core pipeline) ran out";
+  return EXT_ETIMEOUT;
+}
+
 // Full solve of the slots of W (inputs already bound); writes outputs and results.
 static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const float* const* fs,
                      float* const* outs, const int* dirs, ext_result* results,
@@ -1441,13 +1450,7 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
       harvest(ctx);
       harvest_graph(ctx, W->graph_events);
     }
-    if (ctx->h_err[seen]) {
-      BX_CUDA(cudaStreamSynchronize(s));
-      BX_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), s));
-      BX_CUDA(cudaStreamSynchronize(s));
-      g_last_error = "a bounded device wait (tensor copy or tensor-core pipeline) ran out";
-      return EXT_ETIMEOUT;
-    }
+    if (ctx->h_err[seen]) return timed_out(ctx);
     end = W->h_sc + seen * count;
     bool running = false;
     for (int i = 0; i < count; ++i)
@@ -1596,9 +1599,9 @@ int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out) {
   BX_CUDA(stencil_init());
   BX_CUDA(cudaMalloc(&ctx->d_err, sizeof(int)));
   BX_CUDA(cudaMemset(ctx->d_err, 0, sizeof(int)));
-  BX_CUDA(cudaMallocHost(&ctx->h_err, 2 * sizeof(int)));
+  BX_CUDA(cudaMallocHost(&ctx->h_err, 5 * sizeof(int)));
   for (cudaEvent_t& e : ctx->blk_ev) BX_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  ctx->h_err[0] = ctx->h_err[1] = 0;
+  std::fill(ctx->h_err, ctx->h_err + 5, 0);
   BX_CUDA(cudaMallocHost(&ctx->h_sc3, 2 * sizeof(SlotScalars)));
   if (cuda_stream) {
     ctx->stream = (cudaStream_t)cuda_stream;
@@ -1742,6 +1745,7 @@ static int args3(ext_ctx* ctx, const ext_problem3* p, Solve3Args& a) {
   a.stream = ctx->stream;
   a.sm_count = ctx->sm_count;
   a.h_sc = ctx->h_sc3;
+  a.h_err = ctx->h_err + 2;
   if (on_tc)
     a.tc_build = [ctx, &a](const Tc3Io& io, Tc3& t) { return tc3_build(ctx, a, io, t); };
   return EXT_OK;
@@ -2069,6 +2073,13 @@ static int stage_setup(ext_ctx* ctx, const ext_problem* prob, const float* phi, 
   return EXT_OK;
 }
 
+// The end of a single-stage call: EXT_ETIMEOUT, and the flag down again, if a kernel's wait ran out.
+static int stage_done(ext_ctx* ctx) {
+  BX_CUDA(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  BX_CUDA(cudaStreamSynchronize(ctx->stream));
+  return *ctx->h_err ? timed_out(ctx) : EXT_OK;
+}
+
 int ext_apply_biharmonic(ext_ctx* ctx, const ext_problem* prob, const float* phi, const float* p,
                          float* q, double* sum_pq) {
   if (!ctx || !is_device_ptr(p) || !is_device_ptr(q)) return EXT_EINVAL;
@@ -2088,14 +2099,8 @@ int ext_apply_biharmonic(ext_ctx* ctx, const ext_problem* prob, const float* phi
   BX_CUDA(cudaMemcpyAsync(q, sl.d.q, 4 * N, cudaMemcpyDeviceToDevice, s));
   std::vector<double> part((size_t)((prob->ny + 15) / 16) * ((prob->nx + kStTileX - 1) / kStTileX));
   BX_CUDA(cudaMemcpyAsync(part.data(), sl.d.pq_part, 8 * part.size(), cudaMemcpyDeviceToHost, s));
-  BX_CUDA(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-  BX_CUDA(cudaStreamSynchronize(s));
-  if (*ctx->h_err) {
-    BX_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), s));
-    BX_CUDA(cudaStreamSynchronize(s));
-    g_last_error = "a bounded device wait (stencil tensor copy) ran out";
-    return EXT_ETIMEOUT;
-  }
+  rc = stage_done(ctx);
+  if (rc) return rc;
   if (sum_pq) {
     double acc = 0.0;
     for (double v : part) acc += v;
@@ -2128,7 +2133,8 @@ int ext_apply_preconditioner(ext_ctx* ctx, const ext_problem* prob, const float*
   launch_prec(ctx, W, 2);
   BX_CUDA(cudaGetLastError());
   BX_CUDA(cudaMemcpyAsync(z, sl.d.z, 4 * N, cudaMemcpyDefault, ctx->stream));
-  BX_CUDA(cudaStreamSynchronize(ctx->stream));
+  rc = stage_done(ctx);
+  if (rc) return rc;
   if (scale) {
     const double a = 1.0 / (prob->hx * prob->hx), c = 1.0 / (prob->hy * prob->hy);
     const double m = std::max(a, c);
@@ -2548,10 +2554,10 @@ static void serve_loop(ext_ctx* ctx) {
     if (!rc) {
       const int cap = (int)S->slots.size();
       if (cudaMemcpyAsync(W->h_sc, W->d_sc, sizeof(SlotScalars) * cap, cudaMemcpyDeviceToHost, W->stream) != cudaSuccess ||
-          cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, W->stream) != cudaSuccess ||
+          cudaMemcpyAsync(ctx->h_err + 4, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, W->stream) != cudaSuccess ||
           cudaStreamSynchronize(W->stream) != cudaSuccess)
         rc = EXT_ECUDA;
-      else if (*ctx->h_err)
+      else if (ctx->h_err[4])
         rc = EXT_ETIMEOUT;
     }
     if (!rc) {

@@ -145,6 +145,7 @@ struct Solve3Args {
   long long* launches;     // incremented by every kernel launch (host counter)
   int sm_count;
   SlotScalars* h_sc;       // pinned, two entries: the scalars as blocks of iterations leave them
+  int* h_err;              // pinned, two entries: the time-out flag with them
   // builds the tensor-core preconditioner for the given vectors (empty: CUDA-core transforms)
   std::function<int(const Tc3Io&, Tc3&)> tc_build;
 };

@@ -839,6 +839,21 @@ int setup_mask(const Solve3Args& a, State3& s, const float* phi, const float* f,
 
 constexpr int kBlockIters = 8;  // iterations between two readings of the scalars
 
+// Copies the tensor-core kernels' time-out flag to the host (the CUDA-core kernels have no waits).
+int read_flag(const Solve3Args& a, const State3& s, int* flag, std::string* err) {
+  *flag = 0;
+  if (s.tc.on) BX3(cudaMemcpyAsync(flag, s.tc.d_err, sizeof(int), cudaMemcpyDeviceToHost, a.stream));
+  return EXT_OK;
+}
+// A bounded wait ran out: the flag goes down once the stream has finished, so the next call starts afresh.
+int timed_out(const Solve3Args& a, const State3& s, std::string* err) {
+  BX3(cudaStreamSynchronize(a.stream));
+  BX3(cudaMemsetAsync(s.tc.d_err, 0, sizeof(int), a.stream));
+  BX3(cudaStreamSynchronize(a.stream));
+  *err = "a bounded device wait (tensor-core pipeline) ran out";
+  return EXT_ETIMEOUT;
+}
+
 }  // namespace
 
 int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* out, ext_result* res,
@@ -922,10 +937,13 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
     enqueue_tail(a, G, s, wnorm);
     BX3(cudaGetLastError());
     BX3(cudaMemcpyAsync(&a.h_sc[blk & 1], s.sc, sizeof(SlotScalars), cudaMemcpyDeviceToHost, st));
+    rc = read_flag(a, s, &a.h_err[blk & 1], err);
+    if (rc) return rc;
     BX3(cudaEventRecord(s.ev[blk & 1], st));
     // one block stays ahead of the reading; with nothing left to do it passes by its flags
     if (blk == 0 && blk < max_blocks) continue;
     BX3(cudaEventSynchronize(s.ev[(blk & 1) ^ 1]));
+    if (a.h_err[(blk & 1) ^ 1]) return timed_out(a, s, err);
     last = a.h_sc[(blk & 1) ^ 1];
     if (last.status != ST_RUNNING) break;
   }
@@ -941,18 +959,6 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
   ++*a.launches;
   BX3(cudaGetLastError());
   BX3(cudaStreamSynchronize(st));
-  if (s.tc.on) {
-    // a bounded wait of the tensor-core kernels that ran out
-    int flag = 0;
-    BX3(cudaMemcpy(&flag, s.tc.d_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (flag) {
-      BX3(cudaMemsetAsync(s.tc.d_err, 0, sizeof(int), st));
-      BX3(cudaStreamSynchronize(st));
-      *err = "a bounded device wait (tensor-core pipeline) ran out";
-      res->status = EXT_ETIMEOUT;
-      return EXT_ETIMEOUT;
-    }
-  }
   res->status = status;
   return status;
 }
@@ -1001,7 +1007,10 @@ int apply3d_preconditioner(const Solve3Args& a, const float* phi, const float* r
   precondition(a, s, wnorm, rh, rl, s.zh, s.zl, 2);
   BX3(cudaMemcpyAsync(z, s.zh, 4 * s.n, cudaMemcpyDeviceToDevice, a.stream));
   BX3(cudaGetLastError());
+  rc = read_flag(a, s, a.h_err, err);
+  if (rc) return rc;
   BX3(cudaStreamSynchronize(a.stream));
+  if (*a.h_err) return timed_out(a, s, err);
   // weights are (L^2)^+ scaled by wnorm, times the square of the stencil scaling (max 1/h^2)^-2
   const double m = std::max(1.0 / (a.h[0] * a.h[0]), std::max(1.0 / (a.h[1] * a.h[1]), 1.0 / (a.h[2] * a.h[2])));
   if (scale) *scale = (double)wnorm * m * m;

@@ -138,3 +138,29 @@ for i, call in enumerate(CALLS):
     assert n > 3, n
 """)
     assert out.strip() == ""
+
+
+def test_a_wait_that_runs_out_is_told_by_the_call_it_ran_out_in(fake_cuda):
+    """Both preconditioner calls return EXT_ETIMEOUT when a transform product raises the flag, and the next
+    call on the context starts with the flag down; a 3-D solve leaves after the block that raised it, not
+    after all of its blocks."""
+    out = fake_cuda("""
+T = ext.EXT_ETIMEOUT
+phi, f, z = [Dev(128 ** 3) for _ in range(3)]
+prob, prob3 = ext.problem(200, 150), ext.problem3(128, 128, 128)
+for prec in ("fp32", "mixed_bf16"):
+    c = ext.ext_create(ext.options(prec, maxit=400))
+    for name, call, p in (("2-D", ext.load().ext_apply_preconditioner, prob),
+                          ("3-D", ext.load().ext_apply_preconditioner3d, prob3)):
+        for err_after, want in ((1, T), (0, 0)):
+            fake.fake_model(1, 0, err_after)
+            rc = call(c, C.byref(p), phi.p, f.p, z.p, None)
+            if rc != want: print(prec, name, err_after, rc)
+    for err_after, ok_after, want in ((30, 0, T), (0, 5, 0)):
+        fake.fake_model(1, ok_after, err_after)
+        r = ext.ext_solve3d(c, prob3, phi, f, z, check=False)
+        if r["rc"] != want or r["status"] != want or fake.fake_blocks() > 6: print(prec, r, fake.fake_blocks())
+    ext.ext_destroy(c)
+print(faults())
+""")
+    assert out.strip() == ""
