@@ -1433,17 +1433,21 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
   max_blocks = max_blocks / std::max(1, ctx->opt.iters_per_launch) + 8;
   // The host stays one block ahead: block k + 1 is launched before the scalars that block k left are
   // read, so the device never waits for the host; with nothing left to do a block passes by the slots'
-  // flags.  (A profiled solve reads each block's events before the next one records over them.)
+  // flags.  Every block's scalars are read, the last one's with nothing launched behind it.  (A profiled
+  // solve reads each block's events before the next one records over them.)
   const int ahead = ctx->opt.profile ? 0 : 1;
   const SlotScalars* end = W->h_sc;  // the scalars last read
-  for (int blk = 0; blk < max_blocks; ++blk) {
-    BX_CUDA(cudaGraphLaunch(graph.exec, s));
-    ctx->launches += graph.nodes;
-    BX_CUDA(cudaMemcpyAsync(W->h_sc + (blk & 1) * count, W->d_sc, sizeof(SlotScalars) * count, cudaMemcpyDeviceToHost, s));
-    BX_CUDA(cudaMemcpyAsync(ctx->h_err + (blk & 1), ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BX_CUDA(cudaEventRecord(ctx->blk_ev[blk & 1], s));
-    if (blk < ahead && blk + 1 < max_blocks) continue;
-    const int seen = (blk & 1) ^ ahead;
+  for (int blk = 0; blk < max_blocks + ahead; ++blk) {
+    if (blk < max_blocks) {
+      const int set = blk & 1;
+      BX_CUDA(cudaGraphLaunch(graph.exec, s));
+      ctx->launches += graph.nodes;
+      BX_CUDA(cudaMemcpyAsync(W->h_sc + set * count, W->d_sc, sizeof(SlotScalars) * count, cudaMemcpyDeviceToHost, s));
+      BX_CUDA(cudaMemcpyAsync(ctx->h_err + set, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+      BX_CUDA(cudaEventRecord(ctx->blk_ev[set], s));
+    }
+    if (blk < ahead) continue;
+    const int seen = (blk - ahead) & 1;
     BX_CUDA(cudaEventSynchronize(ctx->blk_ev[seen]));
     if (ctx->opt.profile) {
       BX_CUDA(cudaStreamSynchronize(s));

@@ -931,20 +931,24 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
   for (cudaEvent_t& v : s.ev) BX3(cudaEventCreateWithFlags(&v, cudaEventDisableTiming));
   precondition(a, s, wnorm, s.rh, s.rl, s.zh, s.zl, 1);
   SlotScalars last{};
-  const long long max_blocks = 2LL * (maxit / kBlockIters) + 8;
+  const long long max_blocks = 2LL * (maxit / kBlockIters) + 9;
+  // one block stays ahead of the reading; with nothing left to do it passes by its flags
   for (long long blk = 0; blk <= max_blocks; ++blk) {
-    for (int i = 0; i < kBlockIters; ++i) enqueue_iteration(a, G, s, wnorm);
-    enqueue_tail(a, G, s, wnorm);
-    BX3(cudaGetLastError());
-    BX3(cudaMemcpyAsync(&a.h_sc[blk & 1], s.sc, sizeof(SlotScalars), cudaMemcpyDeviceToHost, st));
-    rc = read_flag(a, s, &a.h_err[blk & 1], err);
-    if (rc) return rc;
-    BX3(cudaEventRecord(s.ev[blk & 1], st));
-    // one block stays ahead of the reading; with nothing left to do it passes by its flags
-    if (blk == 0 && blk < max_blocks) continue;
-    BX3(cudaEventSynchronize(s.ev[(blk & 1) ^ 1]));
-    if (a.h_err[(blk & 1) ^ 1]) return timed_out(a, s, err);
-    last = a.h_sc[(blk & 1) ^ 1];
+    if (blk < max_blocks) {
+      const int set = blk & 1;
+      for (int i = 0; i < kBlockIters; ++i) enqueue_iteration(a, G, s, wnorm);
+      enqueue_tail(a, G, s, wnorm);
+      BX3(cudaGetLastError());
+      BX3(cudaMemcpyAsync(&a.h_sc[set], s.sc, sizeof(SlotScalars), cudaMemcpyDeviceToHost, st));
+      rc = read_flag(a, s, &a.h_err[set], err);
+      if (rc) return rc;
+      BX3(cudaEventRecord(s.ev[set], st));
+    }
+    if (blk == 0) continue;
+    const int seen = (blk - 1) & 1;
+    BX3(cudaEventSynchronize(s.ev[seen]));
+    if (a.h_err[seen]) return timed_out(a, s, err);
+    last = a.h_sc[seen];
     if (last.status != ST_RUNNING) break;
   }
   BX3(cudaStreamSynchronize(st));

@@ -164,3 +164,33 @@ for prec in ("fp32", "mixed_bf16"):
 print(faults())
 """)
     assert out.strip() == ""
+
+
+def test_the_last_block_of_iterations_is_read(fake_cuda):
+    """A solve that converges, or whose wait runs out, in the last block its limit allows reports that."""
+    out = fake_cuda("""
+phi, f, z = [Dev(128 ** 3) for _ in range(3)]
+G, maxit = 10, 40
+for prec, profile in (("fp32", 0), ("mixed_bf16", 0), ("mixed_bf16", 1)):
+    c = ext.ext_create(ext.options(prec, maxit=maxit, iters_per_launch=G, profile=profile))
+    prob = ext.problem(200, 150, "dirichlet")
+    blocks = maxit // G + 8
+    fake.fake_model(1, blocks, 0)
+    r = ext.ext_solve(c, prob, phi, f, z, check=False)
+    if (r["rc"], r["iters"]) != (0, blocks): print("2-D", prec, r)
+    # the first product of the last block, after the first pass's four, a block's 4 G and its tail's 4
+    fake.fake_model(1, 0, 4 + (blocks - 1) * 4 * (G + 1) + 1)
+    r = ext.ext_solve(c, prob, phi, f, z, check=False)
+    if r["rc"] != ext.EXT_ETIMEOUT: print("2-D flag", prec, r)
+    fake.fake_model(1, 2, 0)
+    r = ext.ext_solve(c, prob, phi, f, z, check=False)
+    if (r["rc"], r["iters"]) != (0, 2): print("2-D after a time-out", prec, r)
+    ext.ext_destroy(c)
+c = ext.ext_create(ext.options("fp32", maxit=64))
+fake.fake_model(1, 25, 0)
+r = ext.ext_solve3d(c, ext.problem3(12, 12, 12), phi, f, z, check=False)
+if (r["rc"], r["iters"]) != (0, 25): print("3-D", r)
+ext.ext_destroy(c)
+print(faults())
+""")
+    assert out.strip() == ""
