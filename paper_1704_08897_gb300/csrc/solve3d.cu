@@ -931,7 +931,9 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
   for (cudaEvent_t& v : s.ev) BX3(cudaEventCreateWithFlags(&v, cudaEventDisableTiming));
   precondition(a, s, wnorm, s.rh, s.rl, s.zh, s.zl, 1);
   SlotScalars last{};
-  const long long max_blocks = 2LL * (maxit / kBlockIters) + 9;
+  // a block of a solve that runs completes an iteration at least (one whose recursive residual converges
+  // in each, the true one not, no more than that), so maxit ends the solve before the blocks do
+  const long long max_blocks = maxit + 1LL;
   // one block stays ahead of the reading; with nothing left to do it passes by its flags
   for (long long blk = 0; blk <= max_blocks; ++blk) {
     if (blk < max_blocks) {

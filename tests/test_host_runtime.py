@@ -194,3 +194,18 @@ ext.ext_destroy(c)
 print(faults())
 """)
     assert out.strip() == ""
+
+
+def test_a_3d_solve_that_stagnates_runs_to_its_iteration_limit(fake_cuda):
+    """One iteration a block, as when the recursive residual converges again and again and the true one does
+    not: the solve ends as not converged at maxit."""
+    out = fake_cuda("""
+phi, f, z = [Dev(12 ** 3) for _ in range(3)]
+for maxit in (1, 8, 64, 333):
+    c = ext.ext_create(ext.options("fp32", maxit=maxit))
+    fake.fake_model(1, 0, 0)
+    r = ext.ext_solve3d(c, ext.problem3(12, 12, 12), phi, f, z, check=False)
+    if (r["rc"], r["status"], r["iters"]) != (ext.EXT_ENOTCONV, ext.EXT_ENOTCONV, maxit): print(maxit, r)
+    ext.ext_destroy(c)
+""")
+    assert out.strip() == ""
