@@ -86,6 +86,7 @@ struct __align__(16) SlotScalars {
   double aro_total;
   double aro_ring[8];
   int aro_n;
+  int it_ref;       // iterations completed at the last residual replacement
 };
 constexpr int kErrDelay = 8;
 
@@ -610,7 +611,7 @@ __device__ __forceinline__ void finish_pq(SlotScalars* sc, double pq) {
 
 // One thread, after an update with ||r||^2 = s: count the iteration and decide stop or residual
 // replacement.
-__device__ __forceinline__ void decide_update(SlotScalars* sc, double s) {
+__host__ __device__ __forceinline__ void decide_update(SlotScalars* sc, double s) {
   sc->rr = s;
   const int itn = sc->it + 1;
   sc->it = itn;
@@ -621,12 +622,26 @@ __device__ __forceinline__ void decide_update(SlotScalars* sc, double s) {
     sc->fold = 1;
   }
 }
+// The same in three dimensions, where blocks of iterations have a fixed length: a replacement that is due
+// (fold_every counts from the last one) stops the iterations, so that it comes at this one and not at the
+// block's end; decide_true lets them go on.
+__host__ __device__ __forceinline__ void decide_update3(SlotScalars* sc, double s) {
+  sc->rr = s;
+  const int itn = sc->it + 1;
+  sc->it = itn;
+  if (s <= sc->rtol2 * sc->bb || itn >= sc->maxit || !isfinite(s) || s < sc->delta2 * sc->rr_ref ||
+      itn - sc->it_ref >= sc->fold_every) {
+    sc->active = 0;
+    sc->fold = 1;
+  }
+}
 // One thread, after the true residual's ||r||^2 = s: converged, stopped, or continue with a fresh
 // preconditioner pass.
-__device__ __forceinline__ void decide_true(SlotScalars* sc, double s) {
+__host__ __device__ __forceinline__ void decide_true(SlotScalars* sc, double s) {
   sc->rr_true = s;
   sc->rr = s;
   sc->rr_ref = s;
+  sc->it_ref = sc->it;
   sc->fold = 0;
   sc->active = 0;
   sc->need_prec = 0;

@@ -19,7 +19,8 @@
 // The iteration is preconditioned CG from x = 0 with the Fletcher-Reeves beta.  Its scalars live on
 // the device (the two-dimensional path's SlotScalars and its decisions: stop, residual
 // replacement, breakdown) and its kernels follow one another as dependent launches, in blocks of
-// kBlockIters iterations with the replacement work at the block's end; the host stays one block
+// kBlockIters iterations with the replacement work at the block's end (an iteration that calls for a
+// replacement is the block's last: those behind it pass by); the host stays one block
 // ahead, reading the scalars that the block before left, so the device never waits for it.  (Read
 // after every reduction, three times an iteration, the scalars cost a 72 x 60 x 50 solve 80 of
 // its 330 us an iteration.)  Kernels whose flag is down return at once.  Every reduction sums
@@ -433,7 +434,7 @@ k3_finish(SlotScalars* sc, const double* part, int n, int stride, int mode) {
   __syncwarp();  // every lane has read its flag
   if (threadIdx.x != 0) return;
   if (KIND == 0) finish_pq(sc, v);
-  if (KIND == 1) decide_update(sc, v);
+  if (KIND == 1) decide_update3(sc, v);
   if (KIND == 2) finish_preconditioner(sc, v, 0.0, mode);
   if (KIND == 3) decide_true(sc, v);
 }

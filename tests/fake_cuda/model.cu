@@ -1,7 +1,9 @@
 // The few kernels that the runtime without a device models: the end of a block of iterations
 // (k_true_residual; in three dimensions k3_finish<3>), which counts fake_model's iterations and decides;
-// the 3-D set-up's counts and norm; and the transform products, which raise the time-out flag on demand.
+// the 3-D iteration's decisions on a given run of residuals; the 3-D set-up's counts and norm; and the transform products, which raise the time-out flag on demand.
 #include "model.h"
+
+#include <vector>
 
 #include "../../paper_1704_08897_gb300/csrc/common.cuh"
 
@@ -11,6 +13,9 @@ static struct Model {
   int err_after = 0;     // transform products until one raises the time-out flag (0: none)
   int blocks = 0, products = 0;
 } model;
+
+static std::vector<double> residuals;   // 3-D: ||r||^2 / ||b||^2 after each iteration
+static std::vector<int> replaced;       // the iterations at which the residual was replaced
 
 // what the kernel does, with its arguments read now
 std::function<void()> body(const std::string& k, void** a) {
@@ -38,9 +43,20 @@ std::function<void()> body(const std::string& k, void** a) {
         if (items[i].tile == 0) block_end(slots[items[i].slot].sc);
     };
   }
+  if (k.find("k3_finishILi1E") != std::string::npos && !residuals.empty()) {
+    auto sc = *(SlotScalars**)a[0];
+    return [=] {
+      if (sc->active) bx::decide_update3(sc, sc->bb * residuals.at(sc->it));
+    };
+  }
   if (k.find("k3_finishILi3E") != std::string::npos) {
     auto sc = *(SlotScalars**)a[0];
-    return [=] { block_end(sc); };
+    return [=] {
+      if (residuals.empty()) return block_end(sc);
+      if (!sc->fold) return;
+      replaced.push_back(sc->it);
+      bx::decide_true(sc, sc->bb * residuals.at(sc->it - 1) * 1.0001);
+    };
   }
   if (k.find("k3_setup") != std::string::npos) {
     const size_t n = *(size_t*)a[0];
@@ -62,6 +78,14 @@ std::function<void()> body(const std::string& k, void** a) {
 
 extern "C" {
 void fake_model(int its, int ok_after, int err_after) { model = Model{its, ok_after, err_after, 0, 0}; }
+void fake_residuals(const double* r, int n) {
+  residuals.assign(r, r + n);
+  replaced.clear();
+}
+int fake_replaced(int* its, int n) {
+  for (int i = 0; i < n && i < (int)replaced.size(); ++i) its[i] = replaced[i];
+  return (int)replaced.size();
+}
 int fake_blocks() { return model.blocks; }
 int fake_products() { return model.products; }
 }

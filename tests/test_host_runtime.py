@@ -209,3 +209,33 @@ for maxit in (1, 8, 64, 333):
     ext.ext_destroy(c)
 """)
     assert out.strip() == ""
+
+
+def test_3d_residual_replacements_come_when_they_are_due(fake_cuda):
+    """The 3-D solve replaces its residual at the iteration that calls for it: a fall by replace_factor
+    since the last replacement, true_res_every iterations since then, or the recursive residual's
+    convergence, whatever the length of the blocks that it enqueues.  The residuals are given, the
+    decisions the library's own; the rule is restated here."""
+    out = fake_cuda("""
+phi, f, z = [Dev(12 ** 3) for _ in range(3)]
+rng = np.random.default_rng(1)
+for every, factor, fall in itertools.product((1, 5, 11, 200), (1e-1, 1e-2), (0.25, 0.7)):
+    rr = np.cumprod(fall * np.exp(0.8 * rng.standard_normal(400)))
+    want, ref, since = [], 1.0, 0
+    for it, v in enumerate(rr, 1):
+        since += 1
+        if v <= 1e-16 or v < factor ** 2 * ref or since >= every:
+            want.append(it)
+            ref, since = v * 1.0001, 0
+            if v * 1.0001 <= 1e-16: break
+    c = ext.ext_create(ext.options("fp32", maxit=400, iters_per_launch=1, true_res_every=every, replace_factor=factor))
+    fake.fake_residuals(rr.ctypes.data_as(C.POINTER(C.c_double)), len(rr))
+    r = ext.ext_solve3d(c, ext.problem3(12, 12, 12), phi, f, z, check=False)
+    got = (C.c_int * 400)()
+    n = fake.fake_replaced(got, 400)
+    if list(got[:n]) != want or r["iters"] != want[-1] or r["rc"] != 0:
+        print(every, factor, fall, list(got[:n]), want, r)
+    ext.ext_destroy(c)
+print(faults())
+""")
+    assert out.strip() == ""
