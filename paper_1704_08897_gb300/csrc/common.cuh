@@ -87,6 +87,7 @@ struct __align__(16) SlotScalars {
   double aro_ring[8];
   int aro_n;
   int it_ref;       // iterations completed at the last residual replacement
+  double rr_rec;    // 3-D: the recursive ||r||^2 of the last iteration
 };
 constexpr int kErrDelay = 8;
 
@@ -626,7 +627,7 @@ __host__ __device__ __forceinline__ void decide_update(SlotScalars* sc, double s
 // (fold_every counts from the last one) stops the iterations, so that it comes at this one and not at the
 // block's end; decide_true lets them go on.
 __host__ __device__ __forceinline__ void decide_update3(SlotScalars* sc, double s) {
-  sc->rr = s;
+  sc->rr = sc->rr_rec = s;
   const int itn = sc->it + 1;
   sc->it = itn;
   if (s <= sc->rtol2 * sc->bb || itn >= sc->maxit || !isfinite(s) || s < sc->delta2 * sc->rr_ref ||

@@ -917,7 +917,7 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
   const double bn = bnorm * scale;
   SlotScalars& h0 = a.h_sc[0];
   h0 = SlotScalars{};
-  h0.bb = h0.rr = h0.rr_true = h0.rr_ref = bn * bn;
+  h0.bb = h0.rr = h0.rr_rec = h0.rr_true = h0.rr_ref = bn * bn;
   h0.rtol2 = a.rtol * a.rtol;
   h0.delta2 = a.replace_factor * a.replace_factor;
   h0.fold_every = a.true_res_every;
@@ -958,7 +958,7 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
   int status = last.status == ST_RUNNING ? EXT_ETIMEOUT : last.status;
   res->iters = last.it;
   res->relres_true = std::sqrt(last.rr_true) / bn;
-  res->relres_rec = std::sqrt(last.rr) / bn;
+  res->relres_rec = std::sqrt(last.rr_rec) / bn;
   double tail = 0.0;
   for (int k = 0; k < std::min(last.aro_n, kErrDelay); ++k) tail += last.aro_ring[k];
   res->err_est = last.aro_total > 0.0 ? std::sqrt(std::max(0.0, tail) / last.aro_total) : 0.0;

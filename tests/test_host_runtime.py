@@ -239,3 +239,19 @@ for every, factor, fall in itertools.product((1, 5, 11, 200), (1e-1, 1e-2), (0.2
 print(faults())
 """)
     assert out.strip() == ""
+
+
+@pytest.mark.parametrize("maxit", [400, 7])
+def test_3d_result_tells_both_residuals(fake_cuda, maxit):
+    """relres_rec is the recursive residual of the last iteration, relres_true the one recomputed."""
+    out = fake_cuda("""
+phi, f, z = [Dev(12 ** 3) for _ in range(3)]
+rr = 0.3 ** np.arange(1, 100)
+c = ext.ext_create(ext.options("fp32", maxit=%d))
+fake.fake_residuals(rr.ctypes.data_as(C.POINTER(C.c_double)), len(rr))
+r = ext.ext_solve3d(c, ext.problem3(12, 12, 12), phi, f, z, check=False)
+v = rr[r["iters"] - 1]
+assert r["iters"] > 5
+if abs(r["relres_rec"] ** 2 / v - 1) > 1e-12 or abs(r["relres_true"] ** 2 / (v * 1.0001) - 1) > 1e-12: print(r, v)
+""" % maxit)
+    assert out.strip() == ""
