@@ -217,34 +217,38 @@ __device__ __forceinline__ int block_exp(float amax) {
   int e;
   frexpf(amax, &e);
   if (amax * pow2f(8 - e) >= 255.5f) ++e;
-  return max(e, -70);  // keeps 2^(48-E) and 2^(E-16-8d) normal
+  // 2^(16-E) stays finite, and the block's sums are scaled by 2^(E-16) >= 2^-126: smaller blocks lose
+  // what FP32's own unit of 2^-149 takes from them
+  return max(e, -110);
 }
 
-// The NSL integer slices of double-float values (hi, lo) for block exponent E, given up = 2^(16-E)
-// and dn = -2^(E-16), on two lanes with their own block factors.  The value is taken sixteen bits
-// at a time: w = the integer nearest to the leading plane at that scale, removed exactly (the
-// product is exact in the FMA), the remainder joined with the lo plane; and each w is cut into its
-// two digits w = 256 c0 + c1, |c1| <= 128.  The slices carry the value to 2^-32 (NSL = 4) or 2^-48
-// (6) of the block.  Roundings to the nearest integer add and remove 1.5 * 2^23 on packed FP32x2
+// The NSL integer slices of double-float values (hi, lo) for block exponent E, given up = 2^(16-E), on
+// two lanes with their own block factors.  The value is brought to the block's scale (exactly: below
+// 2^16 in magnitude at any E) and taken sixteen bits at a time: w = the integer nearest to the leading
+// plane, removed exactly, the remainder joined with the lo plane and scaled up by 2^16; and each w is cut
+// into its two digits w = 256 c0 + c1, |c1| <= 128.  The slices carry the value to 2^-32 (NSL = 4) or
+// 2^-48 (6) of the block.  Roundings to the nearest integer add and remove 1.5 * 2^23 on packed FP32x2
 // (exact for magnitudes below 2^22; ties to even); a digit is an integer of magnitude at most 256,
 // exact in BF16, whose bits are the upper half of the FP32 bits (one byte permutation packs the two
 // lanes' codes).  FP16 codes come from the packed two-value conversion.  About 4 packed operations
 // a digit; the form before, one digit at a time with a renormalised remainder, took 12.
 template <bool BF16, int NSL>
-__device__ __forceinline__ void slice_codes2_df(float2 vh, float2 vl, float2 up, float2 dn,
-                                                uint32_t (&code)[NSL]) {
+__device__ __forceinline__ void slice_codes2_df(float2 vh, float2 vl, float2 up, uint32_t (&code)[NSL]) {
   static_assert(NSL == 4 || NSL == 6, "slices in pairs");
   const float2 rnd = make_float2(12582912.f, 12582912.f), rnd_n = make_float2(-12582912.f, -12582912.f);
-  float2 rh = vh, rl = vl;
+  float2 rh = __fmul2_rn(vh, up), rl = __fmul2_rn(vl, up);
 #pragma unroll
   for (int k = 0; k < NSL; k += 2) {
-    const float2 w = __fadd2_rn(__fadd2_rn(__fmul2_rn(rh, up), rnd), rnd_n);
+    const float2 w = __fadd2_rn(__fadd2_rn(rh, rnd), rnd_n);
     if (k + 2 < NSL) {
-      const float2 h = __ffma2_rn(w, dn, rh);
-      if (k + 4 < NSL) two_sum2(h, rl, rh, rl);
-      else rh = __fadd2_rn(h, rl);
-      up = mul2(65536.f, up);
-      dn = mul2(1.52587890625e-05f, dn);
+      const float2 h = sub2(rh, w);
+      if (k + 4 < NSL) {
+        two_sum2(h, rl, rh, rl);
+        rl = mul2(65536.f, rl);
+      } else {
+        rh = __fadd2_rn(h, rl);
+      }
+      rh = mul2(65536.f, rh);
     }
     float2 c[2];
     c[0] = __fadd2_rn(__ffma2_rn(w, make_float2(0.00390625f, 0.00390625f), rnd), rnd_n);
@@ -770,10 +774,9 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
           const int e0 = __shfl_sync(0xffffffffu, E_mine, 8 * cb + 2 * tc);
           const int e1 = __shfl_sync(0xffffffffu, E_mine, 8 * cb + 2 * tc + 1);
           const float2 up = make_float2(pow2f(16 - e0), pow2f(16 - e1));
-          const float2 dn = make_float2(-pow2f(e0 - 16), -pow2f(e1 - 16));
           uint32_t code[4][NSL];
 #pragma unroll
-          for (int rb = 0; rb < 4; ++rb) slice_codes2_df<BF16, NSL>(hi[cb][rb], lo[cb][rb], up, dn, code[rb]);
+          for (int rb = 0; rb < 4; ++rb) slice_codes2_df<BF16, NSL>(hi[cb][rb], lo[cb][rb], up, code[rb]);
 #pragma unroll
           for (int q0 = 0; q0 < NSL; q0 += G::kGroup) {
             if (cb > 0 || q0 > 0) {
@@ -927,17 +930,17 @@ __device__ __forceinline__ void slice_row(const float2 (&vh)[2], const float2 (&
 #pragma unroll
   for (int k = 0; k < 2; ++k) amax = fmaxf(amax, fmaxf(fabsf(vh[k].x), fabsf(vh[k].y)));
   const int E = block_exp(warp_max(amax));
-  const float2 up = make_float2(pow2f(16 - E), pow2f(16 - E)), dn = make_float2(-pow2f(E - 16), -pow2f(E - 16));
+  const float2 up = make_float2(pow2f(16 - E), pow2f(16 - E));
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     if (nr == kLowNS) {
       uint32_t code[kLowNS];
-      slice_codes2_df<BF16, kLowNS>(vh[k], vl[k], up, dn, code);
+      slice_codes2_df<BF16, kLowNS>(vh[k], vl[k], up, code);
 #pragma unroll
       for (int q = 0; q < kLowNS; ++q) out32[q * half + idx + 32 * k] = code[q];
     } else {
       uint32_t code[4];
-      slice_codes2_df<BF16, 4>(vh[k], vl[k], up, dn, code);
+      slice_codes2_df<BF16, 4>(vh[k], vl[k], up, code);
 #pragma unroll
       for (int q = 0; q < 4; ++q) out32[q * half + idx + 32 * k] = code[q];
     }
@@ -1365,11 +1368,9 @@ static_assert(kLowM == 32 && kLowK3 == kLowM, "the inverse product's k is one st
 
 // The slices of one double-float value on a single lane (the packed routine on lane x).
 template <bool BF16>
-__device__ __forceinline__ void slice_codes_df(float vh, float vl, float up, float dn,
-                                               uint16_t (&code)[kLowNS]) {
+__device__ __forceinline__ void slice_codes_df(float vh, float vl, float up, uint16_t (&code)[kLowNS]) {
   uint32_t c2[kLowNS];
-  slice_codes2_df<BF16, kLowNS>(make_float2(vh, 0.f), make_float2(vl, 0.f), make_float2(up, up),
-                                make_float2(dn, dn), c2);
+  slice_codes2_df<BF16, kLowNS>(make_float2(vh, 0.f), make_float2(vl, 0.f), make_float2(up, up), c2);
 #pragma unroll
   for (int k = 0; k < kLowNS; ++k) code[k] = static_cast<uint16_t>(c2[k] & 0xffffu);
 }
@@ -1442,7 +1443,7 @@ k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
       const f2 j = (r & 1) ? df_norm(d.s.y, d.c.y) : df_norm(d.s.x, d.c.x);
       const int E = block_exp(warp_max(fabsf(j.hi)));
       uint16_t code[kLowNS];
-      slice_codes_df<BF16>(j.hi, j.lo, pow2f(16 - E), -pow2f(E - 16), code);
+      slice_codes_df<BF16>(j.hi, j.lo, pow2f(16 - E), code);
 #pragma unroll
       for (int p = 0; p < kLowNS; ++p) jt[p * plane + static_cast<size_t>(x) * kLowK3 + lane] = code[p];
       if (lane == 0) S.low_jt_e[x] = static_cast<int8_t>(E);

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from oracle import biharmonic as ob
+from oracle import biharmonic3d as o3
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -38,5 +39,33 @@ def test_preconditioner_reports_a_wait_that_ran_out(ext, prec):
             with pytest.raises(ext.ExtError) as e:
                 call(c, prob, torch.ones_like(r), r, torch.empty_like(r))
             assert e.value.code == ext.EXT_ETIMEOUT
+    finally:
+        ext.ext_destroy(c)
+
+
+@pytest.mark.parametrize("prec,kw", [("fp32", {}), ("mixed_bf16", {}), ("mixed_fp16", dict(low_modes=0)),
+                                     ("mixed_bf16", dict(low_modes=1))])
+@pytest.mark.parametrize("shape", [(70, 60), (250, 300), (128, 128, 128)])
+def test_preconditioner_of_a_small_residual(ext, prec, kw, shape):
+    """Residuals far below one against the oracle's box solve, within the bound of the other preconditioner
+    tests at magnitude one, 5e-6 of the largest entry.  (What FP32's range takes is below that down to
+    1e-31: an element of r or T1..T3 is off by 2^-143 at most, one of z by 4 sqrt(N) 2^-143.)"""
+    phi = _phi(shape, 5)
+    r0 = np.where(phi < 0, 0, np.random.default_rng(6).standard_normal(shape))
+    two = len(shape) == 2
+    bcs = ("symmetric", "dirichlet") if two else ("symmetric", "dirichlet", "periodic")
+    prob = ext.problem(*shape[::-1], *bcs) if two else ext.problem3(*shape[::-1], *bcs)
+    call = ext.ext_apply_preconditioner if two else ext.ext_apply_preconditioner3d
+    c = ext.ext_create(ext.options(prec, **kw))
+    try:
+        for size in (1.0, 1e-25, 1e-28, 1e-31):
+            r = (r0 * size).astype(np.float32)
+            z = torch.empty(shape, device="cuda")
+            scale = call(c, prob, dev(phi), dev(r), z)
+            r = r.astype(np.float64)
+            ref = ob.poisson_squared_pinv(r, *bcs) if two else o3.poisson_squared_pinv3(r, bcs)
+            ref[phi < 0] = 0
+            np.testing.assert_allclose(z.cpu().numpy().astype(np.float64) / scale, ref, rtol=0,
+                                       atol=5e-6 * np.abs(ref).max(), err_msg=f"magnitude {size}")
     finally:
         ext.ext_destroy(c)
