@@ -201,6 +201,14 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// One warp: the sum of the eight warps' values sh[0..7] of a block of 256 threads, in every lane.
+__device__ __forceinline__ double sum_of_eight(const double* sh) {
+  double v = sh[threadIdx.x & 7];
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // Block sum of up to two values; result valid in thread 0.  `sh` holds >= 2*32 doubles.
 template <int NT>
 __device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
@@ -350,6 +358,35 @@ __device__ __forceinline__ double block_sum_comp(CompDot d, float2* sh) {
   }
   return t;
 }
+
+// Sum of exact products in three FP32 numbers (TwoProd, and a TwoSum for every rounding but the last
+// number's): about 70 bits while no product's error term leaves FP32's range, so that its FP64 value is
+// as good as a sum kept in FP64, at the rate of FP32.
+struct Sum3 {
+  float s = 0.f, c = 0.f, d = 0.f;
+  __device__ __forceinline__ void join(float s2, float c2, float d2) {
+    float e, t;
+    two_sum(s, s2, s, e);
+    two_sum(c, c2, c, t);
+    d = __fadd_rn(d, __fadd_rn(d2, t));
+    two_sum(c, e, c, t);
+    d = __fadd_rn(d, t);
+  }
+  __device__ __forceinline__ void add_prod(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    join(p, __fmaf_rn(a, b, -p), 0.f);
+  }
+  // the sum over groups of W consecutive lanes in a fixed butterfly
+  template <int W>
+  __device__ __forceinline__ void reduce() {
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) {
+      const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
+      join(s2, c2, __shfl_xor_sync(0xffffffffu, d, o));
+    }
+  }
+  __device__ __forceinline__ double value() const { return (double)s + ((double)c + (double)d); }
+};
 
 // ------------------------------------------------------------------------------------------
 // Double-float arithmetic (Dekker, Knuth): a value is an unevaluated FP32 pair hi + lo with

@@ -1068,9 +1068,10 @@ k_output64(const SlotDesc* __restrict__ slots, const float* __restrict__ f, doub
 // ---------------------------------------------------------------------------------------------
 // q = M L^2 p for a caller-supplied FP32 p (the solver's compensated evaluation; used by the entry
 // point that allocates nothing): mask from phi's sign, 64 x 16 tiles, the window of p in shared
-// memory, p.q per tile in compensated FP32 (an FP64 product per node took longer than the rest of
-// the kernel).  12 bytes a node; a call on 1000 x 700 nodes is bound by its launches and the copy
-// of p.q back, so the descriptor travels as a kernel argument.
+// memory.  p.q, of whatever magnitude the caller's p has, is an FP64 sum: a warp whose products are
+// within the range that Sum3 is exact in adds them so (an FP64 product per node took longer than the
+// rest of the kernel), any other in FP64.  12 bytes a node; a call on 1000 x 700 nodes is bound by its
+// launches and the copy of p.q back, so the descriptor travels as a kernel argument.
 // ---------------------------------------------------------------------------------------------
 template <bool ANISO>
 __global__ void __launch_bounds__(kStThreads)
@@ -1079,7 +1080,7 @@ k_apply(const __grid_constant__ SlotDesc S, const float* __restrict__ phi, int e
   constexpr int TY = kApplyTileY;
   __shared__ __align__(16) float win[kWX * (TY + 4)];  // rows y0-2 .., columns x0-4 ..
   __shared__ __align__(16) float lap[ANISO ? 1 : 2][ANISO ? 4 : kWX * (TY + 4)];  // g(p), hi and lo
-  __shared__ float2 red[kStThreads / 32];
+  __shared__ double red[kStThreads / 32];
   const int ntx = (S.nx + kStTileX - 1) / kStTileX;
   const int tile = blockIdx.x;
   const int x0 = (tile % ntx) * kStTileX, y0 = (tile / ntx) * TY;
@@ -1101,9 +1102,12 @@ k_apply(const __grid_constant__ SlotDesc S, const float* __restrict__ phi, int e
     lap_tile<TY, kWX, false>(win, nullptr, lap[0], lap[ANISO ? 0 : 1]);
     __syncthreads();
   }
-  CompDot dot;
+  constexpr int kOwn = kStTileX * TY / (2 * kStThreads);  // node pairs per thread
+  float pv[2 * kOwn], qv[2 * kOwn];                       // p and q of the products (zeros elsewhere)
 #pragma unroll
-  for (int k = threadIdx.x; k < kStTileX * TY / 2; k += kStThreads) {
+  for (int j = 0; j < kOwn; ++j) {
+    const int k = threadIdx.x + j * kStThreads;
+    pv[2 * j] = pv[2 * j + 1] = qv[2 * j] = qv[2 * j + 1] = 0.f;
     const int ly = k / (kStTileX / 2), lx = 2 * (k - ly * (kStTileX / 2));
     const int gx = x0 + lx, gy = y0 + ly;
     if (gx >= S.nx || gy >= S.ny) continue;
@@ -1125,15 +1129,41 @@ k_apply(const __grid_constant__ SlotDesc S, const float* __restrict__ phi, int e
     }
     const float q0 = u0 ? r.x : 0.f, q1 = u1 ? r.y : 0.f;
     q[g] = q0;
-    dot.add(c[0], q0);
+    pv[2 * j] = c[0];
+    qv[2 * j] = q0;
     if (two) {
       q[g + 1] = q1;
-      dot.add(c[1], q1);
+      pv[2 * j + 1] = c[1];
+      qv[2 * j + 1] = q1;
     }
   }
-  const double t = block_sum_comp<kStThreads>(dot, red);
-  if (threadIdx.x == 0) part[tile] = t;
+  // a product is zero because a factor is, or it and its error term are normal numbers
+  bool plain = true;
+#pragma unroll
+  for (int i = 0; i < 2 * kOwn; ++i) {
+    const float m = fabsf(__fmul_rn(pv[i], qv[i]));
+    plain = plain && ((m > 0x1p-90f && m < 0x1p100f) || (m == 0.f && (pv[i] == 0.f || qv[i] == 0.f)));
+  }
+  double t = 0.0;
+  if (__all_sync(0xffffffffu, plain)) {
+    Sum3 sum;
+#pragma unroll
+    for (int i = 0; i < 2 * kOwn; ++i) sum.add_prod(pv[i], qv[i]);
+    sum.reduce<32>();
+    t = sum.value();
+  } else {
+#pragma unroll
+    for (int i = 0; i < 2 * kOwn; ++i) t += (double)pv[i] * (double)qv[i];
+    t = warp_sum(t);
+  }
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    t = sum_of_eight(red);
+    if (threadIdx.x == 0) part[tile] = t;
+  }
 }
+
 
 // ---------------------------------------------------------------------------------------------
 // Launchers

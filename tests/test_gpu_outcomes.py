@@ -69,3 +69,24 @@ def test_preconditioner_of_a_small_residual(ext, prec, kw, shape):
                                        atol=5e-6 * np.abs(ref).max(), err_msg=f"magnitude {size}")
     finally:
         ext.ext_destroy(c)
+
+
+@pytest.mark.parametrize("size", ["1", "1e-25", "1e20", "1e-40", "spread"])
+@pytest.mark.parametrize("nx,ny", [(5, 4), (65, 17), (700, 430)])
+def test_sum_of_the_operator_without_a_context(ext, nx, ny, size):
+    """p.q against the exact sum of the products p q of the q returned.  Tolerance: a tile's and the call's
+    sums are FP64, at most 4 + 5 + 8 + 30 additions deep (512 x 512 nodes; a thread's, a warp's, a block's,
+    the tiles'), each 2^-53 of the sum of magnitudes: 47 2^-53."""
+    from fractions import Fraction
+    rng = np.random.default_rng(nx)
+    p = rng.standard_normal((ny, nx))
+    p = p * (10.0 ** rng.uniform(-30, 15, (ny, nx)) if size == "spread" else float(size))
+    phi = _phi((ny, nx), 2)
+    p[phi < 0] = 0
+    p = p.astype(np.float32)
+    q = torch.empty((ny, nx), device="cuda")
+    rc, got = ext.ext_apply_biharmonic_noalloc(ext.problem(nx, ny, "symmetric", "periodic"), dev(phi), dev(p), q)
+    assert rc == ext.EXT_OK
+    terms = [Fraction(float(a)) * Fraction(float(b)) for a, b in zip(p.ravel(), q.cpu().numpy().ravel()) if a and b]
+    want, size_of = sum(terms), sum(abs(t) for t in terms)
+    assert size_of > 0 and abs(Fraction(got) - want) <= 47 * size_of / 2 ** 53
