@@ -338,10 +338,19 @@ __device__ __forceinline__ void group_sum_pair(float& s, float& c) {
   }
 }
 
-// Block sum of compensated per-thread accumulators by FP32 TwoSum butterflies, inside the warps
-// and then across them; FP64 only for the result.  The SM adds two FP64 numbers a cycle (a warp
-// instruction takes 16), so FP64 stays out of every step that each warp would repeat.  Result
-// valid in thread 0.  `sh` >= NT / 32 float2.
+// One warp: the FP64 sum of the pairs sh[0..7] of a block's eight warps, in every lane.
+__device__ __forceinline__ double sum_of_eight(const float2* sh) {
+  const float2 p = sh[threadIdx.x & 7];
+  double v = (double)p.x + (double)p.y;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Block sum of compensated per-thread accumulators: FP32 TwoSum butterflies inside the warps, FP64 across
+// them, by one warp.  The SM adds two FP64 numbers a cycle (a warp instruction takes 16), so FP64
+// stays out of every step that each warp would repeat.  Result valid in the first warp.
+// `sh` >= NT / 32 float2.
 template <int NT>
 __device__ __forceinline__ double block_sum_comp(CompDot d, float2* sh) {
   static_assert(NT / 32 == 8, "eight warps");
@@ -349,14 +358,7 @@ __device__ __forceinline__ double block_sum_comp(CompDot d, float2* sh) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   if (l == 0) sh[w] = make_float2(d.s, d.c);
   __syncthreads();
-  double t = 0.0;
-  if (w == 0) {
-    const float2 v = sh[l & 7];
-    float s = v.x, c = v.y;
-    group_sum_pair<8>(s, c);
-    if (l == 0) t = (double)s + (double)c;
-  }
-  return t;
+  return w == 0 ? sum_of_eight(sh) : 0.0;
 }
 
 // Sum of exact products in three FP32 numbers (TwoProd, and a TwoSum for every rounding but the last

@@ -765,12 +765,9 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     // next tile writes blk_sm only after its own block barriers, which these threads join later
     if (threadIdx.x < 32) {
       const int j = (lane >> 3) & (TY / 16 - 1);  // eight lanes per block, one per warp's pair
-      const float2 v = blk_sm[j][lane & 7];
-      float sv = v.x, cv = v.y;
-      group_sum_pair<8>(sv, cv);
+      const double v = sum_of_eight(blk_sm[j]);
       const int by = (y0 >> 4) + j;
-      if ((lane & 7) == 0 && lane < TY / 2 && 16 * by < S.ny)
-        S.pq_part[by * nbx + x0 / kStTileX] = (double)sv + (double)cv;
+      if ((lane & 7) == 0 && lane < TY / 2 && 16 * by < S.ny) S.pq_part[by * nbx + x0 / kStTileX] = v;
     }
   }
   }

@@ -90,3 +90,23 @@ def test_sum_of_the_operator_without_a_context(ext, nx, ny, size):
     terms = [Fraction(float(a)) * Fraction(float(b)) for a, b in zip(p.ravel(), q.cpu().numpy().ravel()) if a and b]
     want, size_of = sum(terms), sum(abs(t) for t in terms)
     assert size_of > 0 and abs(Fraction(got) - want) <= 47 * size_of / 2 ** 53
+
+
+@pytest.mark.parametrize("tile_y", [16, 32])
+def test_direction_sums_are_fp64_across_warps(ext, tile_y):
+    """p.q of the stencil, one 64 x 16 block: a single node of p per warp, three columns apart, so that
+    each warp's sum is one product 20 p^2, exact in a pair of FP32 numbers; the eight together span 53 bits,
+    exact in FP64 and not in such a pair."""
+    nx, ny = 64, 16
+    p = np.zeros((ny, nx), np.float32)
+    vals = [(2 ** 19 - 1) * 2 ** 6] + [2 ** 19 - 1 - 2 * k for k in range(1, 6)]
+    for w, v in enumerate(vals):
+        p[2 + w, 4 + 6 * w] = v  # rows 2..7: the warps that hold them, away from the edges
+    q = torch.empty((ny, nx), device="cuda")
+    c = ext.ext_create(ext.options("fp32", autotune=0, tile_y=tile_y))
+    try:
+        got = ext.ext_apply_biharmonic(c, ext.problem(nx, ny), dev(np.ones_like(p)), dev(p), q)
+    finally:
+        ext.ext_destroy(c)
+    want = 20 * sum(v * v for v in vals)
+    assert want.bit_length() - 2 <= 53 and int(got) == want, (got, want)
