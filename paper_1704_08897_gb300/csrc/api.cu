@@ -1007,6 +1007,7 @@ static int get_workspace(ext_ctx* ctx, int count, const ext_problem* probs, bool
 static LaunchCfg cfg_of(ext_ctx* ctx, Workspace* W, int which) {
   LaunchCfg c;
   c.wait_cycles = ctx->opt.wait_cycles;
+  c.dots3 = ctx->opt.prec == EXT_PREC_FP32;
   c.pdl = !ctx->opt.profile;  // a profiled kernel is bracketed by event records
   c.slots = W->d_slots;
   c.tcp = W->d_tcp;
@@ -1917,6 +1918,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   t.d_descs = descs;
   t.split = ctx->split;
   t.ns = NS;
+  t.dots3 = ctx->opt.prec == EXT_PREC_FP32;
   t.d_err = ctx->d_err;
   t.wait_cycles = ctx->opt.wait_cycles;
   t.sm_count = ctx->sm_count;

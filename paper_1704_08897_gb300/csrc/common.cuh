@@ -366,6 +366,8 @@ __device__ __forceinline__ double block_sum_comp(CompDot d, float2* sh) {
 // as good as a sum kept in FP64, at the rate of FP32.
 struct Sum3 {
   float s = 0.f, c = 0.f, d = 0.f;
+  __device__ __forceinline__ Sum3() {}
+  __device__ __forceinline__ Sum3(float s0, float c0, float d0 = 0.f) : s(s0), c(c0), d(d0) {}
   __device__ __forceinline__ void join(float s2, float c2, float d2) {
     float e, t;
     two_sum(s, s2, s, e);
@@ -387,8 +389,18 @@ struct Sum3 {
       join(s2, c2, __shfl_xor_sync(0xffffffffu, d, o));
     }
   }
-  __device__ __forceinline__ double value() const { return (double)s + ((double)c + (double)d); }
+  template <bool THIRD = true>
+  __device__ __forceinline__ double value() const {
+    return (double)s + (THIRD ? (double)c + (double)d : (double)c);
+  }
 };
+// The preconditioner's dot products over W lanes: as good as FP64 sums in FP32 mode (DOTS3), in pairs in the
+// mixed modes (as one form for both, 1 us of 60 an iteration slower: more registers in the unfold).
+template <int W, bool DOTS3>
+__device__ __forceinline__ void reduce_dots(Sum3& v) {
+  if (DOTS3) v.reduce<W>();
+  else group_sum_pair<W>(v.s, v.c);
+}
 
 // ------------------------------------------------------------------------------------------
 // Double-float arithmetic (Dekker, Knuth): a value is an unevaluated FP32 pair hi + lo with

@@ -23,6 +23,7 @@ struct LaunchCfg {
   // programmatic dependent launch: the grid may start its prologue while the stream's previous
   // kernel still runs (every kernel launched this way begins its reads with pdl_wait)
   bool pdl = false;
+  bool dots3 = false;  // FP32 mode: r.z and z.q are added as three FP32 numbers (reduce_dots)
 };
 
 // Launch `kernel` under `c` (its stream and dependence form).
@@ -112,6 +113,7 @@ struct Tc3 {
   const int* d_counts = nullptr;  // [7]
   int n_items[7] = {};
   int split = 0, ns = 4;
+  bool dots3 = false;             // LaunchCfg::dots3
   int* d_err = nullptr;
   long long wait_cycles = 0;
   int sm_count = 148;

@@ -122,7 +122,7 @@ struct Ctl {
   uint64_t drain;
   uint32_t tmem;
   int abort_flag;
-  float4 red[kEpiWarps];                  // stage 3: per-warp compensated r.z and z.q
+  Sum3 red[2][kEpiWarps];                 // stage 3: per-warp r.z and z.q
   float colmax[4][16][4];                 // [column group][column][lane quarter]
 };
 static_assert(sizeof(Ctl) <= 2048, "control block too large");
@@ -346,7 +346,8 @@ __device__ __forceinline__ void merge_orders(const float2 (&v)[NSL], float2 scl,
   }
 }
 
-template <bool BF16, int STAGE, int NSL>
+// DOTS3: FP32 mode's stage 3 (reduce_dots)
+template <bool BF16, int STAGE, int NSL, bool DOTS3 = false>
 __global__ void __maxnreg__(kMaxRegs)
 k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items,
           const int* __restrict__ n_items, int mode, int* __restrict__ err, long long wait_cycles) {
@@ -887,20 +888,25 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
             }
         }
         if (mir_out) continue;  // a class problem leaves no partial sums
-        // tile partials of r.z and z.q: butterflies in the warps, then across them by warp 0;
-        // k_prec_finish forms rho and beta from them
-        group_sum_pair<32>(c_rz.s, c_rz.c);
-        if (with_zq) group_sum_pair<32>(c_zq.s, c_zq.c);
-        if (lane == 0) ctl->red[ew] = make_float4(c_rz.s, c_rz.c, c_zq.s, c_zq.c);
+        // tile partials of r.z and z.q: butterflies in the warps, then across them by warp 0; k_prec_finish forms rho and beta from them
+        Sum3 rz(c_rz.s, c_rz.c), zq(c_zq.s, c_zq.c);
+        reduce_dots<32, DOTS3>(rz);
+        if (with_zq) reduce_dots<32, DOTS3>(zq);
+        if (lane == 0) {
+          ctl->red[0][ew] = rz;
+          if (with_zq) ctl->red[1][ew] = zq;
+        }
         epi_bar();
         if (ew == 0) {
-          const float4 t = ctl->red[lane % kEpiWarps];
-          float sv = t.x, cv = t.y, sq = t.z, cq = t.w;
-          group_sum_pair<kEpiWarps>(sv, cv);
-          if (with_zq) group_sum_pair<kEpiWarps>(sq, cq);
+          rz = ctl->red[0][lane % kEpiWarps];
+          reduce_dots<kEpiWarps, DOTS3>(rz);
+          if (with_zq) {
+            zq = ctl->red[1][lane % kEpiWarps];
+            reduce_dots<kEpiWarps, DOTS3>(zq);
+          }
           if (lane == 0) {
-            S.part[it.tile * 4 + 2] = (double)sv + (double)cv;
-            S.part[it.tile * 4 + 3] = with_zq ? (double)sq + (double)cq : 0.0;
+            S.part[it.tile * 4 + 2] = rz.value<DOTS3>();
+            S.part[it.tile * 4 + 3] = with_zq ? zq.value<DOTS3>() : 0.0;
           }
         }
         // ctl->red is rewritten only after the next tile's vote, which this warp joins later
@@ -1261,10 +1267,12 @@ k_update_slice(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ 
 
 // One thread per class node (tiles of 32 x 8): z at the node and its mirrors, masked, with the
 // tile's compensated r.z and z.q partials.
+template <bool DOTS3>
 __global__ void __launch_bounds__(256)
 k_unfold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
          const WorkItem* __restrict__ items, const int* __restrict__ n_items, int mode) {
-  __shared__ float4 red[8];
+  __shared__ float4 red[8];  // r.z and z.q of each warp
+  __shared__ float2 red_d[DOTS3 ? 8 : 1];
   const int total = *n_items;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_wait();
@@ -1324,18 +1332,24 @@ k_unfold(const SlotDesc* __restrict__ slots, const SlotDesc* __restrict__ tcp,
       }
     }
     // the tile's sums: butterflies inside the warps and, by warp 0, across the eight
-    group_sum_pair<32>(c_rz.s, c_rz.c);
-    if (with_zq) group_sum_pair<32>(c_zq.s, c_zq.c);
-    if (lane == 0) red[warp] = make_float4(c_rz.s, c_rz.c, c_zq.s, c_zq.c);
+    Sum3 rz(c_rz.s, c_rz.c), zq(c_zq.s, c_zq.c);
+    reduce_dots<32, DOTS3>(rz);
+    if (with_zq) reduce_dots<32, DOTS3>(zq);
+    if (lane == 0) {
+      red[warp] = make_float4(rz.s, rz.c, zq.s, zq.c);
+      if (DOTS3) red_d[warp] = make_float2(rz.d, zq.d);
+    }
     __syncthreads();
     if (warp == 0) {
       const float4 v = red[lane & 7];
-      float sv = v.x, cv = v.y, sq = v.z, cq = v.w;
-      group_sum_pair<8>(sv, cv);
-      if (with_zq) group_sum_pair<8>(sq, cq);
+      const float2 d = DOTS3 ? red_d[lane & 7] : make_float2(0.f, 0.f);
+      rz = Sum3(v.x, v.y, d.x);
+      zq = Sum3(v.z, v.w, d.y);
+      reduce_dots<8, DOTS3>(rz);
+      if (with_zq) reduce_dots<8, DOTS3>(zq);
       if (lane == 0) {
-        S.part[it.tile * 4 + 2] = (double)sv + (double)cv;
-        S.part[it.tile * 4 + 3] = with_zq ? (double)sq + (double)cq : 0.0;
+        S.part[it.tile * 4 + 2] = rz.value<DOTS3>();
+        S.part[it.tile * 4 + 3] = with_zq ? zq.value<DOTS3>() : 0.0;
       }
     }
     __syncthreads();
@@ -1452,16 +1466,16 @@ k_low_mid(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   }
 }
 
-template <bool BF16, int STAGE, int NSL>
+template <bool BF16, int STAGE, int NSL, bool DOTS3 = false>
 cudaError_t set_attr() {
-  return cudaFuncSetAttribute(k_prec_tc<BF16, STAGE, NSL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(k_prec_tc<BF16, STAGE, NSL, DOTS3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               TcGeom<STAGE, NSL>::kSmem);
 }
 
-template <bool BF16, int STAGE, int NSL>
+template <bool BF16, int STAGE, int NSL, bool DOTS3 = false>
 void launch_one(const LaunchCfg& c, int mode, int* err) {
   const long long wc = c.wait_cycles > 0 ? c.wait_cycles : kWaitCycles;
-  launch_cfg(c, k_prec_tc<BF16, STAGE, NSL>, c.grid, kThreads, TcGeom<STAGE, NSL>::kSmem, c.slots, c.items,
+  launch_cfg(c, k_prec_tc<BF16, STAGE, NSL, DOTS3>, c.grid, kThreads, TcGeom<STAGE, NSL>::kSmem, c.slots, c.items,
              c.n_items, mode, err, wc);
 }
 
@@ -1471,7 +1485,9 @@ void launch_all(const LaunchCfg& c, int stage, int mode, int* err) {
     case 0: launch_one<BF16, 0, NSL>(c, mode, err); break;
     case 1: launch_one<BF16, 1, NSL>(c, mode, err); break;
     case 2: launch_one<BF16, 2, NSL>(c, mode, err); break;
-    default: launch_one<BF16, 3, NSL>(c, mode, err); break;
+    default:
+      if (NSL == 6 && c.dots3) launch_one<BF16, 3, NSL, NSL == 6>(c, mode, err);
+      else launch_one<BF16, 3, NSL>(c, mode, err);
   }
 }
 
@@ -1503,14 +1519,15 @@ int tc_block() { return KC; }
 
 cudaError_t tc_init() {
   cudaError_t e = cudaSuccess;
-  const cudaError_t r[20] = {set_attr<false, 0, 4>(), set_attr<false, 1, 4>(), set_attr<false, 2, 4>(),
+  const cudaError_t r[22] = {set_attr<false, 0, 4>(), set_attr<false, 1, 4>(), set_attr<false, 2, 4>(),
                              set_attr<false, 3, 4>(), set_attr<true, 0, 4>(),  set_attr<true, 1, 4>(),
                              set_attr<true, 2, 4>(),  set_attr<true, 3, 4>(),  set_attr<true, 0, 6>(),
                              set_attr<true, 1, 6>(),  set_attr<true, 2, 6>(),  set_attr<true, 3, 6>(),
                              set_attr<false, 0, 6>(), set_attr<false, 1, 6>(), set_attr<false, 2, 6>(),
                              set_attr<false, 3, 6>(),
                              set_attr<false, kLowFwd, 6>(), set_attr<false, kLowInv, 6>(),
-                             set_attr<true, kLowFwd, 6>(), set_attr<true, kLowInv, 6>()};
+                             set_attr<true, kLowFwd, 6>(), set_attr<true, kLowInv, 6>(),
+                             set_attr<false, 3, 6, true>(), set_attr<true, 3, 6, true>()};
   for (cudaError_t x : r)
     if (x != cudaSuccess) e = x;
   return e;
@@ -1542,7 +1559,8 @@ void launch_update_slice(const LaunchCfg& c, int split_kind, bool fuse_pq) {
 }
 
 void launch_unfold(const LaunchCfg& c, int mode) {
-  launch_cfg(c, k_unfold, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
+  if (c.dots3) launch_cfg(c, k_unfold<true>, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
+  else launch_cfg(c, k_unfold<false>, c.grid, 256, 0, c.slots, c.tcp, c.items, c.n_items, mode);
 }
 
 void launch_prec_tc(const LaunchCfg& c, int stage, int mode, int split_kind, int ns, int* err) {

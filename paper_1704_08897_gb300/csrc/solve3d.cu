@@ -363,7 +363,7 @@ k3_init(size_t n, const double* __restrict__ b, double s, float* __restrict__ rh
 __global__ void __launch_bounds__(kT, 4)
 k3_update(size_t n, const SlotScalars* sc, const float* ph, const float* pl, const float* qh,
           const float* ql, float* xh, float* xl, float* rh, float* rl, double* __restrict__ part) {
-  __shared__ float2 sh[kT / 32];
+  __shared__ double sh[kT / 32];
   if (gate_shut(&sc->active)) return;
   const f2 alpha{sc->alpha_f[0], sc->alpha_f[1]}, na{-alpha.hi, -alpha.lo};
   CompDotDF rr;
@@ -396,8 +396,14 @@ k3_update(size_t n, const SlotScalars* sc, const float* ph, const float* pl, con
       df_axpy(rh[i], rl[i], na, qh[i], ql[i]);
       rr.add(rh[i], rl[i], rh[i], rl[i]);
     }
-  const double s = block_sum_comp<kT>(rr.as_comp(), sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  Sum3 v(rr.s, rr.c);
+  v.reduce<32>();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v.value();
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double s = sum_of_eight(sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+  }
 }
 
 // p = z + beta p (double-float)
@@ -511,7 +517,7 @@ __global__ void __launch_bounds__(kGt)
 k3_gemm(Gemm3 g, const int* __restrict__ gate) {
   __shared__ __align__(16) float As[2][2][GK][GM + 1];  // [buffer][hi, lo][k][m]
   __shared__ __align__(16) float Bs[2][2][GK][GN + 4];
-  __shared__ float2 sh[kGt / 32];
+  __shared__ double sh[kGt / 32];
   if (gate_shut(gate)) return;
   const float* Bl = g.B + static_cast<size_t>(g.ldb) * g.ldb;
   const int m0 = blockIdx.x * GM, n0 = blockIdx.y * GN;
@@ -587,15 +593,12 @@ k3_gemm(Gemm3 g, const int* __restrict__ gate) {
       g.outl[o] = v.lo;
     }
   if (FORM == 2) {
-    group_sum_pair<32>(dot.s, dot.c);
-    if ((t & 31) == 0) sh[t >> 5] = make_float2(dot.s, dot.c);
+    Sum3 v(dot.s, dot.c);
+    v.reduce<32>();
+    if ((t & 31) == 0) sh[t >> 5] = v.value();
     __syncthreads();
-    if (t < 32) {
-      const float2 v = sh[t & 3];
-      float s = v.x, c = v.y;
-      group_sum_pair<4>(s, c);
-      if (t == 0) g.part[blockIdx.y * gridDim.x + blockIdx.x] = (double)s + (double)c;
-    }
+    static_assert(kGt == 128, "four warps");
+    if (t == 0) g.part[blockIdx.y * gridDim.x + blockIdx.x] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
   }
 }
 
@@ -752,6 +755,7 @@ void precondition(const Solve3Args& a, const State3& s, float wnorm, const float
     const Tc3& t = s.tc;
     c.slots = t.d_descs;
     c.wait_cycles = t.wait_cycles;
+    c.dots3 = t.dots3;
     c.items = t.d_items[0];
     c.n_items = t.d_counts;
     c.grid = std::max(1, std::min(t.n_items[0], t.sm_count * 8));
