@@ -74,8 +74,10 @@ typedef struct {
   double replace_factor;   /* replace once ||r|| < replace_factor * ||r at last replacement||;
                               default 1e-2                                                     */
   int32_t iters_per_launch;/* CG iterations per CUDA-graph replay; default 10                 */
-  size_t hbm_budget;       /* bytes the serving queue may hold for admitted requests; 0 = 50%
-                              of free device memory at ext_create                             */
+  size_t hbm_budget;       /* bytes of vectors and transform operands that the serving queue may
+                              hold for admitted requests (their tensor maps, exponents and
+                              partial sums, a few KB and below 0.1%, are not counted); 0 = 50% of
+                              free device memory at ext_create                                */
   int32_t flexible;        /* 1 = flexible (Polak-Ribiere) beta, 0 = Fletcher-Reeves beta;
                               default 0: on the benchmark grids it takes fewer iterations and
                               ends nearer the exact solution at the same residual              */

@@ -78,6 +78,7 @@ struct SlotHost {
   int n_tcp = 0;
   char* arena = nullptr;
   size_t bytes = 0;
+  size_t foot = 0;  // of it vectors and transform operands, without descriptors, exponents and partial sums
   float* phi_stage = nullptr;  // device copies when the caller passes host arrays
   float* f_stage = nullptr;
   float* out_stage = nullptr;
@@ -530,8 +531,8 @@ static std::string shape_key(int count, const ext_problem* probs, bool host_io) 
 }
 
 // Device state of one problem: plans, arena layout (allocated here unless `arena` is given), slot
-// descriptor, its tensor-core problems and their tensor maps.  With size_only, only s.bytes is
-// computed.
+// descriptor, its tensor-core problems and their tensor maps.  With size_only, only s.bytes and
+// s.foot are computed.
 static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotHost& s,
                       char* arena = nullptr, bool size_only = false, bool large_call = false) {
   std::lock_guard<std::recursive_mutex> plk(ctx->plan_mu);
@@ -597,9 +598,11 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   // arena layout
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
+  size_t minor = 0;
+  auto take_minor = [&](size_t bytes) { minor += align_up(bytes, 256); return take(bytes); };
   const size_t o_b = take(8 * N), o_x = take(4 * N), o_xl = take(4 * N);
-  const size_t o_part = take(8 * 4 * (size_t)n_part);
-  const size_t o_pqp = take(8 * (size_t)((ny + 15) / 16) * ((nx + 31) / 32));
+  const size_t o_part = take_minor(8 * 4 * (size_t)n_part);
+  const size_t o_pqp = take_minor(8 * (size_t)((ny + 15) / 16) * ((nx + kStTileX - 1) / kStTileX));
   const size_t o_r = take(4 * N), o_p0 = take(4 * N), o_p1 = take(4 * N);
   const size_t o_q = take(4 * N), o_z = take(4 * N), o_mask = take(N);
   const size_t o_rl = take(4 * N), o_p0l = take(4 * N), o_p1l = take(4 * N);
@@ -608,7 +611,7 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
   size_t o_io = 0;
   if (host_io) o_io = take(12 * N);
   const bool st_copy = stencil_copies_fit(nx);
-  const size_t o_smaps = st_copy ? take(kStMaps * sizeof(CUtensorMap)) : 0;
+  const size_t o_smaps = st_copy ? take_minor(kStMaps * sizeof(CUtensorMap)) : 0;
   // tensor-core problems: the slot itself, or its classes c = 2 cls_y + cls_x
   struct TcLay {
     int c = 0;
@@ -628,12 +631,12 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
         if (rc) return rc;
         const size_t Npc = (size_t)L.px->np * L.py->np;
         {
-          L.o_tr = take(2 * nr * Npc);
-          L.o_tt1 = take(2 * NS * Npc);
-          L.o_tt2 = take(2 * NS * Npc);
-          L.o_tt3 = take(2 * NS * Npc);
-          L.o_maps = take(kTcMaps * sizeof(CUtensorMap));
-          L.o_ex = take(4 * (Npc / 64));
+          // stage 1 writes T2 over the residual's slices, which stage 0 was the last to read, and stage 2
+          // T3 over T1; their exponents likewise
+          L.o_tr = L.o_tt2 = take(2 * nr * Npc);
+          L.o_tt1 = L.o_tt3 = take(2 * NS * Npc);
+          L.o_maps = take_minor(kTcMaps * sizeof(CUtensorMap));
+          L.o_ex = take_minor(2 * (Npc / 128));
         }
         if (d.mir) {
           L.o_lx = take(4 * (size_t)L.px->np);
@@ -645,12 +648,13 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
           L.o_ljt = take(2 * (size_t)kLowNS * L.px->np * kLowK3);
           L.o_ljte = take((size_t)L.px->np);
           L.o_lz = take(2 * 4 * (size_t)L.px->n * L.py->n);
-          L.o_lmaps = take(4 * sizeof(CUtensorMap));
+          L.o_lmaps = take_minor(4 * sizeof(CUtensorMap));
         }
         tl.push_back(L);
       }
   }
   s.bytes = off;
+  s.foot = off - minor;
   if (size_only) return EXT_OK;
   if (arena) {
     s.arena = arena;
@@ -753,21 +757,22 @@ static int build_slot(ext_ctx* ctx, const ext_problem& prob, bool host_io, SlotH
       t.lamx = (const float*)(A + L.o_lx);
       t.lamy = (const float*)(A + L.o_ly);
     }
-    const size_t Npc = (size_t)t.nxp * t.nyp, nex = Npc / 64;
+    const size_t Npc = (size_t)t.nxp * t.nyp, nex = Npc / 128;
     t.tc_r = A + L.o_tr;
     t.tc_nr = nr;
     t.tc_t1 = A + L.o_tt1;
     t.tc_t2 = A + L.o_tt2;
     t.tc_t3 = A + L.o_tt3;
     t.tmaps = A + L.o_maps;
-    for (int k = 0; k < 4; ++k) t.tc_e[k] = (int8_t*)(A + L.o_ex + k * nex);
+    for (int k = 0; k < 4; ++k) t.tc_e[k] = (int8_t*)(A + L.o_ex + (k & 1) * nex);
     t.tc_eb[0] = plan_exps(qx, NS, 1);  // Qx^T rows
     t.tc_eb[1] = plan_exps(qy, NS, 1);  // Qy^T rows
     t.tc_eb[2] = plan_exps(qx, NS, 0);  // Qx rows
     t.tc_eb[3] = plan_exps(qy, NS, 0);  // Qy rows
-    // the operands' padding is never written: zero it once (T1..T3 follow the residual in the arena)
-    BX_CUDA(cudaMemset(t.tc_r, 0, L.o_tt3 + 2 * NS * Npc - L.o_tr));
-    BX_CUDA(cudaMemset(A + L.o_ex, 0, 4 * nex));
+    // the operands' padding is never written with anything but zeros: zero it once (T1 follows the
+    // residual in the arena)
+    BX_CUDA(cudaMemset(t.tc_r, 0, L.o_tt1 + 2 * NS * Npc - L.o_tr));
+    BX_CUDA(cudaMemset(A + L.o_ex, 0, 2 * nex));
     CUtensorMap maps[kTcMaps];
     const size_t pxp = (size_t)t.nxp * t.nxp, pyp = (size_t)t.nyp * t.nyp;
     uint16_t* qxb = (uint16_t*)qx->tc[NS == 6];
@@ -2182,7 +2187,7 @@ struct Req {
 struct ServeSlot {
   bool used = false;
   Req* req = nullptr;
-  size_t bytes = 0;
+  size_t bytes = 0, foot = 0;
 };
 
 }  // namespace
@@ -2378,17 +2383,18 @@ static std::vector<int> serve_admit(ext_ctx* ctx) {
       finish_req(S, r, rc);
       continue;
     }
-    if (probe.bytes > S->budget) {
+    if (probe.foot > S->budget) {
       S->queue.pop_front();
       finish_req(S, r, EXT_EADMIT);
       continue;
     }
-    if (S->used + probe.bytes > S->budget) break;  // wait for running solves to free memory
+    if (S->used + probe.foot > S->budget) break;  // wait for running solves to free memory
     S->queue.pop_front();
     S->slots[free_slot].used = true;
     S->slots[free_slot].req = r;
     S->slots[free_slot].bytes = probe.bytes;
-    S->used += probe.bytes;
+    S->slots[free_slot].foot = probe.foot;
+    S->used += probe.foot;
     r->t_admit = Clock::now();
     admitted.push_back(free_slot);
   }
@@ -2510,7 +2516,7 @@ static int serve_retire(ext_ctx* ctx, const std::vector<int>& done) {
     r->res.err_est = err_estimate(sc);
     S->pool.emplace(S->slots[i].bytes, W->slots[i].arena);
     W->slots[i].arena = nullptr;
-    S->used -= S->slots[i].bytes;
+    S->used -= S->slots[i].foot;
     S->slots[i] = ServeSlot{};
     finish_req(S, r, st);
   }

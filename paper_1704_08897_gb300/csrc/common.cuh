@@ -128,9 +128,9 @@ struct SlotDesc {
   int tc_ns;         // slices per transform operand: 4 or 6
   int tc_nr;         // slices of the residual: tc_ns, or 6 where the low-mode correction reads them
   void* tc_t1;       // [NS][nxp][nyp]
-  void* tc_t2;       // [NS][nyp][nxp]
-  void* tc_t3;       // [NS][nxp][nyp]
-  int8_t* tc_e[4];   // block exponents of the A operand of stage s: [rows][K/128]
+  void* tc_t2;       // [NS][nyp][nxp] (in place of the residual)
+  void* tc_t3;       // [NS][nxp][nyp] (in place of T1)
+  int8_t* tc_e[4];   // block exponents of the A operand of stage s: [rows][K/128], 0 and 2, 1 and 3 one array
   const int8_t* tc_eb[4];  // block exponents of the B operand of stage s (transform matrices)
   const void* tmaps; // kTcMaps CUtensorMap (64-byte aligned): A operand of stages 0..3, B of 0..3,
                      // the results of stages 0..2 (store boxes)

@@ -666,6 +666,18 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
             hi[cb][rb] = t.hi;
             lo[cb][rb] = t.lo;
           }
+        // the tile's rows n beyond the grid lie in the padding of the residual's operand, which only zeros
+        // may reach: a residual of NaNs makes NaNs of their zero sums
+        if (n0 + BN > v.n) {
+#pragma unroll
+          for (int cb = 0; cb < kCb; ++cb)
+#pragma unroll
+            for (int rb = 0; rb < 4; ++rb) {
+              const int n = ng + 32 * cb + 2 * tc;
+              if (n >= v.n) hi[cb][rb].x = lo[cb][rb].x = 0.f;
+              if (n + 1 >= v.n) hi[cb][rb].y = lo[cb][rb].y = 0.f;
+            }
+        }
       }
       if (STAGE == kLowFwd) {
         // the tile's share of G = Qy_low^T H (its 128 rows of y), by compensated dot products of

@@ -110,3 +110,26 @@ def test_direction_sums_are_fp64_across_warps(ext, tile_y):
         ext.ext_destroy(c)
     want = 20 * sum(v * v for v in vals)
     assert want.bit_length() - 2 <= 53 and int(got) == want, (got, want)
+
+
+@pytest.mark.parametrize("prec,kw", [("fp32", {}), ("mixed_bf16", {}), ("mixed_bf16", dict(low_modes=1))])
+@pytest.mark.parametrize("nx,ny", [(70, 61), (130, 140), (389, 251), (300, 257)])
+def test_a_residual_of_nans_leaves_nothing_behind(ext, prec, kw, nx, ny):
+    """The transform stages' operands share memory: after a residual of NaNs the same context gives a finite
+    one the z that a fresh context gives, bit for bit."""
+    phi = _phi((ny, nx), 3)
+    r = np.where(phi < 0, 0, np.random.default_rng(4).standard_normal((ny, nx))).astype(np.float32)
+    prob = ext.problem(nx, ny, "symmetric", "dirichlet")
+    zs = []
+    for before in ([], [np.full_like(r, np.nan), np.full_like(r, np.inf)]):
+        c = ext.ext_create(ext.options(prec, **kw))
+        try:
+            z = torch.empty((ny, nx), device="cuda")
+            for bad in before:
+                ext.ext_apply_preconditioner(c, prob, dev(phi), dev(bad), z)
+                assert not torch.isfinite(z).all()
+            ext.ext_apply_preconditioner(c, prob, dev(phi), dev(r), z)
+        finally:
+            ext.ext_destroy(c)
+        zs.append(z)
+    assert torch.isfinite(zs[0]).all() and torch.equal(*zs)

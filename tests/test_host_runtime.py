@@ -255,3 +255,67 @@ assert r["iters"] > 5
 if abs(r["relres_rec"] ** 2 / v - 1) > 1e-12 or abs(r["relres_true"] ** 2 / (v * 1.0001) - 1) > 1e-12: print(r, v)
 """ % maxit)
     assert out.strip() == ""
+
+
+def _footprint_before(nx, ny, six, low, host):
+    """Bytes of a request's arena while FP32 mode kept double-float transform operands and the mixed modes
+    four slices in four arrays: what a serving budget was set by."""
+    pad = lambda n: (n + 127) // 128 * 128
+    pays = lambda n: 2 * pad((n + 1) // 2) <= pad(n)
+    off = [0]
+
+    def take(b):
+        off[0] = (off[0] + int(b) + 255) // 256 * 256
+    n, nxp, nyp = nx * ny, pad(nx), pad(ny)
+    fx, fy = pays(nx), pays(ny)
+    hx, hy = (nx + 1) // 2 if fx else nx, (ny + 1) // 2 if fy else ny
+    gm = (nxp // 128) * (nyp // 64)
+    unfold = -(-hx // 32) * -(-hy // 8) if fx or fy else 0
+    parts = max(-(-nx // 64) * -(-ny // 32), -(-n // 4096), gm, unfold)
+    for b in (8 * n, 4 * n, 4 * n, 32 * parts, 8 * -(-ny // 16) * -(-nx // 32), *[4 * n] * 5, n, *[4 * n] * 5):
+        take(b)
+    for _ in range(6):
+        take(0 if not six or fx or fy else 4 * nxp * nyp)
+    take(4 * nxp), take(4 * nyp)
+    if host:
+        take(12 * n)
+    if nx % 16 == 0:
+        take(7 * 128)
+    if not six or fx or fy:
+        cx, cy = pad(hx), pad(hy)
+        for _ in range((2 if fx else 1) * (2 if fy else 1)):
+            if six:
+                for _ in range(3):
+                    take(8 * cx * cy)
+                take(8 * hx * hy)
+            else:
+                take(2 * (6 if low else 4) * cx * cy)
+                for _ in range(3):
+                    take(8 * cx * cy)
+                take(8 * 128), take(cx * cy // 16)
+            if fx or fy:
+                take(4 * cx), take(4 * cy), take(8 * hx * hy)
+            if low:
+                take(8 * 32 * 32 * (cy // 128)), take(12 * cx * 32), take(cx), take(8 * hx * hy), take(4 * 128)
+    return off[0]
+
+
+@pytest.mark.parametrize("prec,low", [("fp32", 2), ("mixed_bf16", 2), ("mixed_fp16", 1)])
+def test_a_budget_admits_what_it_admitted(fake_cuda, prec, low):
+    """A request is admitted at the footprint it had with the operands of before: axes that fold and do not, rows of tensor copies and not, host and device arrays."""
+    shapes = [(4, 4), (64, 64), (130, 140), (127, 300), (389, 251), (512, 512), (1024, 700), (300, 2048)]
+    budgets = [(nx, ny, host, _footprint_before(nx, ny, prec == "fp32", prec != "fp32" and (low == 1 or ny >= 2048), host))
+               for nx, ny in shapes for host in (False, True)]
+    out = fake_cuda("""
+for nx, ny, host, budget in %r:
+    arrays = [np.zeros((ny, nx), np.float32) if host else Dev(nx * ny) for _ in range(3)]
+    c = ext.ext_create(ext.options(%r, low_modes=%d, hbm_budget=budget))
+    fake.fake_model(5, 1, 0)
+    t = ext.ext_submit(c, ext.problem(nx, ny, "dirichlet"), *arrays)
+    ext.ext_drain(c)
+    r = ext.ext_poll(c, t)["rc"]
+    if r != 0: print(nx, ny, host, budget, r)
+    ext.ext_destroy(c)
+print(faults())
+""" % (budgets, prec, low))
+    assert out.strip() == ""
