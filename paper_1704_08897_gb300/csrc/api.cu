@@ -123,14 +123,14 @@ struct Workspace {
   int* d_dirs = nullptr;
   void* h_ptrs = nullptr;       // pinned staging for the pointer arrays
   // iteration graphs by graph_key (which kernels the lists need: a serving table meets several)
+  struct Ev { int kind; cudaEvent_t a, b; };
   struct Graph {
     cudaGraphExec_t exec = nullptr;
     int64_t nodes = 0;
+    std::vector<Ev> events;  // profiling: event-record nodes of the graph
   };
   std::map<int, Graph> graphs;
   void* d_tmaps = nullptr;      // per slot 8 CUtensorMap (tensor-core modes)
-  struct Ev { int kind; cudaEvent_t a, b; };
-  std::vector<Ev> graph_events;  // profiling: event-record nodes of the graph
   bool aniso = false;
   bool host_io = false;
   cudaStream_t stream = nullptr;  // the context's stream, or the serving worker's own
@@ -474,7 +474,13 @@ void bx::set_weights(SlotDesc& d, double hx, double hy) {
 }
 
 static void drop_graphs(Workspace* W) {
-  for (auto& g : W->graphs) cudaGraphExecDestroy(g.second.exec);
+  for (auto& g : W->graphs) {
+    cudaGraphExecDestroy(g.second.exec);
+    for (auto& e : g.second.events) {
+      cudaEventDestroy(e.a);
+      cudaEventDestroy(e.b);
+    }
+  }
   W->graphs.clear();
 }
 
@@ -489,10 +495,6 @@ static int graph_key(const Workspace* W) {
 static void free_workspace(Workspace* W) {
   if (!W) return;
   drop_graphs(W);
-  for (auto& e : W->graph_events) {
-    cudaEventDestroy(e.a);
-    cudaEventDestroy(e.b);
-  }
   for (auto& s : W->slots) cudaFree(s.arena);
   cudaFree(W->d_slots);
   cudaFree(W->d_sc);
@@ -1209,7 +1211,7 @@ static int ensure_graph(ext_ctx* ctx, Workspace* W) {
   enqueue_iterations(ctx, W, G);
   made.nodes = ctx->launches - before;
   ctx->launches = before;  // captured, not launched
-  W->graph_events.assign(ctx->pending.begin() + pend0, ctx->pending.end());
+  made.events.assign(ctx->pending.begin() + pend0, ctx->pending.end());
   ctx->pending.resize(pend0);
   cudaError_t e = cudaStreamEndCapture(cstream, &g);
   if (e != cudaSuccess) {
@@ -1222,7 +1224,7 @@ static int ensure_graph(ext_ctx* ctx, Workspace* W) {
     g_last_error = std::string("graph instantiate: ") + cudaGetErrorString(e);
     return EXT_ECUDA;
   }
-  W->graphs[key] = made;
+  W->graphs[key] = std::move(made);
   return EXT_OK;
 }
 
@@ -1427,7 +1429,7 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
   ctx->last_tile_y = W->sten_ty;
   rc = ensure_graph(ctx, W);
   if (rc) return rc;
-  const Workspace::Graph graph = W->graphs[graph_key(W)];
+  const Workspace::Graph& graph = W->graphs[graph_key(W)];
   launch_prec(ctx, W, 1);
   BX_CUDA(cudaGetLastError());
   int max_blocks = 0;
@@ -1458,7 +1460,7 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
     if (ctx->opt.profile) {
       BX_CUDA(cudaStreamSynchronize(s));
       harvest(ctx);
-      harvest_graph(ctx, W->graph_events);
+      harvest_graph(ctx, graph.events);
     }
     if (ctx->h_err[seen]) return timed_out(ctx);
     end = W->h_sc + seen * count;

@@ -319,3 +319,26 @@ for nx, ny, host, budget in %r:
 print(faults())
 """ % (budgets, prec, low))
     assert out.strip() == ""
+
+
+def test_profiled_graphs_own_their_events(fake_cuda):
+    """A serving table whose mixes of requests need several iteration graphs, and solves that capture again
+    after a change of the tile height: every event made is destroyed with the context."""
+    out = fake_cuda("""
+phi, f, out = [Dev(300 * 300) for _ in range(3)]
+before = fake.fake_events()
+c = ext.ext_create(ext.options("mixed_bf16", profile=1, low_modes=2))
+for shape in ((60, 60), (300, 290), (250, 200), (60, 60)):  # unfolded, partly folded, folded
+    fake.fake_model(5, 2, 0)
+    t = ext.ext_submit(c, ext.problem(*shape, "dirichlet"), phi, f, out)
+    ext.ext_drain(c)
+    if ext.ext_poll(c, t)["rc"] != 0: print(shape)
+    fake.fake_model(5, 2, 0)
+    r = ext.ext_solve(c, ext.problem(*shape, "dirichlet"), phi, f, out, check=False)
+    if r["rc"] != 0: print(shape, r)
+# each solve's two blocks of ten iterations are in the totals
+if ext.ext_profile_read(c)["true_residual"][1] != 8: print(ext.ext_profile_read(c))
+ext.ext_destroy(c)
+if fake.fake_events() != before: print(fake.fake_events() - before, "events left")
+""")
+    assert out.strip() == ""
