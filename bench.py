@@ -23,7 +23,6 @@ L2 flush between steps (outside the events); the whole loop bracketed by barrier
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
 import statistics
@@ -37,8 +36,6 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
-CSRC = os.path.join(ROOT, "paper_1704_08897_gb300", "csrc")
 
 
 def parse():
@@ -106,19 +103,19 @@ def make_workload(name, rank, args=None):
                    "nodes": nodes, "prec": "mixed_bf16"}
 
 
-# Slice products the tensor cores execute per useful product in the mixed modes (four slices per
-# operand, orders 0..3: 1 + 2 + 3 + 4), and the tile granularity the operands are padded to.
+# Slice products the tensor cores execute per useful product with four slices per operand (orders 0..3:
+# 1 + 2 + 3 + 4), and the tile granularity the operands are padded to.
 TC_PRODUCTS = 10
 TC_PAD = 128
 
 
-# The low-mode products use six slices per operand: orders 0..5, 21 products per useful product,
-# with k padded to 64 in the inverse product.
+# With six slices per operand (the low-mode products; the stages as stage_products says): orders 0..5, 21
+# products per useful product.
 TC_LOW_PRODUCTS = 21
 
 
 def mirror_classes(n, fold=True):
-    """Node counts of one axis's transform problems in the mixed preconditioner: two mirror
+    """Node counts of one axis's transform problems: two mirror
     classes of ceil(n/2) nodes where both, padded to 128, fit in the padded axis, else the axis."""
     pad = lambda m: -(-m // TC_PAD) * TC_PAD
     h = (n + 1) // 2
@@ -147,7 +144,7 @@ def issued_tensor_flop(probs, kind, fold=None, products=lambda p: TC_PRODUCTS):
                 if kind == "low_fwd":
                     fl += 2 * TC_LOW_PRODUCTS * pad(cy) * 32 * pad(cx)
                 elif kind == "low_inv":
-                    fl += 2 * TC_LOW_PRODUCTS * pad(cx) * pad(cy) * 64
+                    fl += 2 * TC_LOW_PRODUCTS * pad(cx) * pad(cy) * 32
                 else:
                     s = int(kind[-1])
                     fl += 2 * products(p) * pad(cx) * pad(cy) * pad(cx if s in (0, 2) else cy)
@@ -158,9 +155,10 @@ def _fold_default():
     return bool(_OPTION_OVERRIDES.get("fold", 1))
 
 
-def algorithmic_cost(probs, kind, low=False):
+def algorithmic_cost(probs, kind, low=False, prec=None):
     """(amount, unit) per launch of one kernel kind over the workload's instances; low: the
-    low-mode correction ran (the residual is then cut into six slices instead of four)."""
+    low-mode correction ran (the residual is then cut into six slices instead of four); prec: the
+    precision mode, whose grids may take six slices by themselves (None: four)."""
     if kind in ("low_fwd", "low_inv"):
         # the lowest 32 modes of one axis against the whole grid: 2 * nx * ny * 32 flop
         return sum(2 * p.nx * p.ny * min(32, p.nx) for p in probs), "flop"
@@ -178,8 +176,8 @@ def algorithmic_cost(probs, kind, low=False):
         return sum(48 * p.nx * p.ny for p in probs), "byte"
     if kind in ("split", "fold"):  # read r (8); write four (six) 16-bit slices: unfolded / folded
         f = kind == "fold"
-        per_node = 8 + 2 * (6 if low else 4)
-        return sum(per_node * p.nx * p.ny for p in probs
+        six = lambda p: low or (prec is not None and stage_products(p, prec, low) == TC_LOW_PRODUCTS)
+        return sum((20 if six(p) else 16) * p.nx * p.ny for p in probs
                    if (len(mirror_classes(p.nx, _fold_default())) > 1 or
                        len(mirror_classes(p.ny, _fold_default())) > 1) == f), "byte"
     if kind == "unfold":    # read the classes' g (8), r (8), mask (1); write z (8); q (8) is read
@@ -238,15 +236,6 @@ class ClockSampler:
 # ----------------------------------------------------------------------------------------------
 # our implementation
 # ----------------------------------------------------------------------------------------------
-def kernel_hash(kind, prec="fp32"):
-    if kind.startswith("prec") or kind in ("split", "fold", "unfold") or kind.startswith("low"):
-        f = "kernels_gemm_tc.cu"
-    else:
-        f = "kernels_grid.cu"
-    with open(os.path.join(CSRC, f), "rb") as fh:
-        return hashlib.sha256(fh.read()).hexdigest()[:16]
-
-
 def reduce_over_ranks(value, op, device):
     """Max or sum of a per-rank number over all ranks (torch.distributed initialised)."""
     import torch
@@ -429,7 +418,7 @@ def run_ours(args, rank, world):
                    for k, (ms, n) in prof.items() if n}
         dom = max(prof, key=lambda k: prof[k][0])
         ms, n = prof[dom]
-        amount, unit = algorithmic_cost(probs, dom, low="low_fwd" in kernels)
+        amount, unit = algorithmic_cost(probs, dom, low="low_fwd" in kernels, prec=prec)
         if amount is not None and n:
             per_launch_s = ms / n / 1e3
             if unit == "flop":
@@ -446,23 +435,16 @@ def run_ours(args, rank, world):
                 with open(PEAKS_FILE) as fh:
                     peak = json.load(fh)["hbm_gbs"]
                 bound, u, peak_src = "hbm", "GB/s", "measured hbm_gbs"
-            traffic = None
-            if os.path.exists(TRAFFIC_FILE):
-                with open(TRAFFIC_FILE) as fh:
-                    tr = json.load(fh)
-                ent = tr.get(f"{dom}:{prec}:{cfg['workload']}")
-                if ent and ent.get("source_hash") == kernel_hash(dom, prec):
-                    traffic = ent.get("bytes_per_launch")
             roofline = {"kernel": dom, "bound": bound, "achieved": round(achieved, 3),
                         "peak": round(peak, 3), "unit": u, "frac": round(achieved / peak, 4),
-                        "traffic": traffic, "peak_source": peak_src,
+                        "peak_source": peak_src,
                         "algorithmic_per_launch": amount, "algorithmic_unit": unit}
             # the memory-bound kernels against the measured copy bandwidth, from the same pass
             with open(PEAKS_FILE) as fh:
                 hbm_peak = json.load(fh)["hbm_gbs"]
             hbm = {}
             for kd in ("stencil", "update", "split", "fold", "unfold"):
-                amt, un = algorithmic_cost(probs, kd, low="low_fwd" in kernels)
+                amt, un = algorithmic_cost(probs, kd, low="low_fwd" in kernels, prec=prec)
                 if kd in prof and prof[kd][1] and un == "byte":
                     gbs = amt / (prof[kd][0] / prof[kd][1] / 1e3) / 1e9
                     hbm[kd] = {"achieved_gbs": round(gbs, 1), "frac": round(gbs / hbm_peak, 4),
