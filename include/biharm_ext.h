@@ -42,9 +42,10 @@ typedef enum { EXT_BC_SYMMETRIC = 0, EXT_BC_PERIODIC = 1, EXT_BC_DIRICHLET = 2 }
  * outside (phi > 0).  phi == 0 is an unknown node in both directions. */
 typedef enum { EXT_EXTEND_OUT = 0, EXT_EXTEND_IN = 1 } ext_dir;
 
-/* Arithmetic of the iteration.  In every mode the CG inner products are FP64, the iterate x is
- * updated in FP64 every iteration, and the recursive residual is replaced by the FP64 true
- * residual b - A x whenever it has fallen by replace_factor since the last replacement, at
+/* Arithmetic of the iteration.  In every mode the CG scalars are FP64, the vectors and the iterate x
+ * double-float (inner products in compensated FP32 within a warp, FP64 across warps and blocks;
+ * FP32 mode's r.z and z.q as good as FP64 throughout), and the recursive residual is replaced by the FP64
+ * true residual b - A x whenever it has fallen by replace_factor since the last replacement, at
  * least every true_res_every iterations, and before convergence is declared.
  *   FP32        : double-float vectors (pairs of FP32), compensated stencil, transforms on the tcgen05
  *                 tensor cores with every operand as six exact 8-bit integer slices per 128-wide
@@ -149,7 +150,8 @@ typedef struct {
   int32_t status;      /* EXT_OK, EXT_ENOTCONV, EXT_EBREAKDOWN, ...                            */
   int32_t iters;       /* CG iterations taken                                                  */
   double relres_true;  /* FP64 ||b - A x|| / ||b|| of the returned x, recomputed on the GPU     */
-  double relres_rec;   /* the recursively updated residual at exit                            */
+  double relres_rec;   /* the recursively updated residual at exit (2-D solves end with it
+                          replaced: relres_true)                                              */
   int32_t n_unknown;   /* |D \ Omega|                                                          */
   int32_t n_known;     /* |Omega|                                                              */
   double ms_queue;     /* serving: submit -> admission                                         */
@@ -181,8 +183,8 @@ typedef struct ext_ctx ext_ctx;
 void ext_options_default(ext_options* opt);
 
 /* Create a context bound to the current CUDA device and to cuda_stream (a cudaStream_t; NULL =
- * a stream the context creates).  opt may be NULL (defaults).  Returns EXT_ENOTSUP when the
- * mixed modes are requested on a device without tcgen05 (compute capability 10.x). */
+ * a stream the context creates).  opt may be NULL (defaults).  Returns EXT_ENOTSUP on a device without
+ * tcgen05 (compute capability 10.x): every mode's transforms run there. */
 int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out);
 
 /* One extension (Sec. 2.1 problem, Algorithm 1 solve): out = f at known nodes (bit copy),
@@ -282,8 +284,9 @@ int ext_axis_basis(int32_t n, ext_bc bc, double* Q, double* lam);
  * known nodes (bit copy), the extension elsewhere; out may alias f.  res (may be NULL) receives
  * status, iterations, the true and recursive relative residuals, counts and err_est.  Returns
  * EXT_OK, EXT_EINVAL (sizes, spacings, enums, NaN phi, a non-finite known value, host pointers),
- * EXT_ENOKNOWN, EXT_ENOMEM, EXT_ENOTCONV (out holds the last iterate), EXT_EBREAKDOWN or
- * EXT_ECUDA.  Allocates its workspace per call (about 90 bytes per node). */
+ * EXT_ENOKNOWN, EXT_ENOMEM, EXT_ENOTCONV (out holds the last iterate), EXT_EBREAKDOWN,
+ * EXT_ETIMEOUT (out is not written) or EXT_ECUDA.  Allocates its workspace per call (about 80 bytes per
+ * node; on the tensor cores 100, with six slices 110). */
 int ext_solve3d(ext_ctx* ctx, const ext_problem3* prob, const float* phi, const float* f, float* out,
                 ext_result* res);
 

@@ -74,7 +74,7 @@ struct PlanDev {
 struct SlotHost {
   ext_problem prob{};
   SlotDesc d{};
-  SlotDesc tcp[kMirClasses]{};  // tensor-core problems (mixed modes): the slot, or its classes
+  SlotDesc tcp[kMirClasses]{};  // transform problems: the slot, or its classes
   int n_tcp = 0;
   char* arena = nullptr;
   size_t bytes = 0;
@@ -109,7 +109,7 @@ struct Workspace {
   bool fuse = false;            // scalar steps inside the update and stencil (few slots)
   WorkItem *d_l1 = nullptr, *d_l2 = nullptr, *d_l3 = nullptr;  // low-mode forward, middle, inverse
   int n_l1 = 0, n_l2 = 0, n_l3 = 0;
-  // tensor-core problems (mixed modes): kMirClasses entries per slot, the slot's own descriptor
+  // transform problems: kMirClasses entries per slot, the slot's own descriptor
   // or its mirror classes; items of the fold and unfold kernels and of the slicing update
   SlotDesc* d_tcp = nullptr;
   WorkItem *d_fold = nullptr, *d_unfold = nullptr, *d_upd = nullptr;
@@ -130,7 +130,6 @@ struct Workspace {
     std::vector<Ev> events;  // profiling: event-record nodes of the graph
   };
   std::map<int, Graph> graphs;
-  void* d_tmaps = nullptr;      // per slot 8 CUtensorMap (tensor-core modes)
   bool aniso = false;
   bool host_io = false;
   cudaStream_t stream = nullptr;  // the context's stream, or the serving worker's own

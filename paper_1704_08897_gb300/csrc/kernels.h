@@ -14,7 +14,7 @@ namespace bx {
 
 struct LaunchCfg {
   const SlotDesc* slots;   // device array of slot descriptors
-  const SlotDesc* tcp = nullptr;  // tensor-core problems (kMirClasses per slot), mixed modes
+  const SlotDesc* tcp = nullptr;  // transform problems (kMirClasses per slot)
   const WorkItem* items;   // device work list
   const int* n_items;      // device count of valid items (persistent kernels read it)
   int grid;
@@ -103,7 +103,7 @@ void launch_unfold(const LaunchCfg& c, int mode);
 int tc_block();
 bool tc_supported();
 
-// Tensor-core preconditioner of the 3-D path (mixed modes, every side a multiple of 128): the
+// Tensor-core preconditioner of the 3-D path (boxes whose sides are multiples of 128, in every mode): the
 // residual slicing and the six transform products as launches of the 2-D kernels over prepared
 // descriptors (one per launch, [0] = slicing, [1..6] = products), built by the context.
 struct Tc3 {
