@@ -1609,7 +1609,6 @@ int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out) {
   BX_CUDA(tc_init());
   BX_CUDA(stencil_init());
   BX_CUDA(cudaMalloc(&ctx->d_err, sizeof(int)));
-  BX_CUDA(cudaMemset(ctx->d_err, 0, sizeof(int)));
   BX_CUDA(cudaMallocHost(&ctx->h_err, 5 * sizeof(int)));
   for (cudaEvent_t& e : ctx->blk_ev) BX_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   std::fill(ctx->h_err, ctx->h_err + 5, 0);
@@ -1620,8 +1619,9 @@ int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out) {
     BX_CUDA(cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking));
     ctx->own_stream = true;
   }
-  const int rc = set_up_done();
-  if (rc) return rc;
+  // on the context's stream, in order with all that reads it (the serving worker's stream waits for it
+  // in serve_init): nothing here waits for work of the caller's
+  BX_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
   *out = ctx.release();
   return EXT_OK;
 }
@@ -2262,11 +2262,11 @@ static int serve_init(ext_ctx* ctx) {
   BX_CUDA(cudaMalloc(&W->d_slots, sizeof(SlotDesc) * cap));
   BX_CUDA(cudaMalloc(&W->d_tcp, sizeof(SlotDesc) * kMirClasses * cap));
   BX_CUDA(cudaMalloc(&W->d_sc, sizeof(SlotScalars) * cap));
-  BX_CUDA(cudaMemset(W->d_sc, 0, sizeof(SlotScalars) * cap));
+  BX_CUDA(cudaMemsetAsync(W->d_sc, 0, sizeof(SlotScalars) * cap, W->stream));
   BX_CUDA(cudaMallocHost(&W->h_sc, sizeof(SlotScalars) * cap));
   memset(W->h_sc, 0, sizeof(SlotScalars) * cap);
   BX_CUDA(cudaMalloc(&W->d_counts, 13 * sizeof(int)));
-  BX_CUDA(cudaMemset(W->d_counts, 0, 13 * sizeof(int)));
+  BX_CUDA(cudaMemsetAsync(W->d_counts, 0, 13 * sizeof(int), W->stream));
   BX_CUDA(cudaMalloc(&W->d_sl, sizeof(WorkItem) * cap));
   W->n_sl = cap;  // the per-slot grid is sized for the slot table
   BX_CUDA(cudaMalloc(&W->d_phis, sizeof(void*) * cap));
@@ -2276,8 +2276,10 @@ static int serve_init(ext_ctx* ctx) {
   BX_CUDA(cudaMallocHost(&W->h_ptrs, (3 * sizeof(void*) + sizeof(int)) * cap));
   BX_CUDA(cudaMalloc(&S->d_aux, 2 * sizeof(int)));
   BX_CUDA(cudaMallocHost(&S->h_aux, 2 * sizeof(int)));
+  // the time-out flag's first value, set on the context's stream (no solve is under way here)
+  BX_CUDA(cudaEventRecord(ctx->blk_ev[0], ctx->stream));
+  BX_CUDA(cudaStreamWaitEvent(W->stream, ctx->blk_ev[0], 0));
   int rc = serve_alloc_lists(S.get(), 1 << 16);
-  if (!rc) rc = set_up_done();
   if (rc) return rc;
   size_t fr = 0, tot = 0;
   BX_CUDA(cudaMemGetInfo(&fr, &tot));

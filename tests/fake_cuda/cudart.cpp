@@ -28,6 +28,7 @@ std::map<char*, size_t> live;
 std::map<const void*, std::string> kernels;
 std::vector<std::string> faults;
 int pending = 0;         // legacy-stream operations that may be in flight
+int legacy_waits = 0;    // how often the host waited for the legacy stream, and so for the caller's work on it
 long mallocs = 0, fail_malloc = -1;
 std::string trace;       // names of the kernels launched, one per line
 
@@ -106,6 +107,7 @@ void fake_fail_malloc(long n) {
   fail_malloc = n < 0 ? -1 : mallocs + n;
 }
 long fake_mallocs() { return mallocs; }
+int fake_legacy_waits() { return legacy_waits; }
 size_t fake_live_bytes() {
   Lock l(mu);
   size_t b = 0;
@@ -262,7 +264,10 @@ cudaError_t cudaStreamDestroy(cudaStream_t s) {
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
   Lock l(mu);
-  if (legacy(s)) pending = 0;
+  if (legacy(s)) {
+    pending = 0;
+    ++legacy_waits;
+  }
   return cudaSuccess;
 }
 cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode) {
@@ -317,6 +322,7 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) {
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventRecordWithFlags(cudaEvent_t, cudaStream_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) {
   *ms = 1.f;
   return cudaSuccess;

@@ -342,3 +342,14 @@ ext.ext_destroy(c)
 if fake.fake_events() != before: print(fake.fake_events() - before, "events left")
 """)
     assert out.strip() == ""
+
+
+def test_creating_a_context_waits_for_no_work_of_the_caller(fake_cuda):
+    """The caller's default stream may be busy with the inputs of the next call."""
+    out = fake_cuda("""
+before = fake.fake_legacy_waits()
+c = ext.ext_create(ext.options("mixed_bf16"))
+if fake.fake_legacy_waits() != before: print(fake.fake_legacy_waits() - before)
+print(faults())
+""")
+    assert out.strip() == ""
