@@ -201,14 +201,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// One warp: the sum of the eight warps' values sh[0..7] of a block of 256 threads, in every lane.
-__device__ __forceinline__ double sum_of_eight(const double* sh) {
-  double v = sh[threadIdx.x & 7];
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Block sum of up to two values; result valid in thread 0.  `sh` holds >= 2*32 doubles.
 template <int NT>
 __device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
@@ -394,6 +386,18 @@ struct Sum3 {
     return (double)s + (THIRD ? (double)c + (double)d : (double)c);
   }
 };
+// The sum over W warps of one Sum3 each (the same in all its lanes): FP64 for the result only (the SM adds
+// two FP64 numbers a cycle).  Result valid in the first warp.
+template <int W>
+__device__ __forceinline__ double across_warps(Sum3 v, float (&sh)[3][W]) {
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  if (l == 0) sh[0][w] = v.s, sh[1][w] = v.c, sh[2][w] = v.d;
+  __syncthreads();
+  if (w != 0) return 0.0;
+  v = Sum3(sh[0][l % W], sh[1][l % W], sh[2][l % W]);
+  v.reduce<W>();
+  return v.value();
+}
 // The preconditioner's dot products over W lanes: as good as FP64 sums in FP32 mode (DOTS3), in pairs in the
 // mixed modes (as one form for both, 1 us of 60 an iteration slower: more registers in the unfold).
 template <int W, bool DOTS3>

@@ -324,9 +324,11 @@ k_stage_setup(const SlotDesc* __restrict__ slots, const float* __restrict__ phi,
 //
 // The p.q partials do not depend on TY: they are per 64 x 16 block (a tile holds TY / 16 of
 // them), each thread adds its nodes of a block in step order (the steps cover the block's rows
-// in the same order for either TY), the warp adds its lanes in a fixed butterfly and one thread
-// the eight warps in order; k_pq_finish adds the blocks in index order, so every tile height
-// gives the same bits.
+// in the same order for either TY), the warp adds its lanes in a fixed butterfly and the producer
+// warp the eight warps in FP64 while the next tile is computed (added by a computing warp, the FP64 chain
+// held up each tile: 281 us an operator call on 4096^2 nodes, 277 now), but for a block's last tile, whose
+// sum the computing warps have sooner (1 us an iteration of 60 at 389 x 251); k_pq_finish adds the
+// blocks in index order, so every tile height gives the same bits.
 // ---------------------------------------------------------------------------------------------
 constexpr int kWX = kStWinX;  // 72: window row, floats
 static_assert(kStWinX == kStTileX + 8, "window columns");
@@ -397,6 +399,7 @@ struct StTile {
   const SlotDesc* S;  // null: the end of the list
   int x0, y0, par, copied;
   float beta_hi, beta_lo;
+  bool last;          // the block's last item: the computing warps add its p.q themselves
 };
 constexpr int kStBlock = kStThreads + 32;  // the computing warps and the producer
 
@@ -415,17 +418,37 @@ __device__ __forceinline__ bool st_bar_or(bool v) {
   return any != 0;
 }
 
+// One warp: p.q of a tile's 16-row blocks (TY / 16 of them, so the partials do not depend on TY), each the FP64
+// sum of eight warps' pairs.
+template <int TY>
+__device__ __forceinline__ void put_pq(const StTile& t, const float2 (&blk)[TY / 16][kStThreads / 32]) {
+  const int lane = threadIdx.x & 31;
+  const int j = (lane >> 3) & (TY / 16 - 1);  // eight lanes per block, one per warp's pair
+  const double v = sum_of_eight(blk[j]);
+  const int by = (t.y0 >> 4) + j;
+  if ((lane & 7) == 0 && lane < TY / 2 && 16 * by < t.S->ny)
+    t.S->pq_part[by * ((t.S->nx + kStTileX - 1) / kStTileX) + t.x0 / kStTileX] = v;
+}
+
 // The producer warp: for each of the block's tiles (those whose slot iterates) it waits for a free
 // window set, starts the tensor copies (lane 0), forms beta (FUSE: from the preconditioner's partials,
-// once per slot) and hands the tile over.  Done by a computing thread between two tiles, these dependent
-// loads, tensor-map fences and copies took 3.5 K of a tile's 11.5 K cycles.
+// once per slot), stores p.q of the tile that the set held before and hands the tile over.  Done by a
+// computing thread between two tiles, these dependent loads, tensor-map fences and copies took 3.5 K of a
+// tile's 11.5 K cycles.
 template <int TY, bool FUSE>
 __device__ __forceinline__ void stencil_producer(const SlotDesc* __restrict__ slots,
                                                  const WorkItem* __restrict__ items, int total, unsigned char* sbuf,
                                                  uint64_t* full, uint64_t* empty, StTile* info,
+                                                 const float2 (*blk_sm)[TY / 16][kStThreads / 32],
                                                  volatile int* abort_flag, long long wait_cycles) {
   using G = StGeom<TY>;
   const int lane = threadIdx.x & 31;
+  // p.q of the tile that set b held, once the computing warps have released it
+  auto flush = [&](int b) {
+    const StTile t = info[b];
+    if (!t.last) put_pq<TY>(t, blk_sm[b]);
+    __syncwarp();  // the set's entry is written again next
+  };
   int n = 0, slot = -1;
   f2 beta = {0.f, 0.f};
   auto acquire = [&](const SlotDesc& S) {
@@ -484,17 +507,32 @@ __device__ __forceinline__ void stencil_producer(const SlotDesc* __restrict__ sl
         beta = f2{sc->beta_f[0], sc->beta_f[1]};
       }
     }
+    __syncwarp();  // every lane behind the wait for the set
+    if (n >= 2) flush(b);
     if (lane == 0) {
-      info[b] = StTile{&S, x0, y0, par, maps != nullptr, beta.hi, beta.lo};
+      info[b] = StTile{&S, x0, y0, par, maps != nullptr, beta.hi, beta.lo, w + static_cast<int>(gridDim.x) >= total};
       mbar_arrive(&full[b]);
     }
     ++n;
   }
+  // the end of the list, and p.q of the last two tiles
+  auto released = [&](int k) {  // tile k's set, by the computing warps
+    bool r = true;
+    if (lane == 0) r = mbar_wait(&empty[k & 1], (k >> 1) & 1, abort_flag, wait_cycles);
+    r = __shfl_sync(0xffffffffu, r, 0);
+    __syncwarp();
+    return r;
+  };
+  if (ok && n >= 2) {
+    ok = released(n - 2);
+    if (ok) flush(n & 1);
+  }
+  if (ok && lane == 0) {
+    info[n & 1].S = nullptr;
+    mbar_arrive(&full[n & 1]);
+  }
+  if (ok && n >= 1 && released(n - 1)) flush((n - 1) & 1);
   if (lane == 0) {
-    if (ok && mbar_wait(&empty[n & 1], ((n >> 1) & 1) ^ 1, abort_flag, wait_cycles)) {
-      info[n & 1].S = nullptr;
-      mbar_arrive(&full[n & 1]);
-    }
     // after an abort: the copies already issued (the last into each set) land before the block's
     // memory is released
     if (*abort_flag) {
@@ -531,7 +569,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   __shared__ __align__(8) uint64_t full[2], empty[2];
   __shared__ StTile info[2];
   __shared__ int s_abort;
-  __shared__ float2 blk_sm[TY / 16][kStThreads / 32];  // p.q of each warp in each 16-row block
+  __shared__ float2 blk_sm[2][TY / 16][kStThreads / 32];  // p.q of each warp in each 16-row block, by window set
   const int total = *n_items;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
@@ -546,7 +584,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   __syncthreads();
   volatile int* abort_flag = &s_abort;
   if (warp == kStThreads / 32) {
-    stencil_producer<TY, FUSE>(slots, items, total, sbuf, full, empty, info, abort_flag, wait_cycles);
+    stencil_producer<TY, FUSE>(slots, items, total, sbuf, full, empty, info, blk_sm, abort_flag, wait_cycles);
   } else {
   pdl_wait();
   for (int n = 0;; ++n) {
@@ -668,9 +706,8 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     const uint8_t* mt = buf + 4 * G::kWinBytes;
     float* __restrict__ qh = S.q;
     float* __restrict__ ql = S.q_lo;
-    const int nbx = (S.nx + kStTileX - 1) / kStTileX;  // 64-node blocks per grid row
     // p.q of the tile's 64 x 16 blocks: each thread sums its nodes of one block in step order, the
-    // warp its lanes in a fixed butterfly, and one thread the eight warps in order
+    // warp its lanes in a fixed butterfly, and the producer the eight warps
     CompDotDF dot;
     if (!ANISO) {
       float* sh = reinterpret_cast<float*>(buf + 2 * G::kWinBytes);  // g(p), in place of p_old
@@ -726,7 +763,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         }
         // the end of a 16-row block: every lane joins the butterfly
         group_sum_pair<32>(dot.s, dot.c);
-        if (lane == 0) blk_sm[j][warp] = make_float2(dot.s, dot.c);
+        if (lane == 0) blk_sm[b][j][warp] = make_float2(dot.s, dot.c);
         dot = CompDotDF{};
       }
     } else {
@@ -754,21 +791,15 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
         }
         if ((j & 3) == 3) {
           group_sum_pair<32>(dot.s, dot.c);
-          if (lane == 0) blk_sm[j >> 2][threadIdx.x >> 5] = make_float2(dot.s, dot.c);
+          if (lane == 0) blk_sm[b][j >> 2][warp] = make_float2(dot.s, dot.c);
           dot = CompDotDF{};
         }
       }
     }
     st_bar();
-    if (threadIdx.x == 0) mbar_arrive(&empty[b]);  // the window set and the tile's entry are free
-    // the 16-row blocks of the tile (TY / 16 of them, so the partials do not depend on TY); the
-    // next tile writes blk_sm only after its own block barriers, which these threads join later
-    if (threadIdx.x < 32) {
-      const int j = (lane >> 3) & (TY / 16 - 1);  // eight lanes per block, one per warp's pair
-      const double v = sum_of_eight(blk_sm[j]);
-      const int by = (y0 >> 4) + j;
-      if ((lane & 7) == 0 && lane < TY / 2 && 16 * by < S.ny) S.pq_part[by * nbx + x0 / kStTileX] = v;
-    }
+    // the window set, the tile's entry and its sums go back to the producer, which adds up the sums
+    if (threadIdx.x == 0) mbar_arrive(&empty[b]);
+    if (tile.last && warp == 0) put_pq<TY>(tile, blk_sm[b]);
   }
   }
   __syncthreads();
@@ -1077,7 +1108,9 @@ k_apply(const __grid_constant__ SlotDesc S, const float* __restrict__ phi, int e
   constexpr int TY = kApplyTileY;
   __shared__ __align__(16) float win[kWX * (TY + 4)];  // rows y0-2 .., columns x0-4 ..
   __shared__ __align__(16) float lap[ANISO ? 1 : 2][ANISO ? 4 : kWX * (TY + 4)];  // g(p), hi and lo
-  __shared__ double red[kStThreads / 32];
+  __shared__ float red[3][kStThreads / 32];  // the warps' sums as Sum3 ...
+  __shared__ double red_wide[kStThreads / 32];  // ... or, where `wide`, in FP64
+  __shared__ bool wide[kStThreads / 32];
   const int ntx = (S.nx + kStTileX - 1) / kStTileX;
   const int tile = blockIdx.x;
   const int x0 = (tile % ntx) * kStTileX, y0 = (tile / ntx) * TY;
@@ -1141,26 +1174,35 @@ k_apply(const __grid_constant__ SlotDesc S, const float* __restrict__ phi, int e
     const float m = fabsf(__fmul_rn(pv[i], qv[i]));
     plain = plain && ((m > 0x1p-90f && m < 0x1p100f) || (m == 0.f && (pv[i] == 0.f || qv[i] == 0.f)));
   }
-  double t = 0.0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (__all_sync(0xffffffffu, plain)) {
     Sum3 sum;
 #pragma unroll
     for (int i = 0; i < 2 * kOwn; ++i) sum.add_prod(pv[i], qv[i]);
     sum.reduce<32>();
-    t = sum.value();
+    if (lane == 0) {
+      red[0][warp] = sum.s, red[1][warp] = sum.c, red[2][warp] = sum.d;
+      wide[warp] = false;
+    }
   } else {
+    double t = 0.0;
 #pragma unroll
     for (int i = 0; i < 2 * kOwn; ++i) t += (double)pv[i] * (double)qv[i];
     t = warp_sum(t);
+    if (lane == 0) {
+      red_wide[warp] = t;
+      wide[warp] = true;
+    }
   }
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    t = sum_of_eight(red);
-    if (threadIdx.x == 0) part[tile] = t;
+  if (warp == 0) {
+    const int w = lane & 7;
+    double t = wide[w] ? red_wide[w] : Sum3(red[0][w], red[1][w], red[2][w]).value();
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) part[tile] = t;
   }
 }
-
 
 // ---------------------------------------------------------------------------------------------
 // Launchers

@@ -363,7 +363,7 @@ k3_init(size_t n, const double* __restrict__ b, double s, float* __restrict__ rh
 __global__ void __launch_bounds__(kT, 4)
 k3_update(size_t n, const SlotScalars* sc, const float* ph, const float* pl, const float* qh,
           const float* ql, float* xh, float* xl, float* rh, float* rl, double* __restrict__ part) {
-  __shared__ double sh[kT / 32];
+  __shared__ float sh[3][kT / 32];
   if (gate_shut(&sc->active)) return;
   const f2 alpha{sc->alpha_f[0], sc->alpha_f[1]}, na{-alpha.hi, -alpha.lo};
   CompDotDF rr;
@@ -398,12 +398,8 @@ k3_update(size_t n, const SlotScalars* sc, const float* ph, const float* pl, con
     }
   Sum3 v(rr.s, rr.c);
   v.reduce<32>();
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v.value();
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const double s = sum_of_eight(sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
-  }
+  const double s = across_warps<kT / 32>(v, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
 // p = z + beta p (double-float)
@@ -517,7 +513,7 @@ __global__ void __launch_bounds__(kGt)
 k3_gemm(Gemm3 g, const int* __restrict__ gate) {
   __shared__ __align__(16) float As[2][2][GK][GM + 1];  // [buffer][hi, lo][k][m]
   __shared__ __align__(16) float Bs[2][2][GK][GN + 4];
-  __shared__ double sh[kGt / 32];
+  __shared__ float sh[3][kGt / 32];
   if (gate_shut(gate)) return;
   const float* Bl = g.B + static_cast<size_t>(g.ldb) * g.ldb;
   const int m0 = blockIdx.x * GM, n0 = blockIdx.y * GN;
@@ -595,10 +591,8 @@ k3_gemm(Gemm3 g, const int* __restrict__ gate) {
   if (FORM == 2) {
     Sum3 v(dot.s, dot.c);
     v.reduce<32>();
-    if ((t & 31) == 0) sh[t >> 5] = v.value();
-    __syncthreads();
-    static_assert(kGt == 128, "four warps");
-    if (t == 0) g.part[blockIdx.y * gridDim.x + blockIdx.x] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
+    const double s = across_warps<kGt / 32>(v, sh);
+    if (t == 0) g.part[blockIdx.y * gridDim.x + blockIdx.x] = s;
   }
 }
 
