@@ -326,7 +326,7 @@ k_stage_setup(const SlotDesc* __restrict__ slots, const float* __restrict__ phi,
 // them), each thread adds its nodes of a block in step order (the steps cover the block's rows
 // in the same order for either TY), the warp adds its lanes in a fixed butterfly and the producer
 // warp the eight warps in FP64 while the next tile is computed (added by a computing warp, the FP64 chain
-// held up each tile: 281 us an operator call on 4096^2 nodes, 277 now), but for a block's last tile, whose
+// held up each tile: 288 us an operator call on 4096^2 nodes, 277 now), but for a block's last tile, whose
 // sum the computing warps have sooner (1 us an iteration of 60 at 389 x 251); k_pq_finish adds the
 // blocks in index order, so every tile height gives the same bits.
 // ---------------------------------------------------------------------------------------------
@@ -450,6 +450,7 @@ __device__ __forceinline__ void stencil_producer(const SlotDesc* __restrict__ sl
     __syncwarp();  // the set's entry is written again next
   };
   int n = 0, slot = -1;
+  bool last = true;  // of the tile handed over last
   f2 beta = {0.f, 0.f};
   auto acquire = [&](const SlotDesc& S) {
     if (lane < kStMaps && S.st_maps != nullptr)
@@ -509,8 +510,9 @@ __device__ __forceinline__ void stencil_producer(const SlotDesc* __restrict__ sl
     }
     __syncwarp();  // every lane behind the wait for the set
     if (n >= 2) flush(b);
+    last = w + static_cast<int>(gridDim.x) >= total;
     if (lane == 0) {
-      info[b] = StTile{&S, x0, y0, par, maps != nullptr, beta.hi, beta.lo, w + static_cast<int>(gridDim.x) >= total};
+      info[b] = StTile{&S, x0, y0, par, maps != nullptr, beta.hi, beta.lo, last};
       mbar_arrive(&full[b]);
     }
     ++n;
@@ -531,7 +533,7 @@ __device__ __forceinline__ void stencil_producer(const SlotDesc* __restrict__ sl
     info[n & 1].S = nullptr;
     mbar_arrive(&full[n & 1]);
   }
-  if (ok && n >= 1 && released(n - 1)) flush((n - 1) & 1);
+  if (ok && !last && released(n - 1)) flush((n - 1) & 1);
   if (lane == 0) {
     // after an abort: the copies already issued (the last into each set) land before the block's
     // memory is released
