@@ -156,8 +156,9 @@ struct ext_ctx {
   int ns = 4;         // integer slices per transform operand: 6 in FP32 mode; 4 in mixed modes, where
                       // build_slot may give a grid 6
   int split = 0;      // their type: 0 = FP16, 1 = BF16
-  int* d_err = nullptr;   // device flag raised by a bounded wait that ran out
-  int* h_err = nullptr;   // pinned copies: two of a solve, two of a 3-D solve, the serving worker's
+  // raised by a kernel whose bounded wait ran out: in pinned host memory, so that the host reads it behind
+  // any synchronisation of the stream without a copy (one took 6 us of a preconditioner call)
+  int* err = nullptr;
   cudaEvent_t blk_ev[2] = {nullptr, nullptr};  // the ends of a solve's blocks of iterations
   SlotScalars* h_sc3 = nullptr;  // pinned, two entries (3-D solves)
   // launch accounting and optional per-kernel timing (ext_options.profile)
@@ -1148,16 +1149,16 @@ static void launch_prec(ext_ctx* ctx, Workspace* W, int mode, bool with_finish =
     // the lowest modes in high precision: forward product, middle, inverse product
     LaunchCfg c1 = cfg_of(ctx, W, 5), cm = cfg_of(ctx, W, 12), c3 = cfg_of(ctx, W, 6);
     c1.slots = cm.slots = c3.slots = W->d_tcp;
-    timed(ctx, EXT_KERNEL_LOW_FWD, [&] { launch_low_tc(c1, 0, mode, ctx->split, ctx->d_err); }, g.stream);
+    timed(ctx, EXT_KERNEL_LOW_FWD, [&] { launch_low_tc(c1, 0, mode, ctx->split, ctx->err); }, g.stream);
     cm.pdl = false;  // see settled(): in a call of few grids too
     timed(ctx, EXT_KERNEL_LOW_MID, [&] { launch_low_mid(cm, mode, ctx->split); }, g.stream);
-    timed(ctx, EXT_KERNEL_LOW_INV, [&] { launch_low_tc(c3, 1, mode, ctx->split, ctx->d_err); }, g.stream);
+    timed(ctx, EXT_KERNEL_LOW_INV, [&] { launch_low_tc(c3, 1, mode, ctx->split, ctx->err); }, g.stream);
   }
   for (int s = 0; s < 4; ++s) {
     if (W->n_gm[0] > 0)
-      timed(ctx, EXT_KERNEL_PREC0 + s, [&] { launch_prec_tc(g, s, mode, ctx->split, 4, ctx->d_err); }, g.stream);
+      timed(ctx, EXT_KERNEL_PREC0 + s, [&] { launch_prec_tc(g, s, mode, ctx->split, 4, ctx->err); }, g.stream);
     if (W->n_gm[1] > 0)
-      timed(ctx, EXT_KERNEL_PREC0 + s, [&] { launch_prec_tc(g6, s, mode, ctx->split, 6, ctx->d_err); }, g.stream);
+      timed(ctx, EXT_KERNEL_PREC0 + s, [&] { launch_prec_tc(g6, s, mode, ctx->split, 6, ctx->err); }, g.stream);
   }
   if (W->n_unfold > 0)
     timed(ctx, EXT_KERNEL_UNFOLD, [&] { launch_unfold(settled(W, cfg_of(ctx, W, 8)), mode); }, g.stream);
@@ -1174,7 +1175,7 @@ static void enqueue_iterations(ext_ctx* ctx, Workspace* W, int iters) {
   for (int i = 0; i < iters; ++i) {
     // the first stencil follows a pass with its own finish (the tail's, or the first one)
     const bool fz = fuse && i > 0;
-    timed(ctx, EXT_KERNEL_STENCIL, [&] { launch_stencil(sc, W->aniso, W->sten_ty, ctx->d_err, fz); }, st.stream);
+    timed(ctx, EXT_KERNEL_STENCIL, [&] { launch_stencil(sc, W->aniso, W->sten_ty, ctx->err, fz); }, st.stream);
     const LaunchCfg pf = cfg_of(ctx, W, 3);  // one block per slot
     if (!fuse) timed(ctx, EXT_KERNEL_PQ_FINISH, [&] { launch_pq_finish(pf); }, st.stream);
     timed(ctx, EXT_KERNEL_UPDATE, [&] {
@@ -1326,10 +1327,10 @@ static int autotune_stencil(ext_ctx* ctx, Workspace* W) {
       int rc = set_stencil_shape(ctx, W, cand);
       if (rc) return rc;
       const LaunchCfg sc = cfg_of(ctx, W, 4);
-      launch_stencil(sc, W->aniso, cand, ctx->d_err);  // warm
+      launch_stencil(sc, W->aniso, cand, ctx->err);  // warm
       BX_CUDA(cudaEventRecord(e0, s));
       constexpr int kReps = 5;
-      for (int r = 0; r < kReps; ++r) launch_stencil(sc, W->aniso, cand, ctx->d_err);
+      for (int r = 0; r < kReps; ++r) launch_stencil(sc, W->aniso, cand, ctx->err);
       BX_CUDA(cudaEventRecord(e1, s));
       BX_CUDA(cudaEventSynchronize(e1));
       ctx->launches += kReps + 1;
@@ -1363,11 +1364,12 @@ static int map_status(int st, int n_known, const ext_problem& p) {
   return st;
 }
 
+static bool wait_ran_out(const ext_ctx* ctx) { return *static_cast<volatile const int*>(ctx->err) != 0; }
+
 // A bounded wait ran out: the flag goes down once the stream has finished, so the next call starts afresh.
 static int timed_out(ext_ctx* ctx) {
   BX_CUDA(cudaStreamSynchronize(ctx->stream));
-  BX_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
-  BX_CUDA(cudaStreamSynchronize(ctx->stream));
+  *ctx->err = 0;
   g_last_error = "a bounded device wait (tensor copy or tensor-core pipeline) ran out";
   return EXT_ETIMEOUT;
 }
@@ -1450,7 +1452,6 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
       BX_CUDA(cudaGraphLaunch(graph.exec, s));
       ctx->launches += graph.nodes;
       BX_CUDA(cudaMemcpyAsync(W->h_sc + set * count, W->d_sc, sizeof(SlotScalars) * count, cudaMemcpyDeviceToHost, s));
-      BX_CUDA(cudaMemcpyAsync(ctx->h_err + set, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
       BX_CUDA(cudaEventRecord(ctx->blk_ev[set], s));
     }
     if (blk < ahead) continue;
@@ -1461,7 +1462,7 @@ static int run_solve(ext_ctx* ctx, Workspace* W, const float* const* phis, const
       harvest(ctx);
       harvest_graph(ctx, graph.events);
     }
-    if (ctx->h_err[seen]) return timed_out(ctx);
+    if (wait_ran_out(ctx)) return timed_out(ctx);
     end = W->h_sc + seen * count;
     bool running = false;
     for (int i = 0; i < count; ++i)
@@ -1608,10 +1609,9 @@ int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out) {
   ctx->split = o.prec == EXT_PREC_MIXED_FP16 ? 0 : 1;
   BX_CUDA(tc_init());
   BX_CUDA(stencil_init());
-  BX_CUDA(cudaMalloc(&ctx->d_err, sizeof(int)));
-  BX_CUDA(cudaMallocHost(&ctx->h_err, 5 * sizeof(int)));
+  BX_CUDA(cudaMallocHost(&ctx->err, sizeof(int)));
+  *ctx->err = 0;
   for (cudaEvent_t& e : ctx->blk_ev) BX_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  std::fill(ctx->h_err, ctx->h_err + 5, 0);
   BX_CUDA(cudaMallocHost(&ctx->h_sc3, 2 * sizeof(SlotScalars)));
   if (cuda_stream) {
     ctx->stream = (cudaStream_t)cuda_stream;
@@ -1619,9 +1619,6 @@ int ext_create(const ext_options* opt, void* cuda_stream, ext_ctx** out) {
     BX_CUDA(cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking));
     ctx->own_stream = true;
   }
-  // on the context's stream, in order with all that reads it (the serving worker's stream waits for it
-  // in serve_init): nothing here waits for work of the caller's
-  BX_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
   *out = ctx.release();
   return EXT_OK;
 }
@@ -1641,8 +1638,7 @@ void ext_destroy(ext_ctx* ctx) {
     cudaFree(kv.second.low);
   }
   harvest(ctx);
-  cudaFree(ctx->d_err);
-  cudaFreeHost(ctx->h_err);
+  cudaFreeHost(ctx->err);
   for (cudaEvent_t e : ctx->blk_ev)
     if (e) cudaEventDestroy(e);
   cudaFreeHost(ctx->h_sc3);
@@ -1756,7 +1752,6 @@ static int args3(ext_ctx* ctx, const ext_problem3* p, Solve3Args& a) {
   a.stream = ctx->stream;
   a.sm_count = ctx->sm_count;
   a.h_sc = ctx->h_sc3;
-  a.h_err = ctx->h_err + 2;
   if (on_tc)
     a.tc_build = [ctx, &a](const Tc3Io& io, Tc3& t) { return tc3_build(ctx, a, io, t); };
   return EXT_OK;
@@ -1925,7 +1920,7 @@ static int tc3_build(ext_ctx* ctx, const Solve3Args& a, const Tc3Io& io, Tc3& t)
   t.split = ctx->split;
   t.ns = NS;
   t.dots3 = ctx->opt.prec == EXT_PREC_FP32;
-  t.d_err = ctx->d_err;
+  t.err = ctx->err;
   t.wait_cycles = ctx->opt.wait_cycles;
   t.sm_count = ctx->sm_count;
   t.part = part;
@@ -2087,9 +2082,8 @@ static int stage_setup(ext_ctx* ctx, const ext_problem* prob, const float* phi, 
 
 // The end of a single-stage call: EXT_ETIMEOUT, and the flag down again, if a kernel's wait ran out.
 static int stage_done(ext_ctx* ctx) {
-  BX_CUDA(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   BX_CUDA(cudaStreamSynchronize(ctx->stream));
-  return *ctx->h_err ? timed_out(ctx) : EXT_OK;
+  return wait_ran_out(ctx) ? timed_out(ctx) : EXT_OK;
 }
 
 int ext_apply_biharmonic(ext_ctx* ctx, const ext_problem* prob, const float* phi, const float* p,
@@ -2106,7 +2100,7 @@ int ext_apply_biharmonic(ext_ctx* ctx, const ext_problem* prob, const float* phi
   cudaStream_t s = ctx->stream;
   const size_t N = (size_t)prob->nx * prob->ny;
   const LaunchCfg sc = cfg_of(ctx, W, 4);
-  timed(ctx, EXT_KERNEL_STENCIL, [&] { launch_stencil(sc, W->aniso, W->sten_ty, ctx->d_err); });
+  timed(ctx, EXT_KERNEL_STENCIL, [&] { launch_stencil(sc, W->aniso, W->sten_ty, ctx->err); });
   BX_CUDA(cudaGetLastError());
   BX_CUDA(cudaMemcpyAsync(q, sl.d.q, 4 * N, cudaMemcpyDeviceToDevice, s));
   std::vector<double> part((size_t)((prob->ny + 15) / 16) * ((prob->nx + kStTileX - 1) / kStTileX));
@@ -2276,9 +2270,6 @@ static int serve_init(ext_ctx* ctx) {
   BX_CUDA(cudaMallocHost(&W->h_ptrs, (3 * sizeof(void*) + sizeof(int)) * cap));
   BX_CUDA(cudaMalloc(&S->d_aux, 2 * sizeof(int)));
   BX_CUDA(cudaMallocHost(&S->h_aux, 2 * sizeof(int)));
-  // the time-out flag's first value, set on the context's stream (no solve is under way here)
-  BX_CUDA(cudaEventRecord(ctx->blk_ev[0], ctx->stream));
-  BX_CUDA(cudaStreamWaitEvent(W->stream, ctx->blk_ev[0], 0));
   int rc = serve_alloc_lists(S.get(), 1 << 16);
   if (rc) return rc;
   size_t fr = 0, tot = 0;
@@ -2569,10 +2560,9 @@ static void serve_loop(ext_ctx* ctx) {
     if (!rc) {
       const int cap = (int)S->slots.size();
       if (cudaMemcpyAsync(W->h_sc, W->d_sc, sizeof(SlotScalars) * cap, cudaMemcpyDeviceToHost, W->stream) != cudaSuccess ||
-          cudaMemcpyAsync(ctx->h_err + 4, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, W->stream) != cudaSuccess ||
           cudaStreamSynchronize(W->stream) != cudaSuccess)
         rc = EXT_ECUDA;
-      else if (ctx->h_err[4])
+      else if (wait_ran_out(ctx))
         rc = EXT_ETIMEOUT;
     }
     if (!rc) {

@@ -10,6 +10,12 @@
 
 namespace bx {
 
+// Tells the host (err: pinned memory that it reads once the stream has come so far) that a wait ran out.
+__device__ __forceinline__ void raise_flag(int* err) {
+  *reinterpret_cast<volatile int*>(err) = 1;
+  __threadfence_system();
+}
+
 constexpr long long kWaitCycles = 4000000000LL;  // about two seconds at 2 GHz
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

@@ -114,7 +114,7 @@ struct Tc3 {
   int n_items[7] = {};
   int split = 0, ns = 4;
   bool dots3 = false;             // LaunchCfg::dots3
-  int* d_err = nullptr;
+  int* err = nullptr;             // pinned host memory
   long long wait_cycles = 0;
   int sm_count = 148;
   double* part = nullptr;         // the last product's tile partials (4 doubles per tile)
@@ -147,7 +147,6 @@ struct Solve3Args {
   long long* launches;     // incremented by every kernel launch (host counter)
   int sm_count;
   SlotScalars* h_sc;       // pinned, two entries: the scalars as blocks of iterations leave them
-  int* h_err;              // pinned, two entries: the time-out flag with them
   // builds the tensor-core preconditioner for the given vectors (empty: CUDA-core transforms)
   std::function<int(const Tc3Io&, Tc3&)> tc_build;
 };

@@ -934,7 +934,7 @@ k_prec_tc(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols)
                  : "memory");
   }
-  if (threadIdx.x == 0 && ctl->abort_flag) atomicExch(err, 1);
+  if (threadIdx.x == 0 && ctl->abort_flag) raise_flag(err);
 }
 
 // One row of a transform operand: the warp's 128 columns (lane pairs 64 k + 2 lane) under their common

@@ -805,7 +805,7 @@ k_stencil(const SlotDesc* __restrict__ slots, const WorkItem* __restrict__ items
   }
   }
   __syncthreads();
-  if (threadIdx.x == 0 && s_abort) atomicExch(err, 1);
+  if (threadIdx.x == 0 && s_abort) raise_flag(err);
 }
 
 // One block per slot (the slot's tile-0 item of the per-slot list): p.q from the stencil's

@@ -759,7 +759,7 @@ void precondition(const Solve3Args& a, const State3& s, float wnorm, const float
       c.items = t.d_items[k];
       c.n_items = t.d_counts + k;
       c.grid = std::max(1, std::min(t.n_items[k], t.sm_count));
-      launch_prec_tc(c, kForm[k], mode, t.split, t.ns, t.d_err);
+      launch_prec_tc(c, kForm[k], mode, t.split, t.ns, t.err);
     }
     *a.launches += 7;
   } else {
@@ -838,17 +838,12 @@ int setup_mask(const Solve3Args& a, State3& s, const float* phi, const float* f,
 
 constexpr int kBlockIters = 8;  // iterations between two readings of the scalars
 
-// Copies the tensor-core kernels' time-out flag to the host (the CUDA-core kernels have no waits).
-int read_flag(const Solve3Args& a, const State3& s, int* flag, std::string* err) {
-  *flag = 0;
-  if (s.tc.on) BX3(cudaMemcpyAsync(flag, s.tc.d_err, sizeof(int), cudaMemcpyDeviceToHost, a.stream));
-  return EXT_OK;
-}
-// A bounded wait ran out: the flag goes down once the stream has finished, so the next call starts afresh.
+// Whether a wait of the tensor-core kernels ran out (the CUDA-core kernels have none).
+bool wait_ran_out(const State3& s) { return s.tc.on && *static_cast<volatile const int*>(s.tc.err) != 0; }
+// Then the flag goes down once the stream has finished, so the next call starts afresh.
 int timed_out(const Solve3Args& a, const State3& s, std::string* err) {
   BX3(cudaStreamSynchronize(a.stream));
-  BX3(cudaMemsetAsync(s.tc.d_err, 0, sizeof(int), a.stream));
-  BX3(cudaStreamSynchronize(a.stream));
+  *s.tc.err = 0;
   *err = "a bounded device wait (tensor-core pipeline) ran out";
   return EXT_ETIMEOUT;
 }
@@ -941,14 +936,12 @@ int solve3d_run(const Solve3Args& a, const float* phi, const float* f, float* ou
       enqueue_tail(a, G, s, wnorm);
       BX3(cudaGetLastError());
       BX3(cudaMemcpyAsync(&a.h_sc[set], s.sc, sizeof(SlotScalars), cudaMemcpyDeviceToHost, st));
-      rc = read_flag(a, s, &a.h_err[set], err);
-      if (rc) return rc;
       BX3(cudaEventRecord(s.ev[set], st));
     }
     if (blk == 0) continue;
     const int seen = (blk - 1) & 1;
     BX3(cudaEventSynchronize(s.ev[seen]));
-    if (a.h_err[seen]) return timed_out(a, s, err);
+    if (wait_ran_out(s)) return timed_out(a, s, err);
     last = a.h_sc[seen];
     if (last.status != ST_RUNNING) break;
   }
@@ -1012,10 +1005,8 @@ int apply3d_preconditioner(const Solve3Args& a, const float* phi, const float* r
   precondition(a, s, wnorm, rh, rl, s.zh, s.zl, 2);
   BX3(cudaMemcpyAsync(z, s.zh, 4 * s.n, cudaMemcpyDeviceToDevice, a.stream));
   BX3(cudaGetLastError());
-  rc = read_flag(a, s, a.h_err, err);
-  if (rc) return rc;
   BX3(cudaStreamSynchronize(a.stream));
-  if (*a.h_err) return timed_out(a, s, err);
+  if (wait_ran_out(s)) return timed_out(a, s, err);
   // weights are (L^2)^+ scaled by wnorm, times the square of the stencil scaling (max 1/h^2)^-2
   const double m = std::max(1.0 / (a.h[0] * a.h[0]), std::max(1.0 / (a.h[1] * a.h[1]), 1.0 / (a.h[2] * a.h[2])));
   if (scale) *scale = (double)wnorm * m * m;
